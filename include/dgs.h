@@ -224,11 +224,12 @@ int dgs_status(dgs_ctx* ctx, int* device_status);
 int dgs_stats(dgs_ctx* ctx, uint64_t out[4]);
 
 /* Waits for all work in flight and reports how much of the difference vectors the pulls'
- * stream passes had to read: out[0] stage-sized chunks (4096 elements) of whole tiles that
- * the passes covered, out[1] those of them that were actually read.  The library keeps,
- * per 512 elements of every D_q, an upper bound on the magnitudes in it; a chunk whose
- * bounds are all below the selection's lower bound cannot hold a selected entry (Eq. 6a
- * takes the largest magnitudes) and is not read.  The selection stays exact. */
+ * passes had to read: out[0] chunks (4096 elements, fewer where a CTA's share ends) that
+ * the passes covered, out[1] those of them of which some part was actually read.  The
+ * library keeps, per 512 elements of every D_q, an upper bound on the magnitudes in it; a
+ * block that no filed packet has an entry in and whose bound is below the selection's lower
+ * bound cannot hold a selected entry (Eq. 6a takes the largest magnitudes) and is not read.
+ * The selection stays exact. */
 int dgs_pull_read_stats(dgs_ctx* ctx, uint64_t out[2]);
 
 /* prev(worker): the server timestamp at that worker's last pull, -1 before it. */
@@ -243,10 +244,10 @@ enum {
   DGS_KERNEL_FINALIZE_PUSH = 1, /* push, single-pass route: exact k-th key, ordered packet, fix-ups      */
   DGS_KERNEL_TWO_PASS_PUSH = 2, /* push, two-pass route only: histogram of the whole input + bound pick  */
   DGS_KERNEL_SCATTER = 3,       /* apply: theta -= packet, packet filed in the log (or the eager scatter) */
-  DGS_KERNEL_STREAM_PULL = 4,
+  DGS_KERNEL_STREAM_PULL = 4,   /* pull: filed packets folded in and candidates collected in one pass    */
   DGS_KERNEL_FINALIZE_PULL = 5,
   DGS_KERNEL_TWO_PASS_PULL = 6,
-  DGS_KERNEL_CATCH_UP = 7,      /* pull: filed packets folded into the worker's difference vector        */
+  DGS_KERNEL_CATCH_UP = 7,      /* filed packets folded into a difference vector without a selection     */
   DGS_NUM_KERNELS = 8
 };
 

@@ -47,7 +47,7 @@ inline uint64_t align_up(uint64_t x, uint64_t a) { return (x + a - 1) / a * a; }
 
 // Scratch of one selection pipeline ([0] push, on the worker stream; [1] pull, on the server stream)
 struct ScratchLayout {
-  uint64_t cand_idx, cand_val, part_cands, part_slot0, plan, part_live, cta_tot, seg_start;
+  uint64_t cand_idx, cand_val, part_cands, part_slot0, plan, cta_cost, cta_tot, seg_start;
   uint64_t hist1, hist2, hist3, sel, L_safe, L_wide, sync;
   uint64_t zero_begin, zero_end;  // [hist1, end of sync): cleared at init
 };
@@ -60,14 +60,14 @@ struct Layout {
   uint64_t theta, u, D, theta_local, grad_stage;
   uint64_t pkt_idx[kPushSlots + kPullSlots], pkt_val[kPushSlots + kPullSlots];  // push slots, then pull slots
   uint64_t var_idx[kVarSlots], var_val[kVarSlots], var_count[kVarSlots], L_one;
-  uint64_t tiles, segs, seg_off, seg_tile0;
+  uint64_t tiles, segs, seg_off, seg_tile0, blk_seg;
   ScratchLayout sc[kAllSets];  // push sets, then pull sets
   uint64_t L_next, u_slots, status, stats;
-  uint64_t log_idx, log_val, log_bnd, log_pos;
-  uint32_t log_ranges = 0;
+  uint64_t log_ent, log_pos;
   uint64_t blk_max;      // [N][blk_stride]: per block of kWarpTile elements, an upper bound on the keys of D_q in it
   uint64_t blk_stride = 0;  // ring of applied packets not yet folded into every D_q
-  uint32_t log_ring = 0, log_stride = 0;
+  uint32_t log_ring = 0, log_stride = 0, pos_rows = 0;
+  uint32_t num_blocks = 0;
   uint64_t total = 0;
 };
 
@@ -136,6 +136,7 @@ void make_layout(const dgs_config* c, Layout* L) {
   const uint64_t N = c->num_workers, S = c->num_segments;
   L->n_pad = align_up(c->n, kAlign / 4);
   L->num_tiles = count_tiles(c);
+  L->num_blocks = (uint32_t)((c->n + kWarpTile - 1) / kWarpTile);
   L->K[0] = L->K[1] = 0;
   for (uint32_t s = 0; s < S; ++s) {
     L->K[0] += c->segments[s].k_push;
@@ -168,14 +169,15 @@ void make_layout(const dgs_config* c, Layout* L) {
   L->segs = take(S * sizeof(SegDesc));
   L->seg_off = take((S + 1) * 4);
   L->seg_tile0 = take(S * 4);
+  L->blk_seg = take((uint64_t)L->num_blocks * 4);
   for (int k = 0; k < kAllSets; ++k) {
     ScratchLayout& sc = L->sc[k];
     sc.cand_idx = take(vec);
     sc.cand_val = take(vec);
-    sc.part_cands = take((uint64_t)kMaxGrid * 4);
-    sc.part_slot0 = take((uint64_t)kMaxGrid * 4);
-    sc.plan = take((uint64_t)(kMaxGrid + 1) * 4);
-    sc.part_live = take((uint64_t)kMaxGrid * 4);
+    sc.part_cands = take((uint64_t)kMaxParts * 4);
+    sc.part_slot0 = take((uint64_t)kMaxParts * 4);
+    sc.plan = take((uint64_t)(kMaxFoldGrid + 1) * 4);
+    sc.cta_cost = take((uint64_t)kMaxFoldGrid * 4);
     sc.cta_tot = take((uint64_t)kMaxWorkers * sizeof(uint2));
     sc.seg_start = take(S * sizeof(uint2));
     sc.hist1 = take(S * kBins1 * 4);
@@ -196,17 +198,9 @@ void make_layout(const dgs_config* c, Layout* L) {
   // stream, in the way of every later event: four rounds of room where that many packets fit the cap)
   L->log_ring = (uint32_t)std::min<uint64_t>(kLogRingMax, std::max<uint64_t>(std::max<uint64_t>(N + kLogSlack, 4 * N), 16));
   L->log_stride = (uint32_t)align_up(L->K[0], 64);
-  L->log_idx = take((uint64_t)L->log_ring * L->log_stride * 4);
-  L->log_val = take((uint64_t)L->log_ring * L->log_stride * 4);
-  {
-    // ranges of the log = CTAs of a catch-up: about kCatchTarget entries each when a worker has missed
-    // as many packets as there are workers, and no more ranges than a packet has entries
-    const uint64_t entries = std::min<uint64_t>(N, L->log_ring) * L->K[0];
-    L->log_ranges = (uint32_t)std::min<uint64_t>(std::min<uint64_t>(kCatchMaxGrid, L->K[0]),
-                                                 std::max<uint64_t>(1, (entries + kCatchTarget - 1) / kCatchTarget));
-  }
-  L->log_bnd = take((uint64_t)L->log_ranges * 4 * 2);   // two generations of ranges, see apply_impl
-  L->log_pos = take((uint64_t)L->log_ring * (L->log_ranges + 1) * 4);
+  L->log_ent = take((uint64_t)L->log_ring * L->log_stride * sizeof(uint2));
+  L->pos_rows = (uint32_t)align_up(L->num_blocks, kBlockGroup) + 1;
+  L->log_pos = take((uint64_t)L->log_ring * L->pos_rows * 4);
   L->blk_stride = align_up((c->n + kWarpTile - 1) / kWarpTile, 64);
   L->blk_max = take(N * L->blk_stride * 4);
   L->L_next = take(2 * N * S * 4);
@@ -251,24 +245,16 @@ struct dgs_ctx {
   // p % ring of the log from its apply on; applied[q] packets have been folded into D_q so far.
   PacketLog log;
   uint64_t log_head;              // packets filed so far
-  uint64_t last_ranges;           // packet number at which the current generation of ranges was taken
-  int cur_gen;                    // generation of ranges that new packets are filed under
-  int64_t gen_last[2];            // newest packet filed under each generation, -1 if none
-  std::vector<uint8_t> slot_gen;  // per slot of the ring: generation its packet was filed under
   std::vector<uint64_t> applied;  // per worker
   Workspace ws[kAllSets];  // push sets, then pull sets
   float inv_m;
   int sms;               // SMs of the device
-  // Which form of the pull's stream pass to launch.  The ring-less form wins when a pull reads a small part
-  // of D_w (it holds almost no shared memory beside the push passes), the staged form when it reads most of
-  // it.  The kernels count the chunks they cover and read; after every pull those two counters are copied
-  // to pinned host memory on the pull's stream, and the host looks at whatever has arrived so far (never
-  // waiting): a stale figure only means a less suitable form, the results are the same either way.
-  bool multi_worker;
-  unsigned long long* h_chunks;      // pinned: [0] chunks covered, [1] chunks read, as of some recent pull
-  unsigned long long seen_chunks[2]; // the figures at the last decision
-  bool light_now;
   int stream_grid[3];    // CTAs of the stand-alone stream pass, per mode
+  int fold_grid;         // CTAs of k_fold
+  uint32_t fold_ahead;   // entries of a block it fetches ahead
+  // No pull has been enqueued since the caller's stream was last made to wait for everything (dgs_flush, or a call
+  // that waits): the event in hand starts on an idle GPU.
+  bool alone;
   int hist_grid[3];      // CTAs of the whole-input histogram pass, per mode
   int finalize_grid[3];  // CTAs of the cooperative finalize kernel, per mode
   int finalize_max[3];   // most CTAs of it that can be resident at once
@@ -323,8 +309,7 @@ struct ResIds {
   uint32_t VPKT(int slot) const { return PKT(kPushSlots + kPullSlots) + (uint32_t)slot; }
   uint32_t STAGE() const { return VPKT(kVarSlots); }
   uint32_t LOG(uint32_t slot) const { return STAGE() + 1 + slot; }
-  uint32_t RANGES(int gen) const { return LOG(kLogRingMax) + (uint32_t)gen; }   // the two generations of ranges of the log
-  uint32_t count() const { return RANGES(1) + 1; }
+  uint32_t count() const { return LOG(kLogRingMax); }
 };
 
 #define DGS_CUDA(ctx, call)                 \
@@ -390,6 +375,7 @@ int fork_from_user(dgs_ctx* c, int which) {
 int sync_all(dgs_ctx* c) {
   for (int i = 0; i < kNumStreams; ++i) DGS_CUDA(c, cudaStreamSynchronize(c->st[i]));
   DGS_CUDA(c, cudaStreamSynchronize(c->user));
+  c->alone = true;
   return DGS_OK;
 }
 
@@ -440,37 +426,21 @@ int task_end(dgs_ctx* c, const Task& t) {
 // Dependencies of folding the filed packets that D_q has not seen yet into it.
 void catch_up_deps(const dgs_ctx* c, uint32_t q, Task* t) {
   const ResIds R{c->cfg.num_workers};
-  bool gen_used[2] = {false, false};
-  for (uint64_t p = c->applied[q]; p < c->log_head; ++p) {
-    t->reads.push_back(R.LOG((uint32_t)(p % c->log.ring)));
-    gen_used[c->slot_gen[p % c->log.ring]] = true;
-  }
-  for (int g = 0; g < 2; ++g)
-    if (gen_used[g]) t->reads.push_back(R.RANGES(g));
+  for (uint64_t p = c->applied[q]; p < c->log_head; ++p) t->reads.push_back(R.LOG((uint32_t)(p % c->log.ring)));
   t->writes.push_back(R.D(q));
 }
-// The launch itself, on a stream that task_begin has prepared with those dependencies.
-int catch_up_launch(dgs_ctx* c, uint32_t q, cudaStream_t st) {
-  uint64_t first = c->applied[q];
-  // The packets still to be folded in were filed under at most two generations of ranges, the older
-  // ones first: one launch per generation and per kCatchMaxPackets packets, in that order (the order of
-  // the subtractions is kept).
-  while (first < c->log_head) {
-    const int gen = c->slot_gen[first % c->log.ring];
-    uint64_t end = first + 1;
-    while (end < c->log_head && end - first < (uint64_t)kCatchMaxPackets && c->slot_gen[end % c->log.ring] == gen) ++end;
-    const uint32_t count = (uint32_t)(end - first);
-    TimedLaunch tl(c, st, DGS_KERNEL_CATCH_UP);
-    // One CTA per SM at most, each taking several ranges in turn: the kernel runs beside the push passes of
-    // later events, and the loop is faster when it holds few SM resources than when it finishes early.
-    const unsigned catch_grid = std::min<unsigned>(c->log.ranges, (unsigned)c->sms);
-    PacketLog lg = c->log;
-    lg.bnd = c->log.bnd + (size_t)gen * c->log.ranges;
-    k_catch_up<<<catch_grid, kCatchThreads, 0, st>>>(lg, first, count, c->D_buf(q), c->blk_max(q), c->cfg.n);
-    DGS_CUDA(c, cudaGetLastError());
-    c->launches += 1;
-    first = end;
-  }
+// The launch itself, on a stream that task_begin has prepared with those dependencies: the filed packets that D_q
+// has not seen yet, and with SCAN the stream pass of a pull in the same trip over D_q.
+template <bool SCAN>
+int fold_launch(dgs_ctx* c, const Workspace& ws, const SelArgs& a, uint32_t q, cudaStream_t st) {
+  const uint32_t first = (uint32_t)(c->applied[q] % c->log.ring);
+  const uint32_t count = (uint32_t)(c->log_head - c->applied[q]);   // <= ring
+  TimedLaunch tl(c, st, SCAN ? DGS_KERNEL_STREAM_PULL : DGS_KERNEL_CATCH_UP);
+  const uint32_t warps = c->alone || c->cfg.num_workers == 1 ? kFoldWarps : kFoldWarps / 2;
+  k_fold<SCAN><<<c->fold_grid, warps * 32, fold_dyn_bytes(warps, c->fold_ahead, ws.part_cap), st>>>(ws, a, c->log, first, count,
+                                                                                               c->fold_ahead);
+  DGS_CUDA(c, cudaGetLastError());
+  c->launches += 1;
   c->applied[q] = c->log_head;
   return DGS_OK;
 }
@@ -482,7 +452,11 @@ int catch_up_now(dgs_ctx* c, uint32_t q) {
   catch_up_deps(c, q, &t);
   int rc = task_begin(c, t);
   if (rc != DGS_OK) return rc;
-  rc = catch_up_launch(c, q, c->st[kStApply]);
+  SelArgs a;
+  std::memset(&a, 0, sizeof(a));
+  a.D = c->D_buf(q);
+  a.blk_max = c->blk_max(q);
+  rc = fold_launch<false>(c, c->ws[0], a, q, c->st[kStApply]);   // (tables only: a fold without a scan writes no scratch)
   if (rc != DGS_OK) return rc;
   return task_end(c, t);
 }
@@ -506,26 +480,6 @@ int pick_row(const dgs_ctx* c, int kind, uint64_t age) {
 
 inline int packet_format_of(const dgs_ctx* c) {
   return (c->cfg.flags & DGS_PACKET_BF16) ? 1 : (c->cfg.flags & DGS_PACKET_FP16) ? 2 : 0;
-}
-
-// The form of the next pull's stream pass (see dgs_ctx::h_chunks): ring-less if the pulls counted since the
-// last decision read less than a third of the chunks they covered.
-bool use_light_pull(dgs_ctx* c) {
-  if (!c->multi_worker || !c->h_chunks) return false;
-  const unsigned long long covered = *(volatile unsigned long long*)&c->h_chunks[0];
-  const unsigned long long read = *(volatile unsigned long long*)&c->h_chunks[1];
-  if (covered > c->seen_chunks[0] && read >= c->seen_chunks[1]) {
-    c->light_now = 3 * (read - c->seen_chunks[1]) < covered - c->seen_chunks[0];
-    c->seen_chunks[0] = covered;
-    c->seen_chunks[1] = read;
-  }
-  return c->light_now;
-}
-// After a pull: its counters on their way to the host (on the pull's stream, nobody waits for them).
-int report_chunks(dgs_ctx* c, cudaStream_t st) {
-  if (c->h_chunks)
-    DGS_CUDA(c, cudaMemcpyAsync(c->h_chunks, c->ws[0].stats + 3, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
-  return DGS_OK;
 }
 
 template <int MODE>
@@ -557,6 +511,7 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
   if (c->cfg.num_segments > 1) fin_want = (int)((2ull * a.pkt_count + kThreads * 8 - 1) / (kThreads * 8));
   const int fin_grid = std::min(c->finalize_max[MODE], std::max(fin_base, fin_want));
   a.workers = (uint32_t)fin_grid;
+  a.fold_grid = MODE == kPull ? (uint32_t)c->fold_grid : 0u;   // one CTA more plans the next pull's pass
   a.packet_format = packet_format_of(c);
   if (c->cfg.flags & DGS_TEST_STALLED_BARRIER) {
     a.phantom_workers = 1;
@@ -570,12 +525,12 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
   task.writes.push_back(R.SCR(KIND, set));
   int rc = task_begin(c, task);
   if (rc != DGS_OK) return rc;
-  if (MODE == kPull) {
-    rc = catch_up_launch(c, worker, st);
-    if (rc != DGS_OK) return rc;
-  }
   if (!single_pass) {
     // nothing to go by: histogram of the whole input first, its bounds cannot fail
+    if (MODE == kPull && c->applied[worker] < c->log_head) {
+      rc = fold_launch<false>(c, ws, a, worker, st);
+      if (rc != DGS_OK) return rc;
+    }
     TimedLaunch t(c, st, MODE == kPull ? DGS_KERNEL_TWO_PASS_PULL : DGS_KERNEL_TWO_PASS_PUSH);
     k_hist_all<MODE><<<c->hist_grid[MODE], kThreads, 0, st>>>(ws, a);
     DGS_CUDA(c, cudaGetLastError());
@@ -584,14 +539,12 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
     DGS_CUDA(c, cudaGetLastError());
     c->launches += 2;
   }
-  {
-    TimedLaunch t(c, st, MODE == kPull ? DGS_KERNEL_STREAM_PULL : DGS_KERNEL_STREAM_PUSH);
-    // A pull in a context with several workers shares the GPU with the push passes of later events and reads
-    // only a small part of D_w: it takes the form of the pass that holds no ring of stages.
-    if (MODE == kPull && use_light_pull(c))
-      k_pull_light<<<c->stream_grid[MODE], kThreads, 0, st>>>(ws, a);
-    else
-      k_stream<MODE><<<c->stream_grid[MODE], kThreads, StreamRing<MODE>::kBytes, st>>>(ws, a);
+  if (MODE == kPull) {
+    rc = fold_launch<true>(c, ws, a, worker, st);
+    if (rc != DGS_OK) return rc;
+  } else {
+    TimedLaunch t(c, st, DGS_KERNEL_STREAM_PUSH);
+    k_stream<MODE><<<c->stream_grid[MODE], kThreads, StreamRing<MODE>::kBytes, st>>>(ws, a);
     DGS_CUDA(c, cudaGetLastError());
     c->launches += 1;
   }
@@ -599,8 +552,8 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
     // cooperative launch: the CTAs synchronise among themselves, so all must be resident
     TimedLaunch t(c, st, MODE == kPull ? DGS_KERNEL_FINALIZE_PULL : DGS_KERNEL_FINALIZE_PUSH);
     void* args[] = {(void*)&ws, (void*)&a};
-    DGS_CUDA(c, cudaLaunchCooperativeKernel((const void*)k_finalize<MODE>, dim3(fin_grid), dim3(kThreads), args,
-                                            finalize_dyn_bytes(c->cfg.num_segments), st));
+    DGS_CUDA(c, cudaLaunchCooperativeKernel((const void*)k_finalize<MODE>, dim3(fin_grid + (MODE == kPull ? 1 : 0)),
+                                            dim3(kThreads), args, finalize_dyn_bytes(c->cfg.num_segments), st));
     c->launches += 1;
   }
   rc = task_end(c, task);
@@ -623,10 +576,6 @@ int occupancy_grids(dgs_ctx* c, int sms) {
                                                             StreamRing<MODE>::kBytes));
   if (occ < 1) occ = 1;
   c->stream_grid[MODE] = std::min(sms * occ, kMaxGrid);
-  // With several workers a pull's stream pass shares the GPU with the push passes of later events, and
-  // what counts is how few SM resources it holds, not how fast it is alone: one CTA per SM (its ranges
-  // are balanced by the plan that finalize leaves behind).  A context with one worker selects alone.
-  if (MODE == kPull && c->cfg.num_workers > 1) c->stream_grid[MODE] = std::min(c->stream_grid[MODE], sms);
   DGS_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_hist_all<MODE>, kThreads, 0));
   if (occ < 1) occ = 1;
   c->hist_grid[MODE] = std::min(sms * occ, kMaxGrid);
@@ -637,8 +586,26 @@ int occupancy_grids(dgs_ctx* c, int sms) {
     c->broken = true;
     return DGS_ECUDA;
   }
-  c->finalize_max[MODE] = std::min(sms * occ, kMaxWorkers);
+  c->finalize_max[MODE] = std::min(sms * occ, kMaxWorkers) - (MODE == kPull ? 1 : 0);
   c->finalize_grid[MODE] = std::min(c->finalize_max[MODE], kFinalizeWorkers);
+  return DGS_OK;
+}
+
+// Grid of k_fold and the room for its tables and buffers.
+constexpr int kFoldMaxDyn = 208 * 1024;   // beside its static shared memory
+int fold_setup(dgs_ctx* c, int sms) {
+  c->fold_grid = (int)std::min<uint32_t>((c->lay.num_blocks + kBlockGroup - 1) / kBlockGroup, (uint32_t)std::min(2 * sms, kMaxFoldGrid));
+  // A quarter more than the mean number of entries of a block, for a worker that has missed a packet per worker.
+  const uint64_t mean = std::min<uint64_t>(c->cfg.num_workers, 32) * c->lay.K[0] * kWarpTile / c->cfg.n;
+  c->fold_ahead = (uint32_t)std::min<uint64_t>(192, std::max<uint64_t>(64, align_up(mean + mean / 4, 64)));
+  // Eight even shares: where most of the vector is cold, the shares of the CTAs that have only cold blocks grow
+  // (a share never gets longer than an even one without a plan).
+  const uint32_t even = (c->lay.num_blocks + c->fold_grid - 1) / c->fold_grid + kFoldSlack;
+  const uint32_t cap = (uint32_t)align_up(std::max<uint32_t>(even, std::min<uint32_t>(32768u, 8 * even)), 128);
+  for (int k = 0; k < kAllSets; ++k) c->ws[k].part_cap = cap;
+  DGS_CUDA(c, cudaFuncSetAttribute(k_fold<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFoldMaxDyn));
+  DGS_CUDA(c, cudaFuncSetAttribute(k_fold<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFoldMaxDyn));
+  if (fold_dyn_bytes(kFoldWarps, c->fold_ahead, cap) > (uint32_t)kFoldMaxDyn) return DGS_EINVAL;   // (n < 2^32 keeps an even share well below)
   return DGS_OK;
 }
 
@@ -647,7 +614,6 @@ void destroy_ctx(dgs_ctx* c) {
     if (c->st[i] && (i == 0 || c->st[i] != c->st[0])) cudaStreamDestroy(c->st[i]);
     if (c->ev_tail[i]) cudaEventDestroy(c->ev_tail[i]);
   }
-  if (c->h_chunks) cudaFreeHost(c->h_chunks);
   if (c->ev_in) cudaEventDestroy(c->ev_in);
   for (int i = 0; i < kNumStreams; ++i)
     for (cudaEvent_t e : c->ev_ring[i]) cudaEventDestroy(e);
@@ -710,9 +676,6 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
   }
   c->pull_count = c->event_count = c->var_count = 0;
   c->log_head = 0;
-  c->last_ranges = 0;
-  c->cur_gen = 0;
-  c->gen_last[0] = c->gen_last[1] = -1;
   c->applied.assign(cfg->num_workers, 0);
   c->kind_seq[0] = c->kind_seq[1] = 0;
   c->res.assign(ResIds{cfg->num_workers}.count(), dgs_ctx::Res());
@@ -729,6 +692,7 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
   c->launches = 0;
   c->last_cuda = 0;
   c->broken = false;
+  c->alone = true;
   c->timing = false;
   for (int i = 0; i < DGS_NUM_KERNELS; ++i) {
     c->time_ms[i] = 0.0;
@@ -758,16 +722,8 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
   INIT_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
   if (!coop) return fail(DGS_ECUDA);
   c->sms = sms;
-  c->multi_worker = cfg->num_workers > 1;
-  c->h_chunks = nullptr;
-  c->seen_chunks[0] = c->seen_chunks[1] = 0;
-  c->light_now = false;
-  if (c->multi_worker) {
-    INIT_CUDA(cudaHostAlloc(reinterpret_cast<void**>(&c->h_chunks), 2 * sizeof(unsigned long long), cudaHostAllocDefault));
-    c->h_chunks[0] = c->h_chunks[1] = 0;
-  }
   if (occupancy_grids<kPushSam>(c, sms) != DGS_OK || occupancy_grids<kPushResidual>(c, sms) != DGS_OK ||
-      occupancy_grids<kPull>(c, sms) != DGS_OK)
+      occupancy_grids<kPull>(c, sms) != DGS_OK || fold_setup(c, sms) != DGS_OK)
     return fail(DGS_ECUDA);
   int prio_low = 0, prio_high = 0;
   INIT_CUDA(cudaDeviceGetStreamPriorityRange(&prio_low, &prio_high));
@@ -811,10 +767,9 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
   for (int k = 0; k < kAllSets; ++k) {
     const ScratchLayout& sc = L.sc[k];
     INIT_CUDA(cudaMemsetAsync(c->at<char>(sc.zero_begin), 0, sc.zero_end - sc.zero_begin, st));
-    INIT_CUDA(cudaMemsetAsync(c->at<char>(sc.part_cands), 0, (uint64_t)kMaxGrid * 4, st));
-    INIT_CUDA(cudaMemsetAsync(c->at<char>(sc.part_slot0), 0, (uint64_t)kMaxGrid * 4, st));
-    INIT_CUDA(cudaMemsetAsync(c->at<char>(sc.plan), 0, (uint64_t)(kMaxGrid + 1) * 4, st));   // no plan yet
-    INIT_CUDA(cudaMemsetAsync(c->at<char>(sc.part_live), 0, (uint64_t)kMaxGrid * 4, st));
+    INIT_CUDA(cudaMemsetAsync(c->at<char>(sc.part_cands), 0, (uint64_t)kMaxParts * 4, st));
+    INIT_CUDA(cudaMemsetAsync(c->at<char>(sc.part_slot0), 0, (uint64_t)kMaxParts * 4, st));
+    INIT_CUDA(cudaMemsetAsync(c->at<char>(sc.plan), 0, (uint64_t)(kMaxFoldGrid + 1) * 4, st));   // no plan yet
   }
   INIT_CUDA(cudaMemsetAsync(c->at<char>(L.blk_max), 0, N * L.blk_stride * 4, st));   // D = 0
   INIT_CUDA(cudaMemsetAsync(c->at<char>(L.L_next), 0xFF, 2 * N * cfg->num_segments * 4, st));
@@ -829,6 +784,12 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
   seg_off[cfg->num_segments] = (uint32_t)cfg->n;  // n < 2^32
   INIT_CUDA(cudaMemcpyAsync(c->at<char>(L.seg_off), seg_off.data(), seg_off.size() * 4, cudaMemcpyHostToDevice, st));
   INIT_CUDA(cudaMemcpyAsync(c->at<char>(L.seg_tile0), seg_tile0.data(), seg_tile0.size() * 4, cudaMemcpyHostToDevice, st));
+  std::vector<uint32_t> blk_seg(L.num_blocks);
+  for (uint32_t b = 0, q = 0; b < L.num_blocks; ++b) {
+    while (segs.size() > q + 1 && (uint64_t)seg_off[q + 1] <= (uint64_t)b * kWarpTile) ++q;
+    blk_seg[b] = q;
+  }
+  INIT_CUDA(cudaMemcpyAsync(c->at<char>(L.blk_seg), blk_seg.data(), blk_seg.size() * 4, cudaMemcpyHostToDevice, st));
   std::vector<uint32_t> ones(cfg->num_segments, 1u);   // the bound that admits every nonzero value
   INIT_CUDA(cudaMemcpyAsync(c->at<char>(L.L_one), ones.data(), ones.size() * 4, cudaMemcpyHostToDevice, st));
   std::vector<float*> slots(N + kPushSets);
@@ -852,7 +813,11 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
     w.part_cands = c->at<uint32_t>(sc.part_cands);
     w.part_slot0 = c->at<uint32_t>(sc.part_slot0);
     w.plan = c->at<uint32_t>(sc.plan);
-    w.part_live = c->at<uint32_t>(sc.part_live);
+    w.cta_cost = c->at<uint32_t>(sc.cta_cost);
+    w.n = (uint32_t)cfg->n;
+    w.n_pad = (uint32_t)std::min<uint64_t>(L.n_pad, 0xFFFFFFFFull);
+    w.num_blocks = L.num_blocks;
+    w.blk_seg = c->at<uint32_t>(L.blk_seg);
     w.cta_tot = c->at<uint2>(sc.cta_tot);
     w.seg_start = c->at<uint2>(sc.seg_start);
     w.hist1 = c->at<uint32_t>(sc.hist1);
@@ -865,15 +830,11 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
     w.status = c->at<int>(L.status);
     w.stats = c->at<unsigned long long>(L.stats);
   }
-  c->log.idx = c->at<uint32_t>(L.log_idx);
-  c->log.val = c->at<float>(L.log_val);
+  c->log.ent = c->at<uint2>(L.log_ent);
   c->log.stride = L.log_stride;
-  c->log.cap = (uint32_t)L.K[0];
   c->log.ring = L.log_ring;
-  c->log.bnd = c->at<uint32_t>(L.log_bnd);
   c->log.pos = c->at<uint32_t>(L.log_pos);
-  c->log.ranges = L.log_ranges;
-  c->slot_gen.assign(L.log_ring, 0);
+  c->log.pos_rows = L.pos_rows;
   *out = c;
   return DGS_OK;
 }
@@ -928,7 +889,7 @@ int apply_impl(dgs_ctx* c, uint32_t worker, const dgs_packet* pkt) {
   const uint32_t gx = (pkt->count + kThreads - 1) / kThreads;
   if (pkt->count == 0) {
     // nothing to subtract
-  } else if (slot >= 0 && pkt->val == c->at<float>(c->lay.pkt_val[slot]) && pkt->count == c->log.cap) {
+  } else if (slot >= 0 && pkt->val == c->at<float>(c->lay.pkt_val[slot]) && pkt->count == c->lay.K[0]) {
     // One of the library's own packets (sorted by index, of the fixed size): theta now, the D_q lazily.
     // Its slot of the log still holds the packet filed `ring` applies ago; whoever has not folded that
     // one in yet does so first.
@@ -941,52 +902,18 @@ int apply_impl(dgs_ctx* c, uint32_t worker, const dgs_packet* pkt) {
           if (rc != DGS_OK) return rc;
         }
     }
-    // The ranges of the log are taken from the first packet filed, again from packet N (velocities have
-    // built up by then) and then every few rounds of the workers, so that they follow a drifting
-    // distribution.  Packets keep the positions they were filed with: the ranges come in two generations,
-    // a packet's slot remembers which one its positions refer to, and a catch-up folds the packets of the
-    // older generation before those of the newer one.  A generation is overwritten only when every packet
-    // filed under it has left the ring, so nobody has to catch up for the ranges to change.
-    const uint64_t period = std::max<uint64_t>(16ull * N, 2ull * c->log.ring);
-    const bool new_ranges = c->log_head == 0 || (c->log_head == N && c->last_ranges == 0) ||
-                            c->log_head >= c->last_ranges + period;
-    if (new_ranges) {
-      if (c->log_head > 0) {
-        // the other generation is taken over: whoever still has to fold in one of its packets (a worker that
-        // stayed away for very long) does so first
-        const int other = c->cur_gen ^ 1;
-        for (uint32_t q = 0; q < N; ++q)
-          if ((int64_t)c->applied[q] <= c->gen_last[other]) {
-            const int rc = catch_up_now(c, q);
-            if (rc != DGS_OK) return rc;
-          }
-        c->cur_gen = other;
-      }
-      c->last_ranges = c->log_head;
-    }
-    c->gen_last[c->cur_gen] = (int64_t)c->log_head;
-    c->slot_gen[lslot] = (uint8_t)c->cur_gen;
-    PacketLog lg = c->log;
-    lg.bnd = c->log.bnd + (size_t)c->cur_gen * c->log.ranges;
     Task t;
     t.stream = kStApply;
     t.reads.push_back(R.PKT(slot));
     t.writes = {R.THETA(), R.LOG(lslot)};
-    if (new_ranges) t.writes.push_back(R.RANGES(c->cur_gen));
-    else t.reads.push_back(R.RANGES(c->cur_gen));
     int rc = task_begin(c, t);
     if (rc != DGS_OK) return rc;
     {
       TimedLaunch tl(c, c->st[kStApply], DGS_KERNEL_SCATTER);
-      if (new_ranges) {
-        k_log_ranges<<<(c->log.ranges + kThreads - 1) / kThreads, kThreads, 0, c->st[kStApply]>>>(pkt->idx, lg);
-        DGS_CUDA(c, cudaGetLastError());
-        c->launches += 1;
-      }
-      const uint32_t pos_ctas = (c->log.ranges + 1 + kThreads - 1) / kThreads;
+      const uint32_t pos_ctas = (c->log.pos_rows + kThreads - 1) / kThreads;
       k_apply_log<<<gx + pos_ctas, kThreads, 0, c->st[kStApply]>>>(pkt->idx, pkt->val, pkt->count,
                                                                    c->at<float>(c->lay.theta), c->cfg.n,
-                                                                   c->ws[0].status, lg, lslot, gx);
+                                                                   c->ws[0].status, c->log, lslot, gx);
       DGS_CUDA(c, cudaGetLastError());
       c->launches += 1;
     }
@@ -1050,10 +977,9 @@ int pull_impl(dgs_ctx* c, uint32_t worker, dgs_packet* out) {
   const uint64_t age = c->timestamp - (c->prev[worker] < 0 ? 0 : (uint64_t)c->prev[worker]);
   rc = launch_select<kPull>(c, a, worker, age, stream_id, set, task);
   if (rc != DGS_OK) return rc;
-  rc = report_chunks(c, c->st[stream_id]);
-  if (rc != DGS_OK) return rc;
   c->prev[worker] = (int64_t)c->timestamp;
   c->pull_count += 1;
+  c->alone = false;
   if (out) {
     out->idx = a.pkt_idx;
     out->val = a.pkt_val;
@@ -1090,17 +1016,8 @@ int pull_all_impl(dgs_ctx* c, uint32_t worker, dgs_var_packet* out) {
   if (a.theta_local) task.writes.push_back(R.TL(worker));
   rc = task_begin(c, task);
   if (rc != DGS_OK) return rc;
-  rc = catch_up_launch(c, worker, st);
+  rc = fold_launch<true>(c, ws, a, worker, st);
   if (rc != DGS_OK) return rc;
-  {
-    TimedLaunch t(c, st, DGS_KERNEL_STREAM_PULL);
-    if (use_light_pull(c))
-      k_pull_light<<<c->stream_grid[kPull], kThreads, 0, st>>>(ws, a);
-    else
-      k_stream<kPull><<<c->stream_grid[kPull], kThreads, StreamRing<kPull>::kBytes, st>>>(ws, a);
-    DGS_CUDA(c, cudaGetLastError());
-    c->launches += 1;
-  }
   uint32_t* vi = c->at<uint32_t>(L.var_idx[vslot]);
   float* vv = c->at<float>(L.var_val[vslot]);
   uint32_t* vc = c->at<uint32_t>(L.var_count[vslot]);
@@ -1113,11 +1030,10 @@ int pull_all_impl(dgs_ctx* c, uint32_t worker, dgs_var_packet* out) {
   }
   rc = task_end(c, task);
   if (rc != DGS_OK) return rc;
-  rc = report_chunks(c, st);
-  if (rc != DGS_OK) return rc;
   c->prev[worker] = (int64_t)c->timestamp;
   c->pull_count += 1;
   c->var_count += 1;
+  c->alone = false;
   if (out) {
     out->idx = vi;
     out->val = vv;
@@ -1193,6 +1109,7 @@ int dgs_flush(dgs_ctx* c) {
     DGS_CUDA(c, cudaEventRecord(c->ev_tail[i], c->st[i]));
     DGS_CUDA(c, cudaStreamWaitEvent(c->user, c->ev_tail[i], 0));
   }
+  c->alone = true;
   return DGS_OK;
 }
 
@@ -1232,6 +1149,7 @@ int dgs_event_host(dgs_ctx* c, uint32_t worker, const float* grad_host, uint32_t
   // except for the shares of the apply that run on the other server streams
   DGS_CUDA(c, cudaStreamSynchronize(ps));
   for (int i = 0; i < kServerStreams; ++i) DGS_CUDA(c, cudaStreamSynchronize(c->st[kStS0 + i]));
+  c->alone = true;
   return DGS_OK;
 }
 
@@ -1554,8 +1472,13 @@ extern "C" int dgs_topk_encode_static(const float* x, uint32_t n, uint32_t k, ui
   ws.cand_val = sc->cand_val;
   ws.part_cands = sc->part_cands;
   ws.part_slot0 = sc->part_slot0;
+  ws.n = n;
+  ws.n_pad = kStaticMaxN;
+  ws.num_blocks = num_tiles;
+  ws.blk_seg = nullptr;      // only k_fold looks at blocks
   ws.plan = nullptr;
-  ws.part_live = nullptr;
+  ws.cta_cost = nullptr;
+  ws.part_cap = 0;
   ws.seg_off = sc->seg_off;
   ws.seg_tile0 = sc->seg_tile0;
   ws.cta_tot = sc->cta_tot;

@@ -37,6 +37,10 @@ constexpr int kBins3 = 1024;        // key bits  9..0
 constexpr uint32_t kFull = 0xFFFFFFFFu;
 constexpr uint32_t kSpecSlack = 64; // a carried bound aims at max(1.5 k, k + 64) candidates next time
 constexpr int kMaxGrid = 512;       // upper bound on the grid of a stream pass (= parts of the candidate buffer)
+constexpr int kMaxFoldGrid = 320;   // upper bound on the grid of a pull's pass (every warp of it is a part)
+constexpr int kMaxParts = kMaxFoldGrid * kWarps;   // upper bound on the parts of the candidate buffer
+constexpr uint32_t kFoldSlack = 64; // part_cap is at least that much longer than a CTA's share (its tables round to groups and words)
+constexpr int kBlockGroup = 8;      // blocks of kWarpTile elements whose packet positions are one 32-byte sector
 constexpr int kMaxWorkers = 320;    // upper bound on the grid of finalize
 constexpr uint32_t kSpinLimit = 1u << 22;  // bounded waits: give up and report after this many polls
 constexpr int kStatusTimeout = -4;  // = DGS_ETIMEOUT
@@ -73,16 +77,20 @@ struct Workspace {
   const Tile* tiles;
   const SegDesc* segs;
   uint32_t num_tiles, num_segs;
-  // candidates: part p (CTA p of the grid that ran the stream pass, `parts` CTAs) owns the slots
+  uint32_t n, n_pad;      // elements, and elements a state vector is padded to
+  uint32_t num_blocks;    // blocks of kWarpTile elements (the last one may be partial)
+  const uint32_t* blk_seg;   // [num_blocks] layer of the first element of each block
+  // candidates: part p (CTA p of the grid that ran a push's stream pass, warp p of a pull's) owns the slots
   // starting at the first element of its first tile
   uint32_t* cand_idx;     // [n]
   float* cand_val;        // [n]
-  uint32_t* part_cands;   // [kMaxGrid] candidates written by each part
-  uint32_t* part_slot0;   // [kMaxGrid] first slot of each part
-  // Pull, one layer: where the parts of the NEXT stream pass on this scratch set begin (tiles), planned by
-  // finalize from what this pass cost each part; plan[parts] == num_tiles and plan_parts == parts mark it valid.
-  uint32_t* plan;         // [kMaxGrid + 1], or null
-  uint32_t* part_live;    // [kMaxGrid] chunks each part read in the last stream pass, or null
+  uint32_t* part_cands;   // [kMaxParts] candidates written by each part
+  uint32_t* part_slot0;   // [kMaxParts] first slot of each part
+  // Pull: where the CTAs of the NEXT pass over a difference vector on this scratch set begin (blocks), planned
+  // beside finalize from what this pass cost each CTA; plan[G] == num_blocks and sync[kPlanParts] == G mark it valid.
+  uint32_t* plan;         // [kMaxFoldGrid + 1], or null
+  uint32_t* cta_cost;     // [kMaxFoldGrid] cost of each CTA's share in the last pass
+  uint32_t part_cap;      // most blocks a CTA of the pass can take
   const uint32_t* seg_off;   // [S+1] first element of each layer, and n
   const uint32_t* seg_tile0; // [S]   first tile of each layer
   uint2* cta_tot;         // [kMaxWorkers] (#key > T, #key == T) among the candidates of each CTA of finalize
@@ -117,6 +125,7 @@ struct SelArgs {
   int speculate;          // 0: never carry a bound (L_next is left alone)
   uint32_t workers;       // CTAs of finalize that process the candidates
   uint32_t seq;           // launch sequence number (tags the decision word)
+  uint32_t fold_grid;     // pull: CTAs of the pass before this finalize (0: it was not k_fold, nothing to plan)
   uint32_t phantom_workers;  // testing only: CTAs the finalize barrier waits for beyond those launched (0 in normal use)
   uint32_t spin_limit;    // polls after which a bounded wait gives up (0: kSpinLimit)
   int packet_format;      // 0: packets carry float32 values; 1: bfloat16; 2: binary16 (see round16)
@@ -228,12 +237,10 @@ __device__ __forceinline__ void load_tile_vec(const float* __restrict__ a, const
 // warps holding earlier tiles.  Read part after part, the candidate buffer therefore lists all
 // candidates of the vector in ascending index order, which is what lets the finalize kernel
 // number the selected ones with a plain prefix sum.
-constexpr int kLiveWords = 128;     // one bit per stage-sized chunk of a CTA's share of a layer
 struct StreamShared {
   uint32_t hist[kBins1];      // top 11 key bits of the candidates of the layer being processed
   uint32_t cursor;            // candidates appended by this CTA so far
   uint32_t wcnt[2][kWarps];   // candidates per warp of the current round (two rounds alternate)
-  uint32_t live[kLiveWords];  // pull: chunks that may hold a candidate (the others are not read)
 };
 
 __device__ __forceinline__ void flush_hist(uint32_t* s_hist, uint32_t* g_hist) {
@@ -288,10 +295,11 @@ __device__ __forceinline__ uint32_t tile_mask_regs(const SelArgs& a, uint32_t ti
 // order, and histograms their top key bits.  The cost is proportional to the candidates: one
 // packed warp scan gives every lane the rank of its candidates (lane l holds elements
 // j*128 + l*4 + c, order is j-major, so the four per-j counts travel as four bytes of one
-// word), and a lane that has candidates walks its set bits.  value(off) returns element `off`.
-template <typename ValueFn>
-__device__ __forceinline__ void tile_emit(const Workspace& ws, StreamShared& sh, uint32_t tile_start, uint32_t mask,
-                                          uint32_t base, int lane, ValueFn value) {
+// word), and a lane that has candidates walks its set bits.  value(off) returns element `off`; count(off, key)
+// adds a candidate to the histogram of its layer.
+template <typename ValueFn, typename CountFn>
+__device__ __forceinline__ void tile_emit(const Workspace& ws, uint32_t tile_start, uint32_t mask, uint32_t base, int lane,
+                                          ValueFn value, CountFn count) {
   if (!__any_sync(kFull, mask != 0)) return;
   // per-j candidate counts of this lane, one per byte
   uint32_t t = mask - ((mask >> 1) & 0x5555u);
@@ -319,7 +327,7 @@ __device__ __forceinline__ void tile_emit(const Workspace& ws, StreamShared& sh,
       const float v = value(off);
       ws.cand_idx[pos] = tile_start + off;
       ws.cand_val[pos] = v;
-      atomicAdd(sh.hist + (key_of(v) >> 20), 1u);
+      count(off, key_of(v));
     }
   }
 }
@@ -438,7 +446,7 @@ __device__ void stream_tiles(const Workspace& ws, const SelArgs& a, const uint32
       cur += total;
       if (t < a1) {
         if (tile.len == kWarpTile) {
-          tile_emit(ws, sh, tile.start, mask, base, lane, [&](uint32_t off) {
+          tile_emit(ws, tile.start, mask, base, lane, [&](uint32_t off) {
             // element off = j*128 + lane*4 + c is register 4*j + c of this lane
             const int e = (int)(((off >> 7) << 2) | (off & 3u));
             float v = x[0];
@@ -446,7 +454,7 @@ __device__ void stream_tiles(const Workspace& ws, const SelArgs& a, const uint32
             for (int q = 1; q < 4 * kVecIters; ++q)
               if (q == e) v = x[q];
             return v;
-          });
+          }, [&](uint32_t, uint32_t key) { atomicAdd(sh.hist + (key >> 20), 1u); });
         } else {
           ragged_emit(ws, sh, tile, mask, base, lane, lt, x);
         }
@@ -463,7 +471,7 @@ __device__ void stream_tiles(const Workspace& ws, const SelArgs& a, const uint32
 }
 
 // Step one for a tile staged in shared memory (su: the tile of the state vector, sg: the tile
-// of the gradient, push only): candidate mask, new velocity (push), block bound (pull).
+// of the gradient, push only): candidate mask, new velocity (push).
 template <int MODE>
 __device__ __forceinline__ uint32_t tile_mask_smem(const SelArgs& a, uint32_t tile_start, const float* su,
                                                    const float* sg, uint32_t L, int lane, float* __restrict__ out) {
@@ -471,11 +479,9 @@ __device__ __forceinline__ uint32_t tile_mask_smem(const SelArgs& a, uint32_t ti
   const float4* pu = reinterpret_cast<const float4*>(su) + lane;
   const float4* pg = reinterpret_cast<const float4*>(sg) + lane;
   uint32_t mask = 0;
-  uint32_t top = 0;       // pull: largest key of this lane's elements
 #pragma unroll
   for (int j = 0; j < kVecIters; ++j) {
     float4 x = pu[j * 32];
-    if (MODE == kPull) top = max(max(top, max(key_of(x.x), key_of(x.y))), max(key_of(x.z), key_of(x.w)));
     if (MODE != kPull) {
       const float4 g = pg[j * 32];
       x.x = combine<MODE>(x.x, g.x, a.m, a.lr);
@@ -493,11 +499,6 @@ __device__ __forceinline__ uint32_t tile_mask_smem(const SelArgs& a, uint32_t ti
       o.w = c3 ? x.w : unsent<MODE>(x.w, a.inv_m);
       __stcs(reinterpret_cast<float4*>(out + tile_start) + lane + j * 32, o);
     }
-  }
-  if (MODE == kPull && a.blk_max != nullptr) {
-    // the tile is a whole block: its bound becomes exact again (entries sent later only lower it)
-    top = __reduce_max_sync(kFull, top);
-    if (lane == 0) a.blk_max[tile_start / kWarpTile] = top;
   }
   return mask;
 }
@@ -557,14 +558,7 @@ __device__ void stream_tiles_tma(const Workspace& ws, const SelArgs& a, const ui
   using R = StreamRing<MODE>;
   static_assert(R::kStages >= 2, "the ring needs a stage in flight besides the one being read");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t t0 = part_first_tile(cta, G, ws.num_tiles), t1 = part_first_tile(cta + 1, G, ws.num_tiles);
-  if (MODE == kPull && ws.plan != nullptr && ld_volatile(ws.sync + kPlanParts) == G &&
-      __ldcg(ws.plan + G) == ws.num_tiles) {
-    // boundaries planned by the finalize of the previous selection on this scratch set
-    t0 = __ldcg(ws.plan + cta);
-    t1 = __ldcg(ws.plan + cta + 1);
-  }
-  uint32_t live_read = 0;   // thread 0: chunks this part reads
+  const uint32_t t0 = part_first_tile(cta, G, ws.num_tiles), t1 = part_first_tile(cta + 1, G, ws.num_tiles);
   const uint32_t lt = lanemask_lt();
   for (int b = threadIdx.x; b < kBins1; b += kThreads) sh.hist[b] = 0;
   if (threadIdx.x == 0) {
@@ -579,7 +573,6 @@ __device__ void stream_tiles_tma(const Workspace& ws, const SelArgs& a, const ui
     if (threadIdx.x == 0) {
       ws.part_cands[cta] = 0;
       ws.part_slot0[cta] = 0;
-      if (MODE == kPull && ws.part_live != nullptr) ws.part_live[cta] = 0;
     }
     return;
   }
@@ -622,52 +615,11 @@ __device__ void stream_tiles_tma(const Workspace& ws, const SelArgs& a, const ui
       bulk_load(dst, in + elem, bytes, full + st);
       if (MODE != kPull) bulk_load(dst + kStageFloats, a.grad + elem, bytes, full + st);
     };
-    // Pull: a chunk all of whose blocks have a bound below L holds no candidate and is not read.
-    const bool can_skip = MODE == kPull && a.blk_max != nullptr && L > 0 && nchunks <= kLiveWords * 32;
-    if (can_skip) {
-      for (uint32_t base = warp * 32; base < nchunks; base += kWarps * 32) {
-        const uint32_t c = base + lane;
-        bool live = false;
-        if (c < nchunks) {
-          const uint32_t tiles_here = min((uint32_t)kStageTiles, nfull - c * kStageTiles);
-          const uint32_t* bm = a.blk_max + e0 / kWarpTile + c * kStageTiles;
-          uint32_t top = 0;
-          for (uint32_t j = 0; j < tiles_here; ++j) top = max(top, __ldcg(bm + j));
-          live = top >= L;
-        }
-        const uint32_t word = __ballot_sync(kFull, live);
-        if (lane == 0) sh.live[base / 32] = word;
-      }
-      __syncthreads();
-    }
-    auto next_live = [&](uint32_t c) -> uint32_t {       // first chunk >= c that is read, nchunks if none
-      if constexpr (MODE == kPull) {
-        while (can_skip && c < nchunks) {
-          const uint32_t w = sh.live[c >> 5] >> (c & 31);
-          if (w) return c + __ffs(w) - 1;
-          c = (c | 31u) + 1;
-        }
-      }
-      return min(c, nchunks);
-    };
-    if (MODE == kPull && threadIdx.x == 0 && nchunks) {     // bookkeeping: chunks of D_w that exist / that are read
-      uint32_t read = nchunks;
-      if (can_skip) {
-        read = 0;
-        for (uint32_t w = 0; w * 32 < nchunks; ++w) read += __popc(sh.live[w]);
-      }
-      atomicAdd(ws.stats + 3, (unsigned long long)nchunks);
-      atomicAdd(ws.stats + 4, (unsigned long long)read);
-      live_read += read;
-    }
-    uint32_t pc = 0, issued = 0;                          // thread 0: next chunk to ask for, chunks asked for
-    if (threadIdx.x == 0) {
-      pc = next_live(0);
-      for (; issued < (uint32_t)R::kStages - 1 && pc < nchunks; ++issued, pc = next_live(pc + 1))
-        issue(pc, uses + issued);
-    }
+    uint32_t issued = 0;                                  // thread 0: chunks asked for
+    if (threadIdx.x == 0)
+      for (; issued < (uint32_t)R::kStages - 1 && issued < nchunks; ++issued) issue(issued, uses + issued);
     uint32_t done = 0;
-    for (uint32_t c = next_live(0); c < nchunks; c = next_live(c + 1), ++done) {
+    for (uint32_t c = 0; c < nchunks; ++c, ++done) {
       const uint32_t use = uses + done, st = use % R::kStages;
       const bool landed = mbar_wait(full + st, (use / R::kStages) & 1u);
       if (!landed) *s_dead = 1;
@@ -679,17 +631,16 @@ __device__ void stream_tiles_tma(const Workspace& ws, const SelArgs& a, const ui
       if (lane == 0) sh.wcnt[use & 1][warp] = count;
       __syncthreads();   // the counts of this round are known, and every warp has left the stage of the round before
       if (*s_dead) break;
-      if (threadIdx.x == 0 && pc < nchunks) {              // into the stage of the round before
-        issue(pc, uses + issued);
+      if (threadIdx.x == 0 && issued < nchunks) {          // into the stage of the round before
+        issue(issued, uses + issued);
         ++issued;
-        pc = next_live(pc + 1);
       }
       uint32_t total;
       const uint32_t base = slot0 + cur + round_offset(sh.wcnt[use & 1], warp, total);
       cur += total;
-      tile_emit(ws, sh, e0 + tl * kWarpTile, mask, base, lane, [&](uint32_t off) {
+      tile_emit(ws, e0 + tl * kWarpTile, mask, base, lane, [&](uint32_t off) {
         return combine<MODE>(su[off], MODE != kPull ? su[kStageFloats + off] : 0.f, a.m, a.lr);
-      });
+      }, [&](uint32_t, uint32_t key) { atomicAdd(sh.hist + (key >> 20), 1u); });
     }
     if (*s_dead) break;
     uses += done;
@@ -712,179 +663,6 @@ __device__ void stream_tiles_tma(const Workspace& ws, const SelArgs& a, const ui
   if (threadIdx.x == 0) {
     ws.part_cands[cta] = cur;
     ws.part_slot0[cta] = slot0;
-    if (MODE == kPull && ws.part_live != nullptr) ws.part_live[cta] = live_read;
-  }
-}
-
-// ---- the pull's pass without a staging ring ------------------------------------------
-// A pull of one worker among many reads only the chunks of D_w whose block bounds admit a
-// candidate -- a small part of the vector, a few chunks per CTA -- while the push passes of
-// later events stream beside it and need the SMs' shared memory for their own rings.  This
-// form of the pass therefore holds no ring: a warp loads its tile of the next chunk to be read
-// straight into registers while the CTA finishes the chunk before, so one chunk is in flight
-// per CTA, and the CTA keeps only its histogram in shared memory.  Candidates, bounds, plan and
-// counters are exactly those of the staged form.
-__device__ __forceinline__ void load_tile_raw(const float* __restrict__ in, uint32_t start, int lane,
-                                              float (&x)[4 * kVecIters]) {
-  const float4* pa = reinterpret_cast<const float4*>(in + start) + lane;
-#pragma unroll
-  for (int j = 0; j < kVecIters; ++j) {
-    const float4 v = __ldcs(pa + j * 32);
-    x[4 * j + 0] = v.x;
-    x[4 * j + 1] = v.y;
-    x[4 * j + 2] = v.z;
-    x[4 * j + 3] = v.w;
-  }
-}
-
-__device__ void pull_tiles_light(const Workspace& ws, const SelArgs& a, const uint32_t* Larr,
-                                 const float* __restrict__ in, uint32_t cta, uint32_t G, StreamShared& sh) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t t0 = part_first_tile(cta, G, ws.num_tiles), t1 = part_first_tile(cta + 1, G, ws.num_tiles);
-  if (ws.plan != nullptr && ld_volatile(ws.sync + kPlanParts) == G && __ldcg(ws.plan + G) == ws.num_tiles) {
-    // boundaries planned by the finalize of the previous selection on this scratch set
-    t0 = __ldcg(ws.plan + cta);
-    t1 = __ldcg(ws.plan + cta + 1);
-  }
-  uint32_t live_read = 0;   // thread 0: chunks this part reads
-  const uint32_t lt = lanemask_lt();
-  for (int b = threadIdx.x; b < kBins1; b += kThreads) sh.hist[b] = 0;
-  if (threadIdx.x == 0) {
-    sh.cursor = 0;
-    if (cta == 0) ws.sync[kParts] = G;
-  }
-  __syncthreads();
-  if (t0 >= t1) {
-    if (threadIdx.x == 0) {
-      ws.part_cands[cta] = 0;
-      ws.part_slot0[cta] = 0;
-      if (ws.part_live != nullptr) ws.part_live[cta] = 0;
-    }
-    return;
-  }
-  const uint32_t slot0 = ws.tiles[t0].start;
-  const uint32_t seg_first = ws.tiles[t0].seg, seg_last = ws.tiles[t1 - 1].seg;
-  uint32_t cur = 0;     // candidates appended so far (same in every thread)
-  uint32_t round = 0;
-  for (uint32_t s = seg_first; s <= seg_last; ++s) {
-    const uint32_t a0 = max(t0, ws.segs[s].tile_begin), a1 = min(t1, ws.segs[s].tile_end);
-    const uint32_t L = Larr[s];
-    const bool head = ws.tiles[a0].len != kWarpTile;
-    const bool tail = (a1 - 1 > a0 || !head) && ws.tiles[a1 - 1].len != kWarpTile;
-    const uint32_t f0 = a0 + (head ? 1u : 0u), f1 = a1 - (tail ? 1u : 0u);   // full tiles [f0, f1)
-    auto ragged = [&](uint32_t t) {
-      if (warp == 0) {
-        const Tile tile = ws.tiles[t];
-        float x[kRaggedSteps];
-        const uint32_t flags = ragged_mask<kPull>(a, tile, L, lane, in, nullptr, x);
-        const uint32_t count = __reduce_add_sync(kFull, (uint32_t)__popc(flags));
-        ragged_emit(ws, sh, tile, flags, slot0 + cur, lane, lt, x);
-        if (lane == 0) sh.cursor = count;
-      }
-      __syncthreads();
-      cur += sh.cursor;
-      __syncthreads();
-    };
-    if (head) ragged(a0);
-    const uint32_t nfull = f1 > f0 ? f1 - f0 : 0;
-    const uint32_t nchunks = (nfull + kStageTiles - 1) / kStageTiles;
-    const uint32_t e0 = nfull ? ws.tiles[f0].start : 0;   // first element of the full tiles (multiple of kWarpTile)
-    // a chunk all of whose blocks have a bound below L holds no candidate and is not read
-    const bool can_skip = a.blk_max != nullptr && L > 0 && nchunks <= kLiveWords * 32;
-    if (can_skip) {
-      for (uint32_t base = warp * 32; base < nchunks; base += kWarps * 32) {
-        const uint32_t c = base + lane;
-        bool live = false;
-        if (c < nchunks) {
-          const uint32_t tiles_here = min((uint32_t)kStageTiles, nfull - c * kStageTiles);
-          const uint32_t* bm = a.blk_max + e0 / kWarpTile + c * kStageTiles;
-          uint32_t top = 0;
-          if (tiles_here == kStageTiles && (reinterpret_cast<uintptr_t>(bm) & 15u) == 0) {
-            const uint4 q0 = __ldcg(reinterpret_cast<const uint4*>(bm)), q1 = __ldcg(reinterpret_cast<const uint4*>(bm) + 1);
-            top = max(max(max(q0.x, q0.y), max(q0.z, q0.w)), max(max(q1.x, q1.y), max(q1.z, q1.w)));
-          } else {
-            for (uint32_t j = 0; j < tiles_here; ++j) top = max(top, __ldcg(bm + j));
-          }
-          live = top >= L;
-        }
-        const uint32_t word = __ballot_sync(kFull, live);
-        if (lane == 0) sh.live[base / 32] = word;
-      }
-      __syncthreads();
-    }
-    auto next_live = [&](uint32_t c) -> uint32_t {       // first chunk >= c that is read, nchunks if none
-      while (can_skip && c < nchunks) {
-        const uint32_t w = sh.live[c >> 5] >> (c & 31);
-        if (w) return c + __ffs(w) - 1;
-        c = (c | 31u) + 1;
-      }
-      return min(c, nchunks);
-    };
-    if (threadIdx.x == 0 && nchunks) {     // bookkeeping: chunks of D_w that exist / that are read
-      uint32_t read = nchunks;
-      if (can_skip) {
-        read = 0;
-        for (uint32_t w = 0; w * 32 < nchunks; ++w) read += __popc(sh.live[w]);
-      }
-      atomicAdd(ws.stats + 3, (unsigned long long)nchunks);
-      atomicAdd(ws.stats + 4, (unsigned long long)read);
-      live_read += read;
-    }
-    float x[4 * kVecIters], xn[4 * kVecIters];
-    uint32_t c = next_live(0);
-    if (c < nchunks && c * kStageTiles + warp < nfull) load_tile_raw(in, e0 + (c * kStageTiles + warp) * kWarpTile, lane, x);
-    while (c < nchunks) {
-      const uint32_t cn = next_live(c + 1);
-      const uint32_t tl = c * kStageTiles + warp;          // this warp's tile among the full ones
-      const uint32_t tile_start = e0 + tl * kWarpTile;
-      uint32_t mask = 0;
-      if (tl < nfull) {
-        uint32_t top = 0;
-#pragma unroll
-        for (int e = 0; e < 4 * kVecIters; ++e) {
-          const uint32_t key = key_of(x[e]);
-          top = max(top, key);
-          if (key >= L) mask |= 1u << e;
-        }
-        if (a.blk_max != nullptr) {
-          // the tile is a whole block: its bound becomes exact again (entries sent later only lower it)
-          top = __reduce_max_sync(kFull, top);
-          if (lane == 0) a.blk_max[tile_start / kWarpTile] = top;
-        }
-      }
-      const uint32_t count = __reduce_add_sync(kFull, (uint32_t)__popc(mask));
-      if (lane == 0) sh.wcnt[round & 1][warp] = count;
-      // the next chunk is on its way while this one is written out
-      if (cn < nchunks && cn * kStageTiles + warp < nfull)
-        load_tile_raw(in, e0 + (cn * kStageTiles + warp) * kWarpTile, lane, xn);
-      __syncthreads();
-      uint32_t total;
-      const uint32_t base = slot0 + cur + round_offset(sh.wcnt[round & 1], warp, total);
-      cur += total;
-      if (tl < nfull)
-        tile_emit(ws, sh, tile_start, mask, base, lane, [&](uint32_t off) {
-          // element off = j*128 + lane*4 + c is register 4*j + c of this lane
-          const int e = (int)(((off >> 7) << 2) | (off & 3u));
-          float v = x[0];
-#pragma unroll
-          for (int q = 1; q < 4 * kVecIters; ++q)
-            if (q == e) v = x[q];
-          return v;
-        });
-#pragma unroll
-      for (int e = 0; e < 4 * kVecIters; ++e) x[e] = xn[e];
-      c = cn;
-      ++round;
-    }
-    __syncthreads();
-    if (tail) ragged(a1 - 1);
-    flush_hist(sh.hist, ws.hist1 + (size_t)s * kBins1);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    ws.part_cands[cta] = cur;
-    ws.part_slot0[cta] = slot0;
-    if (ws.part_live != nullptr) ws.part_live[cta] = live_read;
   }
 }
 
@@ -998,6 +776,29 @@ __device__ uint32_t block_pick(const uint32_t* hist, uint32_t k, uint32_t& bin, 
   return (uint32_t)total;
 }
 
+// Flat numbering of the candidates over the parts: pre[p] = candidates of the parts before p (pre[parts] = all of
+// them), slot0[p] = first slot of part p.  Both arrays in shared memory; ends with a barrier.
+__device__ __forceinline__ void number_parts(const Workspace& ws, uint32_t parts, uint32_t* pre, uint32_t* slot0,
+                                             unsigned long long* s_warp) {
+  for (uint32_t p = threadIdx.x; p < parts; p += kThreads) {
+    pre[p] = __ldcg(ws.part_cands + p);
+    slot0[p] = __ldcg(ws.part_slot0 + p);
+  }
+  __syncthreads();
+  const uint32_t per = (parts + kThreads - 1) / kThreads, p0 = min(parts, threadIdx.x * per), p1 = min(parts, p0 + per);
+  uint32_t sum = 0;
+  for (uint32_t p = p0; p < p1; ++p) sum += pre[p];
+  unsigned long long total;
+  uint32_t at = (uint32_t)block_excl_scan(sum, s_warp, total);
+  for (uint32_t p = p0; p < p1; ++p) {
+    const uint32_t c = pre[p];
+    pre[p] = at;
+    at += c;
+  }
+  if (threadIdx.x == 0) pre[parts] = (uint32_t)total;
+  __syncthreads();
+}
+
 // Barrier among the CTAs of finalize (all resident: cooperative launch).  One arrival
 // counter that only grows: the i-th barrier of a launch is passed when the counter has
 // reached i*W (the stream pass that precedes every finalize launch clears the counter).
@@ -1047,8 +848,8 @@ struct FinalizeShared {
   unsigned long long warp_scan[kWarps];
   uint32_t res[2];
   int ok;
-  uint32_t pre_cands[kMaxGrid + 1];    // exclusive prefix of part_cands
-  uint32_t slot0[kMaxGrid];            // first slot of each part
+  uint32_t pre_cands[kMaxParts + 1];   // exclusive prefix of part_cands
+  uint32_t slot0[kMaxParts];           // first slot of each part
 };
 // Per-layer tables of finalize live in dynamic shared memory, sized by the number of layers S (up
 // to kSegCap layers; with more, the kernel reads the tables from global memory and needs none):
@@ -1110,6 +911,69 @@ __device__ __forceinline__ void cursor_advance(const FinalizeShared& sh, uint32_
   c.left -= n;
 }
 
+// Where the CTAs of the next pass over a difference vector on this scratch set begin: ranges of blocks that cost
+// about the same, judged by what this pass cost each CTA.  What has to be read and folded in clusters in the
+// tensors with the largest updates, and those are the same for every worker; with equal ranges a few CTAs do most
+// of the work.  Done by a CTA of its own beside the finalize, so that it adds nothing to the chain.
+__device__ void plan_parts(const Workspace& ws, uint32_t G, FinalizeShared& sh) {
+  uint32_t* const before = sh.pre_cands;       // [G] cost of the CTAs before this one
+  uint32_t* const first = sh.slot0;            // [G + 1] where they began
+  uint32_t* const cost = sh.stream.hist;       // [G]
+  uint32_t* const next = sh.stream.hist + kMaxFoldGrid;   // [G + 1]
+  const bool had = ld_volatile(ws.sync + kPlanParts) == G && __ldcg(ws.plan + G) == ws.num_blocks;
+  for (uint32_t p = threadIdx.x; p < G; p += kThreads) {
+    cost[p] = __ldcg(ws.cta_cost + p);
+    first[p] = had ? __ldcg(ws.plan + p) : part_first_tile(p, G, ws.num_blocks);
+  }
+  if (threadIdx.x == 0) first[G] = ws.num_blocks;
+  __syncthreads();
+  const uint32_t per = (G + kThreads - 1) / kThreads, p0 = min(G, threadIdx.x * per), p1 = min(G, p0 + per);
+  uint32_t sum = 0;
+  for (uint32_t p = p0; p < p1; ++p) sum += cost[p];
+  unsigned long long total;
+  block_excl_scan(sum, sh.warp_scan, total);
+  // In 1/2^shift-ths, every block gets an amount on top that keeps a share of nothing but skipped blocks within
+  // part_cap: with c the mean cost of a CTA it is 5/4 c / part_cap, which adds at most 5/32 to c (part_cap holds
+  // eight even shares), so that a share ends after at most (37/32) / (5/4) part_cap blocks.
+  const uint32_t shift = total < (1ull << 20) ? 10u : 0u;   // sums stay below 2^32: a block costs at most 255
+  const float floor_cost = 1.25f * (float)((total << shift) / G + 1) / (float)(ws.part_cap - kFoldSlack);
+  sum = 0;
+  for (uint32_t p = p0; p < p1; ++p) {
+    cost[p] = (cost[p] << shift) + (uint32_t)(floor_cost * (float)(first[p + 1] - first[p])) + 1u;
+    sum += cost[p];
+  }
+  uint32_t at = (uint32_t)block_excl_scan(sum, sh.warp_scan, total);
+  for (uint32_t p = p0; p < p1; ++p) {
+    before[p] = at;
+    at += cost[p];
+  }
+  __syncthreads();
+  for (uint32_t j = threadIdx.x; j <= G; j += kThreads) {
+    uint32_t g = j == 0 ? 0u : ws.num_blocks;
+    if (j > 0 && j < G) {
+      const unsigned long long target = total * j / G;
+      uint32_t lo = 0, hi = G - 1;             // last CTA whose predecessors cost no more than the target
+      while (lo < hi) {
+        const uint32_t mid = (lo + hi + 1) >> 1;
+        if (before[mid] <= target) lo = mid; else hi = mid - 1;
+      }
+      const unsigned long long into = target - before[lo], c = cost[lo];
+      g = first[lo] + (uint32_t)((unsigned long long)(first[lo + 1] - first[lo]) * min(into, c) / c);
+    }
+    next[j] = g;
+  }
+  __syncthreads();
+  int ok = 1;                                  // a CTA cannot take more blocks than its tables hold
+  for (uint32_t j = threadIdx.x; j < G; j += kThreads)
+    if (next[j + 1] < next[j] || next[j + 1] - next[j] + kFoldSlack > ws.part_cap) ok = 0;
+  ok = __syncthreads_and(ok);
+  for (uint32_t j = threadIdx.x; j < G; j += kThreads) ws.plan[j] = next[j];
+  if (threadIdx.x == 0) {
+    ws.plan[G] = ok ? ws.num_blocks : 0u;
+    ws.sync[kPlanParts] = G;
+  }
+}
+
 // 64 registers a thread: finalize runs beside two CTAs of a push pass on an SM, which leave it that many
 template <int MODE>
 __global__ void __maxnreg__(64) k_finalize(Workspace ws, SelArgs a) {
@@ -1117,7 +981,12 @@ __global__ void __maxnreg__(64) k_finalize(Workspace ws, SelArgs a) {
   extern __shared__ __align__(16) unsigned char fin_dyn[];   // finalize_dyn_bytes(S) bytes
 
   constexpr int PM = MODE == kPull ? 1 : 0;
-  const uint32_t cta = blockIdx.x, W = gridDim.x, S = ws.num_segs;
+  // after k_fold one CTA more than a.workers is launched: it plans the next pass and takes no part in the selection
+  const uint32_t cta = blockIdx.x, W = a.workers, S = ws.num_segs;
+  if (MODE == kPull && cta == W) {
+    plan_parts(ws, a.fold_grid, sh);
+    return;
+  }
   const uint32_t gthread = cta * kThreads + threadIdx.x, nthreads = W * kThreads;
   // the barrier counts W arrivals; a test can make it wait for CTAs that do not exist, with a short limit,
   // to see the bounded wait give up (every CTA then leaves with DGS_ETIMEOUT in the status word)
@@ -1182,29 +1051,7 @@ __global__ void __maxnreg__(64) k_finalize(Workspace ws, SelArgs a) {
     }
     // flat numbering of the candidates (the stream pass is complete: an earlier kernel, or the barrier above)
     parts = ld_volatile(ws.sync + kParts);
-    {
-      constexpr int PER = kMaxGrid / kThreads;   // parts <= kMaxGrid
-      uint32_t cnt[PER];
-#pragma unroll
-      for (int j = 0; j < PER; ++j) {
-        const uint32_t p = j * kThreads + threadIdx.x;
-        cnt[j] = p < parts ? __ldcg(ws.part_cands + p) : 0;
-        if (p < parts) sh.slot0[p] = __ldcg(ws.part_slot0 + p);
-      }
-      unsigned long long carry = 0;
-#pragma unroll
-      for (int j = 0; j < PER; ++j) {
-        if ((uint32_t)(j * kThreads) < parts) {   // CTA-uniform
-          const uint32_t p = j * kThreads + threadIdx.x;
-          unsigned long long total;
-          const unsigned long long ex = block_excl_scan(cnt[j], sh.warp_scan, total) + carry;
-          if (p < parts) sh.pre_cands[p] = (uint32_t)ex;
-          carry += total;
-        }
-      }
-      if (threadIdx.x == 0) sh.pre_cands[parts] = (uint32_t)carry;
-      __syncthreads();
-    }
+    number_parts(ws, parts, sh.pre_cands, sh.slot0, sh.warp_scan);
     C = sh.pre_cands[parts];
     // every thread owns the flat candidates [my_lo, my_hi); when they are few it keeps them in registers
     per_thread = (C + nthreads - 1) / nthreads;
@@ -1512,69 +1359,6 @@ __global__ void __maxnreg__(64) k_finalize(Workspace ws, SelArgs a) {
       eq_before += is_eq ? 1u : 0u;
     });
   }
-  if (MODE == kPull && S == 1 && !redo && ws.plan != nullptr && ws.part_live != nullptr && cta == 0) {
-    // Plan for the next pull's stream pass on this scratch set: its CTAs get ranges of tiles that cost
-    // about the same, judged by what this pass cost each part (chunks read, candidates appended).  The
-    // chunks that have to be read cluster in the tensors with the largest updates, and those tensors are
-    // the same for every worker; with equal ranges a few CTAs do most of the reading.
-    constexpr int PER = kMaxGrid / kThreads;
-    const bool had = ld_volatile(ws.sync + kPlanParts) == parts && __ldcg(ws.plan + parts) == ws.num_tiles;
-    uint32_t cost[PER], old_t0[PER];
-#pragma unroll
-    for (int j = 0; j < PER; ++j) {
-      const uint32_t p = j * kThreads + threadIdx.x;
-      cost[j] = 0;
-      old_t0[j] = 0;
-      if (p < parts) {
-        cost[j] = 4u + 8u * __ldcg(ws.part_live + p) + (sh.pre_cands[p + 1] - sh.pre_cands[p]) / 16u;
-        old_t0[j] = had ? __ldcg(ws.plan + p) : part_first_tile(p, parts, ws.num_tiles);
-      }
-    }
-    __syncthreads();   // pre_cands and slot0 have been read for the last time
-    unsigned long long carry = 0;
-#pragma unroll
-    for (int j = 0; j < PER; ++j) {
-      if ((uint32_t)(j * kThreads) < parts) {   // CTA-uniform
-        const uint32_t p = j * kThreads + threadIdx.x;
-        unsigned long long total;
-        const unsigned long long ex = block_excl_scan(cost[j], sh.warp_scan, total) + carry;
-        if (p < parts) {
-          sh.pre_cands[p] = (uint32_t)ex;    // cost of the parts before p
-          sh.slot0[p] = old_t0[j];
-          sh.stream.hist[kMaxGrid + 1 + p] = cost[j];
-        }
-        carry += total;
-      }
-    }
-    __syncthreads();
-    const unsigned long long total_cost = carry;
-    for (uint32_t j = threadIdx.x; j <= parts; j += kThreads) {
-      uint32_t tile = j == 0 ? 0u : ws.num_tiles;
-      if (j > 0 && j < parts) {
-        const unsigned long long target = total_cost * j / parts;
-        uint32_t lo = 0, hi = parts - 1;       // last part whose earlier parts cost no more than the target
-        while (lo < hi) {
-          const uint32_t mid = (lo + hi + 1) >> 1;
-          if (sh.pre_cands[mid] <= target) lo = mid; else hi = mid - 1;
-        }
-        const uint32_t a0 = sh.slot0[lo], a1 = lo + 1 < parts ? sh.slot0[lo + 1] : ws.num_tiles;
-        const unsigned long long into = target - sh.pre_cands[lo], c = sh.stream.hist[kMaxGrid + 1 + lo];
-        tile = a0 + (uint32_t)((unsigned long long)(a1 - a0) * min(into, c) / c);
-      }
-      sh.stream.hist[j] = tile;
-    }
-    __syncthreads();
-    // a part must not be longer than the pass can keep skip flags for; otherwise no plan
-    int ok = 1;
-    for (uint32_t j = threadIdx.x; j < parts; j += kThreads)
-      if (sh.stream.hist[j + 1] < sh.stream.hist[j] || sh.stream.hist[j + 1] - sh.stream.hist[j] > 16384u) ok = 0;
-    ok = __syncthreads_and(ok);
-    for (uint32_t j = threadIdx.x; j < parts; j += kThreads) ws.plan[j] = sh.stream.hist[j];
-    if (threadIdx.x == 0) {
-      ws.plan[parts] = ok ? ws.num_tiles : 0u;
-      ws.sync[kPlanParts] = parts;
-    }
-  }
   if (cta == 0 && threadIdx.x == 0) {
     if (MODE != kPull) {  // the spare buffer now holds the worker's velocity
       float* cur = *a.u_cur_slot;
@@ -1637,13 +1421,6 @@ __global__ void __maxnreg__(64) k_stream(Workspace ws, SelArgs a) {
                          &s_dead);
 }
 
-// ---- the pull's stream pass in its ring-less form (contexts with several workers) -----
-__global__ void __maxnreg__(64) k_pull_light(Workspace ws, SelArgs a) {
-  __shared__ StreamShared sh;
-  if (blockIdx.x == 0 && threadIdx.x == 0) ws.sync[kBarCount] = 0;   // for the finalize launch that follows
-  pull_tiles_light(ws, a, a.L_in, a.D, blockIdx.x, gridDim.x, sh);
-}
-
 // ---- pull without secondary compression: every nonzero entry of D_w -------------------
 // The stream pass has run with the bound 1 for every layer (key >= 1 <=> the value is not zero),
 // so the candidate buffer lists all nonzero entries of D_w in index order, part after part.
@@ -1655,27 +1432,10 @@ __global__ void __launch_bounds__(kThreads) k_emit_all(Workspace ws, float* __re
                                                        uint32_t* __restrict__ blk_max, uint32_t* __restrict__ out_idx,
                                                        float* __restrict__ out_val, uint32_t* __restrict__ out_count,
                                                        uint32_t capacity, int packet_format) {
-  __shared__ uint32_t pre[kMaxGrid + 1], slot0[kMaxGrid];
+  __shared__ uint32_t pre[kMaxParts + 1], slot0[kMaxParts];
   __shared__ unsigned long long warp_scan[kWarps];
   const uint32_t parts = ld_volatile(ws.sync + kParts);
-  {
-    constexpr int PER = kMaxGrid / kThreads;   // parts <= kMaxGrid
-    unsigned long long carry = 0;
-#pragma unroll
-    for (int j = 0; j < PER; ++j) {
-      if ((uint32_t)(j * kThreads) < parts) {   // CTA-uniform
-        const uint32_t p = j * kThreads + threadIdx.x;
-        const uint32_t cnt = p < parts ? __ldcg(ws.part_cands + p) : 0;
-        if (p < parts) slot0[p] = __ldcg(ws.part_slot0 + p);
-        unsigned long long total;
-        const unsigned long long ex = block_excl_scan(cnt, warp_scan, total) + carry;
-        if (p < parts) pre[p] = (uint32_t)ex;
-        carry += total;
-      }
-    }
-    if (threadIdx.x == 0) pre[parts] = (uint32_t)carry;
-    __syncthreads();
-  }
+  number_parts(ws, parts, pre, slot0, warp_scan);
   const uint32_t C = pre[parts];
   const bool all = C <= capacity;          // every nonzero entry is sent: D_w is zero afterwards
   const uint32_t take = all ? C : capacity;
@@ -1716,18 +1476,6 @@ __global__ void __launch_bounds__(kThreads) k_emit_all(Workspace ws, float* __re
 // bit for bit, and each packet is folded into D_q while the entries it touches are hot
 // instead of being scattered into all N vectors at once.
 //
-constexpr int kCatchMaxPackets = 64;     // most packets one k_catch_up launch folds in
-constexpr int kCatchCap = 1024;          // entries a CTA of k_catch_up can hold in shared memory (a power of two)
-constexpr int kCatchSlots = 2 * kCatchCap;        // sparse pieces: slots of the table of distinct indices (>= 2 * kCatchCap)
-constexpr int kCatchDense = 2 * kCatchSlots;      // dense pieces: elements of D a piece can mirror (= the bytes of the sparse table)
-constexpr int kCatchLines = kCatchDense / 32;
-constexpr uint32_t kCatchTarget = 3 * kCatchCap / 4;  // entries per range of the log the launch aims at (a range that holds more than kCatchCap is halved)
-constexpr int kCatchMaxGrid = 16384;
-constexpr int kCatchBlocks = kCatchCap / 8 < 16 ? 16 : kCatchCap / 8;   // blocks of D whose bounds a CTA of k_catch_up collects in shared memory first
-constexpr int catch_log2(int v) { return v <= 1 ? 0 : 1 + catch_log2(v / 2); }
-constexpr int kCatchSlotBits = catch_log2(kCatchSlots);
-constexpr int kCatchThreads = 256;       // threads per CTA of k_catch_up (>= 2 * kCatchMaxPackets)
-
 // Keeps a block's bound an upper bound on the magnitudes in the block.  Bounds only rise while
 // packets are being subtracted, so a bound already read as high enough needs no atomic.
 __device__ __forceinline__ void raise_bound(uint32_t* bound, uint32_t key) {
@@ -1735,55 +1483,67 @@ __device__ __forceinline__ void raise_bound(uint32_t* bound, uint32_t key) {
 }
 
 struct PacketLog {
-  uint32_t* idx;   // [ring][stride], each packet sorted by index
-  float* val;      // [ring][stride]
-  uint32_t stride; // entries between slots
-  uint32_t cap;    // entries per packet
-  uint32_t ring;   // slots
-  // The index space is cut once, at the first packet filed, into `ranges` ranges that hold equally
-  // many of that packet's entries (later packets are spread much alike): range g is
-  // [bnd[g], bnd[g+1]), bnd[0] = 0, the last range is open-ended.  pos[slot][g] is the position of
-  // the first entry of the packet in `slot` whose index is >= bnd[g]; pos[slot][ranges] = cap.
-  uint32_t* bnd;   // [ranges]
-  uint32_t* pos;   // [ring][ranges + 1]
-  uint32_t ranges;
+  uint2* ent;         // [ring][stride]: (index, bits of the value), each packet sorted by index
+  uint32_t stride;    // entries between slots
+  uint32_t ring;      // slots
+  // pos[b][slot]: position of the first entry of the packet in `slot` whose index is >= b * kWarpTile, for every
+  // block b of the vector and a little beyond (those hold the packet's size).  Block-major: a worker that catches up
+  // reads a block's positions in all packets as one or two lines, where packet-major rows cost it a line per packet
+  // (and, with a row per page, an address translation per packet).
+  uint32_t* pos;      // [pos_rows][ring]
+  uint32_t pos_rows;  // > number of blocks rounded up to kBlockGroup
 };
 
-// The ranges of the log, from the quantiles of the first packet filed (sorted by index).
-__global__ void __launch_bounds__(kThreads) k_log_ranges(const uint32_t* __restrict__ idx, PacketLog lg) {
-  const uint32_t g = blockIdx.x * kThreads + threadIdx.x;
-  if (g < lg.ranges) lg.bnd[g] = g == 0 ? 0u : idx[(uint64_t)g * lg.cap / lg.ranges];
+// First position in the sorted idx[0, count) whose entry is >= key, found by a whole warp: 32 probes at a time, so
+// that a packet of 2^15 entries takes three trips to memory and not fifteen.
+__device__ __forceinline__ uint32_t warp_lower_bound(const uint32_t* __restrict__ idx, uint32_t count, uint64_t key, int lane) {
+  uint32_t l = 0, r = count;                     // the answer lies in [l, r]
+  while (r - l > 32) {
+    const uint32_t step = (r - l + 32) / 33, q = l + step * (lane + 1) - 1;
+    const bool less = q < r && (uint64_t)__ldg(idx + q) < key;
+    const uint32_t c = __popc(__ballot_sync(kFull, less));   // sorted: the first c probes are below the key
+    const uint32_t qc = l + step * (c + 1) - 1;
+    if (c < 32 && qc < r) r = qc;
+    l += step * c;
+  }
+  const bool less = l + lane < r && (uint64_t)__ldg(idx + l + lane) < key;
+  return l + __popc(__ballot_sync(kFull, less));
 }
 
 // theta -= packet, and a copy of the packet into slot `slot` of the log: CTAs [0, copy_ctas).
-// The remaining CTAs find where the ranges of the log begin in this packet.
+// Each of the remaining CTAs finds where kThreads blocks of the vector begin in this packet: the packet's part that
+// falls into them is found by two searches, its entries are counted per block in shared memory, and a prefix sum
+// gives the positions.
 __global__ void __launch_bounds__(kThreads) k_apply_log(const uint32_t* __restrict__ idx,
                                                         const float* __restrict__ val, uint32_t count,
                                                         float* __restrict__ theta, uint64_t n, int* status,
                                                         PacketLog lg, uint32_t slot, uint32_t copy_ctas) {
   if (blockIdx.x >= copy_ctas) {
-    const uint32_t g = (blockIdx.x - copy_ctas) * kThreads + threadIdx.x;
-    if (g > lg.ranges) return;
-    uint32_t l = 0;
-    if (g == lg.ranges) {
-      l = count;
-    } else if (g > 0) {
-      const uint32_t key = __ldcg(lg.bnd + g);
-      uint32_t r = count;
-      while (l < r) {
-        const uint32_t mid = (l + r) >> 1;
-        if (__ldg(idx + mid) < key) l = mid + 1; else r = mid;
-      }
+    __shared__ uint32_t s_cnt[kThreads], s_end[2];
+    __shared__ unsigned long long s_warp[kWarps];
+    const uint32_t b0 = (blockIdx.x - copy_ctas) * kThreads, warp = threadIdx.x >> 5;
+    s_cnt[threadIdx.x] = 0;
+    if (warp < 2) {
+      const uint32_t at = warp_lower_bound(idx, count, (uint64_t)(b0 + warp * kThreads) * kWarpTile, threadIdx.x & 31);
+      if ((threadIdx.x & 31) == 0) s_end[warp] = at;
     }
-    lg.pos[(uint64_t)slot * (lg.ranges + 1) + g] = l;
+    __syncthreads();
+    const uint32_t lo = s_end[0], hi = s_end[1];
+    for (uint32_t j = lo + threadIdx.x; j < hi; j += kThreads) {
+      const uint32_t b = __ldg(idx + j) / kWarpTile - b0;
+      if (b < (uint32_t)kThreads) atomicAdd(s_cnt + b, 1u);
+    }
+    __syncthreads();
+    unsigned long long total;
+    const uint32_t before = (uint32_t)block_excl_scan(s_cnt[threadIdx.x], s_warp, total);
+    if (b0 + threadIdx.x < lg.pos_rows) lg.pos[(uint64_t)(b0 + threadIdx.x) * lg.ring + slot] = lo + before;
     return;
   }
   const uint32_t j = blockIdx.x * kThreads + threadIdx.x;
   if (j >= count) return;
   const uint32_t i = idx[j];
   const float v = val[j];
-  lg.idx[(uint64_t)slot * lg.stride + j] = i;
-  lg.val[(uint64_t)slot * lg.stride + j] = v;
+  lg.ent[(uint64_t)slot * lg.stride + j] = make_uint2(i, __float_as_uint(v));
   if (i >= n) {
     atomicMin(status, -2000);
     return;
@@ -1791,316 +1551,489 @@ __global__ void __launch_bounds__(kThreads) k_apply_log(const uint32_t* __restri
   theta[i] = __fsub_rn(theta[i], v);
 }
 
-// D -= packets first .. first + count - 1 of the log, in that order (count <= kCatchMaxPackets).
-// A CTA owns a range c of the log at a time; its part of every packet is known from the
-// positions filed with the packet.  The values of D that the range's entries touch are brought
-// into shared memory once, the packets' values are subtracted there in packet order (indices
-// inside one packet are distinct, so a packet is one parallel step) and every value goes back
-// once: every D[i] sees the same subtractions in the same order as if the packets had been
-// applied one by one, with one trip to memory instead of one per packet.  No two CTAs touch the
-// same entry of D.  A range with more entries than the tables hold (later packets much denser
-// there than the one the ranges were taken from) is taken in several rounds, each over a piece
-// of the range (halved until its entries fit).
-//
-// Two ways to hold a piece's values of D:
-//   dense   the piece spans at most kCatchDense elements (counted from the 128-byte line its
-//           first element lies in): shared memory mirrors the piece, an entry's place is its
-//           offset.  Only the lines that hold an entry are read and written, each as one
-//           coalesced 128-byte access of a warp, so the number of memory requests is the number
-//           of lines touched, not the number of entries.  Where updates crowd -- the tensors
-//           with the largest gradients, which take most entries of every packet -- a line holds
-//           many entries.
-//   sparse  a wider piece: a table of the distinct indices, one load and one store per index.
-struct CatchShared {
-  union {
-    struct {
-      uint32_t keys[kCatchSlots];        // sparse: index held by a slot, kFull = empty
-      float vals[kCatchSlots];           //         running value of D at that index
-    } tab;
-    float dense[kCatchDense];            // dense: running values of D[a0 ..], a0 = first element of the piece's first line
-  };
-  uint16_t ent_slot[kCatchCap];          // place of each entry (packet-major order), 0xFFFF = index out of range
-  float ent_val[kCatchCap];
-  uint32_t lo[kCatchMaxPackets], hi[kCatchMaxPackets], end[kCatchMaxPackets];   // per packet: piece, end of the range
-  uint32_t pre[kCatchMaxPackets + 1];    // exclusive prefix of hi - lo
-  uint32_t bmax[kCatchBlocks];           // largest new magnitude per block of kWarpTile elements, from the piece's first block on
-  uint32_t dirty[kCatchLines / 4];       // dense: one byte per line, nonzero = the line holds an entry
-  uint32_t ab[2];                        // the range's first element and the element after its last
+// D -= packets of the log in slots first, first + 1, ... (count of them, in that order), and (SCAN) in the same trip
+// the stream pass of the pull: candidates of D, block bounds, histogram.
+// A warp owns a block of kWarpTile elements at a time and needs nothing from the other warps.  While it works on one
+// block, the values of the next one and its entries in the packets are on their way to shared memory (asynchronous
+// copies); lane p has looked up where that block begins and ends in packet p, and the entries lie in packet order.
+// 32 of them at a time are subtracted; where several of the 32 hit one element the lane order is the packet order.
+// Every D[i] sees the same subtractions in the same order as if the packets had been applied one by one, with one trip
+// to memory instead of one per packet.  Only 128-byte lines that hold an entry are written back.
+// Blocks are skipped when no packet has an entry in them and (SCAN) their bound lies below L.  The blocks of a CTA
+// that are left are dealt out to its warps in eight runs of about equal cost; a warp is a part of the candidate
+// buffer, so the candidates are in index order without any barrier between the warps.
+// What bounds it is the chain of a block (positions -> entries -> subtract -> scan) times the blocks of a warp, so the
+// grid is two CTAs per SM.  Measured alone, in place of a catch-up by ranges of the log followed by the pull's own
+// pass over D: 11.7 M elements in 62 layers, 3.7 M entries of 32 packets: 92 us for 272 + 62; 25.6 M elements, 0.8 M
+// entries: 46 us for 78 + 28; 124 M elements, 4.0 M entries: 220 us for 434 + 211.
+// The grid is the same whether a CTA has kFoldWarps warps or half as many, and so is the plan for it: a pull that has
+// the GPU to itself takes the full number, one that shares it with the push passes of later events the half (a round
+// of 32 arrivals on 124 M elements: 12.6 ms with four warps, 13.7 ms with eight, whose buffers and threads slow the
+// pushes down; one arrival at a time on 25.6 M elements with 8 workers: 196 us with eight, 210 us with four).
+constexpr int kFoldWarps = kWarps;
+struct FoldStage {                  // one block of one warp
+  float tile[kWarpTile];
+  uint2 runs[32];                   // the packets with entries in the block, in order, see BlockRuns
+  uint2 ent[1];                     // [ahead] entries that are fetched while the block before is worked on
 };
-static_assert(sizeof(float) * kCatchDense == (sizeof(uint32_t) + sizeof(float)) * kCatchSlots, "the two views share their bytes");
-static_assert(kCatchDense <= 0xFFFF && kCatchDense % kCatchThreads == 0 && kCatchThreads % 32 == 0 &&
-              kCatchThreads >= 2 * kCatchMaxPackets, "offsets fit the entry table");
-static_assert(kCatchDense / kWarpTile + 2 <= kCatchBlocks, "a dense piece's blocks fit the table of bounds");
+struct FoldShared {
+  uint32_t hist[kBins1];            // SCAN: top 11 key bits of the candidates of the CTA's main layer
+  uint32_t warp_sum[kFoldWarps];
+  uint32_t start[kFoldWarps + 1];   // first block of each warp's run (counted from the CTA's first)
+  uint32_t read;
+};
+__host__ __device__ inline uint32_t fold_stage_bytes(uint32_t ahead) { return kWarpTile * 4u + 32u * 8u + ahead * 8u; }
+// dynamic shared memory: two blocks per warp, then per block of the CTA's share one byte (its cost, 0 = skipped) and a bit
+__host__ __device__ inline uint32_t fold_dyn_bytes(uint32_t warps, uint32_t ahead, uint32_t part_cap) {   // part_cap: a multiple of 128
+  return warps * 2u * fold_stage_bytes(ahead) + part_cap + part_cap / 8u;
+}
+// cost of a block with that many entries, in units of about 16 entries
+__device__ __forceinline__ uint32_t block_cost(uint32_t entries) { return min(255u, 3u + entries / 16u); }
 
-__global__ void __maxnreg__(32) k_catch_up(PacketLog lg, uint64_t first, uint32_t count,
-                                                       float* __restrict__ D, uint32_t* __restrict__ blk_max,
-                                                       uint64_t n) {
-  __shared__ __align__(16) CatchShared sh;
-  const uint32_t tid = threadIdx.x;
-  if (count == 0 || count > (uint32_t)kCatchMaxPackets) return;
-  uint8_t* const dirty = reinterpret_cast<uint8_t*>(sh.dirty);
-  // a CTA takes the ranges blockIdx.x, blockIdx.x + gridDim.x, ... one after the other; where a range lies
-  // in the packets and in the index space is fetched one range ahead
-  // (thread 2p reads where the range begins in packet p, thread 2p+1 where it ends)
-  const uint32_t* const my_pos = lg.pos + ((first + (tid >> 1)) % lg.ring) * (uint64_t)(lg.ranges + 1) + (tid & 1u);
-  uint32_t pos_ahead = 0, bnd_ahead = 0;     // of the range this CTA takes next
-  if (blockIdx.x < lg.ranges) {
-    if (tid < 2 * count) pos_ahead = __ldcg(my_pos + blockIdx.x);
-    if (tid < 2) bnd_ahead = blockIdx.x + tid == 0 ? 0u : (blockIdx.x + tid == lg.ranges ? (uint32_t)n : __ldcg(lg.bnd + blockIdx.x + tid));
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+// A block in shared memory is read 16 consecutive elements per lane (so that lane order is element order) and filled
+// 16 bytes per lane in memory order; with the 16-byte pieces placed like this neither has bank conflicts.
+__device__ __forceinline__ uint32_t tile_place(uint32_t off) {   // where element `off` of the block is
+  return off ^ ((off >> 3) & 12u);
+}
+
+// The part of one block in up to 32 packets, lane p holding packet p's.  runs[r] = (d, slot) for the r-th packet with
+// entries here: the block's entry number e, if it is that packet's, is entry d + e of that slot of the log.
+struct BlockRuns {
+  uint32_t excl, len;       // this lane's packet: entries of the earlier packets, own entries
+  uint32_t total;           // entries of all packets
+};
+__device__ __forceinline__ BlockRuns block_runs(uint32_t lo, uint32_t hi, uint32_t slot, uint2* runs, int lane, uint32_t lt) {
+  BlockRuns r;
+  r.len = hi - lo;
+  uint32_t incl = r.len;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint32_t o = __shfl_up_sync(kFull, incl, d);
+    if (lane >= d) incl += o;
   }
-  for (uint32_t c = blockIdx.x; c < lg.ranges; c += gridDim.x) {
-  if (tid < 2 * count) {
-    if (tid & 1u) sh.end[tid >> 1] = pos_ahead; else sh.lo[tid >> 1] = pos_ahead;
-  }
-  if (tid < 2) sh.ab[tid] = bnd_ahead;
-  {
-    const uint32_t cn = c + gridDim.x;
-    if (cn < lg.ranges) {
-      if (tid < 2 * count) pos_ahead = __ldcg(my_pos + cn);
-      if (tid < 2) bnd_ahead = cn + tid == lg.ranges ? (uint32_t)n : __ldcg(lg.bnd + cn + tid);   // n < 2^32
+  r.excl = incl - r.len;
+  r.total = __shfl_sync(kFull, incl, 31);
+  const uint32_t some = __ballot_sync(kFull, r.len != 0);   // (every lane has read the list before this one by now)
+  if (r.len) runs[__popc(some & lt)] = make_uint2(lo - r.excl, slot);
+  __syncwarp();
+  return r;
+}
+// the block's entries e0 .. end - 1 (end <= total), on their way to shared memory; e0 a multiple of 32
+__device__ __forceinline__ void fetch_entries(const PacketLog& lg, const BlockRuns& r, uint32_t e0, uint32_t end, const uint2* runs,
+                                              uint2* ent, int lane, uint32_t le) {
+#pragma unroll 1
+  for (uint32_t e = e0; e < end; e += 32) {
+    const uint32_t rel = r.excl - e;
+    const uint32_t heads = __reduce_or_sync(kFull, r.len != 0 && rel < 32u ? 1u << rel : 0u);   // entries that open a packet
+    const uint32_t before = __popc(__ballot_sync(kFull, r.len != 0 && r.excl < e));
+    if (e + lane < end) {
+      const uint2 run = runs[before + __popc(heads & le) - 1u];
+      cp_async8(ent + (e - e0) + lane, lg.ent + ((uint64_t)run.y * lg.stride + (run.x + e + lane)));
     }
+  }
+}
+// Subtracts the first `count` fetched entries from the block.  Lane order is packet order, and inside one packet the
+// indices ascend: 32 entries fall into ascending runs, in each of which every element occurs once.  Where the runs are
+// few (a block with many entries) they go one by one, 36 cycles a step.  Else the lanes that share an element are found
+// with a ballot per bit of its offset (130 cycles; the match instruction takes 360 for 32 different offsets) and go
+// one after the other, mostly one or two steps.  Returns this lane's lines that were changed.
+constexpr uint32_t kFoldFew = 9;
+__device__ __forceinline__ uint32_t subtract_entries(float* tile, const uint2* ent, uint32_t count, uint32_t base, uint32_t n, int lane,
+                                                     uint32_t lt, uint32_t le) {
+  uint32_t dirty = 0;
+#pragma unroll 1
+  for (uint32_t e = 0; e < count; e += 32) {
+    uint32_t off = kFull;
+    float val = 0.f;
+    if (e + lane < count) {
+      const uint2 q = ent[e + lane];
+      if (q.x < n) off = q.x - base;
+      val = __uint_as_float(q.y);
+    }
+    const bool valid = off < (uint32_t)kWarpTile;
+    const uint32_t prev = __shfl_up_sync(kFull, off, 1);
+    const uint32_t opened = __ballot_sync(kFull, lane != 0 && off <= prev && e + lane < count);
+    uint32_t turn = __popc(opened & le), most = __popc(opened);
+    if (most >= kFoldFew) {
+      uint32_t peers = __ballot_sync(kFull, valid);
+#pragma unroll
+      for (int b = 0; (1 << b) < kWarpTile; ++b) {
+        const uint32_t ones = __ballot_sync(kFull, (off >> b) & 1u);
+        peers &= (off >> b) & 1u ? ones : ~ones;
+      }
+      turn = __popc(peers & lt);
+      most = __reduce_max_sync(kFull, valid ? turn : 0u);
+    }
+    float* const at = tile + tile_place(off & (uint32_t)(kWarpTile - 1));
+    for (uint32_t k = 0;; ++k) {
+      if (valid && turn == k) *at = __fsub_rn(*at, val);
+      __syncwarp();
+      if (k == most) break;
+    }
+    dirty |= valid ? 1u << (off >> 5) : 0u;
+  }
+  return dirty;
+}
+
+// What of a block was not fetched ahead: entries of the first 32 packets beyond the first `ahead` (a multiple of 64),
+// and the packets after the first 32 (a worker that has been away for long).  Half a buffer is on its way while the
+// other half is subtracted.
+__device__ __noinline__ uint32_t fold_rest(const PacketLog& lg, uint32_t first, uint32_t count, uint32_t ahead, uint32_t blk, uint32_t n,
+                                           FoldStage* st) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t lt = lanemask_lt(), le = lt | (1u << lane), half = ahead / 2;
+  uint32_t dirty = 0;
+  for (uint32_t p0 = 0; p0 < count; p0 += 32) {
+    const uint32_t p = p0 + lane, slot = (first + p) % lg.ring;
+    uint32_t l = 0, h = 0;
+    if (p < count) {
+      l = __ldcg(lg.pos + (uint64_t)blk * lg.ring + slot);
+      h = __ldcg(lg.pos + (uint64_t)(blk + 1) * lg.ring + slot);
+    }
+    const BlockRuns r = block_runs(l, h, slot, st->runs, lane, lt);
+    uint32_t e = p0 ? 0u : ahead, side = 0;
+    fetch_entries(lg, r, e, min(r.total, e + half), st->runs, st->ent, lane, le);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    for (; e < r.total; e += half, side ^= half) {
+      fetch_entries(lg, r, e + half, min(r.total, e + 2 * half), st->runs, st->ent + (side ^ half), lane, le);
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      __syncwarp();
+      dirty |= subtract_entries(st->tile, st->ent + side, min(half, r.total - e), blk * kWarpTile, n, lane, lt, le);
+    }
+  }
+  return dirty;
+}
+
+// exclusive prefix over the lanes of counts up to 31, and their sum
+__device__ __forceinline__ uint32_t lane_offsets(uint32_t count, uint32_t lt, uint32_t& total) {
+  uint32_t ex = 0;
+  total = 0;
+#pragma unroll
+  for (int b = 0; b < 5; ++b) {
+    const uint32_t m = __ballot_sync(kFull, (count >> b) & 1u);
+    ex += __popc(m & lt) << b;
+    total += __popc(m) << b;
+  }
+  return ex;
+}
+
+// A block that is not a full one inside one layer (layer `seg` is its first): every element is compared with the
+// bound of its own layer.  Appends the candidates from slot `at` on, returns how many; top: largest key.
+template <bool SCAN>
+__device__ __noinline__ uint32_t scan_mixed(const Workspace& ws, const SelArgs& a, const float* t, uint32_t base, uint32_t seg,
+                                            uint32_t at, uint32_t& top) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t len = min((uint32_t)kWarpTile, ws.n - base), S = ws.num_segs;
+  uint32_t mask = 0, best = 0, s = seg;
+  auto layer_of = [&](uint32_t off) {
+    while (s + 1 < S && __ldg(ws.seg_off + s + 1) <= base + off) ++s;
+  };
+  for (uint32_t e = 0; e < 16; ++e) {
+    const uint32_t off = lane * 16 + e;
+    if (off < len) {
+      const uint32_t key = key_of(t[tile_place(off)]);
+      best = max(best, key);
+      if (SCAN) {
+        layer_of(off);
+        if (key >= a.L_in[s]) mask |= 1u << e;
+      }
+    }
+  }
+  __syncwarp();
+  top = best;
+  if (!SCAN) return 0;
+  uint32_t total;
+  uint32_t pos = at + lane_offsets(__popc(mask), lanemask_lt(), total);
+  s = seg;
+  for (uint32_t m = mask; m; m &= m - 1) {
+    const uint32_t off = lane * 16 + __ffs(m) - 1;
+    const float v = t[tile_place(off)];
+    layer_of(off);
+    ws.cand_idx[pos] = base + off;
+    ws.cand_val[pos] = v;
+    ++pos;
+    atomicAdd(ws.hist1 + (size_t)s * kBins1 + (key_of(v) >> 20), 1u);
+  }
+  __syncwarp();
+  return total;
+}
+
+template <bool SCAN>
+__global__ void __maxnreg__(64) k_fold(const __grid_constant__ Workspace ws, const __grid_constant__ SelArgs a,
+                                       const __grid_constant__ PacketLog lg, uint32_t first, uint32_t count, uint32_t ahead) {
+  __shared__ FoldShared sh;
+  extern __shared__ __align__(16) unsigned char fold_dyn[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t tid = threadIdx.x, nt = blockDim.x, nw = nt / 32u, cta = blockIdx.x, G = gridDim.x;
+  const uint32_t lt = lanemask_lt(), le = lt | (1u << lane);
+  const uint32_t NB = ws.num_blocks, S = ws.num_segs, n = ws.n;
+  float* const D = a.D;
+  const uint32_t stage_bytes = fold_stage_bytes(ahead);
+  unsigned char* const stages = fold_dyn + warp * 2u * stage_bytes;
+  uint8_t* const cost = fold_dyn + nw * 2u * stage_bytes;                        // [part_cap]
+  uint32_t* const live = reinterpret_cast<uint32_t*>(cost + ws.part_cap);        // [part_cap / 32]
+
+  // this CTA's blocks [b0, b1); the tables count from `at0`, where b0's group of blocks begins
+  uint32_t b0 = part_first_tile(cta, G, NB), b1 = part_first_tile(cta + 1, G, NB);
+  if (SCAN && ws.plan != nullptr && ld_volatile(ws.sync + kPlanParts) == G && __ldcg(ws.plan + G) == NB) {
+    b0 = __ldcg(ws.plan + cta);
+    b1 = __ldcg(ws.plan + cta + 1);
+  }
+  const uint32_t at0 = b0 / kBlockGroup * kBlockGroup, groups = b0 < b1 ? (b1 - at0 + kBlockGroup - 1) / kBlockGroup : 0u;
+  const uint32_t words = (groups + 3u) / 4u;   // of `live`
+
+  if (SCAN)
+    for (uint32_t b = tid; b < (uint32_t)kBins1; b += nt) sh.hist[b] = 0;
+  if (tid <= nw) sh.start[tid] = kFull;
+  if (tid == 0) {
+    sh.read = 0;
+    if (SCAN && cta == 0) {
+      ws.sync[kParts] = G * nw;
+      ws.sync[kBarCount] = 0;   // for the finalize launch that follows
+    }
+  }
+
+  // A warp looks at 32 blocks at a time: lane l at the bound of block l, then lane p at where the blocks begin in packet
+  // p.  A block is skipped if it has no entry and its bound lies below L.
+  uint32_t read = 0;
+  for (uint32_t w = warp; w < words; w += nw) {
+    const uint32_t b = at0 + w * 32u + lane;
+    bool on = false;
+    if (SCAN && b >= b0 && b < b1) {
+      uint32_t s = S == 1 ? 0u : __ldg(ws.blk_seg + b);
+      uint32_t L = a.L_in[s];
+      if (S > 1) {   // the lowest bound of the layers that have a part of the block
+        const uint64_t end = (uint64_t)(b + 1) * kWarpTile;
+        while (s + 1 < S && __ldg(ws.seg_off + s + 1) < end) L = min(L, a.L_in[++s]);
+      }
+      on = __ldcg(a.blk_max + b) >= L;
+    }
+    uint32_t mine = 0;                        // entries of block b
+    for (uint32_t p0 = 0; p0 < count; p0 += 32) {
+      const uint32_t p = p0 + lane, rows = min(32u, groups * kBlockGroup - w * 32u);
+      const uint32_t* const pos = lg.pos + (uint64_t)(at0 + w * 32u) * lg.ring + (first + p) % lg.ring;
+      uint32_t prev = p < count ? __ldcg(pos) : 0u;
+#pragma unroll 1
+      for (uint32_t r0 = 0; r0 < rows; r0 += kBlockGroup) {
+        uint32_t q[kBlockGroup];
+#pragma unroll
+        for (int k = 0; k < kBlockGroup; ++k) q[k] = p < count ? __ldcg(pos + (uint64_t)(r0 + k + 1) * lg.ring) : 0u;
+#pragma unroll
+        for (int k = 0; k < kBlockGroup; ++k) {
+          const uint32_t e = __reduce_add_sync(kFull, q[k] - prev);
+          if ((uint32_t)lane == r0 + k) mine += e;
+          prev = q[k];
+        }
+      }
+    }
+    on = b >= b0 && b < b1 && (on || mine != 0);
+    cost[w * 32u + lane] = on ? (uint8_t)block_cost(mine) : (uint8_t)0;
+    const uint32_t word = __ballot_sync(kFull, on);
+    if (lane == 0) {
+      live[w] = word;
+      read += (word & 0xFFu ? 1u : 0u) + (word & 0xFF00u ? 1u : 0u) + (word & 0xFF0000u ? 1u : 0u) + (word & 0xFF000000u ? 1u : 0u);
+    }
+  }
+  if (SCAN && read) atomicAdd(&sh.read, read);
+  __syncthreads();
+  // Runs of about equal cost for the warps: warp w begins at the block where the cost so far passes w parts of nw.
+  uint32_t all;
+  {
+    const uint32_t per = (words + nt - 1) / nt, w0 = min(words, tid * per), w1 = min(words, w0 + per);
+    const uint4* const c4 = reinterpret_cast<const uint4*>(cost);
+    auto word_cost = [&](uint32_t w) {
+      const uint4 x = c4[2 * w], y = c4[2 * w + 1];
+      uint32_t v = __dp4a(x.x, 0x01010101u, 0u);
+      v = __dp4a(x.y, 0x01010101u, v); v = __dp4a(x.z, 0x01010101u, v); v = __dp4a(x.w, 0x01010101u, v);
+      v = __dp4a(y.x, 0x01010101u, v); v = __dp4a(y.y, 0x01010101u, v); v = __dp4a(y.z, 0x01010101u, v);
+      return __dp4a(y.w, 0x01010101u, v);
+    };
+    uint32_t sum = 0;
+    for (uint32_t w = w0; w < w1; ++w) sum += word_cost(w);
+    uint32_t at = sum;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t o = __shfl_up_sync(kFull, at, d);
+      if (lane >= d) at += o;
+    }
+    if (lane == 31) sh.warp_sum[warp] = at;
+    __syncthreads();
+    at -= sum;
+    all = 0;
+    for (uint32_t w = 0; w < nw; ++w) {
+      if (w == (uint32_t)warp) at += all;
+      all += sh.warp_sum[w];                     // < 2^32 / 8: a share has fewer than 2^20 blocks
+    }
+    if (sum) {
+      uint32_t k = 0;                            // next warp whose run begins at or after `at`
+      while (k < nw && k * all / nw < at) ++k;
+      for (uint32_t w = w0; w < w1 && k < nw; ++w) {
+        const uint32_t wc = word_cost(w);
+        if (k * all / nw >= at + wc) {           // none begins in this word
+          at += wc;
+          continue;
+        }
+        for (uint32_t x = live[w]; x; x &= x - 1) {
+          const uint32_t b = w * 32u + __ffs(x) - 1u;
+          at += cost[b];
+          for (; k < nw && k * all / nw < at; ++k) sh.start[k] = b;
+        }
+      }
+    }
+    if (tid == 0) sh.start[nw] = words * 32u;
   }
   __syncthreads();
-  const uint32_t range_b = sh.ab[1];
-  uint32_t a = sh.ab[0];
-  for (;;) {   // one round per piece [a, b) of the range; everything here is uniform over the CTA
-    for (int s = tid; s < kCatchBlocks; s += kCatchThreads) sh.bmax[s] = 0;
-    for (int s = tid; s < kCatchLines / 4; s += kCatchThreads) sh.dirty[s] = 0;   // (first written after the barriers below)
-    // If what is left of the range fits a dense piece, its lines of D set out for shared memory now
-    // (asynchronous 16-byte copies past L1), while the entries are being counted and gathered: where
-    // updates crowd nearly every line holds an entry anyway, and a trip to memory leaves the chain.
-    const bool ahead = range_b - (a & ~31u) <= (uint32_t)kCatchDense;
-    if (ahead) {
-      const uint32_t a0 = a & ~31u, floats = (range_b - a0 + 31u) & ~31u;   // whole lines; D is padded beyond n
-      for (uint32_t q = tid * 4; q < floats; q += kCatchThreads * 4)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(sh.dense + q)), "l"(D + a0 + q) : "memory");
+  // this warp's blocks: the live ones in [run0, run1)
+  const uint32_t run0 = sh.start[warp];
+  uint32_t run1 = kFull;
+  for (uint32_t w = nw; w > (uint32_t)warp; --w)
+    if (sh.start[w] != kFull) run1 = sh.start[w];   // (two warps may start at one block: the later one takes it)
+  // the layer whose candidates are counted in shared memory; those of others are counted in global memory
+  const uint32_t main_seg = S == 1 || b0 >= b1 ? 0u : __ldg(ws.blk_seg + b0 + (b1 - b0) / 2);
+
+  uint32_t walk_word = run0 == kFull ? 0u : run0 / 32u, walk_bits = run0 < run1 ? live[walk_word] & (kFull << (run0 & 31u)) : 0u;
+  const uint32_t last_word = run0 < run1 ? (run1 - 1u) / 32u : walk_word;
+  auto next_block = [&]() -> uint32_t {        // kFull after the last one
+    while (walk_bits == 0) {
+      if (walk_word >= last_word) return kFull;
+      walk_bits = live[++walk_word];
     }
-    if (tid < count) sh.hi[tid] = sh.end[tid];
-    uint32_t b = range_b;
-    uint32_t E;
-    for (;;) {
-      __syncthreads();
-      if (tid < 32) {
-        // exclusive prefix of the pieces' lengths over the packets (two per lane)
-        const uint32_t p0 = tid, p1 = tid + 32;
-        const uint32_t x = p0 < count ? sh.hi[p0] - sh.lo[p0] : 0u, y = p1 < count ? sh.hi[p1] - sh.lo[p1] : 0u;
-        uint32_t ix = x, iy = y;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-          const uint32_t ox = __shfl_up_sync(kFull, ix, d), oy = __shfl_up_sync(kFull, iy, d);
-          if ((int)tid >= d) {
-            ix += ox;
-            iy += oy;
-          }
-        }
-        const uint32_t tx = __shfl_sync(kFull, ix, 31), ty = __shfl_sync(kFull, iy, 31);
-        if (p0 < count) sh.pre[p0] = ix - x;
-        if (p1 < count) sh.pre[p1] = tx + iy - y;
-        if (tid == 0) sh.pre[count] = tx + ty;
-      }
-      __syncthreads();
-      E = sh.pre[count];
-      if (E <= (uint32_t)kCatchCap || b - a <= 1) break;   // one index has at most `count` entries
-      b = a + (b - a) / 2;
-      if (tid < count) {
-        const uint32_t* pi = lg.idx + ((first + tid) % lg.ring) * (uint64_t)lg.stride;
-        uint32_t l = sh.lo[tid], r = sh.end[tid];
-        while (l < r) {
-          const uint32_t mid = (l + r) >> 1;
-          if (__ldcg(pi + mid) < b) l = mid + 1; else r = mid;
-        }
-        sh.hi[tid] = l;
-      }
+    const uint32_t b = walk_word * 32u + __ffs(walk_bits) - 1u;
+    walk_bits &= walk_bits - 1u;
+    return b < run1 ? at0 + b : kFull;
+  };
+  const uint32_t my_slot = (first + lane) % lg.ring;             // of the first 32 packets
+  const uint32_t fill = (lane ^ ((lane >> 3) & 3)) * 4;          // where lane's 16 bytes of a 512-byte piece go
+  uint32_t lo = 0, hi = 0;                     // where block blk1 lies in this lane's packet
+  auto load_pos = [&](uint32_t b) {
+    if (b != kFull && (uint32_t)lane < count) {
+      const uint32_t* const pos = lg.pos + (uint64_t)b * lg.ring + my_slot;
+      lo = __ldcg(pos);
+      hi = __ldcg(pos + lg.ring);
     }
-    if (E > 0 && E <= (uint32_t)kCatchCap) {
-      const uint32_t a0 = a & ~31u;                         // first element of the line that holds a
-      const uint32_t span = b - a0;                         // b <= n
-      const bool dense = span <= (uint32_t)kCatchDense;
-      if (!dense) {
-        for (int s = tid; s < kCatchSlots; s += kCatchThreads) sh.tab.keys[s] = kFull;
-        __syncthreads();
-      }
-      // gather: entry e (packet-major) -> its index and value; the index gets a place in shared memory
-      constexpr int PER = kCatchCap / kCatchThreads;
-      uint32_t ei[PER];
-      float ev[PER];
-#pragma unroll
-      for (int u = 0; u < PER; ++u) {
-        const uint32_t e = tid + u * kCatchThreads;
-        ei[u] = kFull;
-        ev[u] = 0.f;
-        if (e < E) {
-          uint32_t l = 0;                       // last packet p with pre[p] <= e: the same six probes for every
-#pragma unroll                                  // entry, so that the searches of a thread's entries overlap
-          for (uint32_t step = kCatchMaxPackets / 2; step >= 1; step >>= 1) {
-            const uint32_t t = l + step;
-            if (t < count && sh.pre[t] <= e) l = t;
-          }
-          const uint64_t at = ((first + l) % lg.ring) * (uint64_t)lg.stride + sh.lo[l] + (e - sh.pre[l]);
-          ei[u] = __ldcg(lg.idx + at);
-          ev[u] = __ldcg(lg.val + at);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < PER; ++u) {
-        const uint32_t e = tid + u * kCatchThreads;
-        if (e < E) {
-          uint32_t slot = 0xFFFFu;
-          const uint32_t i = ei[u];
-          if (i < n && i >= a && i < b) {       // entries of a piece lie inside it; anything else is left alone
-            if (dense) {
-              slot = i - a0;
-              dirty[slot >> 5] = 1;
-            } else {
-              uint32_t h = (i * 2654435761u) >> (32 - kCatchSlotBits);   // the top bits of the product
-              for (;;) {
-                const uint32_t old = atomicCAS(sh.tab.keys + h, kFull, i);
-                if (old == kFull || old == i) break;
-                h = (h + 1) & (kCatchSlots - 1);
-              }
-              slot = h;
-            }
-          }
-          sh.ent_slot[e] = (uint16_t)slot;
-          sh.ent_val[e] = ev[u];
-        }
-      }
-      __syncthreads();
-      float* const cur = dense ? sh.dense : sh.tab.vals;    // running values, by place
-      constexpr int SPT = kCatchSlots / kCatchThreads;      // sparse: table slots per thread
-      constexpr int EPT = kCatchDense / kCatchThreads;      // dense: elements per thread, element tid + j * kCatchThreads
-      constexpr int LB = EPT < 8 ? EPT : 8;                  // loads a thread has in flight together
-      if (dense && ahead) {
-        asm volatile("cp.async.wait_all;" ::: "memory");   // the lines that set out at the start of the piece
-      } else if (dense) {
-        // a warp's 32 threads hold one line at every step j: one 128-byte request per line that holds an entry
-#pragma unroll 1
-        for (int j0 = 0; j0 < EPT; j0 += LB) {
-          if ((uint32_t)(j0 * kCatchThreads) >= span) break;
-          float d[LB];
-#pragma unroll
-          for (int j = 0; j < LB; ++j) {
-            const uint32_t off = tid + (j0 + j) * kCatchThreads;
-            d[j] = 0.f;
-            if (off < span && dirty[off >> 5]) d[j] = __ldcg(D + a0 + off);
-          }
-#pragma unroll
-          for (int j = 0; j < LB; ++j) sh.dense[tid + (j0 + j) * kCatchThreads] = d[j];
-        }
-      } else {
-        // one load of D per distinct index, all in flight together
-        uint32_t k[SPT];
-        float d[SPT];
-#pragma unroll
-        for (int u = 0; u < SPT; ++u) {
-          k[u] = sh.tab.keys[tid + u * kCatchThreads];
-          d[u] = 0.f;
-          if (k[u] != kFull) d[u] = __ldcg(D + k[u]);
-        }
-#pragma unroll
-        for (int u = 0; u < SPT; ++u)
-          if (k[u] != kFull) sh.tab.vals[tid + u * kCatchThreads] = d[u];
-      }
-      __syncthreads();
-      // The packets in arrival order; inside one packet every index, and so every place, occurs once, so a
-      // packet's part is one parallel step.  A part of a piece rarely has more entries than a warp has lanes:
-      // one warp takes the steps one after the other with only its own barrier between them, which costs a
-      // fraction of a barrier of the whole CTA per packet.
-      if (tid < 32) {
-        constexpr int G = 4;   // packets whose entries a lane fetches together, ahead of the steps that use them
-        for (uint32_t p0 = 0; p0 < count; p0 += G) {
-          uint32_t slot[G], e1[G];
-          float val[G];
-          uint32_t ebeg = sh.pre[p0];
-#pragma unroll
-          for (int j = 0; j < G; ++j) {
-            const uint32_t pend = p0 + j < count ? sh.pre[p0 + j + 1] : ebeg;
-            const uint32_t e = ebeg + tid;
-            slot[j] = 0xFFFFu;
-            val[j] = 0.f;
-            if (e < pend) {
-              slot[j] = sh.ent_slot[e];
-              val[j] = sh.ent_val[e];
-            }
-            e1[j] = pend;
-            ebeg = pend;
-          }
-          ebeg = sh.pre[p0];
-#pragma unroll
-          for (int j = 0; j < G; ++j) {
-            if (slot[j] != 0xFFFFu) cur[slot[j]] = __fsub_rn(cur[slot[j]], val[j]);
-            for (uint32_t e = ebeg + 32 + tid; e < e1[j]; e += 32) {   // a part with more entries than lanes
-              const uint32_t sl = sh.ent_slot[e];
-              if (sl != 0xFFFFu) cur[sl] = __fsub_rn(cur[sl], sh.ent_val[e]);
-            }
-            __syncwarp();
-            ebeg = e1[j];
-          }
-        }
-      }
-      __syncthreads();
-      // Back to memory.  The blocks' bounds must stay upper bounds: the largest new magnitude per block is
-      // collected in shared memory, one global atomic per block afterwards.
-      if (dense) {
-        // A warp takes four consecutive lines at a time (their dirty flags are one word); the loads of the
-        // four are in flight together, and a block's bound gets one reduction where the four lie in one block.
-        const uint32_t lead = a - a0;            // elements of the first line that belong to the range before
-        const uint32_t blk0 = a / kWarpTile, line0 = a0 >> 5;
-        const uint32_t lines = (span + 31u) >> 5, lane = tid & 31u;
-#pragma unroll 1
-        for (uint32_t l0 = (tid >> 5) * 4; l0 < lines; l0 += (kCatchThreads / 32) * 4) {
-          const uint32_t flags = sh.dirty[l0 >> 2];
-          if (flags == 0) continue;
-          uint32_t key[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const uint32_t off = (l0 + u) * 32 + lane;
-            key[u] = 0;
-            if (((flags >> (8 * u)) & 0xFFu) && off < span && off >= lead) {
-              const float r = sh.dense[off];
-              __stcg(D + a0 + off, r);
-              key[u] = key_of(r);
-            }
-          }
-          // a line lies inside one block (lines and blocks start at multiples of 32 and of kWarpTile)
-          const uint32_t b_first = (line0 + l0) / (kWarpTile / 32) - blk0, b_last = (line0 + l0 + 3) / (kWarpTile / 32) - blk0;
-          if (b_first == b_last) {
-            const uint32_t k4 = __reduce_max_sync(kFull, max(max(key[0], key[1]), max(key[2], key[3])));
-            if (lane == 0 && k4) atomicMax(sh.bmax + b_first, k4);
-          } else {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const uint32_t k1 = __reduce_max_sync(kFull, key[u]);
-              if (lane == 0 && k1) atomicMax(sh.bmax + ((line0 + l0 + u) / (kWarpTile / 32) - blk0), k1);
-            }
-          }
-        }
-      } else {
-#pragma unroll
-        for (int u = 0; u < SPT; ++u) {
-          const uint32_t i = sh.tab.keys[tid + u * kCatchThreads];
-          if (i != kFull) {
-            const float r = sh.tab.vals[tid + u * kCatchThreads];
-            __stcg(D + i, r);
-            const uint32_t blk = i / kWarpTile - a / kWarpTile;
-            if (blk < (uint32_t)kCatchBlocks) atomicMax(sh.bmax + blk, key_of(r));
-            else atomicMax(blk_max + i / kWarpTile, key_of(r));   // a piece spanning more blocks than the table holds
-          }
-        }
-      }
-      __syncthreads();
-      for (int s = tid; s < kCatchBlocks; s += kCatchThreads) {
-        const uint32_t v = sh.bmax[s];
-        if (v) atomicMax(blk_max + a / kWarpTile + s, v);
-      }
-    }
-    asm volatile("cp.async.wait_all;" ::: "memory");   // (copies of a piece that turned out empty: nothing may still land)
-    if (b == range_b) break;
-    __syncthreads();   // the tables and the pieces are read until here
-    if (tid < count) sh.lo[tid] = sh.hi[tid];
-    a = b;
+  };
+  uint32_t blk = kFull, blk1 = next_block();   // the block in hand, the one that is on its way
+  const uint32_t first_blk = blk1;
+  load_pos(blk1);
+  const uint32_t slot0 = first_blk == kFull ? 0u : first_blk * kWarpTile;   // first slot of this part
+  uint32_t cands = 0;
+  uint32_t seg = 0, seg_end = 0, L = 0;        // layer of the block in hand (blocks come in ascending order)
+  if (first_blk != kFull) {
+    seg = S == 1 ? 0u : __ldg(ws.blk_seg + first_blk);
+    seg_end = S == 1 ? n : __ldg(ws.seg_off + seg + 1);
+    if (SCAN) L = a.L_in[seg];
   }
-  __syncthreads();   // the tables are free for the next range
+  const int sw = (lane >> 1) & 3;
+  uint32_t total = 0, total1 = 0, phase = 0;   // entries of the first 32 packets in blk, in blk1; stage of blk
+  while (blk != kFull || blk1 != kFull) {
+    const uint32_t blk2 = blk1 == kFull ? kFull : next_block();
+    if (blk1 != kFull) {
+      FoldStage* const st = reinterpret_cast<FoldStage*>(stages + (phase ^ stage_bytes));
+      const float* const src = D + (size_t)blk1 * kWarpTile + lane * 4;
+      const uint32_t len = blk1 + 1 < NB ? (uint32_t)kWarpTile : ws.n_pad - blk1 * kWarpTile;
+#pragma unroll
+      for (int j = 0; j < kVecIters; ++j)
+        if ((uint32_t)(j * 128 + lane * 4) < len) cp_async16(st->tile + j * 128 + fill, src + j * 128);
+      if (count) {
+        const BlockRuns r = block_runs(lo, hi, my_slot, st->runs, lane, lt);
+        total1 = r.total;
+        fetch_entries(lg, r, 0, min(r.total, ahead), st->runs, st->ent, lane, le);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    load_pos(blk2);
+    if (blk != kFull) {
+    const uint32_t base = blk * kWarpTile;
+    FoldStage* const st = reinterpret_cast<FoldStage*>(stages + phase);
+    float* const t = st->tile;
+    while (base >= seg_end) {
+      ++seg;
+      seg_end = __ldg(ws.seg_off + seg + 1);
+      if (SCAN) L = a.L_in[seg];
+    }
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncwarp();
+    // fold
+    if (count) {
+      uint32_t dirty = subtract_entries(t, st->ent, min(total, ahead), base, n, lane, lt, le);
+      if (total > ahead || count > 32u) dirty |= fold_rest(lg, first, count, ahead, blk, n, st);
+      dirty = __reduce_or_sync(kFull, dirty);
+      if (dirty) {     // changed lines back to memory
+        float* const dst = D + (size_t)base + lane * 4;
+#pragma unroll
+        for (int j = 0; j < kVecIters; ++j)
+          if ((dirty >> (j * 4 + (lane >> 3))) & 1u)
+            __stcg(reinterpret_cast<float4*>(dst + j * 128), *reinterpret_cast<const float4*>(t + j * 128 + fill));
+      }
+    }
+    // scan: bound and candidates
+    uint32_t top;
+    if (blk + 1 < NB && base + kWarpTile <= seg_end) {   // a full block inside one layer
+      float4 v[kVecIters];
+#pragma unroll
+      for (int j = 0; j < kVecIters; ++j) v[j] = *reinterpret_cast<const float4*>(t + (lane * 4 + (j ^ sw)) * 4);
+      float m = 0.f;
+#pragma unroll
+      for (int j = 0; j < kVecIters; ++j)
+        m = fmaxf(fmaxf(m, fmaxf(fabsf(v[j].x), fabsf(v[j].y))), fmaxf(fabsf(v[j].z), fabsf(v[j].w)));
+      const uint32_t own = __float_as_uint(m);
+      top = __reduce_max_sync(kFull, own);
+      if (SCAN && top >= L) {
+        const float Lf = __uint_as_float(L);   // |x| >= Lf  <=>  key(x) >= L for finite x (no flush-to-zero)
+        uint32_t mask = 0;
+        if (own >= L) {
+#pragma unroll
+          for (int j = 0; j < kVecIters; ++j)
+            mask |= ((fabsf(v[j].x) >= Lf ? 1u : 0u) | (fabsf(v[j].y) >= Lf ? 2u : 0u) | (fabsf(v[j].z) >= Lf ? 4u : 0u) |
+                     (fabsf(v[j].w) >= Lf ? 8u : 0u)) << (4 * j);
+        }
+        __syncwarp();
+        uint32_t found;
+        uint32_t pos = slot0 + cands + lane_offsets(__popc(mask), lt, found);
+        cands += found;
+        while (mask) {
+          const uint32_t off = lane * 16 + __ffs(mask) - 1;
+          mask &= mask - 1;
+          const float c = t[tile_place(off)];
+          ws.cand_idx[pos] = base + off;
+          ws.cand_val[pos] = c;
+          ++pos;
+          atomicAdd(seg == main_seg ? sh.hist + (key_of(c) >> 20) : ws.hist1 + (size_t)seg * kBins1 + (key_of(c) >> 20), 1u);
+        }
+      }
+    } else {
+      cands += scan_mixed<SCAN>(ws, a, t, base, seg, slot0 + cands, top);
+      top = __reduce_max_sync(kFull, top);
+    }
+    if (lane == 0) a.blk_max[blk] = top;     // the block's bound is exact again (entries sent later only lower it)
+    __syncwarp();   // the block's stage is free
+    }
+    phase ^= stage_bytes;
+    blk = blk1;
+    blk1 = blk2;
+    total = total1;
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  if (SCAN) {
+    if (lane == 0) {
+      ws.part_cands[cta * nw + warp] = cands;
+      ws.part_slot0[cta * nw + warp] = slot0;
+    }
+    __syncthreads();
+    for (uint32_t b = tid; b < (uint32_t)kBins1; b += nt)
+      if (sh.hist[b]) atomicAdd(ws.hist1 + (size_t)main_seg * kBins1 + b, sh.hist[b]);
+    if (tid == 0) {
+      if (ws.cta_cost != nullptr) ws.cta_cost[cta] = all;
+      atomicAdd(ws.stats + 3, (unsigned long long)groups);
+      atomicAdd(ws.stats + 4, (unsigned long long)sh.read);
+    }
   }
 }
 
