@@ -295,9 +295,8 @@ int dgs_free(dgs_ctx* ctx);
  * whose memory plan is frozen (a pre-sized pool that must not grow, a real-time or
  * serving loop that may not call into the allocator), or a plug-in that is handed
  * buffers but no allocator.  Such a caller cannot give dgs_init an arena either.  Here
- * every byte of scratch (a private copy of x, the candidate list, histograms, the
- * barrier words: about 12.6 MB) lives in one fixed array that is part of the library's
- * device image; each GPU that loads the library holds it until the process exits.
+ * all scratch is shared memory of the one kernel that does the selection; the only global
+ * memory is the status word, which is part of the library's device image.
  *
  *   x        DEVICE f32[n], read only
  *   n, k     1 <= k <= n <= DGS_STATIC_MAX_N; a larger n returns DGS_ELIMIT, other bad
@@ -307,18 +306,15 @@ int dgs_free(dgs_ctx* ctx);
  *   stream   cudaStream_t; the work is enqueued there and the call returns
  *
  * The function calls no cudaMalloc / cudaFree and no allocating library routine.  The
- * first call on each device looks up the address of the array for that device (the
- * device must be current, as for every call) and sizes its launches; make that first
- * call outside any stream capture.  All calls on a device share the one array: it keeps
- * what the previous call left, the function clears what has to start at zero itself, and
- * two calls whose work overlaps on the GPU (different streams, no ordering) race on it --
- * order them. */
+ * first call on each device (which must be current, as for every call) sizes the launches;
+ * make that first call outside any stream capture.  Calls whose work overlaps on the GPU
+ * (different streams, no ordering) share nothing but the status word. */
 int dgs_topk_encode_static(const float* x, uint32_t n, uint32_t k, uint32_t* out_idx, float* out_val, void* stream);
 
 /* Device-side outcome of the dgs_topk_encode_static calls enqueued on `stream` so far.  (No
  * counterpart in the paper.)  dgs_topk_encode_static only enqueues work, so it cannot report a
- * failure that happens on the device: a bounded wait that gave up (DGS_ETIMEOUT) or an
- * internal rank check that failed leave out_idx / out_val partly unwritten.  This call waits
+ * failure that happens on the device: an internal rank check that failed leaves
+ * out_idx / out_val partly unwritten.  This call waits
  * for `stream` (host-side wait), then stores in *device_status the status word of the last
  * call's kernels: 0 = the packet is complete, negative = it is not.  Like the selection itself
  * it allocates nothing (one 4-byte copy from the fixed array). */

@@ -244,8 +244,8 @@ def dgs_timing_trace(ctx: int, cap: int = 65536):
 
 
 def dgs_topk_encode_static(x_ptr: int, n: int, k: int, out_idx_ptr: int, out_val_ptr: int, stream: int = 0) -> None:
-    """Top-k + encode of a flat device vector with no allocation anywhere (scratch is a
-    fixed array inside the library, n <= DGS_STATIC_MAX_N).  Enqueues on `stream`."""
+    """Top-k + encode of a flat device vector with no allocation anywhere (all scratch is
+    shared memory of one kernel, n <= DGS_STATIC_MAX_N).  Enqueues on `stream`."""
     _check(lib().dgs_topk_encode_static(x_ptr, n, k, out_idx_ptr, out_val_ptr, stream or None),
            "dgs_topk_encode_static")
 

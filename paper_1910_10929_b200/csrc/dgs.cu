@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "dgs_kernels.cuh"
+#include "dgs_topk.cuh"
 
 using namespace dgs;
 
@@ -539,12 +540,12 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
     DGS_CUDA(c, cudaGetLastError());
     c->launches += 2;
   }
-  if (MODE == kPull) {
+  if constexpr (MODE == kPull) {
     rc = fold_launch<true>(c, ws, a, worker, st);
     if (rc != DGS_OK) return rc;
   } else {
     TimedLaunch t(c, st, DGS_KERNEL_STREAM_PUSH);
-    k_stream<MODE><<<c->stream_grid[MODE], kThreads, StreamRing<MODE>::kBytes, st>>>(ws, a);
+    k_stream<MODE><<<c->stream_grid[MODE], kThreads, StreamRing::kBytes, st>>>(ws, a);
     DGS_CUDA(c, cudaGetLastError());
     c->launches += 1;
   }
@@ -570,12 +571,12 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
 template <int MODE>
 int occupancy_grids(dgs_ctx* c, int sms) {
   int occ = 0;
-  DGS_CUDA(c, cudaFuncSetAttribute(k_stream<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   StreamRing<MODE>::kBytes));
-  DGS_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_stream<MODE>, kThreads,
-                                                            StreamRing<MODE>::kBytes));
-  if (occ < 1) occ = 1;
-  c->stream_grid[MODE] = std::min(sms * occ, kMaxGrid);
+  if constexpr (MODE != kPull) {
+    DGS_CUDA(c, cudaFuncSetAttribute(k_stream<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, StreamRing::kBytes));
+    DGS_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_stream<MODE>, kThreads, StreamRing::kBytes));
+    if (occ < 1) occ = 1;
+    c->stream_grid[MODE] = std::min(sms * occ, kMaxGrid);
+  }
   DGS_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_hist_all<MODE>, kThreads, 0));
   if (occ < 1) occ = 1;
   c->hist_grid[MODE] = std::min(sms * occ, kMaxGrid);
@@ -1341,107 +1342,52 @@ int dgs_free(dgs_ctx* c) {
 
 }  // extern "C"
 
-// ---- top-k + encode with all scratch in the device image (dgs_topk_encode_static) --------
+// ---- top-k + encode without any scratch in global memory (dgs_topk_encode_static) --------
 namespace {
 
-constexpr uint32_t kStaticMaxN = DGS_STATIC_MAX_N;
-constexpr uint32_t kStaticMaxTiles = kStaticMaxN / kWarpTile;  // one layer starting at 0: no ragged head
-
-struct StaticScratch {
-  float x[kStaticMaxN];            // private copy of the input (the selection clears what it sends)
-  uint32_t cand_idx[kStaticMaxN];
-  float cand_val[kStaticMaxN];
-  Tile tiles[kStaticMaxTiles];
-  uint32_t part_cands[kMaxGrid];
-  uint32_t part_slot0[kMaxGrid];
-  uint2 cta_tot[kMaxWorkers];
-  uint2 seg_start[1];
-  uint32_t hist1[kBins1];
-  uint32_t hist2[kBins2];
-  uint32_t hist3[kBins3];
-  SegDesc seg;
-  SegSel sel;
-  uint32_t seg_off[2];
-  uint32_t seg_tile0[1];
-  uint32_t L_safe[1];
-  uint32_t L_wide[1];
-  uint32_t L_next[1];
-  uint32_t sync[kNumSyncWords];
-  int status;
-  unsigned long long stats[kNumStats];   // the kernels index words 0 .. 4
-};
-static_assert(sizeof(((StaticScratch*)nullptr)->stats) == kNumStats * sizeof(unsigned long long),
-              "the static scratch must hold every counter a Workspace has");
-
-// The scratch itself.  In host code this name is only a handle for cudaGetSymbolAddress,
-// never a device address.
-static __device__ __align__(256) unsigned char g_static_scratch[sizeof(StaticScratch)];
-
-// Tables of a one-layer problem and everything that has to start at zero.
-__global__ void k_static_prepare(StaticScratch* sc, uint32_t n, uint32_t k, uint32_t num_tiles) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < num_tiles) {
-    Tile t;
-    t.start = i * kWarpTile;
-    t.len = (uint16_t)min((uint32_t)kWarpTile, n - i * kWarpTile);
-    t.seg = 0;
-    sc->tiles[i] = t;
-  }
-  if (i < kBins1) sc->hist1[i] = 0;
-  if (i < kBins2) sc->hist2[i] = 0;
-  if (i < kBins3) sc->hist3[i] = 0;
-  if (i < kMaxGrid) {
-    sc->part_cands[i] = 0;
-    sc->part_slot0[i] = 0;
-  }
-  if (i == 0) {
-    sc->seg.tile_begin = 0;
-    sc->seg.tile_end = num_tiles;
-    sc->seg.k[0] = sc->seg.k[1] = k;
-    sc->seg.pkt_off[0] = sc->seg.pkt_off[1] = 0;
-    sc->seg_off[0] = 0;
-    sc->seg_off[1] = n;
-    sc->seg_tile0[0] = 0;
-    sc->sync[kBarCount] = 0;
-    sc->sync[kFail] = 0;
-    sc->status = 0;
-  }
-}
-
-struct StaticDevice {
+struct TopkDevice {
   bool ready = false;
-  StaticScratch* scratch = nullptr;  // device address of g_static_scratch on this device
-  int stream_grid = 0, hist_grid = 0, finalize_grid = 0;
+  uint32_t max_cluster = 0;   // CTAs of the largest cluster the device takes
 };
 constexpr int kMaxDevices = 64;
-StaticDevice g_static_dev[kMaxDevices];
-std::mutex g_static_mu;
+TopkDevice g_topk_dev[kMaxDevices];
+std::mutex g_topk_mu;
+
+struct TopkLaunch {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr;
+  TopkLaunch(uint32_t cluster, uint32_t cap, cudaStream_t st) {
+    std::memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3(cluster);
+    cfg.blockDim = dim3(kTopkThreads);
+    cfg.dynamicSmemBytes = (size_t)kTopkWarps * cap * 8;
+    cfg.stream = st;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = cluster;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+  }
+};
 
 // Once per device, with that device current.
-int static_setup(int dev, StaticDevice** out) {
-  std::lock_guard<std::mutex> lock(g_static_mu);
-  StaticDevice& d = g_static_dev[dev];
+int topk_setup(int dev, const TopkDevice** out) {
+  std::lock_guard<std::mutex> lock(g_topk_mu);
+  TopkDevice& d = g_topk_dev[dev];
   if (!d.ready) {
-    void* p = nullptr;
-    if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess || !p) return DGS_ECUDA;
-    int sms = 0, coop = 0, occ = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return DGS_ECUDA;
-    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) return DGS_ECUDA;
-    if (cudaFuncSetAttribute(k_stream<kPull>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             StreamRing<kPull>::kBytes) != cudaSuccess)
+    if (cudaFuncSetAttribute(k_topk, cudaFuncAttributeMaxDynamicSharedMemorySize, kTopkWarps * (int)kTopkCap * 8) != cudaSuccess ||
+        cudaFuncSetAttribute(k_topk, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
       return DGS_ECUDA;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_stream<kPull>, kThreads, StreamRing<kPull>::kBytes) !=
-        cudaSuccess)
-      return DGS_ECUDA;
-    d.stream_grid = std::min(sms * std::max(occ, 1), kMaxGrid);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_hist_all<kPull>, kThreads, 0) != cudaSuccess) return DGS_ECUDA;
-    d.hist_grid = std::min(sms * std::max(occ, 1), kMaxGrid);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_finalize<kPull>, kThreads, finalize_dyn_bytes(1)) !=
-            cudaSuccess ||
-        occ < 1)
-      return DGS_ECUDA;
-    d.finalize_grid = std::min(std::min(sms * occ, kMaxWorkers), kFinalizeWorkers);
-    d.scratch = static_cast<StaticScratch*>(p);
+    for (uint32_t c = kTopkMaxCluster; c >= 1; c /= 2) {
+      const TopkLaunch l(c, kTopkCap, nullptr);
+      int clusters = 0;
+      if (cudaOccupancyMaxActiveClusters(&clusters, k_topk, &l.cfg) == cudaSuccess && clusters > 0) {
+        d.max_cluster = c;
+        break;
+      }
+      cudaGetLastError();
+    }
+    if (d.max_cluster == 0) return DGS_ECUDA;
     d.ready = true;
   }
   *out = &d;
@@ -1453,90 +1399,27 @@ int static_setup(int dev, StaticDevice** out) {
 extern "C" int dgs_topk_encode_static(const float* x, uint32_t n, uint32_t k, uint32_t* out_idx, float* out_val,
                                       void* stream) {
   if (!x || !out_idx || !out_val || n == 0 || k == 0 || k > n) return DGS_EINVAL;
-  if (n > kStaticMaxN) return DGS_ELIMIT;
+  if (n > DGS_STATIC_MAX_N) return DGS_ELIMIT;
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return DGS_ECUDA;
-  StaticDevice* d = nullptr;
-  const int rc = static_setup(dev, &d);
+  const TopkDevice* d = nullptr;
+  const int rc = topk_setup(dev, &d);
   if (rc != DGS_OK) return rc;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  StaticScratch* sc = d->scratch;  // device address: only ever dereferenced by kernels
-  const uint32_t num_tiles = (n + kWarpTile - 1) / kWarpTile;
-
-  Workspace ws;
-  ws.tiles = sc->tiles;
-  ws.segs = &sc->seg;
-  ws.num_tiles = num_tiles;
-  ws.num_segs = 1;
-  ws.cand_idx = sc->cand_idx;
-  ws.cand_val = sc->cand_val;
-  ws.part_cands = sc->part_cands;
-  ws.part_slot0 = sc->part_slot0;
-  ws.n = n;
-  ws.n_pad = kStaticMaxN;
-  ws.num_blocks = num_tiles;
-  ws.blk_seg = nullptr;      // only k_fold looks at blocks
-  ws.plan = nullptr;
-  ws.cta_cost = nullptr;
-  ws.part_cap = 0;
-  ws.seg_off = sc->seg_off;
-  ws.seg_tile0 = sc->seg_tile0;
-  ws.cta_tot = sc->cta_tot;
-  ws.seg_start = sc->seg_start;
-  ws.hist1 = sc->hist1;
-  ws.hist2 = sc->hist2;
-  ws.hist3 = sc->hist3;
-  ws.sel = &sc->sel;
-  ws.L_safe = sc->L_safe;
-  ws.L_wide = sc->L_wide;
-  ws.sync = sc->sync;
-  ws.status = &sc->status;
-  ws.stats = sc->stats;
-
-  SelArgs a;
-  std::memset(&a, 0, sizeof(a));
-  a.D = sc->x;
-  a.L_in = sc->L_safe;
-  a.L_next = sc->L_next;
-  a.pkt_idx = out_idx;
-  a.pkt_val = out_val;
-  a.pkt_count = k;
-  a.m = 1.0f;
-  a.inv_m = 1.0f;
-  a.force_two_pass = 1;
-  a.speculate = 0;
-  a.workers = (uint32_t)d->finalize_grid;
-  a.seq = 0;
-
-  if (cudaMemcpyAsync(sc->x, x, (size_t)n * 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return DGS_ECUDA;
-  // every launch is checked before the next one is enqueued: a kernel that did not start must not be
-  // followed by kernels that count on what it clears (peek: an earlier error of the caller's stays the caller's)
-  const uint32_t prep_items = std::max<uint32_t>(num_tiles, kBins1);
-  k_static_prepare<<<(prep_items + kThreads - 1) / kThreads, kThreads, 0, st>>>(sc, n, k, num_tiles);
-  if (cudaPeekAtLastError() != cudaSuccess) return DGS_ECUDA;
-  k_hist_all<kPull><<<d->hist_grid, kThreads, 0, st>>>(ws, a);
-  if (cudaPeekAtLastError() != cudaSuccess) return DGS_ECUDA;
-  k_pick_lower<kPull><<<1, kThreads, 0, st>>>(ws);
-  if (cudaPeekAtLastError() != cudaSuccess) return DGS_ECUDA;
-  k_stream<kPull><<<d->stream_grid, kThreads, StreamRing<kPull>::kBytes, st>>>(ws, a);
-  if (cudaPeekAtLastError() != cudaSuccess) return DGS_ECUDA;
-  void* args[] = {(void*)&ws, (void*)&a};
-  if (cudaLaunchCooperativeKernel((const void*)k_finalize<kPull>, dim3(d->finalize_grid), dim3(kThreads), args,
-                                  finalize_dyn_bytes(1), st) != cudaSuccess)
-    return DGS_ECUDA;
-  return DGS_OK;
+  // a CTA per 4096 elements (four a thread), up to the largest cluster
+  uint32_t cluster = 1;
+  while (cluster < d->max_cluster && cluster * 4096u < n) cluster *= 2;
+  // the lists hold a warp's whole slice where that fits
+  const uint32_t slice = ((n + 31) / 32 + cluster * kTopkWarps - 1) / (cluster * kTopkWarps) * 32;
+  const uint32_t cap = std::min(kTopkCap, slice);
+  const TopkLaunch l(cluster, cap, static_cast<cudaStream_t>(stream));
+  return cudaLaunchKernelEx(&l.cfg, k_topk, x, n, k, out_idx, out_val, cap) == cudaSuccess ? DGS_OK : DGS_ECUDA;
 }
 
 extern "C" int dgs_topk_encode_static_status(void* stream, int* device_status) {
   if (!device_status) return DGS_EINVAL;
-  int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return DGS_ECUDA;
-  StaticDevice* d = nullptr;
-  const int rc = static_setup(dev, &d);
-  if (rc != DGS_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int word = 0;
-  if (cudaMemcpyAsync(&word, &d->scratch->status, sizeof(word), cudaMemcpyDeviceToHost, st) != cudaSuccess)
+  if (cudaMemcpyFromSymbolAsync(&word, g_topk_status, sizeof(word), 0, cudaMemcpyDeviceToHost, st) != cudaSuccess)
     return DGS_ECUDA;
   if (cudaStreamSynchronize(st) != cudaSuccess) return DGS_ECUDA;
   *device_status = word;

@@ -470,8 +470,8 @@ __device__ void stream_tiles(const Workspace& ws, const SelArgs& a, const uint32
   }
 }
 
-// Step one for a tile staged in shared memory (su: the tile of the state vector, sg: the tile
-// of the gradient, push only): candidate mask, new velocity (push).
+// Step one for a tile of a push staged in shared memory (su: the tile of the state vector, sg: the tile of the
+// gradient): candidate mask, new velocity.
 template <int MODE>
 __device__ __forceinline__ uint32_t tile_mask_smem(const SelArgs& a, uint32_t tile_start, const float* su,
                                                    const float* sg, uint32_t L, int lane, float* __restrict__ out) {
@@ -482,23 +482,19 @@ __device__ __forceinline__ uint32_t tile_mask_smem(const SelArgs& a, uint32_t ti
 #pragma unroll
   for (int j = 0; j < kVecIters; ++j) {
     float4 x = pu[j * 32];
-    if (MODE != kPull) {
-      const float4 g = pg[j * 32];
-      x.x = combine<MODE>(x.x, g.x, a.m, a.lr);
-      x.y = combine<MODE>(x.y, g.y, a.m, a.lr);
-      x.z = combine<MODE>(x.z, g.z, a.m, a.lr);
-      x.w = combine<MODE>(x.w, g.w, a.m, a.lr);
-    }
+    const float4 g = pg[j * 32];
+    x.x = combine<MODE>(x.x, g.x, a.m, a.lr);
+    x.y = combine<MODE>(x.y, g.y, a.m, a.lr);
+    x.z = combine<MODE>(x.z, g.z, a.m, a.lr);
+    x.w = combine<MODE>(x.w, g.w, a.m, a.lr);
     const bool c0 = fabsf(x.x) >= Lf, c1 = fabsf(x.y) >= Lf, c2 = fabsf(x.z) >= Lf, c3 = fabsf(x.w) >= Lf;
     mask |= ((c0 ? 1u : 0u) | (c1 ? 2u : 0u) | (c2 ? 4u : 0u) | (c3 ? 8u : 0u)) << (4 * j);
-    if (MODE != kPull) {
-      float4 o;
-      o.x = c0 ? x.x : unsent<MODE>(x.x, a.inv_m);
-      o.y = c1 ? x.y : unsent<MODE>(x.y, a.inv_m);
-      o.z = c2 ? x.z : unsent<MODE>(x.z, a.inv_m);
-      o.w = c3 ? x.w : unsent<MODE>(x.w, a.inv_m);
-      __stcs(reinterpret_cast<float4*>(out + tile_start) + lane + j * 32, o);
-    }
+    float4 o;
+    o.x = c0 ? x.x : unsent<MODE>(x.x, a.inv_m);
+    o.y = c1 ? x.y : unsent<MODE>(x.y, a.inv_m);
+    o.z = c2 ? x.z : unsent<MODE>(x.z, a.inv_m);
+    o.w = c3 ? x.w : unsent<MODE>(x.w, a.inv_m);
+    __stcs(reinterpret_cast<float4*>(out + tile_start) + lane + j * 32, o);
   }
   return mask;
 }
@@ -513,14 +509,11 @@ __device__ __forceinline__ uint32_t tile_mask_smem(const SelArgs& a, uint32_t ti
 // of them in flight.
 constexpr int kStageTiles = kWarps;                        // one tile per warp and stage
 constexpr int kStageFloats = kStageTiles * kWarpTile;      // per input array
-// The ring: three stages for a push (96 KB, two CTAs per SM, 128 KB of the SM's shared memory in flight),
-// four for the staged form of a pull.
-template <int MODE> struct StreamRing {
-  static constexpr int kInputs = MODE == kPull ? 1 : 2;
-  static constexpr int kStages = MODE == kPull ? 4 : 3;
-  static constexpr int kStageBytes = kInputs * kStageFloats * 4;          // 16 KB per input
-  static constexpr int kRingBytes = kStages * kStageBytes;
-  static constexpr int kBytes = kRingBytes;
+// The ring: three stages (96 KB, two CTAs per SM, 128 KB of the SM's shared memory in flight).
+struct StreamRing {
+  static constexpr int kStages = 3;
+  static constexpr int kStageBytes = 2 * kStageFloats * 4;                // 16 KB per input
+  static constexpr int kBytes = kStages * kStageBytes;
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -555,7 +548,8 @@ template <int MODE>
 __device__ void stream_tiles_tma(const Workspace& ws, const SelArgs& a, const uint32_t* Larr,
                                  const float* __restrict__ in, float* __restrict__ out, uint32_t cta, uint32_t G,
                                  StreamShared& sh, float* ring, uint64_t* full, int* s_dead) {
-  using R = StreamRing<MODE>;
+  using R = StreamRing;
+  static_assert(MODE != kPull, "a pull's pass is k_fold");
   static_assert(R::kStages >= 2, "the ring needs a stage in flight besides the one being read");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t t0 = part_first_tile(cta, G, ws.num_tiles), t1 = part_first_tile(cta + 1, G, ws.num_tiles);
@@ -611,9 +605,9 @@ __device__ void stream_tiles_tma(const Workspace& ws, const SelArgs& a, const ui
       const uint32_t bytes = tiles_here * kWarpTile * 4;
       const size_t elem = (size_t)e0 + (size_t)chunk * kStageFloats;
       float* dst = ring + (size_t)st * (R::kStageBytes / 4);
-      mbar_expect_tx(full + st, bytes * R::kInputs);
+      mbar_expect_tx(full + st, bytes * 2);
       bulk_load(dst, in + elem, bytes, full + st);
-      if (MODE != kPull) bulk_load(dst + kStageFloats, a.grad + elem, bytes, full + st);
+      bulk_load(dst + kStageFloats, a.grad + elem, bytes, full + st);
     };
     uint32_t issued = 0;                                  // thread 0: chunks asked for
     if (threadIdx.x == 0)
@@ -639,7 +633,7 @@ __device__ void stream_tiles_tma(const Workspace& ws, const SelArgs& a, const ui
       const uint32_t base = slot0 + cur + round_offset(sh.wcnt[use & 1], warp, total);
       cur += total;
       tile_emit(ws, e0 + tl * kWarpTile, mask, base, lane, [&](uint32_t off) {
-        return combine<MODE>(su[off], MODE != kPull ? su[kStageFloats + off] : 0.f, a.m, a.lr);
+        return combine<MODE>(su[off], su[kStageFloats + off], a.m, a.lr);
       }, [&](uint32_t, uint32_t key) { atomicAdd(sh.hist + (key >> 20), 1u); });
     }
     if (*s_dead) break;
@@ -1406,16 +1400,10 @@ template <int MODE>
 __global__ void __maxnreg__(64) k_stream(Workspace ws, SelArgs a) {
   extern __shared__ __align__(128) unsigned char dyn_smem[];   // the ring of stages
   __shared__ StreamShared sh;
-  __shared__ __align__(8) uint64_t full[StreamRing<MODE>::kStages];
+  __shared__ __align__(8) uint64_t full[StreamRing::kStages];
   __shared__ int s_dead;
-  const float* in;
-  float* out = nullptr;
-  if (MODE == kPull) {
-    in = a.D;
-  } else {
-    in = *a.u_cur_slot;
-    out = *a.u_spare_slot;
-  }
+  const float* in = *a.u_cur_slot;
+  float* out = *a.u_spare_slot;
   if (blockIdx.x == 0 && threadIdx.x == 0) ws.sync[kBarCount] = 0;   // for the finalize launch that follows
   stream_tiles_tma<MODE>(ws, a, a.L_in, in, out, blockIdx.x, gridDim.x, sh, reinterpret_cast<float*>(dyn_smem), full,
                          &s_dead);

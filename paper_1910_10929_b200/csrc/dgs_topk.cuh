@@ -1,0 +1,254 @@
+// Top-k + encode of one short flat vector in one kernel (dgs_topk_encode_static).
+//
+// One cluster of up to 16 CTAs does the whole selection: its CTAs are resident together and meet at the hardware
+// barrier of the cluster, and their histograms are added up in the shared memory of the first of them.  What bounds it
+// is the chain of those meetings, not the bytes (4 MB at the most, read once or twice).
+//   sample      every CTA takes the same sample of at most kTopkSample elements, evenly spaced over the vector, and
+//               from it a bound L that very likely admits at least k elements and not many more.  No meeting: all
+//               CTAs find the same bound.
+//   list        every warp reads a slice of the vector and lists the elements whose key is at least L, in index order,
+//               in shared memory; their top 11 key bits are counted.
+//   levels      three radix levels (11 + 10 + 10 key bits) over the lists give the k-th largest key T and the number r
+//               of entries equal to T that still fit.
+//   emit        counts of (key > T, key == T) per warp, prefix sums over warps and CTAs, packet in index order.
+// If the lists hold fewer than k elements, or one of them overflows (the sample said nothing about the vector, or most
+// of it is equal), the levels and the emit visit the slices themselves instead.  The result never depends on the sample.
+#pragma once
+#include <cooperative_groups.h>
+
+#include "dgs_kernels.cuh"
+
+namespace dgs {
+
+constexpr int kTopkThreads = 1024, kTopkWarps = kTopkThreads / 32;
+constexpr uint32_t kTopkMaxCluster = 16;   // (more than 8 is not portable to every GPU: the launch asks for it)
+constexpr uint32_t kTopkSample = 4096;
+constexpr uint32_t kTopkCap = 736;         // most elements a warp can list: 184 KB of lists per CTA
+constexpr int kStatusRank = -1002;         // an entry got a rank that cannot be
+
+// Outcome of the last call's kernel on the device: 0, or a negative word if its packet is not complete.
+__device__ int g_topk_status;
+
+struct TopkShared {
+  uint32_t hist[kBins1];                     // this CTA's counts of the level in hand
+  uint32_t sum1[kBins1], again1[kBins1];     // first CTA of the cluster: counts of all CTAs, level 1 (lists; slices)
+  uint32_t sum2[kBins2], sum3[kBins3];       //                                               levels 2 and 3
+  uint32_t warp_sum[kTopkWarps];
+  uint2 warp_tot[kTopkWarps];                // (key > T, key == T) of each warp
+  uint2 cta_tot[kTopkMaxCluster];            // of each CTA of the cluster
+  uint32_t overflow;                         // first CTA: some list was too short
+  uint32_t res[2];
+};
+
+// From a histogram of B bins (anywhere in the cluster's shared memory), counting from the top bin down, the bin that
+// holds the k-th entry and how many entries of that bin are needed.  Returns the total count; bin and need are valid
+// if it is at least k.  The same for every thread of the CTA.
+template <int B>
+__device__ uint32_t topk_pick(const uint32_t* hist, uint32_t k, uint32_t& bin, uint32_t& need, TopkShared& sh) {
+  constexpr int PER = B / kTopkThreads;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t c[PER], sum = 0;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    c[j] = hist[B - 1 - (int)threadIdx.x * PER - j];
+    sum += c[j];
+  }
+  uint32_t incl = sum;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint32_t o = __shfl_up_sync(kFull, incl, d);
+    if (lane >= d) incl += o;
+  }
+  if (lane == 31) sh.warp_sum[warp] = incl;
+  __syncthreads();
+  const uint32_t w = sh.warp_sum[lane];       // as many warps as lanes
+  uint32_t winc = w;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint32_t o = __shfl_up_sync(kFull, winc, d);
+    if (lane >= d) winc += o;
+  }
+  const uint32_t total = __shfl_sync(kFull, winc, 31);
+  uint32_t above = __shfl_sync(kFull, winc - w, warp) + incl - sum;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    if (above < k && k <= above + c[j]) {
+      sh.res[0] = B - 1 - threadIdx.x * PER - j;
+      sh.res[1] = k - above;
+    }
+    above += c[j];
+  }
+  __syncthreads();
+  bin = sh.res[0];
+  need = sh.res[1];
+  return total;
+}
+
+__global__ void __launch_bounds__(kTopkThreads, 1) k_topk(const float* __restrict__ x, uint32_t n, uint32_t k,
+                                                         uint32_t* __restrict__ out_idx, float* __restrict__ out_val,
+                                                         uint32_t cap) {
+  extern __shared__ __align__(16) unsigned char topk_dyn[];
+  __shared__ TopkShared sh;
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const uint32_t C = gridDim.x, cta = blockIdx.x, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, lt = lanemask_lt();
+  uint32_t* const my_idx = reinterpret_cast<uint32_t*>(topk_dyn) + warp * 2u * cap;
+  float* const my_val = reinterpret_cast<float*>(my_idx + cap);
+  TopkShared* const head = cl.map_shared_rank(&sh, 0);
+
+  for (uint32_t b = tid; b < (uint32_t)kBins1; b += kTopkThreads) sh.hist[b] = sh.sum1[b] = sh.again1[b] = 0;
+  sh.sum2[tid] = sh.sum3[tid] = 0;
+  if (tid == 0) {
+    sh.overflow = 0;
+    if (cta == 0) g_topk_status = 0;
+  }
+  __syncthreads();
+  cl.barrier_arrive();            // the first CTA's sums are clear (waited for before anything is added to them)
+
+  // this warp's slice of the vector, in units of 32 elements
+  const uint32_t units = (n + 31u) / 32u, g = cta * kTopkWarps + warp;
+  const uint32_t i0 = (uint32_t)((uint64_t)g * units / (C * kTopkWarps)) * 32u;
+  const uint32_t i1 = min(n, (uint32_t)((uint64_t)(g + 1) * units / (C * kTopkWarps)) * 32u);
+
+  // sample -> bound
+  uint32_t L = 0;
+  {
+    const uint32_t s = min(n, kTopkSample);
+    float v[kTopkSample / kTopkThreads];
+#pragma unroll
+    for (uint32_t j = 0; j < kTopkSample / kTopkThreads; ++j) {
+      const uint32_t q = tid + j * kTopkThreads;
+      v[j] = q < s ? __ldg(x + (uint32_t)((uint64_t)q * n / s)) : 0.f;
+    }
+#pragma unroll
+    for (uint32_t j = 0; j < kTopkSample / kTopkThreads; ++j)
+      if (tid + j * kTopkThreads < s) atomicAdd(sh.hist + (key_of(v[j]) >> 20), 1u);
+    __syncthreads();
+    // Of k in n, k s / n are expected in the sample; four standard deviations and a few more, so that at least k
+    // elements lie above the bound all but surely.  A sample of everything needs no margin.
+    uint32_t want = k;
+    if (s < n) {
+      const float mean = (float)k * ((float)s / (float)n);
+      want = (uint32_t)(mean + 4.f * sqrtf(mean)) + 8u;
+    }
+    uint32_t bin, need;
+    if (topk_pick<kBins1>(sh.hist, want, bin, need, sh) >= want) L = bin << 20;
+    for (uint32_t b = tid; b < (uint32_t)kBins1; b += kTopkThreads) sh.hist[b] = 0;
+    __syncthreads();
+  }
+
+  // list
+  uint32_t listed = 0;
+  for (uint32_t base = i0; base < i1; base += 256) {
+    float v[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const uint32_t i = base + j * 32u + lane;
+      v[j] = i < i1 ? __ldg(x + i) : 0.f;
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const uint32_t i = base + j * 32u + lane;
+      const bool in = i < i1 && key_of(v[j]) >= L;
+      const uint32_t m = __ballot_sync(kFull, in);
+      if (in) {
+        const uint32_t at = listed + __popc(m & lt);
+        if (at < cap) {
+          my_idx[at] = i;
+          my_val[at] = v[j];
+          atomicAdd(sh.hist + (key_of(v[j]) >> 20), 1u);
+        }
+      }
+      listed += __popc(m);
+    }
+  }
+  __syncthreads();
+  cl.barrier_wait();
+  if (lane == 0 && listed > cap) head->overflow = 1;
+  auto add_up = [&](uint32_t* sum, uint32_t bins) {   // this CTA's counts to the first CTA's sums; then all are complete
+    for (uint32_t b = tid; b < bins; b += kTopkThreads) {
+      const uint32_t c = sh.hist[b];
+      if (c) {
+        atomicAdd(sum + b, c);
+        sh.hist[b] = 0;
+      }
+    }
+    cl.sync();
+  };
+  add_up(head->sum1, kBins1);
+  uint32_t bin, need;
+  const uint32_t found = topk_pick<kBins1>(head->sum1, k, bin, need, sh);
+  const bool slices = head->overflow != 0 || found < k;   // the same in the whole cluster
+
+  // visits this warp's elements in index order, 32 at a time: fn(valid, index, value)
+  auto each = [&](auto fn) {
+    if (slices) {
+      for (uint32_t i = i0 + lane; i - lane < i1; i += 32) {
+        const bool valid = i < i1;
+        fn(valid, i, valid ? __ldg(x + i) : 0.f);
+      }
+    } else {
+      for (uint32_t p = lane; p - lane < listed; p += 32) {
+        const bool valid = p < listed;
+        fn(valid, valid ? my_idx[p] : 0u, valid ? my_val[p] : 0.f);
+      }
+    }
+  };
+  if (slices) {
+    each([&](bool valid, uint32_t, float v) { hist_add(sh.hist, key_of(v) >> 20, valid, (int)lane); });
+    __syncthreads();
+    add_up(head->again1, kBins1);
+    topk_pick<kBins1>(head->again1, k, bin, need, sh);
+  }
+  uint32_t prefix = bin;
+#pragma unroll 1
+  for (int level = 2; level <= 3; ++level) {
+    const int shift = level == 2 ? 10 : 0;
+    each([&](bool valid, uint32_t, float v) {
+      const uint32_t key = key_of(v);
+      if (valid && (key >> (shift + 10)) == prefix) atomicAdd(sh.hist + ((key >> shift) & 1023u), 1u);
+    });
+    __syncthreads();
+    uint32_t* const sum = level == 2 ? head->sum2 : head->sum3;
+    add_up(sum, 1024);
+    topk_pick<1024>(sum, need, bin, need, sh);
+    prefix = (prefix << 10) | bin;
+  }
+  const uint32_t T = prefix, r = need;
+
+  // how many of either kind each warp has, and the warps and CTAs before it
+  uint32_t gt = 0, eq = 0;
+  each([&](bool valid, uint32_t, float v) {
+    const uint32_t key = key_of(v);
+    gt += __popc(__ballot_sync(kFull, valid && key > T));
+    eq += __popc(__ballot_sync(kFull, valid && key == T));
+  });
+  if (lane == 0) sh.warp_tot[warp] = make_uint2(gt, eq);
+  __syncthreads();
+  const uint2 q = sh.warp_tot[lane];
+  uint32_t gt_before = __reduce_add_sync(kFull, lane < warp ? q.x : 0u), eq_before = __reduce_add_sync(kFull, lane < warp ? q.y : 0u);
+  const uint32_t gt_all = __reduce_add_sync(kFull, q.x), eq_all = __reduce_add_sync(kFull, q.y);
+  if (tid < C) cl.map_shared_rank(&sh, tid)->cta_tot[cta] = make_uint2(gt_all, eq_all);
+  cl.sync();                      // (nobody looks into another CTA's memory after this)
+  const uint2 o = lane < cta ? sh.cta_tot[lane] : make_uint2(0, 0);
+  gt_before += __reduce_add_sync(kFull, o.x);
+  eq_before += __reduce_add_sync(kFull, o.y);
+  each([&](bool valid, uint32_t i, float v) {
+    const uint32_t key = key_of(v);
+    const uint32_t mg = __ballot_sync(kFull, valid && key > T), me = __ballot_sync(kFull, valid && key == T);
+    const uint32_t eq_rank = eq_before + __popc(me & lt);
+    if (valid && (key > T || (key == T && eq_rank < r))) {
+      const uint32_t pos = gt_before + __popc(mg & lt) + min(eq_rank, r);
+      if (pos < k) {
+        out_idx[pos] = i;
+        out_val[pos] = v;
+      } else {
+        atomicMin(&g_topk_status, kStatusRank);
+      }
+    }
+    gt_before += __popc(mg);
+    eq_before += __popc(me);
+  });
+}
+
+}  // namespace dgs
