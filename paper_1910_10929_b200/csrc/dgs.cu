@@ -1405,11 +1405,13 @@ extern "C" int dgs_topk_encode_static(const float* x, uint32_t n, uint32_t k, ui
   const TopkDevice* d = nullptr;
   const int rc = topk_setup(dev, &d);
   if (rc != DGS_OK) return rc;
-  // a CTA per 4096 elements (four a thread), up to the largest cluster
+  // An element a thread, up to the largest cluster: the barriers of 16 CTAs cost no more than those of 2 (16384
+  // elements: 12.3 us with 16, 13.0 with 4, 14.3 with 1; 262144: 14.3, 21.7, 45).
   uint32_t cluster = 1;
-  while (cluster < d->max_cluster && cluster * 4096u < n) cluster *= 2;
-  // the lists hold a warp's whole slice where that fits
-  const uint32_t slice = ((n + 31) / 32 + cluster * kTopkWarps - 1) / (cluster * kTopkWarps) * 32;
+  while (cluster < d->max_cluster && cluster * (uint32_t)kTopkThreads < n) cluster *= 2;
+  // the lists hold a warp's whole slice where that fits (slices as k_topk cuts them)
+  const uint32_t unit = n >= cluster * kTopkWarps * 512u ? 512u : 32u;
+  const uint32_t slice = ((n + unit - 1) / unit + cluster * kTopkWarps - 1) / (cluster * kTopkWarps) * unit;
   const uint32_t cap = std::min(kTopkCap, slice);
   const TopkLaunch l(cluster, cap, static_cast<cudaStream_t>(stream));
   return cudaLaunchKernelEx(&l.cfg, k_topk, x, n, k, out_idx, out_val, cap) == cudaSuccess ? DGS_OK : DGS_ECUDA;
