@@ -41,6 +41,7 @@ constexpr int kPullSets = kServerStreams;  // scratch sets of the pulls
 constexpr int kAllSets = kPushSets + kPullSets;
 constexpr int kLogRingMax = 128;            // most packets the apply log keeps
 constexpr int kLogSlack = 32;               // slots of the log beyond one per worker
+constexpr uint64_t kListCap = 4096;         // most entries of a layer's list of candidates in the k-th's bin
 enum StreamId : int { kStW0 = 0, kStApply = kWorkerStreams, kStS0 = kWorkerStreams + 1,
                       kNumStreams = kWorkerStreams + 1 + kServerStreams };
 
@@ -48,8 +49,8 @@ inline uint64_t align_up(uint64_t x, uint64_t a) { return (x + a - 1) / a * a; }
 
 // Scratch of one selection pipeline ([0] push, on the worker stream; [1] pull, on the server stream)
 struct ScratchLayout {
-  uint64_t cand_idx, cand_val, part_cands, part_slot0, plan, cta_cost, cta_tot, seg_start;
-  uint64_t hist1, hist2, hist3, sel, L_safe, L_wide, sync;
+  uint64_t cand_idx, cand_val, part_cands, part_slot0, plan, cta_cost, cta_tot, cta_eq, tab, list;
+  uint64_t hist1, list_cnt, sel, L_safe, L_wide, sync;
   uint64_t zero_begin, zero_end;  // [hist1, end of sync): cleared at init
 };
 
@@ -61,7 +62,7 @@ struct Layout {
   uint64_t theta, u, D, theta_local, grad_stage;
   uint64_t pkt_idx[kPushSlots + kPullSlots], pkt_val[kPushSlots + kPullSlots];  // push slots, then pull slots
   uint64_t var_idx[kVarSlots], var_val[kVarSlots], var_count[kVarSlots], L_one;
-  uint64_t tiles, segs, seg_off, seg_tile0, blk_seg;
+  uint64_t tiles, segs, seg_off, blk_seg;
   ScratchLayout sc[kAllSets];  // push sets, then pull sets
   uint64_t L_next, u_slots, status, stats;
   uint64_t log_ent, log_pos;
@@ -95,7 +96,7 @@ int check_config(const dgs_config* c) {
 // Tiles: every layer is cut at the global multiples of kWarpTile, so that all full
 // tiles start 2 KB-aligned and only the first and last tile of a layer can be ragged.
 void build_tiles(const dgs_config* c, std::vector<Tile>* tiles, std::vector<SegDesc>* segs) {
-  uint32_t koff[2] = {0, 0};
+  uint32_t koff[2] = {0, 0}, list_off = 0;
   for (uint32_t s = 0; s < c->num_segments; ++s) {
     const dgs_segment& g = c->segments[s];
     SegDesc d;
@@ -117,6 +118,9 @@ void build_tiles(const dgs_config* c, std::vector<Tile>* tiles, std::vector<SegD
     d.k[1] = g.k_pull;
     d.pkt_off[0] = koff[0];
     d.pkt_off[1] = koff[1];
+    d.list_off = list_off;
+    d.list_cap = (uint32_t)std::min<uint64_t>(g.len, kListCap);
+    list_off += d.list_cap;
     koff[0] += g.k_push;
     koff[1] += g.k_pull;
     segs->push_back(d);
@@ -139,9 +143,11 @@ void make_layout(const dgs_config* c, Layout* L) {
   L->num_tiles = count_tiles(c);
   L->num_blocks = (uint32_t)((c->n + kWarpTile - 1) / kWarpTile);
   L->K[0] = L->K[1] = 0;
+  uint64_t list_entries = 0;
   for (uint32_t s = 0; s < S; ++s) {
     L->K[0] += c->segments[s].k_push;
     L->K[1] += c->segments[s].k_pull;
+    list_entries += std::min<uint64_t>(c->segments[s].len, kListCap);
   }
   uint64_t off = 0;
   auto take = [&](uint64_t bytes) {
@@ -169,7 +175,6 @@ void make_layout(const dgs_config* c, Layout* L) {
   L->tiles = take((uint64_t)L->num_tiles * sizeof(Tile));
   L->segs = take(S * sizeof(SegDesc));
   L->seg_off = take((S + 1) * 4);
-  L->seg_tile0 = take(S * 4);
   L->blk_seg = take((uint64_t)L->num_blocks * 4);
   for (int k = 0; k < kAllSets; ++k) {
     ScratchLayout& sc = L->sc[k];
@@ -180,11 +185,12 @@ void make_layout(const dgs_config* c, Layout* L) {
     sc.plan = take((uint64_t)(kMaxFoldGrid + 1) * 4);
     sc.cta_cost = take((uint64_t)kMaxFoldGrid * 4);
     sc.cta_tot = take((uint64_t)kMaxWorkers * sizeof(uint2));
-    sc.seg_start = take(S * sizeof(uint2));
+    sc.cta_eq = take((uint64_t)kMaxWorkers * 4);
+    sc.tab = take((S + kMaxWorkers) * sizeof(LayerPick));
+    sc.list = take(list_entries * sizeof(uint2));
     sc.hist1 = take(S * kBins1 * 4);
     sc.zero_begin = sc.hist1;
-    sc.hist2 = take(S * kBins2 * 4);
-    sc.hist3 = take(S * kBins3 * 4);
+    sc.list_cnt = take(S * 4);
     sc.sel = take(S * sizeof(SegSel));
     sc.L_safe = take(S * 4);
     sc.L_wide = take(S * 4);
@@ -257,8 +263,7 @@ struct dgs_ctx {
   // that waits): the event in hand starts on an idle GPU.
   bool alone;
   int hist_grid[3];      // CTAs of the whole-input histogram pass, per mode
-  int finalize_grid[3];  // CTAs of the cooperative finalize kernel, per mode
-  int finalize_max[3];   // most CTAs of it that can be resident at once
+  int finalize_max[3];   // most CTAs of the cooperative finalize kernel that can be resident at once, per mode
   uint32_t select_seq;   // selections launched so far
   uint64_t kind_seq[2];  // selections of each kind launched so far
   // Carried bounds: row (kind, worker) of L_next holds the bounds suggested by that worker's
@@ -330,7 +335,7 @@ inline int live(dgs_ctx* c) {
 }
 
 constexpr size_t kMaxTimedLaunches = 1 << 16;
-constexpr int kFinalizeWorkers = 64;  // CTAs of the finalize kernel (more of them take SM slots from the stream passes)
+constexpr uint64_t kFinalizeMin = 32;  // fewest CTAs of the finalize kernel
 
 // Records an event before and after one launch when timing is on.
 struct TimedLaunch {
@@ -484,6 +489,11 @@ inline int packet_format_of(const dgs_ctx* c) {
 }
 
 template <int MODE>
+const void* finalize_kernel(const dgs_ctx* c) {
+  return c->cfg.num_segments > 1 ? (const void*)k_finalize<MODE, true> : (const void*)k_finalize<MODE, false>;
+}
+
+template <int MODE>
 int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age, int stream_id, int set,
                   Task& task) {
   constexpr int KIND = MODE == kPull ? 1 : 0;
@@ -501,17 +511,16 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
   const bool single_pass = row >= 0;
   a.L_next = c->L_next(KIND, worker);
   a.force_two_pass = single_pass ? 0 : 1;
-  // A selection of very many entries (dense packets) gets more CTAs: one more per 4096 entries.  One whose
-  // candidates (about three times the entries) fit the registers of 48 CTAs' threads, eight each, gets only
-  // those 48: finalize runs beside the push passes of later events and should hold few SMs.
-  int fin_base = c->finalize_grid[MODE];
-  if (3ull * a.pkt_count <= 48ull * kThreads * 8) fin_base = std::min(fin_base, 48);
-  // With several layers the threads visit their candidates four times; as many CTAs as keep those candidates
-  // (about twice the entries) in the threads' registers, eight each, save the re-reads.
-  int fin_want = (int)(a.pkt_count / 4096);
-  if (c->cfg.num_segments > 1) fin_want = (int)((2ull * a.pkt_count + kThreads * 8 - 1) / (kThreads * 8));
-  const int fin_grid = std::min(c->finalize_max[MODE], std::max(fin_base, fin_want));
+  // CTAs of finalize: as many as keep the candidates (about 1.7 times the entries) in the threads' registers, but not
+  // fewer than 32, since every step of a warp is a chain, and no more than one per SM (see k_finalize).  A warp per two
+  // layers for the advice.
+  const uint32_t advisers = std::min<uint32_t>(32u, (c->cfg.num_segments + 2 * kWarps - 1) / (2 * kWarps));
+  const uint64_t keep = finalize_keep(c->cfg.num_segments > 1);
+  const uint64_t cands = (uint64_t)a.pkt_count + a.pkt_count / 4 * 3 + 64ull * c->cfg.num_segments;
+  const int fin_grid = (int)std::min<uint64_t>(std::min(c->finalize_max[MODE], c->alone ? 2 * c->sms : c->sms) - (int)advisers,
+                                               std::max<uint64_t>(kFinalizeMin, (cands + kThreads * keep - 1) / (kThreads * keep)));
   a.workers = (uint32_t)fin_grid;
+  a.advisers = advisers;
   a.fold_grid = MODE == kPull ? (uint32_t)c->fold_grid : 0u;   // one CTA more plans the next pull's pass
   a.packet_format = packet_format_of(c);
   if (c->cfg.flags & DGS_TEST_STALLED_BARRIER) {
@@ -553,7 +562,7 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
     // cooperative launch: the CTAs synchronise among themselves, so all must be resident
     TimedLaunch t(c, st, MODE == kPull ? DGS_KERNEL_FINALIZE_PULL : DGS_KERNEL_FINALIZE_PUSH);
     void* args[] = {(void*)&ws, (void*)&a};
-    DGS_CUDA(c, cudaLaunchCooperativeKernel((const void*)k_finalize<MODE>, dim3(fin_grid + (MODE == kPull ? 1 : 0)),
+    DGS_CUDA(c, cudaLaunchCooperativeKernel(finalize_kernel<MODE>(c), dim3(fin_grid + advisers + (MODE == kPull ? 1 : 0)),
                                             dim3(kThreads), args, finalize_dyn_bytes(c->cfg.num_segments), st));
     c->launches += 1;
   }
@@ -580,7 +589,7 @@ int occupancy_grids(dgs_ctx* c, int sms) {
   DGS_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_hist_all<MODE>, kThreads, 0));
   if (occ < 1) occ = 1;
   c->hist_grid[MODE] = std::min(sms * occ, kMaxGrid);
-  DGS_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_finalize<MODE>, kThreads,
+  DGS_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, finalize_kernel<MODE>(c), kThreads,
                                                             finalize_dyn_bytes(c->cfg.num_segments)));
   if (occ < 1) {
     c->last_cuda = (int)cudaErrorCooperativeLaunchTooLarge;
@@ -588,7 +597,6 @@ int occupancy_grids(dgs_ctx* c, int sms) {
     return DGS_ECUDA;
   }
   c->finalize_max[MODE] = std::min(sms * occ, kMaxWorkers) - (MODE == kPull ? 1 : 0);
-  c->finalize_grid[MODE] = std::min(c->finalize_max[MODE], kFinalizeWorkers);
   return DGS_OK;
 }
 
@@ -777,14 +785,12 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
   INIT_CUDA(cudaMemsetAsync(c->at<char>(L.status), 0, L.total - L.status, st));
   INIT_CUDA(cudaMemcpyAsync(c->at<char>(L.tiles), tiles.data(), tiles.size() * sizeof(Tile), cudaMemcpyHostToDevice, st));
   INIT_CUDA(cudaMemcpyAsync(c->at<char>(L.segs), segs.data(), segs.size() * sizeof(SegDesc), cudaMemcpyHostToDevice, st));
-  std::vector<uint32_t> seg_off(cfg->num_segments + 1), seg_tile0(cfg->num_segments);
+  std::vector<uint32_t> seg_off(cfg->num_segments + 1);
   for (uint32_t q = 0; q < cfg->num_segments; ++q) {
     seg_off[q] = (uint32_t)cfg->segments[q].offset;
-    seg_tile0[q] = segs[q].tile_begin;
   }
   seg_off[cfg->num_segments] = (uint32_t)cfg->n;  // n < 2^32
   INIT_CUDA(cudaMemcpyAsync(c->at<char>(L.seg_off), seg_off.data(), seg_off.size() * 4, cudaMemcpyHostToDevice, st));
-  INIT_CUDA(cudaMemcpyAsync(c->at<char>(L.seg_tile0), seg_tile0.data(), seg_tile0.size() * 4, cudaMemcpyHostToDevice, st));
   std::vector<uint32_t> blk_seg(L.num_blocks);
   for (uint32_t b = 0, q = 0; b < L.num_blocks; ++b) {
     while (segs.size() > q + 1 && (uint64_t)seg_off[q + 1] <= (uint64_t)b * kWarpTile) ++q;
@@ -808,7 +814,6 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
     w.num_tiles = L.num_tiles;
     w.num_segs = cfg->num_segments;
     w.seg_off = c->at<uint32_t>(L.seg_off);
-    w.seg_tile0 = c->at<uint32_t>(L.seg_tile0);
     w.cand_idx = c->at<uint32_t>(sc.cand_idx);
     w.cand_val = c->at<float>(sc.cand_val);
     w.part_cands = c->at<uint32_t>(sc.part_cands);
@@ -820,10 +825,11 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
     w.num_blocks = L.num_blocks;
     w.blk_seg = c->at<uint32_t>(L.blk_seg);
     w.cta_tot = c->at<uint2>(sc.cta_tot);
-    w.seg_start = c->at<uint2>(sc.seg_start);
+    w.cta_eq = c->at<uint32_t>(sc.cta_eq);
+    w.tab = c->at<LayerPick>(sc.tab);
+    w.list = c->at<uint2>(sc.list);
+    w.list_cnt = c->at<uint32_t>(sc.list_cnt);
     w.hist1 = c->at<uint32_t>(sc.hist1);
-    w.hist2 = c->at<uint32_t>(sc.hist2);
-    w.hist3 = c->at<uint32_t>(sc.hist3);
     w.sel = c->at<SegSel>(sc.sel);
     w.L_safe = c->at<uint32_t>(sc.L_safe);
     w.L_wide = c->at<uint32_t>(sc.L_wide);

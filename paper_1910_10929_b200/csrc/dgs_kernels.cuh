@@ -10,10 +10,11 @@
 //                 of the candidate buffer.  Everything below L is final at once (the
 //                 push writes t*(1/m) there).
 //   finalize      one small kernel (a few dozen co-resident CTAs with a barrier of
-//                 their own) over the candidates only: three radix levels (11+10+10
-//                 key bits) give the exact k-th largest key T and the number r of
-//                 entries equal to T that still fit; a count / scan / emit writes the
-//                 packet in index order.
+//                 their own) over the candidates only: the histogram that the stream
+//                 pass has counted gives the bin of the k-th largest, a list of that
+//                 bin's candidates the exact k-th largest key T and the number r of
+//                 entries equal to T that still fit; ranks by ballot write the packet
+//                 in index order.
 //
 // L is a guess carried over from an earlier selection of the same kind on that layer
 // (the host picks the most recent one made in a comparable state).  The guess is
@@ -31,9 +32,7 @@ constexpr int kWarpTile = 512;      // elements per tile (one warp, 4 x float4 p
 constexpr int kVecIters = 4;
 constexpr int kThreads = 256;       // threads per CTA in every kernel here
 constexpr int kWarps = kThreads / 32;
-constexpr int kBins1 = 2048;        // key bits 30..20
-constexpr int kBins2 = 1024;        // key bits 19..10
-constexpr int kBins3 = 1024;        // key bits  9..0
+constexpr int kBins1 = 2048;        // bins of a layer's histogram, see bin_of
 constexpr uint32_t kFull = 0xFFFFFFFFu;
 constexpr uint32_t kSpecSlack = 64; // a carried bound aims at max(1.5 k, k + 64) candidates next time
 constexpr int kMaxGrid = 512;       // upper bound on the grid of a stream pass (= parts of the candidate buffer)
@@ -58,20 +57,25 @@ struct SegDesc {
   uint32_t tile_begin, tile_end;  // tiles of this layer
   uint32_t k[2];                  // [0] push, [1] pull
   uint32_t pkt_off[2];            // exclusive prefix of k over layers
+  uint32_t list_off, list_cap;    // the layer's place in Workspace::list
 };
 
-struct SegSel {        // per-layer selection state of the selection in flight
-  uint32_t prefix;     // key bits fixed so far
-  uint32_t krem;       // entries still to take at or below the fixed prefix
-  uint32_t T;          // k-th largest key
-  uint32_t r;          // entries with key == T that are taken (lowest indices)
-  uint32_t neq;        // candidates with key == T
-  uint32_t wrem;       // bound suggested for a later selection: rank of its entry inside the first-level bin of
-                       // the k-th, when it lies in that bin (the second level then places it), else 0
+struct SegSel {        // per layer, finalize
+  uint32_t next;       // bound suggested for a later selection
+  uint32_t prefix;     // radix levels over all candidates: key bits fixed so far
+  uint32_t krem;       //   entries still to take at or below the fixed prefix
+};
+
+struct LayerPick {     // finalize: what a CTA knows of a layer that its candidates lie in
+  uint32_t L;          // bound of the stream pass
+  uint32_t bin, krem, pop;   // bin of the k-th largest, entries needed of it, entries in it (= on the layer's list)
+  uint32_t T, r;       // k-th largest key; entries with key == T that are taken (lowest indices)
+  uint32_t pkt_off, list_off;
+  uint32_t start_gt, start_eq, start_warp;   // a layer that begins in this CTA: what that warp had counted before it
 };
 
 // word indices in Workspace::sync
-enum SyncWord : int { kBarCount = 0, kBarGen = 1, kDecision = 2, kFail = 3, kParts = 4, kPlanParts = 5, kNumSyncWords = 8 };
+enum SyncWord : int { kBarCount = 0, kFail = 3, kParts = 4, kPlanParts = 5, kNumSyncWords = 8 };
 
 struct Workspace {
   const Tile* tiles;
@@ -92,12 +96,12 @@ struct Workspace {
   uint32_t* cta_cost;     // [kMaxFoldGrid] cost of each CTA's share in the last pass
   uint32_t part_cap;      // most blocks a CTA of the pass can take
   const uint32_t* seg_off;   // [S+1] first element of each layer, and n
-  const uint32_t* seg_tile0; // [S]   first tile of each layer
-  uint2* cta_tot;         // [kMaxWorkers] (#key > T, #key == T) among the candidates of each CTA of finalize
-  uint2* seg_start;       // [S] the same counted over all earlier layers
+  uint2* cta_tot;         // [kMaxWorkers] finalize: last layer of each CTA's candidates; how many of them in it lie above the k-th's bin
+  uint32_t* cta_eq;       // [kMaxWorkers] ... and equal T, where the lists were too short (then the count above is exact)
+  LayerPick* tab;         // [S + kMaxWorkers] picks of CTAs with too many layers for shared memory
+  uint2* list;            // candidates in the k-th's bin: (key, flat number), every layer at its own place
+  uint32_t* list_cnt;     // [S]
   uint32_t* hist1;        // [S][kBins1]
-  uint32_t* hist2;        // [S][kBins2]
-  uint32_t* hist3;        // [S][kBins3]
   SegSel* sel;            // [S]
   uint32_t* L_safe;       // [S] bound from the whole-input histogram (two-pass route)
   uint32_t* L_wide;       // [S] from the same histogram: the bound that admits about max(1.5 k, k+64) entries
@@ -124,6 +128,7 @@ struct SelArgs {
   int force_two_pass;
   int speculate;          // 0: never carry a bound (L_next is left alone)
   uint32_t workers;       // CTAs of finalize that process the candidates
+  uint32_t advisers;      // further ones that check the guesses and suggest the next bounds
   uint32_t seq;           // launch sequence number (tags the decision word)
   uint32_t fold_grid;     // pull: CTAs of the pass before this finalize (0: it was not k_fold, nothing to plan)
   uint32_t phantom_workers;  // testing only: CTAs the finalize barrier waits for beyond those launched (0 in normal use)
@@ -171,6 +176,13 @@ __device__ __forceinline__ uint32_t bound_inside_bin(uint32_t bin, uint32_t need
   const float f = fminf(1.f, 1.25f * (float)need / (float)max(pop, 1u) + 0.02f);
   const uint32_t take = (uint32_t)ceilf(f * (float)width);
   return hi - min(width, take);
+}
+// Histogram bin of a candidate of a layer with bound L (key >= L).  The bins start at the bound and are fine, 2^14 keys
+// (an eighth of an octave has 2^20), over the four octaves above it; the last one takes what lies beyond.  A bound near
+// zero says nothing about where the candidates are: then the bins are the top 11 key bits.
+__device__ __forceinline__ uint32_t bin_shift(uint32_t L) { return L < (1u << 25) ? 20u : 14u; }
+__device__ __forceinline__ uint32_t bin_of(uint32_t key, uint32_t L) {
+  return min((uint32_t)kBins1 - 1u, (key - L) >> bin_shift(L));
 }
 __device__ __forceinline__ uint32_t lanemask_lt() {
   uint32_t m;
@@ -238,7 +250,7 @@ __device__ __forceinline__ void load_tile_vec(const float* __restrict__ a, const
 // candidates of the vector in ascending index order, which is what lets the finalize kernel
 // number the selected ones with a plain prefix sum.
 struct StreamShared {
-  uint32_t hist[kBins1];      // top 11 key bits of the candidates of the layer being processed
+  uint32_t hist[kBins1];      // candidates of the layer being processed, by bin_of
   uint32_t cursor;            // candidates appended by this CTA so far
   uint32_t wcnt[2][kWarps];   // candidates per warp of the current round (two rounds alternate)
 };
@@ -292,7 +304,7 @@ __device__ __forceinline__ uint32_t tile_mask_regs(const SelArgs& a, uint32_t ti
 }
 
 // Writes the candidates of a full tile (mask from tile_mask_*) from slot `base` on, in index
-// order, and histograms their top key bits.  The cost is proportional to the candidates: one
+// order, and histograms them.  The cost is proportional to the candidates: one
 // packed warp scan gives every lane the rank of its candidates (lane l holds elements
 // j*128 + l*4 + c, order is j-major, so the four per-j counts travel as four bytes of one
 // word), and a lane that has candidates walks its set bits.  value(off) returns element `off`; count(off, key)
@@ -373,7 +385,7 @@ __device__ __forceinline__ uint32_t ragged_mask(const SelArgs& a, const Tile til
   return flags;
 }
 // Writes its candidates from slot `base` on, in index order.
-__device__ __forceinline__ void ragged_emit(const Workspace& ws, StreamShared& sh, const Tile tile, uint32_t flags,
+__device__ __forceinline__ void ragged_emit(const Workspace& ws, StreamShared& sh, const Tile tile, uint32_t flags, uint32_t L,
                                             uint32_t base, int lane, uint32_t lt, const float (&x)[kRaggedSteps]) {
   if (!__any_sync(kFull, flags != 0)) return;
 #pragma unroll
@@ -385,7 +397,7 @@ __device__ __forceinline__ void ragged_emit(const Workspace& ws, StreamShared& s
         const uint32_t pos = base + __popc(b & lt);
         ws.cand_idx[pos] = tile.start + st * 32 + lane;
         ws.cand_val[pos] = x[st];
-        atomicAdd(sh.hist + (key_of(x[st]) >> 20), 1u);
+        atomicAdd(sh.hist + bin_of(key_of(x[st]), L), 1u);
       }
       base += __popc(b);
     }
@@ -454,9 +466,9 @@ __device__ void stream_tiles(const Workspace& ws, const SelArgs& a, const uint32
             for (int q = 1; q < 4 * kVecIters; ++q)
               if (q == e) v = x[q];
             return v;
-          }, [&](uint32_t, uint32_t key) { atomicAdd(sh.hist + (key >> 20), 1u); });
+          }, [&](uint32_t, uint32_t key) { atomicAdd(sh.hist + bin_of(key, L), 1u); });
         } else {
-          ragged_emit(ws, sh, tile, mask, base, lane, lt, x);
+          ragged_emit(ws, sh, tile, mask, L, base, lane, lt, x);
         }
       }
     }
@@ -588,7 +600,7 @@ __device__ void stream_tiles_tma(const Workspace& ws, const SelArgs& a, const ui
         float x[kRaggedSteps];
         const uint32_t flags = ragged_mask<MODE>(a, tile, L, lane, in, out, x);
         const uint32_t count = __reduce_add_sync(kFull, (uint32_t)__popc(flags));
-        ragged_emit(ws, sh, tile, flags, slot0 + cur, lane, lt, x);
+        ragged_emit(ws, sh, tile, flags, L, slot0 + cur, lane, lt, x);
         if (lane == 0) sh.cursor = count;
       }
       __syncthreads();
@@ -634,7 +646,7 @@ __device__ void stream_tiles_tma(const Workspace& ws, const SelArgs& a, const ui
       cur += total;
       tile_emit(ws, e0 + tl * kWarpTile, mask, base, lane, [&](uint32_t off) {
         return combine<MODE>(su[off], su[kStageFloats + off], a.m, a.lr);
-      }, [&](uint32_t, uint32_t key) { atomicAdd(sh.hist + (key >> 20), 1u); });
+      }, [&](uint32_t, uint32_t key) { atomicAdd(sh.hist + bin_of(key, L), 1u); });
     }
     if (*s_dead) break;
     uses += done;
@@ -759,6 +771,7 @@ __device__ uint32_t block_pick(const uint32_t* hist, uint32_t k, uint32_t& bin, 
       if (acc < k && k <= acc + loc[j]) {
         s_res[0] = (uint32_t)(top - j);
         s_res[1] = k - acc;
+        s_res[2] = loc[j];
       }
       acc += loc[j];
     }
@@ -771,26 +784,47 @@ __device__ uint32_t block_pick(const uint32_t* hist, uint32_t k, uint32_t& bin, 
 }
 
 // Flat numbering of the candidates over the parts: pre[p] = candidates of the parts before p (pre[parts] = all of
-// them), slot0[p] = first slot of part p.  Both arrays in shared memory; ends with a barrier.
-__device__ __forceinline__ void number_parts(const Workspace& ws, uint32_t parts, uint32_t* pre, uint32_t* slot0,
-                                             unsigned long long* s_warp) {
-  for (uint32_t p = threadIdx.x; p < parts; p += kThreads) {
-    pre[p] = __ldcg(ws.part_cands + p);
-    slot0[p] = __ldcg(ws.part_slot0 + p);
-  }
+// them), in shared memory; ends with a barrier.
+template <int MAXPARTS>
+__device__ __forceinline__ void number_parts(const Workspace& ws, uint32_t parts, uint32_t* pre, unsigned long long* s_warp) {
+  constexpr int PER = MAXPARTS / kThreads;
+  static_assert(MAXPARTS % kThreads == 0, "the same number of parts for every thread");
+  uint32_t v[PER], sum = 0;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) v[j] = j * kThreads + threadIdx.x < parts ? __ldcg(ws.part_cands + j * kThreads + threadIdx.x) : 0u;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) pre[j * kThreads + threadIdx.x] = v[j];
   __syncthreads();
-  const uint32_t per = (parts + kThreads - 1) / kThreads, p0 = min(parts, threadIdx.x * per), p1 = min(parts, p0 + per);
-  uint32_t sum = 0;
-  for (uint32_t p = p0; p < p1; ++p) sum += pre[p];
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    v[j] = pre[threadIdx.x * PER + j];
+    sum += v[j];
+  }
   unsigned long long total;
   uint32_t at = (uint32_t)block_excl_scan(sum, s_warp, total);
-  for (uint32_t p = p0; p < p1; ++p) {
-    const uint32_t c = pre[p];
-    pre[p] = at;
-    at += c;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    pre[threadIdx.x * PER + j] = at;
+    at += v[j];
   }
-  if (threadIdx.x == 0) pre[parts] = (uint32_t)total;
+  if (threadIdx.x == 0) pre[parts] = (uint32_t)total;   // (the owner of that place writes the same)
   __syncthreads();
+}
+
+// From the histogram of a whole layer (top 11 key bits; cleared here): L_safe = lower edge of the bin holding the k-th
+// largest key, L_wide = a bound that admits about max(1.5 k, k+64) entries.  By one CTA.
+__device__ void pick_lower(const Workspace& ws, uint32_t s, uint32_t k, unsigned long long* s_warp, uint32_t* s_res) {
+  uint32_t bin, krem, wbin = 0, wrem = 0;
+  uint32_t* const h = ws.hist1 + (size_t)s * kBins1;
+  const uint32_t want = spec_want(k), total = block_pick<kBins1>(h, k, bin, krem, s_warp, s_res);
+  if (total >= want) block_pick<kBins1>(h, want, wbin, wrem, s_warp, s_res);
+  if (threadIdx.x == 0) {
+    ws.L_safe[s] = bin << 20;
+    // 0 (everything) when the layer has fewer than `want` entries
+    ws.L_wide[s] = total >= want ? bound_inside_bin(wbin, wrem, __ldcg(h + wbin), 0u) : 0u;
+  }
+  __syncthreads();
+  for (int b = threadIdx.x; b < kBins1; b += kThreads) h[b] = 0;
 }
 
 // Barrier among the CTAs of finalize (all resident: cooperative launch).  One arrival
@@ -821,97 +855,220 @@ __device__ bool worker_barrier(uint32_t* sync, uint32_t W, int* status, int* s_o
 }
 
 // ---- finalize -------------------------------------------------------------------
-// The candidates are numbered flat over the parts: part p holds part_cands[p] of them in
-// consecutive slots from part_slot0[p] on.  Parts follow one another in index order and every
-// part lists its candidates in index order, so the flat numbering is the index order of all
-// candidates.  Every thread owns a run of consecutive flat candidates (kept in registers when
-// they are few) for all phases:
-//   levels 2 and 3   histograms of the next 10 + 10 key bits among the candidates that share the
-//                    bits fixed so far  ->  exact k-th largest key T and tie quota r per layer
-//   count            (key > T, key == T) per thread, prefix sums inside the CTA, totals per CTA
-//   emit             a candidate's rank among the selected ones of its layer follows from the
-//                    prefix sums (layers are consecutive in the flat order and layer s selects
-//                    exactly k_s entries)  ->  packet in index order, state updates
-// With one layer every CTA works out the picks itself from the shared histograms, which leaves
-// three grid-wide barriers; with several layers the picks are spread over the CTAs.
-constexpr int kSegCap = 1024;  // layers whose tables fit in shared memory; more fall back to global reads
-constexpr int kBatch = 8;       // independent loads a thread issues before using any (latency-bound loops)
+// The candidates are numbered flat over the parts: part p holds part_cands[p] of them in consecutive slots from
+// part_slot0[p] on.  Parts follow one another in index order and every part lists its candidates in index order, so
+// the flat numbering is the index order of all candidates.  Every warp owns a run of consecutive flat candidates, 32
+// of them at a time, kept in registers when they are few:
+//   pick    every CTA finds, in the histograms of the layers its candidates lie in, the bin of the k-th largest
+//   list    the candidates of that bin, and where they stand, go to a short list of the layer.  The bins are fine
+//           (a 64th of an eighth of an octave above the bound), so the list is a fraction of a percent of the
+//           candidates.  Candidates above the bin are counted per warp
+//   -- the only barrier among the CTAs --
+//   exact   a radix selection over the list (a warp per layer) gives the k-th largest key T and the tie quota r.
+//           With the counts above the bin and the places on the list every warp knows how many selected entries
+//           stand before its candidates
+//   emit    ranks by ballot  ->  packet in index order, state updates
+// A few more CTAs check the guesses and work out the next bounds meanwhile, so that this is not on the way.
+// What bounds it is the chain of trips to L2, and the fetching of instructions that run once (39 % of a warp's time in a
+// form that kept four candidates a lane in unrolled code for any number of layers), not bytes.  So there are few
+// phases, a variant for one layer and one for several, little unrolling, and the rare paths stay out of line.
+// Measured between events (about 6 us of that is the events'), against three radix levels over global histograms with
+// three barriers (one layer) or eight (several): 25 K of 47 K candidates, one layer: 23-26 us for 33-35; 120 K of 200 K,
+// 62 layers: 40-42 us for 56-57; 148 layers: 50-57 us for 73-78; 670 K of 1 M, one layer: 63 us for 93.
+constexpr int kSegCap = 1024;   // layers whose offsets fit in shared memory; more are looked up in global memory
+// candidates a lane keeps in registers between the phases, and loads at a time
+__host__ __device__ constexpr int finalize_keep(bool many) { return many ? 4 : 2; }
+constexpr int kTouch = 40;      // layers of a CTA whose picks fit in shared memory; more are kept in global memory
 
+constexpr int kListSmem = kThreads;    // entries of the list that are ranked in shared memory (one layer)
+template <int MAXPARTS>
 struct FinalizeShared {
-  StreamShared stream;                 // redo of the passes (guess failed); its histogram also serves levels 2 and 3
+  StreamShared stream;                 // redo of the passes (guess failed); its histogram also serves the warps' radix steps
   unsigned long long warp_scan[kWarps];
-  uint32_t res[2];
+  uint32_t res[3];
   int ok;
-  uint32_t pre_cands[kMaxParts + 1];   // exclusive prefix of part_cands
-  uint32_t slot0[kMaxParts];           // first slot of each part
+  uint32_t range[3];                   // layers of the candidate before this CTA's, of its first and of its last one
+  uint32_t gt[kWarps], eq[kWarps];     // what each warp has counted
+  LayerPick tab[kTouch];
+  uint32_t pre[MAXPARTS + 1];          // exclusive prefix of part_cands
 };
-// Per-layer tables of finalize live in dynamic shared memory, sized by the number of layers S (up
-// to kSegCap layers; with more, the kernel reads the tables from global memory and needs none):
-//   uint2 seg_start[S]   (key > T, key == T) candidates of all earlier layers
-//   u32 seg_off[S + 1]   first element of each layer, and n
-//   u32 seg_a[S]         per-layer parameter of the current phase (prefix, or T)
-//   u32 seg_b[S]         second one (r)
+static_assert(kWarps * 128 <= kBins1, "a radix step of every warp fits the histogram's place");
+static_assert(2 * kListSmem <= kBins1, "and so does the list");
+// offsets of the layers in dynamic shared memory
 __host__ __device__ inline uint32_t finalize_dyn_bytes(uint32_t S) {
-  return S <= (uint32_t)kSegCap ? 20u * S + 8u : 0u;
+  return S <= (uint32_t)kSegCap ? 4u * (S + 1u) : 0u;
 }
 
-// layer that holds element i: last s with off[s] <= i
-__device__ __forceinline__ uint32_t seg_of(const uint32_t* off, uint32_t S, uint32_t i) {
-  uint32_t lo = 0, hi = S - 1;
+// layer in [lo, hi] that holds element i: last s with off[s] <= i
+__device__ __forceinline__ uint32_t seg_of(const uint32_t* off, uint32_t lo, uint32_t hi, uint32_t i) {
   while (lo < hi) {
     const uint32_t mid = (lo + hi + 1) >> 1;
     if (off[mid] <= i) lo = mid; else hi = mid - 1;
   }
   return lo;
 }
-// The same for a thread that visits candidates in index order: consecutive candidates mostly lie in the
-// same layer, so the layer found last is tried first and the search is only made when it does not hold i.
-__device__ __forceinline__ uint32_t seg_near(const uint32_t* off, uint32_t S, uint32_t i, uint32_t& last) {
-  if (i < off[last] || i >= off[last + 1]) last = seg_of(off, S, i);
-  return last;
-}
-// slot of flat candidate p: last part with pre[part] <= p
-__device__ __forceinline__ uint32_t slot_of(const FinalizeShared& sh, uint32_t parts, uint32_t p, uint32_t* part_out) {
-  uint32_t lo = 0, hi = parts - 1;
+// last part in [lo, hi] with pre[part] <= p
+__device__ __forceinline__ uint32_t part_of(const uint32_t* pre, uint32_t lo, uint32_t hi, uint32_t p) {
+#pragma unroll 1
   while (lo < hi) {
     const uint32_t mid = (lo + hi + 1) >> 1;
-    if (sh.pre_cands[mid] <= p) lo = mid; else hi = mid - 1;
+    if (pre[mid] <= p) lo = mid; else hi = mid - 1;
   }
-  if (part_out) *part_out = lo;
-  return sh.slot0[lo] + (p - sh.pre_cands[lo]);
+  return lo;
+}
+// the same over all parts, found by a whole warp, 32 probes at a time (p the same in every lane)
+__device__ __forceinline__ uint32_t warp_part_of(const uint32_t* pre, uint32_t parts, uint32_t p, int lane) {
+  uint32_t lo = 0, span = parts;                 // the answer lies in [lo, lo + span)
+#pragma unroll 1
+  while (span > 1) {
+    const uint32_t step = (span + 31u) / 32u, at = lo + lane * step;
+    const uint32_t c = __popc(__ballot_sync(kFull, lane * step < span && pre[at] <= p));   // >= 1: pre[lo] <= p
+    span = min(step, span - (c - 1u) * step);
+    lo += (c - 1u) * step;
+  }
+  return lo;
 }
 
-// Walks the flat numbering: a thread owns consecutive flat candidates, finds the first one by
-// binary search and then only steps.
-struct Cursor {
-  uint32_t part, slot, left;   // part of the current candidate, its slot, candidates left in that part (>= 1 if valid)
-};
-__device__ __forceinline__ Cursor cursor_at(const FinalizeShared& sh, uint32_t parts, uint32_t p) {
-  Cursor c;
-  c.slot = slot_of(sh, parts, p, &c.part);
-  c.left = sh.pre_cands[c.part + 1] - p;
-  return c;
-}
-// advance by n candidates; the caller never dereferences a cursor that ran past the last candidate
-__device__ __forceinline__ void cursor_advance(const FinalizeShared& sh, uint32_t parts, Cursor& c, uint32_t n) {
-  while (n >= c.left) {
-    n -= c.left;
-    do { ++c.part; } while (c.part < parts && sh.pre_cands[c.part + 1] == sh.pre_cands[c.part]);
-    if (c.part >= parts) { c.left = 0xFFFFFFFFu; c.slot = 0; return; }   // ran off the end
-    c.slot = sh.slot0[c.part];
-    c.left = sh.pre_cands[c.part + 1] - sh.pre_cands[c.part];
+// From a layer's histogram, counting from the top bin down, the bin that holds the k-th entry; by one warp.
+struct BinPick { uint32_t bin, rem, pop; };   // rem: entries needed of the bin; pop: entries in it
+// lane `lane` of the warp holds bins kBins1 - 64 (lane + 1) .. kBins1 - 1 - 64 lane: how many entries
+__device__ __forceinline__ uint32_t lane_bins(const uint32_t* h, int lane) {
+  const uint4* q = reinterpret_cast<const uint4*>(h + kBins1 - 64 * (lane + 1));
+  uint32_t sum = 0;
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    const uint4 x = __ldcg(q + j);
+    sum += x.x + x.y + x.z + x.w;
   }
-  c.slot += n;
-  c.left -= n;
+  return sum;
+}
+__device__ __forceinline__ uint32_t warp_incl(uint32_t v, int lane) {
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint32_t o = __shfl_up_sync(kFull, v, d);
+    if (lane >= d) v += o;
+  }
+  return v;
+}
+// incl: inclusive prefix over the lanes of lane_bins; k <= its total
+__device__ __forceinline__ BinPick warp_pick(const uint32_t* h, uint32_t incl, uint32_t own, uint32_t k, int lane) {
+  const uint32_t src = __ffs(__ballot_sync(kFull, incl >= k)) - 1u;
+  const uint32_t above = __shfl_sync(kFull, incl - own, src);
+  const uint32_t top = kBins1 - 1u - 64u * src - 2u * lane;     // this lane: bins top, top - 1
+  const uint2 x = __ldcg(reinterpret_cast<const uint2*>(h + top - 1u));
+  const uint32_t in2 = above + warp_incl(x.x + x.y, lane);
+  const uint32_t who = __ffs(__ballot_sync(kFull, in2 >= k)) - 1u;
+  const uint32_t before = in2 - x.x - x.y;
+  const bool high = before + x.y >= k;
+  BinPick r;
+  r.bin = __shfl_sync(kFull, high ? top : top - 1u, who);
+  r.rem = __shfl_sync(kFull, high ? k - before : k - before - x.y, who);
+  r.pop = __shfl_sync(kFull, high ? x.y : x.x, who);
+  return r;
+}
+
+// Bound suggested for a later selection on layer s, by one warp: the one above which about `want` entries lie.
+__device__ __forceinline__ uint32_t next_bound(const Workspace& ws, uint32_t s, const uint32_t* h, uint32_t L, uint32_t total,
+                                               uint32_t want, uint32_t incl, uint32_t own, bool whole, int lane) {
+  uint32_t key;
+  if (total >= want) {
+    const uint32_t roomy = want + want / 16;          // a little beyond, if there are that many
+    key = L + (warp_pick(h, incl, own, roomy <= total ? roomy : want, lane).bin << bin_shift(L));
+  } else if (whole) {
+    key = __ldcg(ws.L_wide + s);                      // known from the histogram of the whole input
+  } else if (L < (1u << 25)) {
+    key = 0;
+  } else {
+    // Fewer candidates than wished for (but at least k) and nothing known below the bound: lower it by as much as would
+    // hold the missing ones at the density seen right above it -- what was never sent piles up below the k-th, so half
+    // an octave down may hold a hundred times the wished-for number -- and by half an octave only where too few keys
+    // lie above the bound to tell.
+    uint2 x = __ldcg(reinterpret_cast<const uint2*>(h) + lane);         // an eighth of an octave: 64 bins
+    uint32_t pop = __reduce_add_sync(kFull, x.x + x.y), width = 1u << 20;
+    if (pop < 64u) {
+      x = __ldcg(reinterpret_cast<const uint2*>(h) + 32 + lane);
+      pop += __reduce_add_sync(kFull, x.x + x.y);
+      width += 1u << 20;
+    }
+    const float step = 1.5f * (float)(want + want / 16 - total) / (float)max(pop, 1u) * (float)width;
+    const uint32_t down = pop >= 64u && step < (float)(4u << 20) ? (uint32_t)step + 1u : 4u << 20;
+    key = L > down ? L - down : 0u;
+  }
+  // A bound of zero makes every element of the layer a candidate (zeros included).  That is fine for a
+  // layer not much larger than the wished-for number of candidates, and for one that is small beside the
+  // whole vector: a layer without enough candidates costs the next selection a histogram and a second pass
+  // over all layers (148 layers of 124 M elements: 570 us a pull when every other one failed on layers of 768
+  // to 3072 elements, 78 us without).  For a large one, no bound at all is the better advice: the next
+  // selection finds nothing, notices, and takes its bound from a histogram.
+  const uint32_t layer_cap = (ws.segs[s].tile_end - ws.segs[s].tile_begin) * (uint32_t)kWarpTile;
+  const bool flood = key == 0 && layer_cap / 8 > want && layer_cap > max(8192u, ws.n / 1024u);
+  return flood ? 0xFFFFFFFFu : key;
+}
+
+// The k-th largest of the `pop` keys of a list, all of them in [base, base + 2^bits), by one warp; hist: 128 words of
+// shared memory of its own.  Returns T and, in r, how many of the keys equal to T are among the k.
+__device__ __noinline__ uint32_t warp_radix(const uint2* list, uint32_t pop, uint32_t k, uint32_t base, int bits, uint32_t* hist,
+                                               int lane, uint32_t& r) {
+  if (pop <= 32u) {                              // ranks by comparing with every other key
+    const uint32_t key = (uint32_t)lane < pop ? __ldcg(&list[lane].x) : 0u;
+    uint32_t above = 0, same = 0;
+    for (uint32_t q = 0; q < pop; ++q) {
+      const uint32_t o = __shfl_sync(kFull, key, q);
+      above += o > key ? 1u : 0u;
+      same += o == key ? 1u : 0u;
+    }
+    const uint32_t who = __ffs(__ballot_sync(kFull, (uint32_t)lane < pop && above < k && k <= above + same)) - 1u;
+    r = __shfl_sync(kFull, k - above, who);
+    return __shfl_sync(kFull, key, who);
+  }
+  constexpr int kKeep = 8;
+  uint32_t prefix = 0, keep[kKeep];
+  auto load = [&](uint32_t q0) {
+#pragma unroll
+    for (int u = 0; u < kKeep; ++u) {
+      const uint32_t q = q0 + u * 32u + lane;
+      keep[u] = q < pop ? __ldcg(&list[q].x) - base : kFull;
+    }
+  };
+  if (pop <= 32u * kKeep) load(0);
+#pragma unroll 1
+  for (int shift = (bits - 1) / 7 * 7; shift >= 0; shift -= 7) {
+    *reinterpret_cast<uint4*>(hist + lane * 4) = make_uint4(0, 0, 0, 0);
+    __syncwarp();
+    for (uint32_t q0 = 0; q0 < pop; q0 += 32u * kKeep) {
+      if (pop > 32u * kKeep) load(q0);
+#pragma unroll
+      for (int u = 0; u < kKeep; ++u)
+        if (q0 + u * 32u + lane < pop && (uint32_t)((uint64_t)keep[u] >> (shift + 7)) == prefix)
+          atomicAdd(hist + ((keep[u] >> shift) & 127u), 1u);
+    }
+    __syncwarp();
+    const uint4 x = *reinterpret_cast<const uint4*>(hist + 124 - lane * 4);   // lane's four bins, .w the highest
+    const uint32_t sum = x.x + x.y + x.z + x.w, incl = warp_incl(sum, lane);
+    const uint32_t who = __ffs(__ballot_sync(kFull, incl >= k)) - 1u;
+    uint32_t left = k - (incl - sum), bin = 127u - lane * 4u;
+    if (left > x.w) {
+      left -= x.w; --bin;
+      if (left > x.z) {
+        left -= x.z; --bin;
+        if (left > x.y) { left -= x.y; --bin; }
+      }
+    }
+    prefix = (prefix << 7) | __shfl_sync(kFull, bin, who);
+    k = __shfl_sync(kFull, left, who);
+    __syncwarp();
+  }
+  r = k;
+  return base + prefix;
 }
 
 // Where the CTAs of the next pass over a difference vector on this scratch set begin: ranges of blocks that cost
 // about the same, judged by what this pass cost each CTA.  What has to be read and folded in clusters in the
 // tensors with the largest updates, and those are the same for every worker; with equal ranges a few CTAs do most
 // of the work.  Done by a CTA of its own beside the finalize, so that it adds nothing to the chain.
-__device__ void plan_parts(const Workspace& ws, uint32_t G, FinalizeShared& sh) {
-  uint32_t* const before = sh.pre_cands;       // [G] cost of the CTAs before this one
-  uint32_t* const first = sh.slot0;            // [G + 1] where they began
+__device__ void plan_parts(const Workspace& ws, uint32_t G, FinalizeShared<kMaxParts>& sh) {
+  uint32_t* const before = sh.pre;             // [G] cost of the CTAs before this one
+  uint32_t* const first = sh.pre + 512;        // [G + 1] where they began
   uint32_t* const cost = sh.stream.hist;       // [G]
   uint32_t* const next = sh.stream.hist + kMaxFoldGrid;   // [G + 1]
   const bool had = ld_volatile(ws.sync + kPlanParts) == G && __ldcg(ws.plan + G) == ws.num_blocks;
@@ -968,23 +1125,53 @@ __device__ void plan_parts(const Workspace& ws, uint32_t G, FinalizeShared& sh) 
   }
 }
 
-// 64 registers a thread: finalize runs beside two CTAs of a push pass on an SM, which leave it that many
+// The guess was too high for some layer: take the bound that cannot fail from a histogram of the whole input and repeat
+// the stream pass, with the few CTAs this kernel has.  False: a barrier gave up.
 template <int MODE>
-__global__ void __maxnreg__(64) k_finalize(Workspace ws, SelArgs a) {
-  __shared__ FinalizeShared sh;
+__device__ __noinline__ bool redo_passes(const Workspace& ws, const SelArgs& a, const float* in, float* out, StreamShared& st,
+                                         unsigned long long* s_warp, uint32_t* s_res, int* s_ok, uint32_t Wb, uint32_t spin_limit,
+                                         uint32_t& bar_target) {
+  const uint32_t cta = blockIdx.x, G = a.workers + a.advisers, S = ws.num_segs;
+  auto barrier = [&]() { return worker_barrier(ws.sync, Wb, ws.status, s_ok, bar_target, spin_limit); };
+  for (size_t w = (size_t)cta * kThreads + threadIdx.x; w < (size_t)S * kBins1; w += (size_t)G * kThreads) ws.hist1[w] = 0;
+  for (uint32_t s = cta * kThreads + threadIdx.x; s < S; s += G * kThreads) ws.list_cnt[s] = 0;
+  if (cta == 0 && threadIdx.x == 0) ws.sync[kFail] = 0;
+  if (!barrier()) return false;
+  hist_all_tiles<MODE>(ws, a, in, cta, G, st.hist);
+  if (!barrier()) return false;
+  for (uint32_t s = cta; s < S; s += G) {
+    pick_lower(ws, s, ws.segs[s].k[MODE == kPull ? 1 : 0], s_warp, s_res);
+    __syncthreads();
+  }
+  if (!barrier()) return false;
+  stream_tiles<MODE>(ws, a, ws.L_safe, in, out, cta, G, st);
+  return barrier();
+}
+
+// 64 registers a thread: finalize runs beside two CTAs of a push pass on an SM, which leave it that many
+template <int MODE, bool MANY>
+__global__ void __maxnreg__(64) k_finalize(const __grid_constant__ Workspace ws, const __grid_constant__ SelArgs a) {
+  constexpr int kPartCap = MODE == kPull ? kMaxParts : kMaxGrid;   // parts that the pass before, or a redo, can leave
+  __shared__ __align__(16) FinalizeShared<kPartCap> sh;
   extern __shared__ __align__(16) unsigned char fin_dyn[];   // finalize_dyn_bytes(S) bytes
 
-  constexpr int PM = MODE == kPull ? 1 : 0;
-  // after k_fold one CTA more than a.workers is launched: it plans the next pass and takes no part in the selection
-  const uint32_t cta = blockIdx.x, W = a.workers, S = ws.num_segs;
-  if (MODE == kPull && cta == W) {
-    plan_parts(ws, a.fold_grid, sh);
-    return;
+  constexpr int PM = MODE == kPull ? 1 : 0, kKeep = finalize_keep(MANY);
+  // CTAs [0, W) process the candidates, [W, W + A) look after the layers' bounds, and after k_fold one more plans the
+  // next pass (it takes no part in the selection)
+  const uint32_t cta = blockIdx.x, W = a.workers, A = a.advisers, S = ws.num_segs;
+  if constexpr (MODE == kPull) {
+    if (cta == W + A) {
+      plan_parts(ws, a.fold_grid, sh);
+      return;
+    }
   }
-  const uint32_t gthread = cta * kThreads + threadIdx.x, nthreads = W * kThreads;
-  // the barrier counts W arrivals; a test can make it wait for CTAs that do not exist, with a short limit,
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t gthread = cta * kThreads + threadIdx.x, nthreads = (W + A) * kThreads, lt = lanemask_lt(), le = lt | (1u << lane);
+  // the barrier counts W + A arrivals; a test can make it wait for CTAs that do not exist, with a short limit,
   // to see the bounded wait give up (every CTA then leaves with DGS_ETIMEOUT in the status word)
-  const uint32_t Wb = W + a.phantom_workers, spin_limit = a.spin_limit ? a.spin_limit : kSpinLimit;
+  const uint32_t Wb = W + A + a.phantom_workers, spin_limit = a.spin_limit ? a.spin_limit : kSpinLimit;
+  uint32_t bar_target = 0;
+  auto barrier = [&]() { return worker_barrier(ws.sync, Wb, ws.status, &sh.ok, bar_target, spin_limit); };
 
   // pointers are read once, before anything may exchange them
   const float* in = nullptr;
@@ -995,368 +1182,479 @@ __global__ void __maxnreg__(64) k_finalize(Workspace ws, SelArgs a) {
     in = *a.u_cur_slot;
     out = *a.u_spare_slot;
   }
-
-  // layer tables
-  const bool seg_smem = S <= (uint32_t)kSegCap;
-  uint2* const sm_seg_start = reinterpret_cast<uint2*>(fin_dyn);
-  uint32_t* const sm_seg_off = reinterpret_cast<uint32_t*>(fin_dyn + 8u * S);
-  uint32_t* const sm_seg_a = sm_seg_off + S + 1;
-  uint32_t* const sm_seg_b = sm_seg_a + S;
-  if (seg_smem)
-    for (uint32_t s = threadIdx.x; s <= S; s += kThreads) sm_seg_off[s] = ws.seg_off[s];
-  const uint32_t* const seg_off = seg_smem ? sm_seg_off : ws.seg_off;
-  __syncthreads();
-
-  // flat numbering of the candidates, and this thread's own candidates
-  uint32_t parts = 0, C = 0, per_thread = 0, my_lo = 0, my_hi = 0;
-  constexpr int kKeep = 8;            // candidates a thread keeps in registers between the phases
-  float rraw[kKeep];
-  uint32_t ridx[kKeep];               // valid when per_thread <= kKeep
-  uint32_t bar_target = 0;
-  uint32_t one_prefix = 0, one_krem = 0;   // S == 1: the layer's selection state, the same in every thread of the grid
-  uint32_t one_wrem = 0;                   // S == 1, CTA 0: SegSel::wrem of the layer
-  bool redo = false;
-  for (int attempt = 0; attempt < 2; ++attempt) {
-    if (redo) {
-      // the guess was too high for some layer: take the bound that cannot fail from a histogram of
-      // the whole input and repeat the stream pass, with the few CTAs this kernel has
-      hist_all_tiles<MODE>(ws, a, in, cta, W, sh.stream.hist);
-      if (!worker_barrier(ws.sync, Wb, ws.status, &sh.ok, bar_target, spin_limit)) return;
-      for (uint32_t s = cta; s < S; s += W) {
-        uint32_t bin, krem;
-        uint32_t* h = ws.hist1 + (size_t)s * kBins1;
-        const uint32_t k = ws.segs[s].k[PM];
-        const uint32_t total = block_pick<kBins1>(h, k, bin, krem, sh.warp_scan, sh.res);
-        uint32_t wbin = 0, wrem = 0;
-        const uint32_t want = spec_want(k);
-        if (total >= want) block_pick<kBins1>(h, want, wbin, wrem, sh.warp_scan, sh.res);
-        if (threadIdx.x == 0) {
-          ws.L_safe[s] = bin << 20;
-          // 0 (everything) when the layer has fewer than `want` entries
-          ws.L_wide[s] = total >= want ? bound_inside_bin(wbin, wrem, __ldcg(h + wbin), 0u) : 0u;
-        }
-        __syncthreads();
-        for (int b = threadIdx.x; b < kBins1; b += kThreads) h[b] = 0;
-      }
-      if (cta == 0 && threadIdx.x == 0) ws.sync[kFail] = 0;
-      if (!worker_barrier(ws.sync, Wb, ws.status, &sh.ok, bar_target, spin_limit)) return;
-      stream_tiles<MODE>(ws, a, ws.L_safe, in, out, cta, W, sh.stream);
-      if (!worker_barrier(ws.sync, Wb, ws.status, &sh.ok, bar_target, spin_limit)) return;
-    }
-    // flat numbering of the candidates (the stream pass is complete: an earlier kernel, or the barrier above)
-    parts = ld_volatile(ws.sync + kParts);
-    number_parts(ws, parts, sh.pre_cands, sh.slot0, sh.warp_scan);
-    C = sh.pre_cands[parts];
-    // every thread owns the flat candidates [my_lo, my_hi); when they are few it keeps them in registers
-    per_thread = (C + nthreads - 1) / nthreads;
-    my_lo = min(C, gthread * per_thread);
-    my_hi = min(C, my_lo + per_thread);
-    if (per_thread <= (uint32_t)kKeep && my_lo < my_hi) {
-      Cursor cur = cursor_at(sh, parts, my_lo);
-#pragma unroll
-      for (int u = 0; u < kKeep; ++u) {
-        rraw[u] = 0.f;
-        ridx[u] = 0;
-        if (my_lo + u < my_hi) {
-          rraw[u] = __ldcg(ws.cand_val + cur.slot);
-          ridx[u] = __ldcg(ws.cand_idx + cur.slot);
-          cursor_advance(sh, parts, cur, 1);
-        }
-      }
-    }
-    // level 1: the bin of the k-th largest among the candidates; checks the guess, suggests the next one
-    bool failed = false;
-    const bool everyone_picks = S == 1;   // one layer: every CTA reads the histogram itself, no barrier needed
-    for (uint32_t s = everyone_picks ? 0 : cta; s < S; s += everyone_picks ? 1 : W) {
-      uint32_t bin, krem;
-      uint32_t* h = ws.hist1 + (size_t)s * kBins1;
-      const uint32_t k = ws.segs[s].k[PM];
-      const uint32_t total = block_pick<kBins1>(h, k, bin, krem, sh.warp_scan, sh.res);
-      const bool owner = !everyone_picks || cta == 0;
-      if (total < k) {
-        failed = true;
-        if (owner && threadIdx.x == 0) atomicOr(ws.sync + kFail, 1u);
-      } else {
-        one_prefix = bin;
-        one_krem = krem;
-        if (owner && threadIdx.x == 0) {
-          ws.sel[s].prefix = bin;
-          ws.sel[s].krem = krem;
-          ws.sel[s].wrem = 0;
-          atomicAdd(ws.stats + 2, (unsigned long long)total);
-        }
-        one_wrem = 0;
-        if (owner && a.speculate) {
-          // bound suggested for a later selection on this layer
-          const uint32_t want = spec_want(k);
-          uint32_t lbin, lrem;
-          uint32_t lkey;   // the bound itself
-          if (total >= want) {
-            block_pick<kBins1>(h, want, lbin, lrem, sh.warp_scan, sh.res);
-            const uint32_t in_force = (redo || a.force_two_pass) ? __ldcg(ws.L_safe + s) : a.L_in[s];
-            lkey = bound_inside_bin(lbin, lrem, __ldcg(h + lbin), in_force);
-            // Inside the bin of the k-th the keys are anything but evenly spread where a push has run for a
-            // while: what was never sent piles up right below the k-th, what lies above it is a thin tail, and
-            // a bound interpolated from the top of the bin lands in the tail (the next selection then finds
-            // fewer than k candidates and starts over).  The second level counts that bin in 1024 parts.
-            if (lbin == bin && bin > 0) {
-              const uint32_t roomy = lrem + want / 16;          // a little beyond, if the bin holds that many
-              one_wrem = roomy <= __ldcg(h + bin) ? roomy : lrem;
-              if (threadIdx.x == 0) ws.sel[s].wrem = one_wrem;
-            }
-          } else if (redo || a.force_two_pass) {
-            lkey = __ldcg(ws.L_wide + s);         // known from the histogram of the whole input
-            lbin = lkey >> 20;
-          } else {
-            // Fewer candidates than wished for (but at least k) and nothing known below the bound: lower it by
-            // as much as would hold the missing ones at the density seen right above it -- what was never sent
-            // piles up below the k-th, so half an octave down may hold a hundred times the wished-for number --
-            // and by half an octave only where too few keys lie above the bound to tell.
-            const uint32_t L_used = a.L_in[s], used = L_used >> 20;
-            uint32_t pop = __ldcg(h + used), width = ((used + 1u) << 20) - L_used;
-            if (pop < 64u && used + 1u < (uint32_t)kBins1) {
-              pop += __ldcg(h + used + 1u);
-              width += 1u << 20;
-            }
-            const float step = 1.5f * (float)(want + want / 16 - total) / (float)max(pop, 1u) * (float)width;
-            if (pop >= 64u && step < (float)(4u << 20)) {
-              const uint32_t down = (uint32_t)step + 1u;
-              lkey = L_used > down ? L_used - down : 0u;
-            } else {
-              lkey = used > 4 ? (used - 4) << 20 : 0u;
-            }
-            lbin = lkey >> 20;
-          }
-          __syncthreads();
-          // A bound of zero makes every element of the layer a candidate (zeros included).  That is fine for a
-          // layer not much larger than the wished-for number of candidates, and for one that is small beside the
-          // whole vector: a layer without enough candidates costs the next selection a histogram and a second pass
-          // over all layers (148 layers of 124 M elements: 570 us a pull when every other one failed on layers of 768
-          // to 3072 elements, 78 us without).  For a large one, no bound at all is the better advice: the next
-          // selection finds nothing, notices, and takes its bound from a histogram.
-          const uint32_t layer_cap = (ws.segs[s].tile_end - ws.segs[s].tile_begin) * (uint32_t)kWarpTile;
-          const bool flood = lkey == 0 && layer_cap / 8 > want && layer_cap > max(8192u, ws.n / 1024u);
-          if (threadIdx.x == 0) a.L_next[s] = flood ? 0xFFFFFFFFu : lkey;
-        }
-      }
-      if (!everyone_picks) {   // the histogram has served; with one layer the others may still be reading it
-        __syncthreads();
-        for (int b = threadIdx.x; b < kBins1; b += kThreads) h[b] = 0;
-      }
-    }
-    if (everyone_picks) {
-      if (!failed || redo) break;
-      // every CTA has seen the same histogram and comes here: clear it once all have read it, then redo
-      if (!worker_barrier(ws.sync, Wb, ws.status, &sh.ok, bar_target, spin_limit)) return;
-      if (cta == 0)
-        for (int b = threadIdx.x; b < kBins1; b += kThreads) ws.hist1[b] = 0;
-      if (!worker_barrier(ws.sync, Wb, ws.status, &sh.ok, bar_target, spin_limit)) return;
-      redo = true;
-    } else {
-      if (!worker_barrier(ws.sync, Wb, ws.status, &sh.ok, bar_target, spin_limit)) return;
-      if (redo || ld_volatile(ws.sync + kFail) == 0) break;
-      redo = true;
-    }
+  const uint32_t* seg_off = ws.seg_off;
+  if (MANY && S <= (uint32_t)kSegCap) {
+    uint32_t* const sm = reinterpret_cast<uint32_t*>(fin_dyn);
+    for (uint32_t s = threadIdx.x; s <= S; s += kThreads) sm[s] = ws.seg_off[s];
+    seg_off = sm;
   }
 
-  uint32_t near_seg = 0;   // layer of the candidate this thread looked at last (S > 1)
-  // visits this thread's candidates in flat order: fn(value, index)
-  auto each_own = [&](auto fn) {
-    if (per_thread <= (uint32_t)kKeep) {
+  uint32_t parts = 0, clo = 0, chi = 0, wlo = 0, whi = 0;   // flat candidates of this CTA, of this warp
+  uint32_t part0 = 0, part1 = 0;         // parts that this warp's candidates lie in
+  bool kept = false;                     // this warp's candidates stay in registers
+  float raw[kKeep];
+  uint32_t idx[kKeep];
+  auto slot_of = [&](uint32_t p, uint32_t lo, uint32_t hi) {
+    const uint32_t part = part_of(sh.pre, lo, hi, p);
+    return __ldcg(ws.part_slot0 + part) + (p - sh.pre[part]);
+  };
+  auto load = [&](uint32_t base) {       // candidates base + 32 u + lane of this warp's run (beyond its end: the last one)
+    uint32_t slot[kKeep];
+#pragma unroll
+    for (int u = 0; u < kKeep; ++u)
+      if (base + u * 32u < whi) slot[u] = slot_of(min(base + u * 32u + lane, whi - 1u), part0, part1);
+#pragma unroll
+    for (int u = 0; u < kKeep; ++u)
+      if (base + u * 32u < whi) {
+        raw[u] = __ldcg(ws.cand_val + slot[u]);
+        idx[u] = __ldcg(ws.cand_idx + slot[u]);
+      }
+  };
+
+  uint32_t s_lo = 0, s_last = 0;         // layers of this CTA's first and last candidate
+  bool goes_on = false;                  // layer s_lo began before this CTA's first candidate
+  LayerPick* tab = sh.tab;               // [s - s_lo]
+  uint32_t near_t = 0, near_b = 1, near_e = 0;   // layer (counted from s_lo) that this lane looked at last
+  auto row_of = [&](uint32_t i) -> LayerPick* {
+    if (MANY && (i < near_b || i >= near_e)) {
+      const uint32_t s = seg_of(seg_off, s_lo, s_last, i);
+      near_t = s - s_lo;
+      near_b = seg_off[s];
+      near_e = seg_off[s + 1];
+    }
+    return tab + near_t;
+  };
+  // Visits this warp's candidates in flat order and counts them: classify(u, row, valid, equal) says whether a candidate
+  // counts as above, and may set `equal`.  Notes where in the count the layers begin; batch(first flat number) is called
+  // after each batch of candidates.  Then the counts of the CTA's last layer are published.
+  auto count = [&](auto classify, auto batch) {
+    uint32_t gt = 0, eq = 0, prev_t = kFull;     // the same in every lane; layer of the candidate before
+    if (MANY && wlo < whi) {
+      if (wlo > clo) {
+        row_of(__ldcg(ws.cand_idx + slot_of(wlo - 1u, 0, parts - 1u)));
+        prev_t = near_t;
+      } else if (goes_on) {
+        prev_t = 0;
+      }
+    }
+#pragma unroll 1
+    for (uint32_t base = wlo; base < whi; base += 32u * kKeep) {
+      if (!kept) load(base);
 #pragma unroll
       for (int u = 0; u < kKeep; ++u)
-        if (my_lo + u < my_hi) fn(rraw[u], ridx[u]);
-    } else if (my_lo < my_hi) {
-      Cursor cur = cursor_at(sh, parts, my_lo);
-      for (uint32_t p = my_lo; p < my_hi; p += kBatch) {
-        // all loads of the batch are issued before any loaded value is touched (a use right
-        // after its load would make the loads wait for one another)
-        float raw[kBatch];
-        uint32_t idx[kBatch];
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-          raw[u] = 0.f;
-          idx[u] = 0;
-          if (p + u < my_hi) {
-            raw[u] = __ldcg(ws.cand_val + cur.slot);
-            idx[u] = __ldcg(ws.cand_idx + cur.slot);
-            cursor_advance(sh, parts, cur, 1);
+        if (base + u * 32u < whi) {
+          const bool valid = base + u * 32u + lane < whi;
+          LayerPick* const t = row_of(idx[u]);
+          bool equal = false;
+          const bool above = classify(u, t, valid, equal);
+          const uint32_t mg = __ballot_sync(kFull, above), me = __ballot_sync(kFull, equal);
+          if (MANY) {
+            uint32_t before = __shfl_up_sync(kFull, near_t, 1);
+            if (lane == 0) before = prev_t;
+            if (valid && before != near_t) {
+              t->start_gt = gt + __popc(mg & lt);
+              t->start_eq = eq + __popc(me & lt);
+              t->start_warp = warp;
+            }
+            prev_t = __shfl_sync(kFull, near_t, 31);
           }
+          gt += __popc(mg);
+          eq += __popc(me);
         }
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u)
-          if (p + u < my_hi) fn(raw[u], idx[u]);
+      batch(base);
+    }
+    if (lane == 0) {
+      sh.gt[warp] = gt;
+      sh.eq[warp] = eq;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && cta < W) {
+      uint32_t g = 0, e = 0;
+      for (int w = 0; w < kWarps; ++w) {
+        g += sh.gt[w];
+        e += sh.eq[w];
       }
+      if (clo < chi && !(goes_on && s_lo == s_last) && MANY) {
+        const LayerPick& t = tab[s_last - s_lo];
+        for (uint32_t w = 0; w < t.start_warp; ++w) {
+          g -= sh.gt[w];
+          e -= sh.eq[w];
+        }
+        g -= t.start_gt;
+        e -= t.start_eq;
+      }
+      ws.cta_tot[cta] = make_uint2(clo < chi ? s_last : kFull, g);
+      ws.cta_eq[cta] = e;
     }
   };
 
-  // ---- levels 2 and 3 ----------------------------------------------------------------
+  bool redo = false;
+  uint32_t flags = 0;
 #pragma unroll 1
-  for (int level = 2; level <= 3; ++level) {
-    uint32_t* hist = level == 2 ? ws.hist2 : ws.hist3;
-    constexpr int B = kBins2;   // both levels have 1024 bins
-    const int SH = level == 2 ? 20 : 10;
-    if (S == 1) {
-      for (int b = threadIdx.x; b < B; b += kThreads) sh.stream.hist[b] = 0;
-      __syncthreads();
-      each_own([&](float v, uint32_t) {
-        const uint32_t key = key_of(v);
-        if ((key >> SH) == one_prefix) atomicAdd(sh.stream.hist + ((key >> (SH - 10)) & 1023u), 1u);
-      });
-      __syncthreads();
-      for (int b = threadIdx.x; b < B; b += kThreads) {
-        const uint32_t v = sh.stream.hist[b];
-        if (v) atomicAdd(hist + b, v);
-      }
-      if (!worker_barrier(ws.sync, Wb, ws.status, &sh.ok, bar_target, spin_limit)) return;
-      // the histogram of the level before has been read by everyone
-      if (cta == 0) {
-        uint32_t* old = level == 2 ? ws.hist1 : ws.hist2;
-        for (int b = threadIdx.x; b < (level == 2 ? kBins1 : kBins2); b += kThreads) old[b] = 0;
-      }
-      uint32_t bin, krem;
-      block_pick<B>(hist, one_krem, bin, krem, sh.warp_scan, sh.res);
-      if (level == 2 && cta == 0 && one_wrem) {   // (CTA-uniform) the suggested bound: lower edge of the part that holds its entry
-        uint32_t wsub, wleft;
-        block_pick<B>(hist, one_wrem, wsub, wleft, sh.warp_scan, sh.res);
-        if (threadIdx.x == 0) a.L_next[0] = ((one_prefix << 10) | wsub) << 10;
-      }
-      one_prefix = (one_prefix << 10) | bin;
-      one_krem = krem;
-    } else {
-      if (seg_smem) {
-        for (uint32_t s = threadIdx.x; s < S; s += kThreads) sm_seg_a[s] = __ldcg(&ws.sel[s].prefix);
-        __syncthreads();
-      }
-      each_own([&](float v, uint32_t idx) {
-        const uint32_t key = key_of(v);
-        const uint32_t seg = seg_near(seg_off, S, idx, near_seg);
-        const uint32_t prefix = seg_smem ? sm_seg_a[seg] : __ldcg(&ws.sel[seg].prefix);
-        if ((key >> SH) == prefix) atomicAdd(hist + (size_t)seg * B + ((key >> (SH - 10)) & 1023u), 1u);
-      });
-      if (!worker_barrier(ws.sync, Wb, ws.status, &sh.ok, bar_target, spin_limit)) return;
-      for (uint32_t s = cta; s < S; s += W) {
-        uint32_t bin, krem;
-        uint32_t* h = hist + (size_t)s * B;
-        block_pick<B>(h, __ldcg(&ws.sel[s].krem), bin, krem, sh.warp_scan, sh.res);
-        const uint32_t wrem = level == 2 ? __ldcg(&ws.sel[s].wrem) : 0u;   // written by this CTA at the first level
-        if (wrem) {
-          uint32_t wsub, wleft;
-          block_pick<B>(h, wrem, wsub, wleft, sh.warp_scan, sh.res);
-          if (threadIdx.x == 0) a.L_next[s] = ((__ldcg(&ws.sel[s].prefix) << 10) | wsub) << 10;
-          __syncthreads();   // the prefix is read before it is extended below
-        }
-        if (threadIdx.x == 0) {
-          const uint32_t pre = (__ldcg(&ws.sel[s].prefix) << 10) | bin;
-          ws.sel[s].prefix = pre;
-          ws.sel[s].krem = krem;
-          if (level == 3) {
-            ws.sel[s].T = pre;   // all 31 key bits are fixed now
-            ws.sel[s].r = krem;
-            ws.sel[s].neq = __ldcg(h + bin);
+  for (int attempt = 0; attempt < 2; ++attempt) {
+    if (redo) {
+      if (!redo_passes<MODE>(ws, a, in, out, sh.stream, sh.warp_scan, sh.res, &sh.ok, Wb, spin_limit, bar_target)) return;
+    }
+    const uint32_t* const L_used = redo ? ws.L_safe : a.L_in;
+    if (cta >= W) {
+      // checks the guesses (a layer needs at least k candidates) and suggests the next bounds
+      uint32_t seen = 0;
+      for (uint32_t s = (cta - W) * kWarps + warp; s < S; s += A * kWarps) {
+        const uint32_t* const h = ws.hist1 + (size_t)s * kBins1;
+        const uint32_t k = ws.segs[s].k[PM], L = __ldcg(L_used + s);
+        const uint32_t sum = lane_bins(h, lane), incl = warp_incl(sum, lane), total = __shfl_sync(kFull, incl, 31);
+        uint32_t flag = 1u;
+        if (total >= k) {
+          flag = warp_pick(h, incl, sum, k, lane).pop > ws.segs[s].list_cap ? 2u : 0u;
+          if (a.speculate) {
+            const uint32_t key = next_bound(ws, s, h, L, total, spec_want(k), incl, sum, redo || a.force_two_pass, lane);
+            if (lane == 0) ws.sel[s].next = key;   // (L_next may be the row that the other CTAs still read L from)
           }
         }
+        if (flag && lane == 0) atomicOr(ws.sync + kFail, flag);
+        seen += total;
+      }
+      if (lane == 0 && seen) atomicAdd(ws.stats + 2, (unsigned long long)seen);
+      clo = chi = wlo = whi = 0;
+    } else {
+      // flat numbering of the candidates (the stream pass is complete: an earlier kernel, or the barrier above)
+      parts = ld_volatile(ws.sync + kParts);
+      number_parts<kPartCap>(ws, parts, sh.pre, sh.warp_scan);
+      const uint32_t C = sh.pre[parts];
+      const uint32_t per_warp = (uint32_t)(((uint64_t)C + W * kWarps * 32u - 1u) / (W * kWarps * 32u)) * 32u;
+      clo = (uint32_t)min((uint64_t)C, (uint64_t)cta * kWarps * per_warp);
+      chi = (uint32_t)min((uint64_t)C, (uint64_t)(cta + 1) * kWarps * per_warp);
+      wlo = (uint32_t)min((uint64_t)chi, (uint64_t)clo + warp * per_warp);
+      whi = (uint32_t)min((uint64_t)chi, (uint64_t)wlo + per_warp);
+      kept = per_warp <= 32u * kKeep;
+      if (wlo < whi) {
+        part0 = warp_part_of(sh.pre, parts, wlo, lane);
+        part1 = warp_part_of(sh.pre, parts, whi - 1u, lane);
+        if (kept) load(wlo);
+      }
+      s_lo = s_last = 0;
+      near_t = 0;
+      near_b = 1;
+      near_e = 0;
+      goes_on = clo > 0;
+      if (MANY) {
+        if (threadIdx.x < 3 && clo < chi) {
+          const uint32_t p = threadIdx.x == 0 ? (clo > 0 ? clo - 1u : clo) : threadIdx.x == 1 ? clo : chi - 1u;
+          sh.range[threadIdx.x] = seg_of(seg_off, 0, S - 1u, __ldcg(ws.cand_idx + slot_of(p, 0, parts - 1u)));
+        }
         __syncthreads();
-        for (int b = threadIdx.x; b < B; b += kThreads) h[b] = 0;
-      }
-      if (!worker_barrier(ws.sync, Wb, ws.status, &sh.ok, bar_target, spin_limit)) return;
-    }
-  }
-
-  // ---- count: (key > T, key == T) among this thread's candidates, prefix inside the CTA -------
-  if (S > 1) {
-    if (seg_smem) {
-      for (uint32_t s = threadIdx.x; s < S; s += kThreads) {
-        sm_seg_a[s] = __ldcg(&ws.sel[s].T);
-        sm_seg_b[s] = __ldcg(&ws.sel[s].r);
+        if (clo < chi) {
+          s_lo = sh.range[1];
+          s_last = sh.range[2];
+          goes_on = clo > 0 && sh.range[0] == s_lo;
+        }
       }
     }
-    if (cta == 0) {
-      // (key > T, key == T) candidates of all earlier layers: layer s selects k_s - r_s of the first kind
-      unsigned long long carry = 0;
-      for (uint32_t base = 0; base < S; base += kThreads) {
-        const uint32_t s = base + threadIdx.x;
-        unsigned long long v = 0;
-        if (s < S) v = ((unsigned long long)(ws.segs[s].k[PM] - __ldcg(&ws.sel[s].r)) << 32) | __ldcg(&ws.sel[s].neq);
-        unsigned long long total;
-        const unsigned long long ex = block_excl_scan(v, sh.warp_scan, total) + carry;
-        if (s < S) ws.seg_start[s] = make_uint2((uint32_t)(ex >> 32), (uint32_t)ex);
-        carry += total;
+    const uint32_t touched = clo < chi ? s_last - s_lo + 1u : 0u;
+    tab = touched <= (uint32_t)kTouch ? sh.tab : ws.tab + s_lo + cta;   // (two CTAs share at most a layer: their rows differ)
+    if (!MANY ? touched != 0 : touched == 1) {
+      uint32_t bin, krem;
+      const uint32_t k = ws.segs[s_lo].k[PM];
+      const uint32_t total = block_pick<kBins1>(ws.hist1 + (size_t)s_lo * kBins1, k, bin, krem, sh.warp_scan, sh.res);
+      if (threadIdx.x == 0) {
+        LayerPick& t = tab[0];
+        const uint32_t pop = sh.res[2];
+        t.L = __ldcg(L_used + s_lo);
+        t.bin = total < k ? kFull : bin;
+        t.krem = krem;
+        t.pop = pop > ws.segs[s_lo].list_cap ? 0u : pop;
+        t.pkt_off = ws.segs[s_lo].pkt_off[PM];
+        t.list_off = ws.segs[s_lo].list_off;
+      }
+    } else if (MANY) {
+#pragma unroll 1
+      for (uint32_t t0 = warp; t0 < touched; t0 += kWarps) {
+        const uint32_t s = s_lo + t0, k = ws.segs[s].k[PM], L = __ldcg(L_used + s);
+        const uint32_t list_cap = ws.segs[s].list_cap, list_off = ws.segs[s].list_off, pkt_off = ws.segs[s].pkt_off[PM];
+        const uint32_t* const h = ws.hist1 + (size_t)s * kBins1;
+        const uint32_t sum = lane_bins(h, lane), incl = warp_incl(sum, lane);
+        BinPick b = {kFull, 0, 0};
+        if (__shfl_sync(kFull, incl, 31) >= k) b = warp_pick(h, incl, sum, k, lane);
+        if (lane == 0) {
+          LayerPick& t = tab[t0];
+          t.L = L;
+          t.bin = b.bin;
+          t.krem = b.rem;
+          t.pop = b.pop > list_cap ? 0u : b.pop;
+          t.pkt_off = pkt_off;
+          t.list_off = list_off;
+        }
       }
     }
     __syncthreads();
+    // candidates above the k-th's bin are counted, those in it go to the layer's list
+    uint32_t hits = 0;
+    count([&](int u, const LayerPick* t, bool valid, bool&) {
+      const uint32_t b = bin_of(key_of(raw[u]), t->L), bin = t->bin;
+      if (valid && b == bin && t->pop) hits |= 1u << u;
+      return valid && bin != kFull && b > bin;
+    }, [&](uint32_t base) {
+      if (!MANY) {                       // one layer: a place for all hits of the warp at once
+        uint32_t n = 0, at = 0;
+#pragma unroll
+        for (int u = 0; u < kKeep; ++u) n += __popc(__ballot_sync(kFull, (hits >> u) & 1u));
+        if (n) {
+          if (lane == 0) at = sh.tab[0].list_off + atomicAdd(ws.list_cnt, n);
+          at = __shfl_sync(kFull, at, 0);
+#pragma unroll
+          for (int u = 0; u < kKeep; ++u) {
+            const uint32_t m = __ballot_sync(kFull, (hits >> u) & 1u);
+            if ((hits >> u) & 1u) ws.list[at + __popc(m & lt)] = make_uint2(key_of(raw[u]), base + u * 32u + lane);
+            at += __popc(m);
+          }
+          hits = 0;
+        }
+      }
+      if (MANY) {
+        uint32_t todo;
+        while ((todo = __ballot_sync(kFull, hits != 0)) != 0) {   // rarely more than one layer
+          uint32_t i = idx[0];
+#pragma unroll
+          for (int u = 1; u < kKeep; ++u)
+            if (hits && u == __ffs(hits) - 1) i = idx[u];
+          const LayerPick* const t = row_of(__shfl_sync(kFull, i, __ffs(todo) - 1));   // the layer of the first hit: for all lanes
+          uint32_t n = 0, at = 0, mine = 0;
+#pragma unroll
+          for (int u = 0; u < kKeep; ++u) {
+            const bool in = ((hits >> u) & 1u) && idx[u] >= near_b && idx[u] < near_e;
+            mine |= in ? 1u << u : 0u;
+            n += __popc(__ballot_sync(kFull, in));
+          }
+          if (lane == 0) at = t->list_off + atomicAdd(ws.list_cnt + s_lo + near_t, n);
+          at = __shfl_sync(kFull, at, 0);
+#pragma unroll
+          for (int u = 0; u < kKeep; ++u) {
+            const uint32_t m = __ballot_sync(kFull, (mine >> u) & 1u);
+            if ((mine >> u) & 1u) ws.list[at + __popc(m & lt)] = make_uint2(key_of(raw[u]), base + u * 32u + lane);
+            at += __popc(m);
+          }
+          hits &= ~mine;
+        }
+      }
+      __syncwarp();
+    });
+    if (!barrier()) return;
+    flags = ld_volatile(ws.sync + kFail);
+    if (!(flags & 1u) || redo) break;
+    if (!barrier()) return;              // everyone has seen the flags
+    redo = true;
   }
-  unsigned long long mine = 0;   // (gt << 32) | eq
-  each_own([&](float v, uint32_t idx) {
-    const uint32_t key = key_of(v);
-    uint32_t T = one_prefix;
-    if (S > 1) {
-      const uint32_t seg = seg_near(seg_off, S, idx, near_seg);
-      T = seg_smem ? sm_seg_a[seg] : __ldcg(&ws.sel[seg].T);
+  const uint32_t touched = clo < chi ? s_last - s_lo + 1u : 0u;
+  // what the next selection expects to find cleared, and the bounds it may use
+  {
+    uint4* const h4 = reinterpret_cast<uint4*>(ws.hist1);
+    for (size_t w = gthread; w < (size_t)S * (kBins1 / 4); w += nthreads) h4[w] = make_uint4(0, 0, 0, 0);
+  }
+  if (cta >= W) {
+    if (a.speculate)
+      for (uint32_t s = (cta - W) * kThreads + threadIdx.x; s < S; s += A * kThreads) a.L_next[s] = __ldcg(&ws.sel[s].next);
+    for (uint32_t s = (cta - W) * kThreads + threadIdx.x; s < S; s += A * kThreads) ws.list_cnt[s] = 0;
+  }
+  uint2* const s_list = reinterpret_cast<uint2*>(sh.stream.hist);   // the list, where it is ranked in shared memory
+  const bool ranked = !MANY && touched && !(flags & 2u) && tab[0].pop <= (uint32_t)kListSmem;
+  if (ranked) {
+    // a thread per entry compares it with every other one
+    const uint32_t pop = tab[0].pop, k = tab[0].krem;
+    uint2 mine = make_uint2(0, 0);
+    if (threadIdx.x < pop) {
+      mine = __ldcg(ws.list + tab[0].list_off + threadIdx.x);
+      s_list[threadIdx.x] = mine;
     }
-    if (key > T) mine += 1ull << 32;
-    else if (key == T) mine += 1ull;
-  });
-  unsigned long long cta_total;
-  unsigned long long before = block_excl_scan(mine, sh.warp_scan, cta_total);
-  if (threadIdx.x == 0) ws.cta_tot[cta] = make_uint2((uint32_t)(cta_total >> 32), (uint32_t)cta_total);
-  if (!worker_barrier(ws.sync, Wb, ws.status, &sh.ok, bar_target, spin_limit)) return;
-  if (S == 1 && cta == 0)
-    for (int b = threadIdx.x; b < kBins3; b += kThreads) ws.hist3[b] = 0;
+    __syncthreads();
+    if (threadIdx.x < pop) {
+      uint32_t above = 0, same = 0;
+#pragma unroll 4
+      for (uint32_t q = 0; q < pop; ++q) {
+        const uint32_t o = s_list[q].x;
+        above += o > mine.x ? 1u : 0u;
+        same += o == mine.x ? 1u : 0u;
+      }
+      if (above < k && k <= above + same) {   // (the same for all that are equal)
+        tab[0].T = mine.x;
+        tab[0].r = k - above;
+      }
+    }
+    __syncthreads();
+  } else if (!(flags & 2u)) {
+#pragma unroll 1
+    for (uint32_t t = warp; t < touched; t += kWarps) {
+      const uint32_t L = tab[t].L, bin = tab[t].bin, sft = bin_shift(L);
+      const bool open = bin == (uint32_t)kBins1 - 1u;    // (the last bin is open-ended)
+      uint32_t r;
+      const uint32_t T = warp_radix(ws.list + tab[t].list_off, tab[t].pop, tab[t].krem, open ? 0u : L + (bin << sft),
+                                    open ? 31 : (int)sft, sh.stream.hist + warp * 128, lane, r);
+      if (lane == 0) {
+        tab[t].T = T;
+        tab[t].r = r;
+      }
+    }
+    __syncthreads();
+  } else {
+    // Some bin holds more candidates than its list (many equal values, or a bound far below the k-th): three radix
+    // levels (11 + 10 + 10 key bits) over all candidates, counted in global memory, the picks spread over the CTAs.
+    if (!barrier()) return;              // the histograms are clear
+#pragma unroll 1
+    for (int level = 1; level <= 3; ++level) {
+      const int sft = level == 1 ? 20 : level == 2 ? 10 : 0;
+#pragma unroll 1
+      for (uint32_t base = wlo; base < whi; base += 32u * kKeep) {
+        if (!kept) load(base);
+#pragma unroll
+        for (int u = 0; u < kKeep; ++u)
+          if (base + u * 32u < whi) {
+            const uint32_t key = key_of(raw[u]);
+            row_of(idx[u]);
+            const uint32_t s = s_lo + near_t;
+            const bool mine = base + u * 32u + lane < whi && (level == 1 || (key >> (sft + 10)) == __ldcg(&ws.sel[s].prefix));
+            const uint32_t at = s * (uint32_t)kBins1 + (level == 1 ? key >> 20 : (key >> sft) & 1023u);
+            // lanes with the first one's bin are counted together: ties crowd into few bins
+            const uint32_t m = __ballot_sync(kFull, mine);
+            if (m) {
+              const uint32_t lead = __shfl_sync(kFull, at, __ffs(m) - 1), same = __ballot_sync(kFull, mine && at == lead);
+              if (lane == __ffs(m) - 1) atomicAdd(ws.hist1 + lead, (uint32_t)__popc(same));
+              if (mine && at != lead) atomicAdd(ws.hist1 + at, 1u);
+            }
+          }
+      }
+      if (!barrier()) return;
+      for (uint32_t s = cta; s < S; s += W + A) {
+        uint32_t bin, krem;
+        uint32_t* const h = ws.hist1 + (size_t)s * kBins1;
+        const uint32_t k = level == 1 ? ws.segs[s].k[PM] : __ldcg(&ws.sel[s].krem);
+        const uint32_t old = level == 1 ? 0u : __ldcg(&ws.sel[s].prefix);
+        block_pick<kBins1>(h, k, bin, krem, sh.warp_scan, sh.res);
+        if (threadIdx.x == 0) {
+          ws.sel[s].prefix = level == 1 ? bin : (old << 10) | bin;
+          ws.sel[s].krem = krem;
+        }
+        __syncthreads();
+        for (int b = threadIdx.x; b < kBins1; b += kThreads) h[b] = 0;
+      }
+      if (!barrier()) return;
+    }
+    for (uint32_t t = threadIdx.x; t < touched; t += kThreads) {
+      tab[t].T = __ldcg(&ws.sel[s_lo + t].prefix);
+      tab[t].r = __ldcg(&ws.sel[s_lo + t].krem);
+    }
+    __syncthreads();
+    count([&](int u, const LayerPick* t, bool valid, bool& equal) {
+      const uint32_t key = key_of(raw[u]), T = t->T;
+      equal = valid && key == T;
+      return valid && key > T;
+    }, [](uint32_t) {});
+    if (!barrier()) return;
+  }
 
   // ---- emit: packet in index order, and the state updates that depend on selection ----
-  {
-    unsigned long long lower = 0;   // totals of the CTAs before this one (W <= kMaxWorkers)
-    for (uint32_t c = threadIdx.x; c < cta; c += kThreads) {
-      const uint2 q = __ldcg(ws.cta_tot + c);
-      lower += ((unsigned long long)q.x << 32) | q.y;
-    }
-    unsigned long long lower_total;
-    block_excl_scan(lower, sh.warp_scan, lower_total);
-    before += lower_total;
-    if (S > 1 && seg_smem) {
-      for (uint32_t s = threadIdx.x; s < S; s += kThreads) sm_seg_start[s] = __ldcg(ws.seg_start + s);
-      __syncthreads();
-    }
-    uint32_t gt_before = (uint32_t)(before >> 32), eq_before = (uint32_t)before;   // over all layers
-    each_own([&](float val, uint32_t idx) {
-      const uint32_t key = key_of(val);
-      uint32_t T = one_prefix, r = one_krem, pkt_off = 0;
-      uint2 start = make_uint2(0, 0);
-      if (S > 1) {
-        const uint32_t seg = seg_near(seg_off, S, idx, near_seg);
-        T = seg_smem ? sm_seg_a[seg] : __ldcg(&ws.sel[seg].T);
-        r = seg_smem ? sm_seg_b[seg] : __ldcg(&ws.sel[seg].r);
-        start = seg_smem ? sm_seg_start[seg] : __ldcg(ws.seg_start + seg);
-        pkt_off = ws.segs[seg].pkt_off[PM];
+  if (wlo < whi) {
+    // selected entries of the first candidate's layer that stand before it
+    uint32_t run_gt = 0, run_eq = 0;
+    if (!kept) load(wlo);
+    const LayerPick* const t0 = row_of(__shfl_sync(kFull, idx[0], 0));
+    uint32_t carry_t = near_t;
+    const bool before = goes_on && carry_t == 0;         // it began before this CTA
+    if (!(flags & 2u)) {
+      const uint32_t T = t0->T, pop = t0->pop;
+      const uint2* const list = ws.list + t0->list_off;
+#pragma unroll 1
+      for (uint32_t q = lane; q < pop; q += 32) {
+        const uint2 e = ranked ? s_list[q] : __ldcg(list + q);
+        if (e.y < wlo) {
+          run_gt += e.x > T ? 1u : 0u;
+          run_eq += e.x == T ? 1u : 0u;
+        }
       }
-      const bool is_gt = key > T, is_eq = key == T;
-      const uint32_t eq_in_layer = eq_before - start.y;
-      const bool sel = is_gt || (is_eq && eq_in_layer < r);
-      if (sel) {
-        const uint32_t pos = pkt_off + (gt_before - start.x) + min(eq_in_layer, r);
-        const float q = round16(val, a.packet_format);   // what the packet carries (val itself with float32 packets)
-        if (pos < a.pkt_count) {
-          a.pkt_idx[pos] = idx;
-          a.pkt_val[pos] = q;
-        } else {
-          atomicMin(ws.status, -1000 - MODE);
+    }
+    if (before)
+#pragma unroll 4
+      for (uint32_t c = lane; c < cta; c += 32) {
+        const uint2 q = __ldcg(ws.cta_tot + c);
+        const uint32_t e = __ldcg(ws.cta_eq + c);
+        if (q.x == s_lo) {
+          run_gt += q.y;
+          run_eq += e;
         }
-        // Algorithm 1: the sent part leaves v (what a rounded packet did not carry stays: val - q, else zero).
-        // Algorithm 3 keeps the sent entry's velocity t (already stored): no residual exists to take val - q.
-        if (MODE == kPushResidual) out[idx] = __fsub_rn(val, q);
-        if (MODE == kPull) {
-          a.D[idx] = __fsub_rn(val, q);                  // Eq. 6b: v_k <- v_k + G; the rounding remainder stays
-          if (a.theta_local) a.theta_local[idx] = __fadd_rn(a.theta_local[idx], q);  // Eq. 5
-        }
+      }
+    if (lane < kWarps && lane < warp) {
+      run_gt += sh.gt[lane];
+      run_eq += sh.eq[lane];
+    }
+    if (MANY && !before && lane <= (int)t0->start_warp) {   // the layer began in this CTA: without what was counted before it
+      if (lane < (int)t0->start_warp) {
+        run_gt -= sh.gt[lane];
+        run_eq -= sh.eq[lane];
       } else {
-        if (MODE == kPushSam) out[idx] = __fmul_rn(val, a.inv_m);  // Eq. 12, lower branch
+        run_gt -= t0->start_gt;
+        run_eq -= t0->start_eq;
       }
-      gt_before += is_gt ? 1u : 0u;
-      eq_before += is_eq ? 1u : 0u;
-    });
+    }
+    run_gt = __reduce_add_sync(kFull, run_gt);
+    run_eq = __reduce_add_sync(kFull, run_eq);
+#pragma unroll 1
+    for (uint32_t base = wlo; base < whi; base += 32u * kKeep) {
+      if (!kept && base != wlo) load(base);
+      uint32_t pos[kKeep];               // place in the packet, kFull: not selected
+#pragma unroll
+      for (int u = 0; u < kKeep; ++u) {
+        pos[u] = kFull;
+        if (base + u * 32u < whi) {
+          const bool valid = base + u * 32u + lane < whi;
+          const LayerPick* const t = row_of(idx[u]);
+          const uint32_t key = key_of(raw[u]), T = t->T;
+          const bool above = valid && key > T, equal = valid && key == T;
+          const uint32_t mg = __ballot_sync(kFull, above), me = __ballot_sync(kFull, equal);
+          uint32_t in_layer = kFull, heads = 0;              // lanes of this lane's layer, counted from its first one
+          if (MANY) {
+            uint32_t prev = __shfl_up_sync(kFull, near_t, 1);
+            if (lane == 0) prev = carry_t;
+            heads = __ballot_sync(kFull, prev != near_t);
+            carry_t = __shfl_sync(kFull, near_t, 31);
+            if (heads & le) in_layer = kFull << (31 - __clz(heads & le));
+          }
+          const bool first = (heads & le) != 0;              // the layer begins among these 32
+          const uint32_t gt_rank = (first ? 0u : run_gt) + __popc(mg & lt & in_layer);
+          const uint32_t eq_rank = (first ? 0u : run_eq) + __popc(me & lt & in_layer);
+          const uint32_t r = t->r;
+          if (above || (equal && eq_rank < r)) pos[u] = t->pkt_off + gt_rank + min(eq_rank, r);
+          const uint32_t tail = heads ? kFull << (31 - __clz(heads)) : kFull;
+          run_gt = (heads ? 0u : run_gt) + __popc(mg & tail);
+          run_eq = (heads ? 0u : run_eq) + __popc(me & tail);
+        }
+      }
+      float local[kKeep];
+      if (MODE == kPull && a.theta_local != nullptr) {
+#pragma unroll
+        for (int u = 0; u < kKeep; ++u) local[u] = pos[u] != kFull ? __ldcg(a.theta_local + idx[u]) : 0.f;
+      }
+#pragma unroll
+      for (int u = 0; u < kKeep; ++u) {
+        if (pos[u] != kFull) {
+          const float q = round16(raw[u], a.packet_format);  // what the packet carries (the value itself with float32 packets)
+          if (pos[u] < a.pkt_count) {
+            a.pkt_idx[pos[u]] = idx[u];
+            a.pkt_val[pos[u]] = q;
+          } else {
+            atomicMin(ws.status, -1000 - MODE);
+          }
+          // Algorithm 1: the sent part leaves v (what a rounded packet did not carry stays: val - q, else zero).
+          // Algorithm 3 keeps the sent entry's velocity t (already stored): no residual exists to take val - q.
+          if (MODE == kPushResidual) out[idx[u]] = __fsub_rn(raw[u], q);
+          if (MODE == kPull) {
+            a.D[idx[u]] = __fsub_rn(raw[u], q);              // Eq. 6b: v_k <- v_k + G; the rounding remainder stays
+            if (a.theta_local) a.theta_local[idx[u]] = __fadd_rn(local[u], q);  // Eq. 5
+          }
+        } else if (MODE == kPushSam && base + u * 32u + lane < whi) {
+          out[idx[u]] = __fmul_rn(raw[u], a.inv_m);          // Eq. 12, lower branch
+        }
+      }
+    }
   }
-  if (cta == 0 && threadIdx.x == 0) {
+  if (cta == W && threadIdx.x == 0) {
     if (MODE != kPull) {  // the spare buffer now holds the worker's velocity
       float* cur = *a.u_cur_slot;
       *a.u_cur_slot = *a.u_spare_slot;
@@ -1374,27 +1672,14 @@ __global__ void __launch_bounds__(kThreads, 4) k_hist_all(Workspace ws, SelArgs 
   hist_all_tiles<MODE>(ws, a, in, blockIdx.x, gridDim.x, s_hist);
 }
 
-// one CTA per layer (strided): L_safe = lower edge of the top-11-bit bin holding the k-th largest key,
-// L_wide = a bound that admits about max(1.5 k, k+64) entries (the bound suggested for later selections)
+// one CTA per layer (strided)
 template <int MODE>
 __global__ void __launch_bounds__(kThreads) k_pick_lower(Workspace ws) {
   __shared__ unsigned long long s_warp[kWarps];
-  __shared__ uint32_t s_res[2];
-  constexpr int PM = MODE == kPull ? 1 : 0;
+  __shared__ uint32_t s_res[3];
   for (uint32_t s = blockIdx.x; s < ws.num_segs; s += gridDim.x) {
-    uint32_t bin, krem;
-    uint32_t* h = ws.hist1 + (size_t)s * kBins1;
-    const uint32_t k = ws.segs[s].k[PM];
-    const uint32_t total = block_pick<kBins1>(h, k, bin, krem, s_warp, s_res);
-    uint32_t wbin = 0, wrem = 0;
-    const uint32_t want = spec_want(k);
-    if (total >= want) block_pick<kBins1>(h, want, wbin, wrem, s_warp, s_res);
-    if (threadIdx.x == 0) {
-      ws.L_safe[s] = bin << 20;
-      ws.L_wide[s] = total >= want ? bound_inside_bin(wbin, wrem, __ldcg(h + wbin), 0u) : 0u;
-    }
+    pick_lower(ws, s, ws.segs[s].k[MODE == kPull ? 1 : 0], s_warp, s_res);
     __syncthreads();
-    for (int b = threadIdx.x; b < kBins1; b += kThreads) h[b] = 0;
   }
 }
 
@@ -1407,7 +1692,7 @@ __global__ void __maxnreg__(64) k_stream(Workspace ws, SelArgs a) {
   __shared__ int s_dead;
   const float* in = *a.u_cur_slot;
   float* out = *a.u_spare_slot;
-  if (blockIdx.x == 0 && threadIdx.x == 0) ws.sync[kBarCount] = 0;   // for the finalize launch that follows
+  if (blockIdx.x == 0 && threadIdx.x == 0) ws.sync[kBarCount] = ws.sync[kFail] = 0;   // for the finalize launch that follows
   stream_tiles_tma<MODE>(ws, a, a.L_in, in, out, blockIdx.x, gridDim.x, sh, reinterpret_cast<float*>(dyn_smem), full,
                          &s_dead);
 }
@@ -1423,10 +1708,10 @@ __global__ void __launch_bounds__(kThreads) k_emit_all(Workspace ws, float* __re
                                                        uint32_t* __restrict__ blk_max, uint32_t* __restrict__ out_idx,
                                                        float* __restrict__ out_val, uint32_t* __restrict__ out_count,
                                                        uint32_t capacity, int packet_format) {
-  __shared__ uint32_t pre[kMaxParts + 1], slot0[kMaxParts];
+  __shared__ uint32_t pre[kMaxParts + 1];
   __shared__ unsigned long long warp_scan[kWarps];
   const uint32_t parts = ld_volatile(ws.sync + kParts);
-  number_parts(ws, parts, pre, slot0, warp_scan);
+  number_parts<kMaxParts>(ws, parts, pre, warp_scan);
   const uint32_t C = pre[parts];
   const bool all = C <= capacity;          // every nonzero entry is sent: D_w is zero afterwards
   const uint32_t take = all ? C : capacity;
@@ -1436,12 +1721,7 @@ __global__ void __launch_bounds__(kThreads) k_emit_all(Workspace ws, float* __re
     atomicAdd(ws.stats + 2, (unsigned long long)C);
   }
   for (uint32_t p = blockIdx.x * kThreads + threadIdx.x; p < take; p += gridDim.x * kThreads) {
-    uint32_t lo = 0, hi = parts - 1;       // last part with pre[part] <= p
-    while (lo < hi) {
-      const uint32_t mid = (lo + hi + 1) >> 1;
-      if (pre[mid] <= p) lo = mid; else hi = mid - 1;
-    }
-    const uint32_t slot = slot0[lo] + (p - pre[lo]);
+    const uint32_t part = part_of(pre, 0, parts - 1u, p), slot = __ldcg(ws.part_slot0 + part) + (p - pre[part]);
     const uint32_t i = __ldcg(ws.cand_idx + slot);
     const float v = __ldcg(ws.cand_val + slot);
     const float q = round16(v, packet_format);
@@ -1453,7 +1733,7 @@ __global__ void __launch_bounds__(kThreads) k_emit_all(Workspace ws, float* __re
     // with everything sent unrounded the whole block is zero now
     if (all && packet_format == 0 && blk_max != nullptr) blk_max[i / kWarpTile] = 0;
   }
-  // the pass has added the candidates' top key bits to the layers' histograms: nobody reads them here
+  // the pass has counted the candidates in the layers' histograms: nobody reads them here
   const size_t words = (size_t)ws.num_segs * kBins1;
   for (size_t w = (size_t)blockIdx.x * kThreads + threadIdx.x; w < words; w += (size_t)gridDim.x * kThreads) ws.hist1[w] = 0;
 }
@@ -1568,7 +1848,7 @@ struct FoldStage {                  // one block of one warp
   uint2 ent[1];                     // [ahead] entries that are fetched while the block before is worked on
 };
 struct FoldShared {
-  uint32_t hist[kBins1];            // SCAN: top 11 key bits of the candidates of the CTA's main layer
+  uint32_t hist[kBins1];            // SCAN: candidates of the CTA's main layer, by bin_of
   uint32_t warp_sum[kFoldWarps];
   uint32_t start[kFoldWarps + 1];   // first block of each warp's run (counted from the CTA's first)
   uint32_t read;
@@ -1750,7 +2030,7 @@ __device__ __noinline__ uint32_t scan_mixed(const Workspace& ws, const SelArgs& 
     ws.cand_idx[pos] = base + off;
     ws.cand_val[pos] = v;
     ++pos;
-    atomicAdd(ws.hist1 + (size_t)s * kBins1 + (key_of(v) >> 20), 1u);
+    atomicAdd(ws.hist1 + (size_t)s * kBins1 + bin_of(key_of(v), a.L_in[s]), 1u);
   }
   __syncwarp();
   return total;
@@ -1787,7 +2067,7 @@ __global__ void __maxnreg__(64) k_fold(const __grid_constant__ Workspace ws, con
     sh.read = 0;
     if (SCAN && cta == 0) {
       ws.sync[kParts] = G * nw;
-      ws.sync[kBarCount] = 0;   // for the finalize launch that follows
+      ws.sync[kBarCount] = ws.sync[kFail] = 0;   // for the finalize launch that follows
     }
   }
 
@@ -1996,7 +2276,8 @@ __global__ void __maxnreg__(64) k_fold(const __grid_constant__ Workspace ws, con
           ws.cand_idx[pos] = base + off;
           ws.cand_val[pos] = c;
           ++pos;
-          atomicAdd(seg == main_seg ? sh.hist + (key_of(c) >> 20) : ws.hist1 + (size_t)seg * kBins1 + (key_of(c) >> 20), 1u);
+          const uint32_t bin = bin_of(key_of(c), L);
+          atomicAdd(seg == main_seg ? sh.hist + bin : ws.hist1 + (size_t)seg * kBins1 + bin, 1u);
         }
       }
     } else {

@@ -26,6 +26,7 @@ namespace dgs {
 
 constexpr int kTopkThreads = 1024, kTopkWarps = kTopkThreads / 32;
 constexpr uint32_t kTopkMaxCluster = 16;   // (more than 8 is not portable to every GPU: the launch asks for it)
+constexpr int kBins2 = 1024;               // levels 2 and 3 (level 1: kBins1, the top 11 key bits)
 constexpr uint32_t kTopkSample = kTopkThreads;   // one element a thread
 constexpr uint32_t kTopkCap = 736;         // most elements a warp can list: 184 KB of lists per CTA
 constexpr int kStatusRank = -1002;         // an entry got a rank that cannot be
@@ -36,7 +37,7 @@ __device__ int g_topk_status;
 struct TopkShared {
   uint32_t hist[kBins1];                     // this CTA's counts of the level in hand
   uint32_t sum1[kBins1], again1[kBins1];     // first CTA of the cluster: counts of all CTAs, level 1 (lists; slices)
-  uint32_t sum2[kBins2], sum3[kBins3];       //                                               levels 2 and 3
+  uint32_t sum2[kBins2], sum3[kBins2];       //                                               levels 2 and 3
   uint32_t warp_sum[kTopkWarps];
   uint2 warp_tot[kTopkWarps];                // (key > T, key == T) of each warp
   uint2 cta_tot[kTopkMaxCluster];            // of each CTA of the cluster
