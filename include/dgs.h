@@ -27,15 +27,16 @@
  *   - DEVICE pointers are marked DEVICE, everything else is host memory.
  *   - The caller owns all device memory (the arena); the library allocates no device
  *     memory.  Calls only enqueue work and return.  The work runs on streams of the
- *     library's own (several for the pushes, one for the apply, several for the pulls, so
- *     that the push of the next events overlaps the server side of the current one; a
- *     dependency tracker keeps, per buffer, the order of the calls); it is ordered after
+ *     library's own (an event's steps follow one another on one of them, and consecutive
+ *     events take several in turn, so that they overlap; a dependency tracker keeps, per
+ *     buffer, the order of the calls); it is ordered after
  *     everything the caller had enqueued on the stream given at dgs_init when the call
  *     was made.  Results (packets, state) are complete for that stream after dgs_flush,
  *     and for the host after any call that is documented to wait.  One host thread per
  *     context.
- *   - The library's streams are eleven (four for pushes, one for the apply, six for pulls).
- *     The CUDA driver maps streams onto a fixed number of hardware queues, 8 unless the
+ *   - The library's streams are eight at most, and about half as many as there are workers; each
+ *     is created when it is first needed, and a caller that calls dgs_flush after every event
+ *     uses one.  The CUDA driver maps streams onto a fixed number of hardware queues, 8 unless the
  *     environment variable CUDA_DEVICE_MAX_CONNECTIONS says otherwise, and streams that
  *     share a queue run one after the other.  The variable is read when the process creates
  *     its CUDA context, so a process that wants the overlap must set it (to 12 or more; 32
@@ -159,8 +160,9 @@ int dgs_worker_push(dgs_ctx* ctx, uint32_t worker, const float* grad, dgs_packet
 /* Server apply (Algorithm 2, "M <- M - decode(g)"; Eq. 1-3): theta[i] -= val and
  * D_q[i] -= val for every worker q, the sender included, for each (i, val) of the
  * packet.  pkt may be the library's own push packet or any DEVICE packet with
- * strictly ascending indices < n.  Also advances the server timestamp t.
- * For the library's own packets the subtraction from D_q is deferred: the packet is
+ * strictly ascending indices < n (the device status word becomes negative if it is not).
+ * Also advances the server timestamp t.
+ * The subtraction from D_q is deferred (unless the packet is longer than the library's own): the packet is
  * filed in a log and folded into D_q, in arrival order, before anything reads D_q
  * (that worker's next pull, dgs_state_ptr); every D_q[i] sees the same subtractions
  * in the same order, so the values are the same bit for bit. */
@@ -190,8 +192,7 @@ int dgs_event(dgs_ctx* ctx, uint32_t worker, const float* grad, dgs_packet* push
 
 /* Makes the stream given at dgs_init wait (on the device, not the host) for all work
  * enqueued by earlier calls: what that stream runs afterwards sees their packets and
- * state.  (No counterpart in the paper: it joins the library's own streams -- four for the
- * pushes, one for the apply, six for the pulls -- to the caller's.) */
+ * state.  (No counterpart in the paper: it joins the library's own streams to the caller's.) */
 int dgs_flush(dgs_ctx* ctx);
 
 /* The same event with HOST buffers (needs DGS_HOST_IO): copies grad (HOST f32[n],
@@ -271,8 +272,8 @@ int dgs_timing_read(dgs_ctx* ctx, double ms[DGS_NUM_KERNELS], uint64_t count[DGS
 int dgs_timing_trace(dgs_ctx* ctx, uint32_t cap, float* start_ms, float* stop_ms, int32_t* kernel, int32_t* stream,
                      uint32_t* count);
 
-/* How many hardware queues the library's streams want (*needed: its own streams plus the caller's)
- * and how many the process asked the driver for (*configured: CUDA_DEVICE_MAX_CONNECTIONS as the
+/* How many hardware queues a process should ask for (*needed: room for the streams of a context, the caller's and
+ * a few more) and how many the process asked the driver for (*configured: CUDA_DEVICE_MAX_CONNECTIONS as the
  * process environment has it now, 8 if unset or unreadable).  configured < needed means that some of
  * the library's streams share a queue and their kernels do not overlap.  No GPU work; either
  * pointer may be NULL.  (No counterpart in the paper.) */

@@ -12,7 +12,7 @@ import ctypes as C
 import os
 from typing import Optional, Sequence, Tuple
 
-# The library spreads its kernels over eleven CUDA streams.  The driver maps streams onto a fixed
+# The library spreads its kernels over several CUDA streams.  The driver maps streams onto a fixed
 # number of hardware queues (8 unless told otherwise) and streams that share a queue run one after
 # the other; the variable is read when the process creates its CUDA context, so it has to be in
 # place before that.  A value the user has set is left alone.

@@ -1,16 +1,18 @@
 // Host side of the C ABI declared in include/dgs.h: argument checks, the layout of
 // the caller's arena, and the kernel launches of one push / apply / pull event.
 //
-// Work runs on streams of the library's own so that independent steps of consecutive
-// events overlap: pushes take kWorkerStreams worker streams in turn, the apply runs on a stream
-// of its own, pulls take kServerStreams server streams in turn.  A push touches only the worker's
-// velocity, the gradient and its own scratch; a pull touches one difference vector.  The
-// small, latency-bound finalize kernels thus share the GPU with the bandwidth-bound passes
-// of other events.  Order is kept by a small dependency tracker: every launch names the
-// buffers it reads and writes, and waits (cudaStreamWaitEvent) for the last writer of what
-// it reads and for the last writer and the readers of what it writes.  Per buffer the order
-// of operations is therefore the order of the calls, which keeps the results bit-identical
-// to a serial run.
+// Work runs on streams of the library's own so that consecutive events overlap: an event's push, apply and pull
+// follow one another on one stream, and events take kStreams streams in turn.  A push touches only the worker's
+// velocity, the gradient and its scratch; a pull touches one difference vector.  The small, latency-bound kernels
+// thus share the GPU with the bandwidth-bound passes of other events.  An event that starts while nothing else is
+// in flight always takes the first stream, and streams are created when they are first taken: a caller that joins
+// after every event uses one.  (Eleven streams per context -- four for pushes, one for applies, six for pulls --
+// cost every event a hop from stream to stream between its steps, and every stream that is alive costs the others:
+// with three contexts alive, one event of 25.6 M elements took 185 us where it took 158 us with one.)
+// Order is kept by a small dependency tracker: every launch names the buffers it reads and writes, and waits
+// (cudaStreamWaitEvent) for the last writer of what it reads and for the last writer and the readers of what it
+// writes.  Per buffer the order of operations is therefore the order of the calls, which keeps the results
+// bit-identical to a serial run.
 #include "dgs.h"
 
 #include <algorithm>
@@ -33,21 +35,25 @@ namespace {
 constexpr uint64_t kAlign = 256;
 constexpr uint32_t kMagic = 0x44475331u;  // "DGS1"
 constexpr int kPushSlots = 8;  // push packet slots, used in turn (a slot is refilled once its apply has read it)
-constexpr int kPullSlots = 6;             // pull packet slots
+constexpr int kPullSlots = 8;             // pull packet slots
 constexpr int kVarSlots = 4;              // packet slots of the pull without secondary compression
-constexpr int kWorkerStreams = 4, kServerStreams = 6;   // library streams for the pushes and for the pulls
-constexpr int kPushSets = kWorkerStreams;  // scratch sets and spare velocity buffers of the pushes
-constexpr int kPullSets = kServerStreams;  // scratch sets of the pulls
-constexpr int kAllSets = kPushSets + kPullSets;
+constexpr int kStreams = 8;               // most events in flight at a time
+constexpr int kSets = kStreams;           // scratch sets and spare velocity buffers: one of each per stream
+// Events in flight at a time: with more than about half of the workers in flight a selection finds no finished one to
+// take its bound from and waits for one that runs (8 workers, 124 M elements, a round of 8: 3.3 ms with 5 streams, 4.5 ms
+// with 7; 32 workers, 25.6 M elements, a round of 32: 2.5 ms with 4, 2.4 with 5, 2.2 with 7).
+int streams_for(const dgs_config* c) {
+  if (c->flags & DGS_SINGLE_STREAM) return 1;   // kernels run one after the other, in call order
+  return (int)std::min<uint32_t>(kStreams, c->num_workers / 2 + 1);
+}
+constexpr int kQueuesWanted = 12;         // hardware queues that keep the streams of two contexts and the caller's apart
 constexpr int kLogRingMax = 128;            // most packets the apply log keeps
 constexpr int kLogSlack = 32;               // slots of the log beyond one per worker
 constexpr uint64_t kListCap = 4096;         // most entries of a layer's list of candidates in the k-th's bin
-enum StreamId : int { kStW0 = 0, kStApply = kWorkerStreams, kStS0 = kWorkerStreams + 1,
-                      kNumStreams = kWorkerStreams + 1 + kServerStreams };
 
 inline uint64_t align_up(uint64_t x, uint64_t a) { return (x + a - 1) / a * a; }
 
-// Scratch of one selection pipeline ([0] push, on the worker stream; [1] pull, on the server stream)
+// Scratch of the selections on one stream
 struct ScratchLayout {
   uint64_t cand_idx, cand_val, part_cands, part_slot0, plan, cta_cost, cta_tot, cta_eq, tab, list;
   uint64_t hist1, list_cnt, sel, L_safe, L_wide, sync;
@@ -63,7 +69,7 @@ struct Layout {
   uint64_t pkt_idx[kPushSlots + kPullSlots], pkt_val[kPushSlots + kPullSlots];  // push slots, then pull slots
   uint64_t var_idx[kVarSlots], var_val[kVarSlots], var_count[kVarSlots], L_one;
   uint64_t tiles, segs, seg_off, blk_seg;
-  ScratchLayout sc[kAllSets];  // push sets, then pull sets
+  ScratchLayout sc[kSets];
   uint64_t L_next, u_slots, status, stats;
   uint64_t log_ent, log_pos;
   uint64_t blk_max;      // [N][blk_stride]: per block of kWarpTile elements, an upper bound on the keys of D_q in it
@@ -157,7 +163,7 @@ void make_layout(const dgs_config* c, Layout* L) {
   };
   const uint64_t vec = L->n_pad * 4;
   L->theta = take(vec);
-  L->u = take(vec * (N + kPushSets));  // N velocities and the spares that pushes write into
+  L->u = take(vec * (N + streams_for(c)));  // N velocities and the spares that pushes write into
   L->D = take(vec * N);
   L->theta_local = (c->flags & DGS_KEEP_LOCAL_MODEL) ? take(vec * N) : 0;
   L->grad_stage = (c->flags & DGS_HOST_IO) ? take(vec) : 0;
@@ -176,7 +182,7 @@ void make_layout(const dgs_config* c, Layout* L) {
   L->segs = take(S * sizeof(SegDesc));
   L->seg_off = take((S + 1) * 4);
   L->blk_seg = take((uint64_t)L->num_blocks * 4);
-  for (int k = 0; k < kAllSets; ++k) {
+  for (int k = 0; k < streams_for(c); ++k) {
     ScratchLayout& sc = L->sc[k];
     sc.cand_idx = take(vec);
     sc.cand_val = take(vec);
@@ -211,7 +217,7 @@ void make_layout(const dgs_config* c, Layout* L) {
   L->blk_stride = align_up((c->n + kWarpTile - 1) / kWarpTile, 64);
   L->blk_max = take(N * L->blk_stride * 4);
   L->L_next = take(2 * N * S * 4);
-  L->u_slots = take((N + kPushSets) * sizeof(float*));
+  L->u_slots = take((N + kSets) * sizeof(float*));
   L->status = take(4);
   L->stats = take((uint64_t)kNumStats * 8);
   L->total = off;
@@ -226,10 +232,16 @@ struct dgs_ctx {
   Layout lay;
   char* base;
   cudaStream_t user;       // the caller's stream: entry point of dependencies, target of dgs_flush
-  cudaStream_t st[kNumStreams];
+  cudaStream_t st[kStreams];   // null until first taken
+  int streams;             // how many of them may be taken (1 under DGS_SINGLE_STREAM)
+  int next_stream;         // the one that the next event takes ...
+  bool idle;               // ... unless nothing has been enqueued since everything was last joined: then the first one
+  bool dirty[kStreams];    // stream has work that the caller's stream has not been made to wait for
+  std::vector<int> worker_stream;   // per worker: stream of its last push if its pull is still to come, else -1
+  int slot_stream[kPushSlots];      // per push packet slot: stream of its push
   cudaEvent_t ev_in;       // "everything the caller had enqueued when the call was made"
-  bool forked[kNumStreams];  // stream already waits for ev_in of the current call
-  cudaEvent_t ev_tail[kNumStreams];  // for dgs_flush
+  bool forked[kStreams];  // stream already waits for ev_in of the current call
+  cudaEvent_t ev_tail[kStreams];  // for dgs_flush
   // dependency tracker
   struct Dep {
     cudaEvent_t ev = nullptr;
@@ -243,17 +255,17 @@ struct dgs_ctx {
   std::vector<Res> res;
   // one "done" event per task, reused in turn; a ring per stream, so that an event is only ever
   // re-recorded later on the same stream and waiting for a reused one still covers the older task
-  std::vector<cudaEvent_t> ev_ring[kNumStreams];
-  size_t ev_next[kNumStreams];
+  std::vector<cudaEvent_t> ev_ring[kStreams];
+  size_t ev_next[kStreams];
   uint64_t task_seq;                               // tasks filed so far
-  uint64_t waited_seq[kNumStreams][kNumStreams];   // [waiting stream][stream]: newest task already waited for
+  uint64_t waited_seq[kStreams][kStreams];   // [waiting stream][stream]: newest task already waited for
   uint64_t push_count, pull_count, event_count, var_count;
   // Lazy difference vectors: packet number p (counted from 0) of the library's own pushes sits in slot
   // p % ring of the log from its apply on; applied[q] packets have been folded into D_q so far.
   PacketLog log;
   uint64_t log_head;              // packets filed so far
   std::vector<uint64_t> applied;  // per worker
-  Workspace ws[kAllSets];  // push sets, then pull sets
+  Workspace ws[kSets];
   float inv_m;
   int sms;               // SMs of the device
   int stream_grid[3];    // CTAs of the stand-alone stream pass, per mode
@@ -310,8 +322,8 @@ struct ResIds {
   uint32_t ROW(int kind, uint32_t w) const { return 3 * N + (uint32_t)kind * N + w; }
   uint32_t THETA() const { return 5 * N; }
   uint32_t SPARE(int j) const { return 5 * N + 1 + j; }
-  uint32_t SCR(int kind, int set) const { return 5 * N + 1 + kPushSets + (kind ? kPushSets : 0) + set; }
-  uint32_t PKT(int slot) const { return 5 * N + 1 + kPushSets + kAllSets + slot; }   // push slots, then pull slots
+  uint32_t SCR(int set) const { return 5 * N + 1 + kSets + set; }
+  uint32_t PKT(int slot) const { return 5 * N + 1 + 2 * kSets + slot; }   // push slots, then pull slots
   uint32_t VPKT(int slot) const { return PKT(kPushSlots + kPullSlots) + (uint32_t)slot; }
   uint32_t STAGE() const { return VPKT(kVarSlots); }
   uint32_t LOG(uint32_t slot) const { return STAGE() + 1 + slot; }
@@ -334,6 +346,7 @@ inline int live(dgs_ctx* c) {
   return DGS_OK;
 }
 
+constexpr int kEventRing = 256;       // "done" events per stream, used in turn
 constexpr size_t kMaxTimedLaunches = 1 << 16;
 constexpr uint64_t kFinalizeMin = 32;  // fewest CTAs of the finalize kernel
 
@@ -354,7 +367,7 @@ struct TimedLaunch {
     stop = c->ev_pool[2 * i + 1];
     c->ev_kernel.push_back(kernel_id);
     int which = -1;
-    for (int j = 0; j < kNumStreams; ++j)
+    for (int j = 0; j < kStreams; ++j)
       if (c->st[j] == st) which = j;
     c->ev_stream.push_back(which);
   }
@@ -367,10 +380,31 @@ struct TimedLaunch {
 // current API call began (ev_in is recorded once per call by begin_call).
 int begin_call(dgs_ctx* c) {
   DGS_CUDA(c, cudaEventRecord(c->ev_in, c->user));
-  for (int i = 0; i < kNumStreams; ++i) c->forked[i] = false;
+  for (int i = 0; i < kStreams; ++i) c->forked[i] = false;
   return DGS_OK;
 }
+int stream_ready(dgs_ctx* c, int which) {
+  if (c->st[which]) return DGS_OK;
+  DGS_CUDA(c, cudaStreamCreateWithFlags(&c->st[which], cudaStreamNonBlocking));
+  DGS_CUDA(c, cudaEventCreateWithFlags(&c->ev_tail[which], cudaEventDisableTiming));
+  for (int i = 0; i < kEventRing; ++i) {
+    cudaEvent_t e;
+    DGS_CUDA(c, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    c->ev_ring[which].push_back(e);
+  }
+  return DGS_OK;
+}
+// The stream of the next event, and taking it.
+int peek_stream(const dgs_ctx* c) { return c->idle ? 0 : c->next_stream; }
+int take_stream(dgs_ctx* c) {
+  const int s = peek_stream(c);
+  c->idle = false;
+  c->next_stream = (s + 1) % c->streams;
+  return s;
+}
 int fork_from_user(dgs_ctx* c, int which) {
+  const int rc = stream_ready(c, which);
+  if (rc != DGS_OK) return rc;
   if (c->forked[which]) return DGS_OK;
   DGS_CUDA(c, cudaStreamWaitEvent(c->st[which], c->ev_in, 0));
   c->forked[which] = true;
@@ -379,9 +413,10 @@ int fork_from_user(dgs_ctx* c, int which) {
 
 // Waits (on the host) for all internal streams and the caller's stream.
 int sync_all(dgs_ctx* c) {
-  for (int i = 0; i < kNumStreams; ++i) DGS_CUDA(c, cudaStreamSynchronize(c->st[i]));
+  for (int i = 0; i < kStreams; ++i)
+    if (c->st[i]) DGS_CUDA(c, cudaStreamSynchronize(c->st[i]));
   DGS_CUDA(c, cudaStreamSynchronize(c->user));
-  c->alone = true;
+  c->alone = c->idle = true;
   return DGS_OK;
 }
 
@@ -393,9 +428,11 @@ struct Task {
   std::vector<uint32_t> reads, writes;
 };
 int task_begin(dgs_ctx* c, const Task& t) {
+  const int ready = stream_ready(c, t.stream);
+  if (ready != DGS_OK) return ready;
   // Tasks of one stream complete in order, so per stream only the newest task that this one depends
   // on matters, and only if the stream has not already waited for that task or a newer one.
-  dgs_ctx::Dep need[kNumStreams];
+  dgs_ctx::Dep need[kStreams];
   auto want = [&](const dgs_ctx::Dep& d) {
     if (!d.ev || d.stream == t.stream) return;   // same stream: already ordered
     if (d.seq > need[d.stream].seq) need[d.stream] = d;
@@ -406,7 +443,7 @@ int task_begin(dgs_ctx* c, const Task& t) {
     want(x.last_write);
     for (const dgs_ctx::Dep& rd : x.reads) want(rd);
   }
-  for (int s = 0; s < kNumStreams; ++s) {
+  for (int s = 0; s < kStreams; ++s) {
     if (!need[s].ev || need[s].seq <= c->waited_seq[t.stream][s]) continue;
     DGS_CUDA(c, cudaStreamWaitEvent(c->st[t.stream], need[s].ev, 0));
     c->waited_seq[t.stream][s] = need[s].seq;
@@ -414,6 +451,7 @@ int task_begin(dgs_ctx* c, const Task& t) {
   return DGS_OK;
 }
 int task_end(dgs_ctx* c, const Task& t) {
+  c->dirty[t.stream] = true;
   dgs_ctx::Dep d;
   d.ev = c->ev_ring[t.stream][c->ev_next[t.stream]];
   d.stream = t.stream;
@@ -450,11 +488,11 @@ int fold_launch(dgs_ctx* c, const Workspace& ws, const SelArgs& a, uint32_t q, c
   c->applied[q] = c->log_head;
   return DGS_OK;
 }
-// Both, as a task of its own on the apply stream.
-int catch_up_now(dgs_ctx* c, uint32_t q) {
+// Both, as a task of its own.
+int catch_up_now(dgs_ctx* c, uint32_t q, int stream) {
   if (c->applied[q] == c->log_head) return DGS_OK;
   Task t;
-  t.stream = kStApply;
+  t.stream = stream;
   catch_up_deps(c, q, &t);
   int rc = task_begin(c, t);
   if (rc != DGS_OK) return rc;
@@ -462,7 +500,7 @@ int catch_up_now(dgs_ctx* c, uint32_t q) {
   std::memset(&a, 0, sizeof(a));
   a.D = c->D_buf(q);
   a.blk_max = c->blk_max(q);
-  rc = fold_launch<false>(c, c->ws[0], a, q, c->st[kStApply]);   // (tables only: a fold without a scan writes no scratch)
+  rc = fold_launch<false>(c, c->ws[0], a, q, c->st[stream]);   // (tables only: a fold without a scan writes no scratch)
   if (rc != DGS_OK) return rc;
   return task_end(c, t);
 }
@@ -473,7 +511,7 @@ int catch_up_now(dgs_ctx* c, uint32_t q) {
 // before them was written on this selection's own stream).  -1 if there is none.
 int pick_row(const dgs_ctx* c, int kind, uint64_t age) {
   int best = -1, best_old = -1;
-  const uint64_t in_flight = (uint64_t)(kind ? kServerStreams : kWorkerStreams) - 1;
+  const uint64_t in_flight = (uint64_t)c->streams - 1;
   const uint64_t newest = c->kind_seq[kind];
   for (uint32_t q = 0; q < c->cfg.num_workers; ++q) {
     if (!c->row_valid[kind][q] || c->row_age[kind][q] > age) continue;
@@ -494,12 +532,11 @@ const void* finalize_kernel(const dgs_ctx* c) {
 }
 
 template <int MODE>
-int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age, int stream_id, int set,
-                  Task& task) {
+int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age, int stream_id, Task& task) {
   constexpr int KIND = MODE == kPull ? 1 : 0;
   const ResIds R{c->cfg.num_workers};
   cudaStream_t st = c->st[stream_id];
-  Workspace& ws = c->ws[(KIND ? kPushSets : 0) + set];
+  Workspace& ws = c->ws[stream_id];
   SelArgs a = a_in;
   a.speculate = (c->cfg.flags & DGS_NO_SPECULATION) ? 0 : 1;
   int row = a.speculate ? pick_row(c, KIND, age) : -1;
@@ -532,7 +569,7 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
   task.stream = stream_id;
   if (single_pass && (uint32_t)row != worker) task.reads.push_back(R.ROW(KIND, (uint32_t)row));
   if (a.speculate) task.writes.push_back(R.ROW(KIND, worker));
-  task.writes.push_back(R.SCR(KIND, set));
+  task.writes.push_back(R.SCR(stream_id));
   int rc = task_begin(c, task);
   if (rc != DGS_OK) return rc;
   if (!single_pass) {
@@ -611,7 +648,7 @@ int fold_setup(dgs_ctx* c, int sms) {
   // (a share never gets longer than an even one without a plan).
   const uint32_t even = (c->lay.num_blocks + c->fold_grid - 1) / c->fold_grid + kFoldSlack;
   const uint32_t cap = (uint32_t)align_up(std::max<uint32_t>(even, std::min<uint32_t>(32768u, 8 * even)), 128);
-  for (int k = 0; k < kAllSets; ++k) c->ws[k].part_cap = cap;
+  for (int k = 0; k < kSets; ++k) c->ws[k].part_cap = cap;
   DGS_CUDA(c, cudaFuncSetAttribute(k_fold<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFoldMaxDyn));
   DGS_CUDA(c, cudaFuncSetAttribute(k_fold<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFoldMaxDyn));
   if (fold_dyn_bytes(kFoldWarps, c->fold_ahead, cap) > (uint32_t)kFoldMaxDyn) return DGS_EINVAL;   // (n < 2^32 keeps an even share well below)
@@ -619,12 +656,12 @@ int fold_setup(dgs_ctx* c, int sms) {
 }
 
 void destroy_ctx(dgs_ctx* c) {
-  for (int i = 0; i < kNumStreams; ++i) {
-    if (c->st[i] && (i == 0 || c->st[i] != c->st[0])) cudaStreamDestroy(c->st[i]);
+  for (int i = 0; i < kStreams; ++i) {
+    if (c->st[i]) cudaStreamDestroy(c->st[i]);
     if (c->ev_tail[i]) cudaEventDestroy(c->ev_tail[i]);
   }
   if (c->ev_in) cudaEventDestroy(c->ev_in);
-  for (int i = 0; i < kNumStreams; ++i)
+  for (int i = 0; i < kStreams; ++i)
     for (cudaEvent_t e : c->ev_ring[i]) cudaEventDestroy(e);
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
   c->magic = 0;
@@ -672,16 +709,21 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
   c->segments.assign(cfg->segments, cfg->segments + cfg->num_segments);
   c->cfg.segments = c->segments.data();
   make_layout(&c->cfg, &c->lay);
-  for (int i = 0; i < kNumStreams; ++i) {
+  for (int i = 0; i < kStreams; ++i) {
     c->st[i] = nullptr;
     c->ev_tail[i] = nullptr;
-    c->forked[i] = false;
+    c->forked[i] = c->dirty[i] = false;
   }
+  c->streams = streams_for(cfg);
+  c->next_stream = 0;
+  c->idle = true;
+  c->worker_stream.assign(cfg->num_workers, -1);
+  for (int i = 0; i < kPushSlots; ++i) c->slot_stream[i] = 0;
   c->ev_in = nullptr;
   c->task_seq = 0;
-  for (int i = 0; i < kNumStreams; ++i) {
+  for (int i = 0; i < kStreams; ++i) {
     c->ev_next[i] = 0;
-    for (int j = 0; j < kNumStreams; ++j) c->waited_seq[i][j] = 0;
+    for (int j = 0; j < kStreams; ++j) c->waited_seq[i][j] = 0;
   }
   c->pull_count = c->event_count = c->var_count = 0;
   c->log_head = 0;
@@ -734,25 +776,8 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
   if (occupancy_grids<kPushSam>(c, sms) != DGS_OK || occupancy_grids<kPushResidual>(c, sms) != DGS_OK ||
       occupancy_grids<kPull>(c, sms) != DGS_OK || fold_setup(c, sms) != DGS_OK)
     return fail(DGS_ECUDA);
-  int prio_low = 0, prio_high = 0;
-  INIT_CUDA(cudaDeviceGetStreamPriorityRange(&prio_low, &prio_high));
-  for (int i = 0; i < kNumStreams; ++i) {
-    // The push passes move most of the bytes and fill every SM; the short kernels of the server side sit on
-    // the longer chain (apply -> catch-up -> pull), so their blocks go first whenever an SM has room.
-    const int prio = i < kStApply ? prio_low : prio_high;
-    if (i > 0 && (cfg->flags & DGS_SINGLE_STREAM))
-      c->st[i] = c->st[0];   // every step on one stream: kernels run one after the other, in call order
-    else
-      INIT_CUDA(cudaStreamCreateWithPriority(&c->st[i], cudaStreamNonBlocking, prio));
-    INIT_CUDA(cudaEventCreateWithFlags(&c->ev_tail[i], cudaEventDisableTiming));
-  }
   INIT_CUDA(cudaEventCreateWithFlags(&c->ev_in, cudaEventDisableTiming));
-  for (int s = 0; s < kNumStreams; ++s)
-    for (int i = 0; i < 256; ++i) {
-      cudaEvent_t e;
-      INIT_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-      c->ev_ring[s].push_back(e);
-    }
+  if (stream_ready(c, 0) != DGS_OK) return fail(DGS_ECUDA);
 
   const Layout& L = c->lay;
   const uint64_t N = cfg->num_workers, vec = L.n_pad * 4;
@@ -763,7 +788,7 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
   if (tiles.size() != L.num_tiles) return fail(DGS_EINVAL);
   cudaStream_t st = c->user;
   // state: u = 0, D = 0 (initialisation lines of Algorithm 3 and Algorithm 2), theta = theta_0
-  INIT_CUDA(cudaMemsetAsync(c->at<char>(L.u), 0, vec * (N + kPushSets), st));
+  INIT_CUDA(cudaMemsetAsync(c->at<char>(L.u), 0, vec * (N + c->streams), st));
   INIT_CUDA(cudaMemsetAsync(c->at<char>(L.D), 0, vec * N, st));
   INIT_CUDA(cudaMemsetAsync(c->at<char>(L.theta), 0, vec, st));
   INIT_CUDA(cudaMemcpyAsync(c->at<char>(L.theta), cfg->theta0, cfg->n * 4, cudaMemcpyDeviceToDevice, st));
@@ -773,7 +798,7 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
       INIT_CUDA(cudaMemcpyAsync(c->theta_local_buf(q), cfg->theta0, cfg->n * 4, cudaMemcpyDeviceToDevice, st));
   }
   // scratch that kernels expect to find cleared, and the static tables
-  for (int k = 0; k < kAllSets; ++k) {
+  for (int k = 0; k < c->streams; ++k) {
     const ScratchLayout& sc = L.sc[k];
     INIT_CUDA(cudaMemsetAsync(c->at<char>(sc.zero_begin), 0, sc.zero_end - sc.zero_begin, st));
     INIT_CUDA(cudaMemsetAsync(c->at<char>(sc.part_cands), 0, (uint64_t)kMaxParts * 4, st));
@@ -799,14 +824,14 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
   INIT_CUDA(cudaMemcpyAsync(c->at<char>(L.blk_seg), blk_seg.data(), blk_seg.size() * 4, cudaMemcpyHostToDevice, st));
   std::vector<uint32_t> ones(cfg->num_segments, 1u);   // the bound that admits every nonzero value
   INIT_CUDA(cudaMemcpyAsync(c->at<char>(L.L_one), ones.data(), ones.size() * 4, cudaMemcpyHostToDevice, st));
-  std::vector<float*> slots(N + kPushSets);
-  for (uint32_t q = 0; q < N + kPushSets; ++q) slots[q] = c->u_buf(q);
+  std::vector<float*> slots(N + c->streams);
+  for (uint32_t q = 0; q < N + c->streams; ++q) slots[q] = c->u_buf(q);
   INIT_CUDA(cudaMemcpyAsync(c->at<char>(L.u_slots), slots.data(), slots.size() * sizeof(float*), cudaMemcpyHostToDevice, st));
   // the host vectors above go out of scope, and the library's own streams start from a ready arena
   INIT_CUDA(cudaStreamSynchronize(st));
 #undef INIT_CUDA
 
-  for (int k = 0; k < kAllSets; ++k) {
+  for (int k = 0; k < c->streams; ++k) {
     Workspace& w = c->ws[k];
     const ScratchLayout& sc = L.sc[k];
     w.tiles = c->at<Tile>(L.tiles);
@@ -848,19 +873,17 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
 
 namespace {
 
-int push_impl(dgs_ctx* c, uint32_t worker, const float* grad, dgs_packet* out, bool grad_is_stage) {
+int push_impl(dgs_ctx* c, uint32_t worker, const float* grad, dgs_packet* out, int stream_id, bool grad_is_stage) {
   const Layout& L = c->lay;
   const ResIds R{c->cfg.num_workers};
   const int slot = (int)(c->push_count % kPushSlots);
-  const int set = (int)(c->push_count % kPushSets);
-  const int stream_id = kStW0 + (int)(c->push_count % kWorkerStreams);
   int rc = fork_from_user(c, stream_id);  // the gradient may have been produced on the caller's stream
   if (rc != DGS_OK) return rc;
   SelArgs a;
   std::memset(&a, 0, sizeof(a));
   a.grad = grad;
   a.u_cur_slot = c->u_slot(worker);
-  a.u_spare_slot = c->u_slot(c->cfg.num_workers + set);
+  a.u_spare_slot = c->u_slot(c->cfg.num_workers + stream_id);
   a.pkt_idx = c->at<uint32_t>(L.pkt_idx[slot]);
   a.pkt_val = c->at<float>(L.pkt_val[slot]);
   a.pkt_count = (uint32_t)L.K[0];
@@ -868,15 +891,17 @@ int push_impl(dgs_ctx* c, uint32_t worker, const float* grad, dgs_packet* out, b
   a.lr = c->cfg.lr;
   a.inv_m = c->inv_m;
   Task task;
-  task.writes = {R.U(worker), R.SPARE(set), R.PKT(slot)};
+  task.writes = {R.U(worker), R.SPARE(stream_id), R.PKT(slot)};
   if (grad_is_stage) task.reads.push_back(R.STAGE());
   const uint64_t age = c->pushes[worker];
   rc = (c->cfg.flags & DGS_RESIDUAL_MODE)
-           ? launch_select<kPushResidual>(c, a, worker, age, stream_id, set, task)
-           : launch_select<kPushSam>(c, a, worker, age, stream_id, set, task);
+           ? launch_select<kPushResidual>(c, a, worker, age, stream_id, task)
+           : launch_select<kPushSam>(c, a, worker, age, stream_id, task);
   if (rc != DGS_OK) return rc;
   c->pushes[worker] += 1;
   c->push_count += 1;
+  c->worker_stream[worker] = stream_id;
+  c->slot_stream[slot] = stream_id;
   if (out) {
     out->idx = a.pkt_idx;
     out->val = a.pkt_val;
@@ -893,11 +918,18 @@ int apply_impl(dgs_ctx* c, uint32_t worker, const dgs_packet* pkt) {
   int slot = -1;
   for (int i = 0; i < kPushSlots; ++i)
     if (pkt->idx == c->at<uint32_t>(c->lay.pkt_idx[i])) slot = i;
+  const bool own = slot >= 0 && pkt->val == c->at<float>(c->lay.pkt_val[slot]) && pkt->count == c->lay.K[0];
+  const int stream_id = own ? c->slot_stream[slot] : peek_stream(c);   // after its push; else where a pull comes next
   const uint32_t gx = (pkt->count + kThreads - 1) / kThreads;
+  int rc = DGS_OK;
+  if (pkt->count > 0 && !own) rc = fork_from_user(c, stream_id);
+  if (rc != DGS_OK) return rc;
   if (pkt->count == 0) {
     // nothing to subtract
-  } else if (slot >= 0 && pkt->val == c->at<float>(c->lay.pkt_val[slot]) && pkt->count == c->lay.K[0]) {
-    // One of the library's own packets (sorted by index, of the fixed size): theta now, the D_q lazily.
+  } else if (pkt->count <= c->log.stride) {
+    // theta now, the D_q lazily.  Any packet that fits a slot of the log is filed, a caller's own as well (16 of them
+    // and 16 pulls on 25.6 M elements: 1136 us with a scatter into theta and all 16 D_q each, which also kept every
+    // event from overlapping the next, 392 us filed).
     // Its slot of the log still holds the packet filed `ring` applies ago; whoever has not folded that
     // one in yet does so first.
     const uint32_t lslot = (uint32_t)(c->log_head % c->log.ring);
@@ -905,22 +937,21 @@ int apply_impl(dgs_ctx* c, uint32_t worker, const dgs_packet* pkt) {
       const uint64_t oldest = c->log_head - c->log.ring;
       for (uint32_t q = 0; q < N; ++q)
         if (c->applied[q] <= oldest) {
-          const int rc = catch_up_now(c, q);
+          rc = catch_up_now(c, q, stream_id);
           if (rc != DGS_OK) return rc;
         }
     }
     Task t;
-    t.stream = kStApply;
-    t.reads.push_back(R.PKT(slot));
+    t.stream = stream_id;
+    if (slot >= 0) t.reads.push_back(R.PKT(slot));
     t.writes = {R.THETA(), R.LOG(lslot)};
-    int rc = task_begin(c, t);
+    rc = task_begin(c, t);
     if (rc != DGS_OK) return rc;
     {
-      TimedLaunch tl(c, c->st[kStApply], DGS_KERNEL_SCATTER);
+      TimedLaunch tl(c, c->st[stream_id], DGS_KERNEL_SCATTER);
       const uint32_t pos_ctas = (c->log.pos_rows + kThreads - 1) / kThreads;
-      k_apply_log<<<gx + pos_ctas, kThreads, 0, c->st[kStApply]>>>(pkt->idx, pkt->val, pkt->count,
-                                                                   c->at<float>(c->lay.theta), c->cfg.n,
-                                                                   c->ws[0].status, c->log, lslot, gx);
+      k_apply_log<<<gx + pos_ctas, kThreads, 0, c->st[stream_id]>>>(pkt->idx, pkt->val, pkt->count, c->at<float>(c->lay.theta),
+                                                                    c->cfg.n, c->ws[0].status, c->log, lslot, gx);
       DGS_CUDA(c, cudaGetLastError());
       c->launches += 1;
     }
@@ -928,23 +959,21 @@ int apply_impl(dgs_ctx* c, uint32_t worker, const dgs_packet* pkt) {
     if (rc != DGS_OK) return rc;
     c->log_head += 1;
   } else {
-    // Any other packet: bring every D_q up to date, then subtract from theta and all of them at once.
+    // A packet too long for the log: bring every D_q up to date, then subtract from theta and all of them at once.
     for (uint32_t q = 0; q < N; ++q) {
-      const int rc = catch_up_now(c, q);
+      rc = catch_up_now(c, q, stream_id);
       if (rc != DGS_OK) return rc;
     }
     Task t;
-    t.stream = kStApply;
+    t.stream = stream_id;
     if (slot >= 0) t.reads.push_back(R.PKT(slot));
     t.writes.push_back(R.THETA());
     for (uint32_t q = 0; q < N; ++q) t.writes.push_back(R.D(q));
-    int rc = slot >= 0 ? DGS_OK : fork_from_user(c, kStApply);
-    if (rc != DGS_OK) return rc;
     rc = task_begin(c, t);
     if (rc != DGS_OK) return rc;
     {
-      TimedLaunch tl(c, c->st[kStApply], DGS_KERNEL_SCATTER);
-      k_scatter_sub<<<dim3(gx, N + 1), kThreads, 0, c->st[kStApply]>>>(
+      TimedLaunch tl(c, c->st[stream_id], DGS_KERNEL_SCATTER);
+      k_scatter_sub<<<dim3(gx, N + 1), kThreads, 0, c->st[stream_id]>>>(
           pkt->idx, pkt->val, pkt->count, c->at<float>(c->lay.theta), c->at<float>(c->lay.D), c->lay.n_pad, N,
           c->cfg.n, c->ws[0].status, c->blk_max(0), c->lay.blk_stride);
       DGS_CUDA(c, cudaGetLastError());
@@ -961,8 +990,7 @@ int pull_impl(dgs_ctx* c, uint32_t worker, dgs_packet* out) {
   const Layout& L = c->lay;
   const ResIds R{c->cfg.num_workers};
   const int slot = kPushSlots + (int)(c->pull_count % kPullSlots);
-  const int set = (int)(c->pull_count % kPullSets);
-  const int stream_id = kStS0 + (int)(c->pull_count % kServerStreams);
+  const int stream_id = c->worker_stream[worker] >= 0 ? c->worker_stream[worker] : take_stream(c);
   int rc = fork_from_user(c, stream_id);  // the caller may still be reading an older pull packet on its stream
   if (rc != DGS_OK) return rc;
   SelArgs a;
@@ -982,10 +1010,11 @@ int pull_impl(dgs_ctx* c, uint32_t worker, dgs_packet* out) {
   if (a.theta_local) task.writes.push_back(R.TL(worker));
   // packets that entered D_worker since its previous pull
   const uint64_t age = c->timestamp - (c->prev[worker] < 0 ? 0 : (uint64_t)c->prev[worker]);
-  rc = launch_select<kPull>(c, a, worker, age, stream_id, set, task);
+  rc = launch_select<kPull>(c, a, worker, age, stream_id, task);
   if (rc != DGS_OK) return rc;
   c->prev[worker] = (int64_t)c->timestamp;
   c->pull_count += 1;
+  c->worker_stream[worker] = -1;
   c->alone = false;
   if (out) {
     out->idx = a.pkt_idx;
@@ -1001,12 +1030,11 @@ int pull_all_impl(dgs_ctx* c, uint32_t worker, dgs_var_packet* out) {
   const Layout& L = c->lay;
   const ResIds R{c->cfg.num_workers};
   const int vslot = (int)(c->var_count % kVarSlots);
-  const int set = (int)(c->pull_count % kPullSets);
-  const int stream_id = kStS0 + (int)(c->pull_count % kServerStreams);
-  cudaStream_t st = c->st[stream_id];
+  const int stream_id = c->worker_stream[worker] >= 0 ? c->worker_stream[worker] : take_stream(c);
   int rc = fork_from_user(c, stream_id);  // the caller may still be reading an older packet on its stream
   if (rc != DGS_OK) return rc;
-  Workspace& ws = c->ws[kPushSets + set];
+  cudaStream_t st = c->st[stream_id];
+  Workspace& ws = c->ws[stream_id];
   SelArgs a;
   std::memset(&a, 0, sizeof(a));
   a.D = c->D_buf(worker);
@@ -1018,7 +1046,7 @@ int pull_all_impl(dgs_ctx* c, uint32_t worker, dgs_var_packet* out) {
   a.inv_m = c->inv_m;
   Task task;
   task.stream = stream_id;
-  task.writes = {R.VPKT(vslot), R.SCR(1, set)};
+  task.writes = {R.VPKT(vslot), R.SCR(stream_id)};
   catch_up_deps(c, worker, &task);  // D_worker is brought up to date first, on the same stream
   if (a.theta_local) task.writes.push_back(R.TL(worker));
   rc = task_begin(c, task);
@@ -1039,6 +1067,7 @@ int pull_all_impl(dgs_ctx* c, uint32_t worker, dgs_var_packet* out) {
   if (rc != DGS_OK) return rc;
   c->prev[worker] = (int64_t)c->timestamp;
   c->pull_count += 1;
+  c->worker_stream[worker] = -1;
   c->var_count += 1;
   c->alone = false;
   if (out) {
@@ -1068,7 +1097,7 @@ int dgs_worker_push(dgs_ctx* c, uint32_t worker, const float* grad, dgs_packet* 
   if ((reinterpret_cast<uintptr_t>(grad) % 16) != 0) return DGS_EINVAL;
   rc = begin_call(c);
   if (rc != DGS_OK) return rc;
-  return push_impl(c, worker, grad, out, false);
+  return push_impl(c, worker, grad, out, take_stream(c), false);
 }
 
 int dgs_server_apply(dgs_ctx* c, uint32_t worker, const dgs_packet* pkt) {
@@ -1098,7 +1127,7 @@ int dgs_event(dgs_ctx* c, uint32_t worker, const float* grad, dgs_packet* push_o
   rc = begin_call(c);
   if (rc != DGS_OK) return rc;
   dgs_packet p, g;
-  rc = push_impl(c, worker, grad, &p, false);
+  rc = push_impl(c, worker, grad, &p, take_stream(c), false);
   if (rc != DGS_OK) return rc;
   rc = apply_impl(c, worker, &p);
   if (rc != DGS_OK) return rc;
@@ -1112,10 +1141,13 @@ int dgs_event(dgs_ctx* c, uint32_t worker, const float* grad, dgs_packet* push_o
 int dgs_flush(dgs_ctx* c) {
   int rc = live(c);
   if (rc != DGS_OK) return rc;
-  for (int i = 0; i < kNumStreams; ++i) {
+  for (int i = 0; i < kStreams; ++i) {
+    if (!c->dirty[i]) continue;              // joined by an earlier call
     DGS_CUDA(c, cudaEventRecord(c->ev_tail[i], c->st[i]));
     DGS_CUDA(c, cudaStreamWaitEvent(c->user, c->ev_tail[i], 0));
+    c->dirty[i] = false;
   }
+  c->idle = true;
   c->alone = true;
   return DGS_OK;
 }
@@ -1128,10 +1160,11 @@ int dgs_event_host(dgs_ctx* c, uint32_t worker, const float* grad_host, uint32_t
   if (rc != DGS_OK) return rc;
   const ResIds R{c->cfg.num_workers};
   float* stage = c->at<float>(c->lay.grad_stage);
+  const int stream_id = take_stream(c);
   {
     // host -> staging buffer, on the stream of the push that will read it
     Task t;
-    t.stream = kStW0 + (int)(c->push_count % kWorkerStreams);
+    t.stream = stream_id;
     t.writes.push_back(R.STAGE());
     rc = fork_from_user(c, t.stream);
     if (rc != DGS_OK) return rc;
@@ -1142,21 +1175,20 @@ int dgs_event_host(dgs_ctx* c, uint32_t worker, const float* grad_host, uint32_t
     if (rc != DGS_OK) return rc;
   }
   dgs_packet p, g;
-  rc = push_impl(c, worker, stage, &p, true);
+  rc = push_impl(c, worker, stage, &p, stream_id, true);
   if (rc != DGS_OK) return rc;
   rc = apply_impl(c, worker, &p);
   if (rc != DGS_OK) return rc;
-  const int pull_stream = kStS0 + (int)(c->pull_count % kServerStreams);
   rc = pull_impl(c, worker, &g);
   if (rc != DGS_OK) return rc;
-  cudaStream_t ps = c->st[pull_stream];
+  cudaStream_t ps = c->st[stream_id];
   if (out_idx) DGS_CUDA(c, cudaMemcpyAsync(out_idx, g.idx, (uint64_t)g.count * 4, cudaMemcpyDeviceToHost, ps));
   if (out_val) DGS_CUDA(c, cudaMemcpyAsync(out_val, g.val, (uint64_t)g.count * 4, cudaMemcpyDeviceToHost, ps));
-  // the event is complete when its pull is (the pull waited for the apply, the apply for the push),
-  // except for the shares of the apply that run on the other server streams
+  // push, apply and pull follow one another on this stream; what other calls have enqueued may still be running
   DGS_CUDA(c, cudaStreamSynchronize(ps));
-  for (int i = 0; i < kServerStreams; ++i) DGS_CUDA(c, cudaStreamSynchronize(c->st[kStS0 + i]));
-  c->alone = true;
+  c->alone = c->idle = true;
+  for (int i = 0; i < kStreams; ++i)
+    if (i != stream_id && c->dirty[i]) c->alone = c->idle = false;
   return DGS_OK;
 }
 
@@ -1168,7 +1200,7 @@ int dgs_state_ptr(dgs_ctx* c, int which, uint32_t worker, const float** out) {
   switch (which) {
     case DGS_THETA: *out = c->at<float>(c->lay.theta); break;
     case DGS_D:
-      rc = catch_up_now(c, worker);
+      rc = catch_up_now(c, worker, 0);
       if (rc != DGS_OK) return rc;
       *out = c->D_buf(worker);
       break;
@@ -1200,7 +1232,7 @@ int dgs_state_load(dgs_ctx* c, int which, uint32_t worker, const float* src) {
   if (rc != DGS_OK) return rc;
   const ResIds R{c->cfg.num_workers};
   Task t;
-  t.stream = kStApply;
+  t.stream = 0;
   t.writes.push_back(which == DGS_THETA ? R.THETA()
                      : which == DGS_U   ? R.U(worker)
                      : which == DGS_D   ? R.D(worker)
@@ -1320,7 +1352,7 @@ int dgs_timing_trace(dgs_ctx* c, uint32_t cap, float* start_ms, float* stop_ms, 
 }
 
 int dgs_hardware_queues(int* needed, int* configured) {
-  if (needed) *needed = kNumStreams + 1;
+  if (needed) *needed = kQueuesWanted;
   if (configured) {
     int v = 8;   // the driver's default
     if (const char* e = std::getenv("CUDA_DEVICE_MAX_CONNECTIONS")) {
@@ -1340,7 +1372,8 @@ int dgs_last_cuda_error(dgs_ctx* c) {
 
 int dgs_free(dgs_ctx* c) {
   if (!c || c->magic != kMagic) return DGS_ESTATE;
-  for (int i = 0; i < kNumStreams; ++i) cudaStreamSynchronize(c->st[i]);
+  for (int i = 0; i < kStreams; ++i)
+    if (c->st[i]) cudaStreamSynchronize(c->st[i]);
   cudaStreamSynchronize(c->user);
   destroy_ctx(c);
   return DGS_OK;

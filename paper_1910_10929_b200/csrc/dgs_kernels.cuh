@@ -1815,10 +1815,8 @@ __global__ void __launch_bounds__(kThreads) k_apply_log(const uint32_t* __restri
   const uint32_t i = idx[j];
   const float v = val[j];
   lg.ent[(uint64_t)slot * lg.stride + j] = make_uint2(i, __float_as_uint(v));
-  if (i >= n) {
-    atomicMin(status, -2000);
-    return;
-  }
+  if (i >= n || (j + 1 < count && idx[j + 1] <= i)) atomicMin(status, -2000);   // out of range, or not ascending
+  if (i >= n) return;
   theta[i] = __fsub_rn(theta[i], v);
 }
 
@@ -2309,8 +2307,7 @@ __global__ void __maxnreg__(64) k_fold(const __grid_constant__ Workspace ws, con
   }
 }
 
-// Eager form, for a packet that is not one of the library's own (any order of indices, any
-// count): buffer q < N is D_q, buffer N is theta.  Indices of one packet are distinct, so every
+// Eager form, for a packet that is too long for the log (any count): buffer q < N is D_q, buffer N is theta.  Indices of one packet are distinct, so every
 // (buffer, entry) pair is touched by exactly one thread: plain load / subtract / store.
 __global__ void __launch_bounds__(kThreads) k_scatter_sub(const uint32_t* __restrict__ idx,
                                                           const float* __restrict__ val, uint32_t count,
