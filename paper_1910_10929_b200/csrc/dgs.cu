@@ -71,10 +71,10 @@ struct Layout {
   uint64_t tiles, segs, seg_off, blk_seg;
   ScratchLayout sc[kSets];
   uint64_t L_next, u_slots, status, stats;
-  uint64_t log_ent, log_pos;
+  uint64_t log_ent, log_pos, log_sum;
   uint64_t blk_max;      // [N][blk_stride]: per block of kWarpTile elements, an upper bound on the keys of D_q in it
   uint64_t blk_stride = 0;  // ring of applied packets not yet folded into every D_q
-  uint32_t log_ring = 0, log_stride = 0, pos_rows = 0;
+  uint32_t log_ring = 0, log_stride = 0, pos_rows = 0, sum_stride = 0;
   uint32_t num_blocks = 0;
   uint64_t total = 0;
 };
@@ -212,8 +212,10 @@ void make_layout(const dgs_config* c, Layout* L) {
   L->log_ring = (uint32_t)std::min<uint64_t>(kLogRingMax, std::max<uint64_t>(std::max<uint64_t>(N + kLogSlack, 4 * N), 16));
   L->log_stride = (uint32_t)align_up(L->K[0], 64);
   L->log_ent = take((uint64_t)L->log_ring * L->log_stride * sizeof(uint2));
-  L->pos_rows = (uint32_t)align_up(L->num_blocks, kBlockGroup) + 1;
+  L->pos_rows = L->num_blocks + 1;
   L->log_pos = take((uint64_t)L->log_ring * L->pos_rows * 4);
+  L->sum_stride = (uint32_t)align_up(L->pos_rows, 64);
+  L->log_sum = take((uint64_t)(L->log_ring + 1) * L->sum_stride * 4);
   L->blk_stride = align_up((c->n + kWarpTile - 1) / kWarpTile, 64);
   L->blk_max = take(N * L->blk_stride * 4);
   L->L_next = take(2 * N * S * 4);
@@ -481,8 +483,9 @@ int fold_launch(dgs_ctx* c, const Workspace& ws, const SelArgs& a, uint32_t q, c
   const uint32_t count = (uint32_t)(c->log_head - c->applied[q]);   // <= ring
   TimedLaunch tl(c, st, SCAN ? DGS_KERNEL_STREAM_PULL : DGS_KERNEL_CATCH_UP);
   const uint32_t warps = c->alone || c->cfg.num_workers == 1 ? kFoldWarps : kFoldWarps / 2;
-  k_fold<SCAN><<<c->fold_grid, warps * 32, fold_dyn_bytes(warps, c->fold_ahead, ws.part_cap), st>>>(ws, a, c->log, first, count,
-                                                                                               c->fold_ahead);
+  k_fold<SCAN><<<c->fold_grid, warps * 32, fold_dyn_bytes(warps, c->fold_ahead, ws.part_cap), st>>>(
+      ws, a, c->log, first, count, (uint32_t)(c->applied[q] % (c->log.ring + 1)), (uint32_t)(c->log_head % (c->log.ring + 1)),
+      c->fold_ahead);
   DGS_CUDA(c, cudaGetLastError());
   c->launches += 1;
   c->applied[q] = c->log_head;
@@ -640,7 +643,7 @@ int occupancy_grids(dgs_ctx* c, int sms) {
 // Grid of k_fold and the room for its tables and buffers.
 constexpr int kFoldMaxDyn = 208 * 1024;   // beside its static shared memory
 int fold_setup(dgs_ctx* c, int sms) {
-  c->fold_grid = (int)std::min<uint32_t>((c->lay.num_blocks + kBlockGroup - 1) / kBlockGroup, (uint32_t)std::min(2 * sms, kMaxFoldGrid));
+  c->fold_grid = (int)std::min<uint32_t>((c->lay.num_blocks + 7) / 8, (uint32_t)std::min(2 * sms, kMaxFoldGrid));
   // A quarter more than the mean number of entries of a block, for a worker that has missed a packet per worker.
   const uint64_t mean = std::min<uint64_t>(c->cfg.num_workers, 32) * c->lay.K[0] * kWarpTile / c->cfg.n;
   c->fold_ahead = (uint32_t)std::min<uint64_t>(192, std::max<uint64_t>(64, align_up(mean + mean / 4, 64)));
@@ -805,6 +808,7 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
     INIT_CUDA(cudaMemsetAsync(c->at<char>(sc.part_slot0), 0, (uint64_t)kMaxParts * 4, st));
     INIT_CUDA(cudaMemsetAsync(c->at<char>(sc.plan), 0, (uint64_t)(kMaxFoldGrid + 1) * 4, st));   // no plan yet
   }
+  INIT_CUDA(cudaMemsetAsync(c->at<char>(L.log_sum), 0, (uint64_t)L.sum_stride * 4, st));   // no packet filed
   INIT_CUDA(cudaMemsetAsync(c->at<char>(L.blk_max), 0, N * L.blk_stride * 4, st));   // D = 0
   INIT_CUDA(cudaMemsetAsync(c->at<char>(L.L_next), 0xFF, 2 * N * cfg->num_segments * 4, st));
   INIT_CUDA(cudaMemsetAsync(c->at<char>(L.status), 0, L.total - L.status, st));
@@ -867,6 +871,8 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
   c->log.ring = L.log_ring;
   c->log.pos = c->at<uint32_t>(L.log_pos);
   c->log.pos_rows = L.pos_rows;
+  c->log.sum = c->at<uint32_t>(L.log_sum);
+  c->log.sum_stride = L.sum_stride;
   *out = c;
   return DGS_OK;
 }
@@ -951,7 +957,8 @@ int apply_impl(dgs_ctx* c, uint32_t worker, const dgs_packet* pkt) {
       TimedLaunch tl(c, c->st[stream_id], DGS_KERNEL_SCATTER);
       const uint32_t pos_ctas = (c->log.pos_rows + kThreads - 1) / kThreads;
       k_apply_log<<<gx + pos_ctas, kThreads, 0, c->st[stream_id]>>>(pkt->idx, pkt->val, pkt->count, c->at<float>(c->lay.theta),
-                                                                    c->cfg.n, c->ws[0].status, c->log, lslot, gx);
+                                                                    c->cfg.n, c->ws[0].status, c->log, lslot,
+                                                                    (uint32_t)(c->log_head % (c->log.ring + 1)), gx);
       DGS_CUDA(c, cudaGetLastError());
       c->launches += 1;
     }

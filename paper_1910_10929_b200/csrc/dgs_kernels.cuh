@@ -39,7 +39,6 @@ constexpr int kMaxGrid = 512;       // upper bound on the grid of a stream pass 
 constexpr int kMaxFoldGrid = 320;   // upper bound on the grid of a pull's pass (every warp of it is a part)
 constexpr int kMaxParts = kMaxFoldGrid * kWarps;   // upper bound on the parts of the candidate buffer
 constexpr uint32_t kFoldSlack = 64; // part_cap is at least that much longer than a CTA's share (its tables round to groups and words)
-constexpr int kBlockGroup = 8;      // blocks of kWarpTile elements whose packet positions are one 32-byte sector
 constexpr int kMaxWorkers = 320;    // upper bound on the grid of finalize
 constexpr uint32_t kSpinLimit = 1u << 22;  // bounded waits: give up and report after this many polls
 constexpr int kStatusTimeout = -4;  // = DGS_ETIMEOUT
@@ -1762,7 +1761,11 @@ struct PacketLog {
   // reads a block's positions in all packets as one or two lines, where packet-major rows cost it a line per packet
   // (and, with a row per page, an address translation per packet).
   uint32_t* pos;      // [pos_rows][ring]
-  uint32_t pos_rows;  // > number of blocks rounded up to kBlockGroup
+  uint32_t pos_rows;  // number of blocks + 1
+  // sum[r][b]: entries in block b of all packets filed so far, when r packets had been (r counted modulo ring + 1; the
+  // sums wrap): what a worker finds in a block is the difference of two rows
+  uint32_t* sum;      // [ring + 1][sum_stride]
+  uint32_t sum_stride;
 };
 
 // First position in the sorted idx[0, count) whose entry is >= key, found by a whole warp: 32 probes at a time, so
@@ -1788,7 +1791,7 @@ __device__ __forceinline__ uint32_t warp_lower_bound(const uint32_t* __restrict_
 __global__ void __launch_bounds__(kThreads) k_apply_log(const uint32_t* __restrict__ idx,
                                                         const float* __restrict__ val, uint32_t count,
                                                         float* __restrict__ theta, uint64_t n, int* status,
-                                                        PacketLog lg, uint32_t slot, uint32_t copy_ctas) {
+                                                        PacketLog lg, uint32_t slot, uint32_t row, uint32_t copy_ctas) {
   if (blockIdx.x >= copy_ctas) {
     __shared__ uint32_t s_cnt[kThreads], s_end[2];
     __shared__ unsigned long long s_warp[kWarps];
@@ -1807,7 +1810,12 @@ __global__ void __launch_bounds__(kThreads) k_apply_log(const uint32_t* __restri
     __syncthreads();
     unsigned long long total;
     const uint32_t before = (uint32_t)block_excl_scan(s_cnt[threadIdx.x], s_warp, total);
-    if (b0 + threadIdx.x < lg.pos_rows) lg.pos[(uint64_t)(b0 + threadIdx.x) * lg.ring + slot] = lo + before;
+    const uint32_t b = b0 + threadIdx.x;
+    if (b < lg.pos_rows) {
+      lg.pos[(uint64_t)b * lg.ring + slot] = lo + before;
+      const uint32_t next = row == lg.ring ? 0u : row + 1u;       // `row`: as of the packet before
+      lg.sum[(uint64_t)next * lg.sum_stride + b] = __ldcg(lg.sum + (uint64_t)row * lg.sum_stride + b) + s_cnt[threadIdx.x];
+    }
     return;
   }
   const uint32_t j = blockIdx.x * kThreads + threadIdx.x;
@@ -1857,7 +1865,7 @@ __host__ __device__ inline uint32_t fold_dyn_bytes(uint32_t warps, uint32_t ahea
   return warps * 2u * fold_stage_bytes(ahead) + part_cap + part_cap / 8u;
 }
 // cost of a block with that many entries, in units of about 16 entries
-__device__ __forceinline__ uint32_t block_cost(uint32_t entries) { return min(255u, 3u + entries / 16u); }
+__device__ __forceinline__ uint32_t block_cost(uint32_t entries) { return min(255u, 4u + entries / 16u); }
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
@@ -1893,71 +1901,70 @@ __device__ __forceinline__ BlockRuns block_runs(uint32_t lo, uint32_t hi, uint32
   __syncwarp();
   return r;
 }
+// where in the log the block's entry e + lane is (e a multiple of 32, e + lane < total)
+__device__ __forceinline__ const uint2* entry_at(const PacketLog& lg, const BlockRuns& r, uint32_t e, const uint2* runs, int lane,
+                                                 uint32_t le) {
+  const uint32_t rel = r.excl - e;
+  const uint32_t heads = __reduce_or_sync(kFull, r.len != 0 && rel < 32u ? 1u << rel : 0u);   // entries that open a packet
+  const uint32_t before = __popc(__ballot_sync(kFull, r.len != 0 && r.excl < e));
+  const uint2 run = runs[max(before + __popc(heads & le), 1u) - 1u];
+  return lg.ent + ((uint64_t)run.y * lg.stride + (run.x + e + lane));
+}
+__device__ __forceinline__ uint2 load_entry(const PacketLog& lg, const BlockRuns& r, uint32_t e, const uint2* runs, int lane, uint32_t le) {
+  const uint2* const at = entry_at(lg, r, e, runs, lane, le);
+  return e + lane < r.total ? __ldcg(at) : make_uint2(kFull, 0u);
+}
 // the block's entries e0 .. end - 1 (end <= total), on their way to shared memory; e0 a multiple of 32
 __device__ __forceinline__ void fetch_entries(const PacketLog& lg, const BlockRuns& r, uint32_t e0, uint32_t end, const uint2* runs,
                                               uint2* ent, int lane, uint32_t le) {
 #pragma unroll 1
   for (uint32_t e = e0; e < end; e += 32) {
-    const uint32_t rel = r.excl - e;
-    const uint32_t heads = __reduce_or_sync(kFull, r.len != 0 && rel < 32u ? 1u << rel : 0u);   // entries that open a packet
-    const uint32_t before = __popc(__ballot_sync(kFull, r.len != 0 && r.excl < e));
-    if (e + lane < end) {
-      const uint2 run = runs[before + __popc(heads & le) - 1u];
-      cp_async8(ent + (e - e0) + lane, lg.ent + ((uint64_t)run.y * lg.stride + (run.x + e + lane)));
-    }
+    const uint2* const at = entry_at(lg, r, e, runs, lane, le);
+    if (e + lane < end) cp_async8(ent + (e - e0) + lane, at);
   }
 }
-// Subtracts the first `count` fetched entries from the block.  Lane order is packet order, and inside one packet the
+// Subtracts up to 32 entries (`has`: this lane has one) from the block.  Lane order is packet order, and inside one packet the
 // indices ascend: 32 entries fall into ascending runs, in each of which every element occurs once.  Where the runs are
 // few (a block with many entries) they go one by one, 36 cycles a step.  Else the lanes that share an element are found
 // with a ballot per bit of its offset (130 cycles; the match instruction takes 360 for 32 different offsets) and go
 // one after the other, mostly one or two steps.  Returns this lane's lines that were changed.
 constexpr uint32_t kFoldFew = 9;
-__device__ __forceinline__ uint32_t subtract_entries(float* tile, const uint2* ent, uint32_t count, uint32_t base, uint32_t n, int lane,
-                                                     uint32_t lt, uint32_t le) {
-  uint32_t dirty = 0;
-#pragma unroll 1
-  for (uint32_t e = 0; e < count; e += 32) {
-    uint32_t off = kFull;
-    float val = 0.f;
-    if (e + lane < count) {
-      const uint2 q = ent[e + lane];
-      if (q.x < n) off = q.x - base;
-      val = __uint_as_float(q.y);
-    }
-    const bool valid = off < (uint32_t)kWarpTile;
-    const uint32_t prev = __shfl_up_sync(kFull, off, 1);
-    const uint32_t opened = __ballot_sync(kFull, lane != 0 && off <= prev && e + lane < count);
-    uint32_t turn = __popc(opened & le), most = __popc(opened);
-    if (most >= kFoldFew) {
-      uint32_t peers = __ballot_sync(kFull, valid);
+__device__ __forceinline__ uint32_t subtract_group(float* tile, uint2 q, bool has, uint32_t base, uint32_t n, int lane, uint32_t lt,
+                                                   uint32_t le) {
+  const uint32_t off = has && q.x < n ? q.x - base : kFull;
+  const bool valid = off < (uint32_t)kWarpTile;
+  const uint32_t prev = __shfl_up_sync(kFull, off, 1);
+  const uint32_t opened = __ballot_sync(kFull, lane != 0 && off <= prev && has);
+  uint32_t turn = __popc(opened & le), most = __popc(opened);
+  if (most >= kFoldFew) {
+    uint32_t peers = __ballot_sync(kFull, valid);
 #pragma unroll
-      for (int b = 0; (1 << b) < kWarpTile; ++b) {
-        const uint32_t ones = __ballot_sync(kFull, (off >> b) & 1u);
-        peers &= (off >> b) & 1u ? ones : ~ones;
-      }
-      turn = __popc(peers & lt);
-      most = __reduce_max_sync(kFull, valid ? turn : 0u);
+    for (int b = 0; (1 << b) < kWarpTile; ++b) {
+      const uint32_t ones = __ballot_sync(kFull, (off >> b) & 1u);
+      peers &= (off >> b) & 1u ? ones : ~ones;
     }
-    float* const at = tile + tile_place(off & (uint32_t)(kWarpTile - 1));
-    for (uint32_t k = 0;; ++k) {
-      if (valid && turn == k) *at = __fsub_rn(*at, val);
-      __syncwarp();
-      if (k == most) break;
-    }
-    dirty |= valid ? 1u << (off >> 5) : 0u;
+    turn = __popc(peers & lt);
+    most = __reduce_max_sync(kFull, valid ? turn : 0u);
   }
-  return dirty;
+  float* const at = tile + tile_place(off & (uint32_t)(kWarpTile - 1));
+  for (uint32_t k = 0;; ++k) {
+    if (valid && turn == k) *at = __fsub_rn(*at, __uint_as_float(q.y));
+    __syncwarp();
+    if (k == most) break;
+  }
+  return valid ? 1u << (off >> 5) : 0u;
 }
 
-// What of a block was not fetched ahead: entries of the first 32 packets beyond the first `ahead` (a multiple of 64),
-// and the packets after the first 32 (a worker that has been away for long).  Half a buffer is on its way while the
-// other half is subtracted.
+// What of a block was not fetched ahead: entries of the first 32 packets beyond the first `ahead` (a multiple of 32),
+// and the packets after the first 32 (a worker that has been away for long).  128 entries are on their way while 128 are
+// subtracted (a block with 1500 entries is a warp's whole share: with 32 on their way it took 50,000 cycles).
 __device__ __noinline__ uint32_t fold_rest(const PacketLog& lg, uint32_t first, uint32_t count, uint32_t ahead, uint32_t blk, uint32_t n,
                                            FoldStage* st) {
+  constexpr int kDeep = 4;
   const int lane = threadIdx.x & 31;
-  const uint32_t lt = lanemask_lt(), le = lt | (1u << lane), half = ahead / 2;
+  const uint32_t lt = lanemask_lt(), le = lt | (1u << lane);
   uint32_t dirty = 0;
+#pragma unroll 1
   for (uint32_t p0 = 0; p0 < count; p0 += 32) {
     const uint32_t p = p0 + lane, slot = (first + p) % lg.ring;
     uint32_t l = 0, h = 0;
@@ -1966,16 +1973,25 @@ __device__ __noinline__ uint32_t fold_rest(const PacketLog& lg, uint32_t first, 
       h = __ldcg(lg.pos + (uint64_t)(blk + 1) * lg.ring + slot);
     }
     const BlockRuns r = block_runs(l, h, slot, st->runs, lane, lt);
-    uint32_t e = p0 ? 0u : ahead, side = 0;
-    fetch_entries(lg, r, e, min(r.total, e + half), st->runs, st->ent, lane, le);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    for (; e < r.total; e += half, side ^= half) {
-      fetch_entries(lg, r, e + half, min(r.total, e + 2 * half), st->runs, st->ent + (side ^ half), lane, le);
-      asm volatile("cp.async.commit_group;" ::: "memory");
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-      __syncwarp();
-      dirty |= subtract_entries(st->tile, st->ent + side, min(half, r.total - e), blk * kWarpTile, n, lane, lt, le);
+    uint2 q[kDeep], next[kDeep];
+    auto load = [&](uint32_t e) {
+#pragma unroll
+      for (int u = 0; u < kDeep; ++u)
+        if (e + 32u * u < r.total) next[u] = load_entry(lg, r, e + 32u * u, st->runs, lane, le);
+    };
+    uint32_t e = p0 ? 0u : ahead;
+    load(e);
+#pragma unroll 1
+    for (; e < r.total; e += 32u * kDeep) {
+#pragma unroll
+      for (int u = 0; u < kDeep; ++u) q[u] = next[u];
+      load(e + 32u * kDeep);
+#pragma unroll
+      for (int u = 0; u < kDeep; ++u)
+        if (e + 32u * u < r.total)
+          dirty |= subtract_group(st->tile, q[u], e + 32u * u + lane < r.total, blk * kWarpTile, n, lane, lt, le);
     }
+    __syncwarp();
   }
   return dirty;
 }
@@ -2034,9 +2050,12 @@ __device__ __noinline__ uint32_t scan_mixed(const Workspace& ws, const SelArgs& 
   return total;
 }
 
+// 72 registers a thread: with 64 the loop over the blocks spills a few (a round of 32 arrivals on 124 M elements: 14.1 ms
+// against 11.9), with 80 and 96 fewer warps of other kernels fit beside it (12.4 ms, 12.4 ms).
 template <bool SCAN>
-__global__ void __maxnreg__(64) k_fold(const __grid_constant__ Workspace ws, const __grid_constant__ SelArgs a,
-                                       const __grid_constant__ PacketLog lg, uint32_t first, uint32_t count, uint32_t ahead) {
+__global__ void __maxnreg__(72) k_fold(const __grid_constant__ Workspace ws, const __grid_constant__ SelArgs a,
+                                       const __grid_constant__ PacketLog lg, uint32_t first, uint32_t count, uint32_t row0,
+                                       uint32_t row1, uint32_t ahead) {
   __shared__ FoldShared sh;
   extern __shared__ __align__(16) unsigned char fold_dyn[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -2049,14 +2068,13 @@ __global__ void __maxnreg__(64) k_fold(const __grid_constant__ Workspace ws, con
   uint8_t* const cost = fold_dyn + nw * 2u * stage_bytes;                        // [part_cap]
   uint32_t* const live = reinterpret_cast<uint32_t*>(cost + ws.part_cap);        // [part_cap / 32]
 
-  // this CTA's blocks [b0, b1); the tables count from `at0`, where b0's group of blocks begins
+  // this CTA's blocks [b0, b1)
   uint32_t b0 = part_first_tile(cta, G, NB), b1 = part_first_tile(cta + 1, G, NB);
   if (SCAN && ws.plan != nullptr && ld_volatile(ws.sync + kPlanParts) == G && __ldcg(ws.plan + G) == NB) {
     b0 = __ldcg(ws.plan + cta);
     b1 = __ldcg(ws.plan + cta + 1);
   }
-  const uint32_t at0 = b0 / kBlockGroup * kBlockGroup, groups = b0 < b1 ? (b1 - at0 + kBlockGroup - 1) / kBlockGroup : 0u;
-  const uint32_t words = (groups + 3u) / 4u;   // of `live`
+  const uint32_t mine = b0 < b1 ? b1 - b0 : 0u, words = (mine + 31u) / 32u;   // words of `live`
 
   if (SCAN)
     for (uint32_t b = tid; b < (uint32_t)kBins1; b += nt) sh.hist[b] = 0;
@@ -2069,41 +2087,27 @@ __global__ void __maxnreg__(64) k_fold(const __grid_constant__ Workspace ws, con
     }
   }
 
-  // A warp looks at 32 blocks at a time: lane l at the bound of block l, then lane p at where the blocks begin in packet
-  // p.  A block is skipped if it has no entry and its bound lies below L.
+  // A block is skipped if no packet has an entry in it and its bound lies below L.
   uint32_t read = 0;
   for (uint32_t w = warp; w < words; w += nw) {
-    const uint32_t b = at0 + w * 32u + lane;
+    const uint32_t b = b0 + w * 32u + lane;
+    uint32_t entries = 0;
     bool on = false;
-    if (SCAN && b >= b0 && b < b1) {
-      uint32_t s = S == 1 ? 0u : __ldg(ws.blk_seg + b);
-      uint32_t L = a.L_in[s];
-      if (S > 1) {   // the lowest bound of the layers that have a part of the block
-        const uint64_t end = (uint64_t)(b + 1) * kWarpTile;
-        while (s + 1 < S && __ldg(ws.seg_off + s + 1) < end) L = min(L, a.L_in[++s]);
-      }
-      on = __ldcg(a.blk_max + b) >= L;
-    }
-    uint32_t mine = 0;                        // entries of block b
-    for (uint32_t p0 = 0; p0 < count; p0 += 32) {
-      const uint32_t p = p0 + lane, rows = min(32u, groups * kBlockGroup - w * 32u);
-      const uint32_t* const pos = lg.pos + (uint64_t)(at0 + w * 32u) * lg.ring + (first + p) % lg.ring;
-      uint32_t prev = p < count ? __ldcg(pos) : 0u;
-#pragma unroll 1
-      for (uint32_t r0 = 0; r0 < rows; r0 += kBlockGroup) {
-        uint32_t q[kBlockGroup];
-#pragma unroll
-        for (int k = 0; k < kBlockGroup; ++k) q[k] = p < count ? __ldcg(pos + (uint64_t)(r0 + k + 1) * lg.ring) : 0u;
-#pragma unroll
-        for (int k = 0; k < kBlockGroup; ++k) {
-          const uint32_t e = __reduce_add_sync(kFull, q[k] - prev);
-          if ((uint32_t)lane == r0 + k) mine += e;
-          prev = q[k];
+    if (b < b1) {
+      if (count) entries = __ldcg(lg.sum + (uint64_t)row1 * lg.sum_stride + b) - __ldcg(lg.sum + (uint64_t)row0 * lg.sum_stride + b);
+      if (SCAN) {
+        const uint32_t bound = __ldcg(a.blk_max + b);
+        uint32_t s = S == 1 ? 0u : __ldg(ws.blk_seg + b);
+        uint32_t L = a.L_in[s];
+        if (S > 1) {   // the lowest bound of the layers that have a part of the block
+          const uint64_t end = (uint64_t)(b + 1) * kWarpTile;
+          while (s + 1 < S && __ldg(ws.seg_off + s + 1) < end) L = min(L, a.L_in[++s]);
         }
+        on = bound >= L;
       }
+      on = on || entries != 0;
     }
-    on = b >= b0 && b < b1 && (on || mine != 0);
-    cost[w * 32u + lane] = on ? (uint8_t)block_cost(mine) : (uint8_t)0;
+    cost[w * 32u + lane] = on ? (uint8_t)block_cost(entries) : (uint8_t)0;
     const uint32_t word = __ballot_sync(kFull, on);
     if (lane == 0) {
       live[w] = word;
@@ -2112,20 +2116,14 @@ __global__ void __maxnreg__(64) k_fold(const __grid_constant__ Workspace ws, con
   }
   if (SCAN && read) atomicAdd(&sh.read, read);
   __syncthreads();
-  // Runs of about equal cost for the warps: warp w begins at the block where the cost so far passes w parts of nw.
+  // Runs of about equal cost for the warps: warp w begins at the block where the cost so far passes w parts of nw.  A
+  // thread adds up `per` consecutive blocks, four at a time.
   uint32_t all;
   {
-    const uint32_t per = (words + nt - 1) / nt, w0 = min(words, tid * per), w1 = min(words, w0 + per);
-    const uint4* const c4 = reinterpret_cast<const uint4*>(cost);
-    auto word_cost = [&](uint32_t w) {
-      const uint4 x = c4[2 * w], y = c4[2 * w + 1];
-      uint32_t v = __dp4a(x.x, 0x01010101u, 0u);
-      v = __dp4a(x.y, 0x01010101u, v); v = __dp4a(x.z, 0x01010101u, v); v = __dp4a(x.w, 0x01010101u, v);
-      v = __dp4a(y.x, 0x01010101u, v); v = __dp4a(y.y, 0x01010101u, v); v = __dp4a(y.z, 0x01010101u, v);
-      return __dp4a(y.w, 0x01010101u, v);
-    };
+    const uint32_t quads = words * 8u, per = (quads + nt - 1) / nt, q0 = min(quads, tid * per), q1 = min(quads, q0 + per);
+    const uint32_t* const c4 = reinterpret_cast<const uint32_t*>(cost);
     uint32_t sum = 0;
-    for (uint32_t w = w0; w < w1; ++w) sum += word_cost(w);
+    for (uint32_t q = q0; q < q1; ++q) sum = __dp4a(c4[q], 0x01010101u, sum);
     uint32_t at = sum;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -2140,20 +2138,16 @@ __global__ void __maxnreg__(64) k_fold(const __grid_constant__ Workspace ws, con
       if (w == (uint32_t)warp) at += all;
       all += sh.warp_sum[w];                     // < 2^32 / 8: a share has fewer than 2^20 blocks
     }
-    if (sum) {
-      uint32_t k = 0;                            // next warp whose run begins at or after `at`
-      while (k < nw && k * all / nw < at) ++k;
-      for (uint32_t w = w0; w < w1 && k < nw; ++w) {
-        const uint32_t wc = word_cost(w);
-        if (k * all / nw >= at + wc) {           // none begins in this word
-          at += wc;
-          continue;
-        }
-        for (uint32_t x = live[w]; x; x &= x - 1) {
-          const uint32_t b = w * 32u + __ffs(x) - 1u;
-          at += cost[b];
-          for (; k < nw && k * all / nw < at; ++k) sh.start[k] = b;
-        }
+    // first warp whose run begins in this thread's blocks or later: the smallest k with k all / nw >= at
+    uint32_t k = sum ? (uint32_t)(((uint64_t)at * nw + all - 1) / all) : nw;
+    while (k > 0 && sum && (k - 1) * all / nw >= at) --k;
+    while (k < nw && k * all / nw < at) ++k;
+    if (sum && k < nw && k * all / nw < at + sum) {
+      for (uint32_t b = q0 * 4u; b < q1 * 4u; ++b) {
+        const uint32_t c = cost[b];
+        if (c == 0) continue;
+        at += c;
+        for (; k < nw && k * all / nw < at; ++k) sh.start[k] = b;
       }
     }
     if (tid == 0) sh.start[nw] = words * 32u;
@@ -2176,7 +2170,7 @@ __global__ void __maxnreg__(64) k_fold(const __grid_constant__ Workspace ws, con
     }
     const uint32_t b = walk_word * 32u + __ffs(walk_bits) - 1u;
     walk_bits &= walk_bits - 1u;
-    return b < run1 ? at0 + b : kFull;
+    return b < run1 ? b0 + b : kFull;
   };
   const uint32_t my_slot = (first + lane) % lg.ring;             // of the first 32 packets
   const uint32_t fill = (lane ^ ((lane >> 3) & 3)) * 4;          // where lane's 16 bytes of a 512-byte piece go
@@ -2231,7 +2225,11 @@ __global__ void __maxnreg__(64) k_fold(const __grid_constant__ Workspace ws, con
     __syncwarp();
     // fold
     if (count) {
-      uint32_t dirty = subtract_entries(t, st->ent, min(total, ahead), base, n, lane, lt, le);
+      uint32_t dirty = 0;
+      const uint32_t ready = min(total, ahead);
+#pragma unroll 1
+      for (uint32_t e = 0; e < ready; e += 32)
+        dirty |= subtract_group(t, st->ent[e + lane], e + lane < ready, base, n, lane, lt, le);   // (ent is a multiple of 32 long)
       if (total > ahead || count > 32u) dirty |= fold_rest(lg, first, count, ahead, blk, n, st);
       dirty = __reduce_or_sync(kFull, dirty);
       if (dirty) {     // changed lines back to memory
@@ -2301,7 +2299,7 @@ __global__ void __maxnreg__(64) k_fold(const __grid_constant__ Workspace ws, con
       if (sh.hist[b]) atomicAdd(ws.hist1 + (size_t)main_seg * kBins1 + b, sh.hist[b]);
     if (tid == 0) {
       if (ws.cta_cost != nullptr) ws.cta_cost[cta] = all;
-      atomicAdd(ws.stats + 3, (unsigned long long)groups);
+      atomicAdd(ws.stats + 3, (unsigned long long)((mine + 7u) / 8u));
       atomicAdd(ws.stats + 4, (unsigned long long)sh.read);
     }
   }
