@@ -1923,29 +1923,18 @@ __device__ __forceinline__ void fetch_entries(const PacketLog& lg, const BlockRu
     if (e + lane < end) cp_async8(ent + (e - e0) + lane, at);
   }
 }
-// Subtracts up to 32 entries (`has`: this lane has one) from the block.  Lane order is packet order, and inside one packet the
-// indices ascend: 32 entries fall into ascending runs, in each of which every element occurs once.  Where the runs are
-// few (a block with many entries) they go one by one, 36 cycles a step.  Else the lanes that share an element are found
-// with a ballot per bit of its offset (130 cycles; the match instruction takes 360 for 32 different offsets) and go
-// one after the other, mostly one or two steps.  Returns this lane's lines that were changed.
-constexpr uint32_t kFoldFew = 9;
-__device__ __forceinline__ uint32_t subtract_group(float* tile, uint2 q, bool has, uint32_t base, uint32_t n, int lane, uint32_t lt,
-                                                   uint32_t le) {
+// Subtracts up to 32 entries (`has`: this lane has one) from the block.  Lane order is packet order, and inside one packet
+// the indices ascend: 32 entries fall into ascending runs, in each of which every element occurs once, and the runs go
+// one after the other, 36 cycles a step.  (Finding the lanes that share an element instead -- with the match instruction,
+// with a ballot per bit of the offsets, or with a tag byte per element -- costs more than the steps it saves: a round of
+// 32 arrivals on 11.7 M elements takes 3.19 ms by runs, 3.25 ms with ballots above 5 runs, 4.29 ms with tags.)
+// Returns this lane's line that was changed.
+__device__ __forceinline__ uint32_t subtract_group(float* tile, uint2 q, bool has, uint32_t base, uint32_t n, int lane, uint32_t le) {
   const uint32_t off = has && q.x < n ? q.x - base : kFull;
   const bool valid = off < (uint32_t)kWarpTile;
   const uint32_t prev = __shfl_up_sync(kFull, off, 1);
-  const uint32_t opened = __ballot_sync(kFull, lane != 0 && off <= prev && has);
-  uint32_t turn = __popc(opened & le), most = __popc(opened);
-  if (most >= kFoldFew) {
-    uint32_t peers = __ballot_sync(kFull, valid);
-#pragma unroll
-    for (int b = 0; (1 << b) < kWarpTile; ++b) {
-      const uint32_t ones = __ballot_sync(kFull, (off >> b) & 1u);
-      peers &= (off >> b) & 1u ? ones : ~ones;
-    }
-    turn = __popc(peers & lt);
-    most = __reduce_max_sync(kFull, valid ? turn : 0u);
-  }
+  const uint32_t opened = __ballot_sync(kFull, lane != 0 && off <= prev && has);   // lanes that open a run, but the first
+  const uint32_t turn = __popc(opened & le), most = __popc(opened);
   float* const at = tile + tile_place(off & (uint32_t)(kWarpTile - 1));
   for (uint32_t k = 0;; ++k) {
     if (valid && turn == k) *at = __fsub_rn(*at, __uint_as_float(q.y));
@@ -1989,7 +1978,7 @@ __device__ __noinline__ uint32_t fold_rest(const PacketLog& lg, uint32_t first, 
 #pragma unroll
       for (int u = 0; u < kDeep; ++u)
         if (e + 32u * u < r.total)
-          dirty |= subtract_group(st->tile, q[u], e + 32u * u + lane < r.total, blk * kWarpTile, n, lane, lt, le);
+          dirty |= subtract_group(st->tile, q[u], e + 32u * u + lane < r.total, blk * kWarpTile, n, lane, le);
     }
     __syncwarp();
   }
@@ -1998,11 +1987,12 @@ __device__ __noinline__ uint32_t fold_rest(const PacketLog& lg, uint32_t first, 
 
 // exclusive prefix over the lanes of counts up to 31, and their sum
 __device__ __forceinline__ uint32_t lane_offsets(uint32_t count, uint32_t lt, uint32_t& total) {
-  uint32_t ex = 0;
-  total = 0;
+  uint32_t m = __ballot_sync(kFull, count & 1u), ex = __popc(m & lt);
+  total = __popc(m);
+  if (!__any_sync(kFull, count > 1)) return ex;    // as it mostly is
 #pragma unroll
-  for (int b = 0; b < 5; ++b) {
-    const uint32_t m = __ballot_sync(kFull, (count >> b) & 1u);
+  for (int b = 1; b < 5; ++b) {
+    m = __ballot_sync(kFull, (count >> b) & 1u);
     ex += __popc(m & lt) << b;
     total += __popc(m) << b;
   }
@@ -2229,7 +2219,7 @@ __global__ void __maxnreg__(72) k_fold(const __grid_constant__ Workspace ws, con
       const uint32_t ready = min(total, ahead);
 #pragma unroll 1
       for (uint32_t e = 0; e < ready; e += 32)
-        dirty |= subtract_group(t, st->ent[e + lane], e + lane < ready, base, n, lane, lt, le);   // (ent is a multiple of 32 long)
+        dirty |= subtract_group(t, st->ent[e + lane], e + lane < ready, base, n, lane, le);   // (ent is a multiple of 32 long)
       if (total > ahead || count > 32u) dirty |= fold_rest(lg, first, count, ahead, blk, n, st);
       dirty = __reduce_or_sync(kFull, dirty);
       if (dirty) {     // changed lines back to memory
