@@ -28,6 +28,8 @@ class Context:
         self.arena_bytes = dgs.dgs_arena_bytes(cfg)
         with torch.cuda.device(self.device):
             self.arena = torch.empty(self.arena_bytes, dtype=torch.uint8, device=self.device)
+            self._base = self.arena.data_ptr()
+            self._typed = {t: self.arena.view(t) for t in (torch.int32, torch.float32)}
             cfg.theta0 = theta0.data_ptr()
             cfg.arena = self.arena.data_ptr()
             cfg.arena_bytes = self.arena_bytes
@@ -81,9 +83,9 @@ class Context:
     # ---- reading results ---------------------------------------------------------
     def _view(self, ptr: int, count: int, dtype: torch.dtype) -> torch.Tensor:
         """A tensor over `count` 4-byte elements at a device address inside the arena."""
-        off = ptr - self.arena.data_ptr()
+        off = ptr - self._base
         assert 0 <= off and off + 4 * count <= self.arena_bytes
-        return self.arena[off:off + 4 * count].view(dtype)
+        return self._typed[dtype].narrow(0, off // 4, count)
 
     def flush(self) -> None:
         """Orders the context's stream after all work enqueued so far."""

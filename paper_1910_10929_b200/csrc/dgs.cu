@@ -46,6 +46,7 @@ int streams_for(const dgs_config* c) {
   if (c->flags & DGS_SINGLE_STREAM) return 1;   // kernels run one after the other, in call order
   return (int)std::min<uint32_t>(kStreams, c->num_workers / 2 + 1);
 }
+constexpr int kCaller = kStreams;         // the caller's stream, where the tracker names streams by number
 constexpr int kQueuesWanted = 12;         // hardware queues that keep the streams of two contexts and the caller's apart
 constexpr int kLogRingMax = 128;            // most packets the apply log keeps
 constexpr int kLogSlack = 32;               // slots of the log beyond one per worker
@@ -234,15 +235,15 @@ struct dgs_ctx {
   Layout lay;
   char* base;
   cudaStream_t user;       // the caller's stream: entry point of dependencies, target of dgs_flush
-  cudaStream_t st[kStreams];   // null until first taken
+  cudaStream_t st[kStreams + 1];   // null until first taken; [kCaller]: the caller's
   int streams;             // how many of them may be taken (1 under DGS_SINGLE_STREAM)
   int next_stream;         // the one that the next event takes ...
   bool idle;               // ... unless nothing has been enqueued since everything was last joined: then the first one
-  bool dirty[kStreams];    // stream has work that the caller's stream has not been made to wait for
+  bool dirty[kStreams + 1];    // stream has work that the caller's stream has not been made to wait for
   std::vector<int> worker_stream;   // per worker: stream of its last push if its pull is still to come, else -1
   int slot_stream[kPushSlots];      // per push packet slot: stream of its push
   cudaEvent_t ev_in;       // "everything the caller had enqueued when the call was made"
-  bool forked[kStreams];  // stream already waits for ev_in of the current call
+  bool forked[kStreams + 1];  // stream already waits for ev_in of the current call
   cudaEvent_t ev_tail[kStreams];  // for dgs_flush
   // dependency tracker
   struct Dep {
@@ -257,10 +258,10 @@ struct dgs_ctx {
   std::vector<Res> res;
   // one "done" event per task, reused in turn; a ring per stream, so that an event is only ever
   // re-recorded later on the same stream and waiting for a reused one still covers the older task
-  std::vector<cudaEvent_t> ev_ring[kStreams];
-  size_t ev_next[kStreams];
+  std::vector<cudaEvent_t> ev_ring[kStreams + 1];
+  size_t ev_next[kStreams + 1];
   uint64_t task_seq;                               // tasks filed so far
-  uint64_t waited_seq[kStreams][kStreams];   // [waiting stream][stream]: newest task already waited for
+  uint64_t waited_seq[kStreams + 1][kStreams + 1];   // [waiting stream][stream]: newest task already waited for
   uint64_t push_count, pull_count, event_count, var_count;
   // Lazy difference vectors: packet number p (counted from 0) of the library's own pushes sits in slot
   // p % ring of the log from its apply on; applied[q] packets have been folded into D_q so far.
@@ -386,9 +387,11 @@ int begin_call(dgs_ctx* c) {
   return DGS_OK;
 }
 int stream_ready(dgs_ctx* c, int which) {
-  if (c->st[which]) return DGS_OK;
-  DGS_CUDA(c, cudaStreamCreateWithFlags(&c->st[which], cudaStreamNonBlocking));
-  DGS_CUDA(c, cudaEventCreateWithFlags(&c->ev_tail[which], cudaEventDisableTiming));
+  if (!c->ev_ring[which].empty()) return DGS_OK;
+  if (which != kCaller) {
+    DGS_CUDA(c, cudaStreamCreateWithFlags(&c->st[which], cudaStreamNonBlocking));
+    DGS_CUDA(c, cudaEventCreateWithFlags(&c->ev_tail[which], cudaEventDisableTiming));
+  }
   for (int i = 0; i < kEventRing; ++i) {
     cudaEvent_t e;
     DGS_CUDA(c, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
@@ -410,6 +413,7 @@ int fork_from_user(dgs_ctx* c, int which) {
   if (c->forked[which]) return DGS_OK;
   DGS_CUDA(c, cudaStreamWaitEvent(c->st[which], c->ev_in, 0));
   c->forked[which] = true;
+  c->waited_seq[which][kCaller] = c->task_seq;   // (ev_in was recorded after the tasks on the caller's stream)
   return DGS_OK;
 }
 
@@ -434,7 +438,7 @@ int task_begin(dgs_ctx* c, const Task& t) {
   if (ready != DGS_OK) return ready;
   // Tasks of one stream complete in order, so per stream only the newest task that this one depends
   // on matters, and only if the stream has not already waited for that task or a newer one.
-  dgs_ctx::Dep need[kStreams];
+  dgs_ctx::Dep need[kStreams + 1];
   auto want = [&](const dgs_ctx::Dep& d) {
     if (!d.ev || d.stream == t.stream) return;   // same stream: already ordered
     if (d.seq > need[d.stream].seq) need[d.stream] = d;
@@ -445,7 +449,7 @@ int task_begin(dgs_ctx* c, const Task& t) {
     want(x.last_write);
     for (const dgs_ctx::Dep& rd : x.reads) want(rd);
   }
-  for (int s = 0; s < kStreams; ++s) {
+  for (int s = 0; s <= kCaller; ++s) {
     if (!need[s].ev || need[s].seq <= c->waited_seq[t.stream][s]) continue;
     DGS_CUDA(c, cudaStreamWaitEvent(c->st[t.stream], need[s].ev, 0));
     c->waited_seq[t.stream][s] = need[s].seq;
@@ -666,7 +670,7 @@ void destroy_ctx(dgs_ctx* c) {
     if (c->ev_tail[i]) cudaEventDestroy(c->ev_tail[i]);
   }
   if (c->ev_in) cudaEventDestroy(c->ev_in);
-  for (int i = 0; i < kStreams; ++i)
+  for (int i = 0; i <= kCaller; ++i)
     for (cudaEvent_t e : c->ev_ring[i]) cudaEventDestroy(e);
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
   c->magic = 0;
@@ -726,10 +730,11 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
   for (int i = 0; i < kPushSlots; ++i) c->slot_stream[i] = 0;
   c->ev_in = nullptr;
   c->task_seq = 0;
-  for (int i = 0; i < kStreams; ++i) {
+  for (int i = 0; i <= kCaller; ++i) {
     c->ev_next[i] = 0;
-    for (int j = 0; j < kStreams; ++j) c->waited_seq[i][j] = 0;
+    for (int j = 0; j <= kCaller; ++j) c->waited_seq[i][j] = 0;
   }
+  c->forked[kCaller] = c->dirty[kCaller] = false;
   c->pull_count = c->event_count = c->var_count = 0;
   c->log_head = 0;
   c->applied.assign(cfg->num_workers, 0);
@@ -740,7 +745,7 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
     return DGS_ENOMEM;
   }
   c->base = static_cast<char*>(cfg->arena);
-  c->user = static_cast<cudaStream_t>(cfg->stream);
+  c->user = c->st[kCaller] = static_cast<cudaStream_t>(cfg->stream);
   c->push_count = 0;
   c->inv_m = 1.0f / cfg->momentum;  // one IEEE division; the kernels multiply by this constant
   c->timestamp = 0;
@@ -1155,6 +1160,7 @@ int dgs_flush(dgs_ctx* c) {
     DGS_CUDA(c, cudaEventRecord(c->ev_tail[i], c->st[i]));
     DGS_CUDA(c, cudaStreamWaitEvent(c->user, c->ev_tail[i], 0));
     c->dirty[i] = false;
+    c->waited_seq[kCaller][i] = c->task_seq;
   }
   c->idle = true;
   c->alone = true;
@@ -1234,25 +1240,40 @@ int dgs_state_load(dgs_ctx* c, int which, uint32_t worker, const float* src) {
   int rc = live(c);
   if (rc != DGS_OK) return rc;
   if (!src) return DGS_EINVAL;
-  const float* dst = nullptr;
-  rc = dgs_state_ptr(c, which, worker, &dst);  // waits for all work in flight
-  if (rc != DGS_OK) return rc;
-  rc = begin_call(c);
-  if (rc != DGS_OK) return rc;
+  if (which != DGS_THETA && worker >= c->cfg.num_workers) return DGS_EINVAL;
   const ResIds R{c->cfg.num_workers};
   Task t;
-  t.stream = 0;
-  t.writes.push_back(which == DGS_THETA ? R.THETA()
-                     : which == DGS_U   ? R.U(worker)
-                     : which == DGS_D   ? R.D(worker)
-                                        : R.TL(worker));
-  rc = fork_from_user(c, t.stream);
-  if (rc != DGS_OK) return rc;
+  t.stream = kCaller;          // src may be given back to a stream-ordered allocator right after the call
+  const float* dst = nullptr;
+  switch (which) {
+    case DGS_THETA:
+      dst = c->at<float>(c->lay.theta);
+      t.writes.push_back(R.THETA());
+      break;
+    case DGS_D:
+      dst = c->D_buf(worker);
+      t.writes.push_back(R.D(worker));
+      break;
+    case DGS_THETA_LOCAL:
+      if (!(c->cfg.flags & DGS_KEEP_LOCAL_MODEL)) return DGS_EINVAL;
+      dst = c->theta_local_buf(worker);
+      t.writes.push_back(R.TL(worker));
+      break;
+    case DGS_U:                // the buffer is known on the device only: waits for all work in flight
+      rc = dgs_state_ptr(c, which, worker, &dst);
+      if (rc != DGS_OK) return rc;
+      t.writes.push_back(R.U(worker));
+      break;
+    default: return DGS_EINVAL;
+  }
   rc = task_begin(c, t);
   if (rc != DGS_OK) return rc;
-  DGS_CUDA(c, cudaMemcpyAsync(const_cast<float*>(dst), src, c->cfg.n * 4, cudaMemcpyDeviceToDevice, c->st[t.stream]));
-  if (which == DGS_D)   // nothing is known about the new contents: every block may hold anything
-    DGS_CUDA(c, cudaMemsetAsync(c->blk_max(worker), 0xFF, c->lay.blk_stride * 4, c->st[t.stream]));
+  DGS_CUDA(c, cudaMemcpyAsync(const_cast<float*>(dst), src, c->cfg.n * 4, cudaMemcpyDeviceToDevice, c->user));
+  if (which == DGS_D) {
+    // Nothing is known about the new contents: every block may hold anything.  Packets filed so far belong to the old.
+    DGS_CUDA(c, cudaMemsetAsync(c->blk_max(worker), 0xFF, c->lay.blk_stride * 4, c->user));
+    c->applied[worker] = c->log_head;
+  }
   return task_end(c, t);
 }
 
