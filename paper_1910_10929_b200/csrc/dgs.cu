@@ -71,7 +71,7 @@ struct Layout {
   uint64_t var_idx[kVarSlots], var_val[kVarSlots], var_count[kVarSlots], L_one;
   uint64_t tiles, segs, seg_off, blk_seg;
   ScratchLayout sc[kSets];
-  uint64_t L_next, u_slots, status, stats;
+  uint64_t L_next, slack, u_slots, status, stats;
   uint64_t log_ent, log_pos, log_sum;
   uint64_t blk_max;      // [N][blk_stride]: per block of kWarpTile elements, an upper bound on the keys of D_q in it
   uint64_t blk_stride = 0;  // ring of applied packets not yet folded into every D_q
@@ -220,6 +220,7 @@ void make_layout(const dgs_config* c, Layout* L) {
   L->blk_stride = align_up((c->n + kWarpTile - 1) / kWarpTile, 64);
   L->blk_max = take(N * L->blk_stride * 4);
   L->L_next = take(2 * N * S * 4);
+  L->slack = take(2 * S * 4);
   L->u_slots = take((N + kSets) * sizeof(float*));
   L->status = take(4);
   L->stats = take((uint64_t)kNumStats * 8);
@@ -279,7 +280,6 @@ struct dgs_ctx {
   bool alone;
   int hist_grid[3];      // CTAs of the whole-input histogram pass, per mode
   int finalize_max[3];   // most CTAs of the cooperative finalize kernel that can be resident at once, per mode
-  uint32_t select_seq;   // selections launched so far
   uint64_t kind_seq[2];  // selections of each kind launched so far
   // Carried bounds: row (kind, worker) of L_next holds the bounds suggested by that worker's
   // latest selection of that kind ([0] push, [1] pull).  row_age says in which state it was
@@ -556,6 +556,7 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
   if (KIND == 1 && age < 2 && c->cfg.num_workers > 1) row = -1;
   const bool single_pass = row >= 0;
   a.L_next = c->L_next(KIND, worker);
+  a.slack = c->at<uint32_t>(c->lay.slack) + (uint64_t)KIND * c->cfg.num_segments;
   a.force_two_pass = single_pass ? 0 : 1;
   // CTAs of finalize: as many as keep the candidates (about 1.7 times the entries) in the threads' registers, but not
   // fewer than 32, since every step of a warp is a chain, and no more than one per SM (see k_finalize).  A warp per two
@@ -573,7 +574,7 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
     a.phantom_workers = 1;
     a.spin_limit = 4096;
   }
-  a.seq = ++c->select_seq;
+  a.seq = (uint32_t)c->kind_seq[KIND];
   a.L_in = single_pass ? c->L_next(KIND, (uint32_t)row) : ws.L_safe;
   task.stream = stream_id;
   if (single_pass && (uint32_t)row != worker) task.reads.push_back(R.ROW(KIND, (uint32_t)row));
@@ -749,7 +750,6 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
   c->push_count = 0;
   c->inv_m = 1.0f / cfg->momentum;  // one IEEE division; the kernels multiply by this constant
   c->timestamp = 0;
-  c->select_seq = 0;
   c->launches = 0;
   c->last_cuda = 0;
   c->broken = false;
@@ -818,6 +818,7 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
   INIT_CUDA(cudaMemsetAsync(c->at<char>(L.log_sum), 0, (uint64_t)L.sum_stride * 4, st));   // no packet filed
   INIT_CUDA(cudaMemsetAsync(c->at<char>(L.blk_max), 0, N * L.blk_stride * 4, st));   // D = 0
   INIT_CUDA(cudaMemsetAsync(c->at<char>(L.L_next), 0xFF, 2 * N * cfg->num_segments * 4, st));
+  INIT_CUDA(cudaMemsetAsync(c->at<char>(L.slack), 0, 2ull * cfg->num_segments * 4, st));
   INIT_CUDA(cudaMemsetAsync(c->at<char>(L.status), 0, L.total - L.status, st));
   INIT_CUDA(cudaMemcpyAsync(c->at<char>(L.tiles), tiles.data(), tiles.size() * sizeof(Tile), cudaMemcpyHostToDevice, st));
   INIT_CUDA(cudaMemcpyAsync(c->at<char>(L.segs), segs.data(), segs.size() * sizeof(SegDesc), cudaMemcpyHostToDevice, st));
