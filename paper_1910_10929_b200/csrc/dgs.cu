@@ -1417,7 +1417,7 @@ namespace {
 
 struct TopkDevice {
   bool ready = false;
-  uint32_t max_cluster = 0;   // CTAs of the largest cluster the device takes
+  uint32_t max_cluster[2] = {0, 0};   // CTAs of the largest cluster the device takes, for either variant of k_topk
 };
 constexpr int kMaxDevices = 64;
 TopkDevice g_topk_dev[kMaxDevices];
@@ -1426,11 +1426,11 @@ std::mutex g_topk_mu;
 struct TopkLaunch {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr;
-  TopkLaunch(uint32_t cluster, uint32_t cap, cudaStream_t st) {
+  TopkLaunch(bool fine, uint32_t cluster, uint32_t cap, cudaStream_t st) {
     std::memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3(cluster);
-    cfg.blockDim = dim3(kTopkThreads);
-    cfg.dynamicSmemBytes = (size_t)kTopkWarps * cap * 8;
+    cfg.blockDim = dim3(topk_threads(fine));
+    cfg.dynamicSmemBytes = (size_t)topk_threads(fine) / 32 * cap * 8;
     cfg.stream = st;
     attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.x = cluster;
@@ -1440,24 +1440,30 @@ struct TopkLaunch {
   }
 };
 
+template <bool FINE>
+bool topk_max_cluster(uint32_t* most) {
+  if (cudaFuncSetAttribute(k_topk<FINE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           topk_threads(FINE) / 32 * (int)topk_cap(FINE) * 8) != cudaSuccess ||
+      cudaFuncSetAttribute(k_topk<FINE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+    return false;
+  for (uint32_t c = kTopkMaxCluster; c >= 1; c /= 2) {
+    const TopkLaunch l(FINE, c, topk_cap(FINE), nullptr);
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, k_topk<FINE>, &l.cfg) == cudaSuccess && clusters > 0) {
+      *most = c;
+      return true;
+    }
+    cudaGetLastError();
+  }
+  return false;
+}
+
 // Once per device, with that device current.
 int topk_setup(int dev, const TopkDevice** out) {
   std::lock_guard<std::mutex> lock(g_topk_mu);
   TopkDevice& d = g_topk_dev[dev];
   if (!d.ready) {
-    if (cudaFuncSetAttribute(k_topk, cudaFuncAttributeMaxDynamicSharedMemorySize, kTopkWarps * (int)kTopkCap * 8) != cudaSuccess ||
-        cudaFuncSetAttribute(k_topk, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
-      return DGS_ECUDA;
-    for (uint32_t c = kTopkMaxCluster; c >= 1; c /= 2) {
-      const TopkLaunch l(c, kTopkCap, nullptr);
-      int clusters = 0;
-      if (cudaOccupancyMaxActiveClusters(&clusters, k_topk, &l.cfg) == cudaSuccess && clusters > 0) {
-        d.max_cluster = c;
-        break;
-      }
-      cudaGetLastError();
-    }
-    if (d.max_cluster == 0) return DGS_ECUDA;
+    if (!topk_max_cluster<false>(&d.max_cluster[0]) || !topk_max_cluster<true>(&d.max_cluster[1])) return DGS_ECUDA;
     d.ready = true;
   }
   *out = &d;
@@ -1475,16 +1481,20 @@ extern "C" int dgs_topk_encode_static(const float* x, uint32_t n, uint32_t k, ui
   const TopkDevice* d = nullptr;
   const int rc = topk_setup(dev, &d);
   if (rc != DGS_OK) return rc;
+  const bool fine = n <= kTopkFine;
   // An element a thread, up to the largest cluster: the barriers of 16 CTAs cost no more than those of 2 (16384
   // elements: 12.3 us with 16, 13.0 with 4, 14.3 with 1; 262144: 14.3, 21.7, 45).
+  const uint32_t warps = (uint32_t)topk_threads(fine) / 32;
   uint32_t cluster = 1;
-  while (cluster < d->max_cluster && cluster * (uint32_t)kTopkThreads < n) cluster *= 2;
+  while (cluster < d->max_cluster[fine] && cluster * warps * 32 < n) cluster *= 2;
   // the lists hold a warp's whole slice where that fits (slices as k_topk cuts them)
-  const uint32_t unit = n >= cluster * kTopkWarps * 512u ? 512u : 32u;
-  const uint32_t slice = ((n + unit - 1) / unit + cluster * kTopkWarps - 1) / (cluster * kTopkWarps) * unit;
-  const uint32_t cap = std::min(kTopkCap, slice);
-  const TopkLaunch l(cluster, cap, static_cast<cudaStream_t>(stream));
-  return cudaLaunchKernelEx(&l.cfg, k_topk, x, n, k, out_idx, out_val, cap) == cudaSuccess ? DGS_OK : DGS_ECUDA;
+  const uint32_t unit = n >= cluster * warps * 512u ? 512u : 32u;
+  const uint32_t slice = ((n + unit - 1) / unit + cluster * warps - 1) / (cluster * warps) * unit;
+  const uint32_t cap = std::min(topk_cap(fine), slice);
+  const TopkLaunch l(fine, cluster, cap, static_cast<cudaStream_t>(stream));
+  const cudaError_t e = fine ? cudaLaunchKernelEx(&l.cfg, k_topk<true>, x, n, k, out_idx, out_val, cap)
+                             : cudaLaunchKernelEx(&l.cfg, k_topk<false>, x, n, k, out_idx, out_val, cap);
+  return e == cudaSuccess ? DGS_OK : DGS_ECUDA;
 }
 
 extern "C" int dgs_topk_encode_static_status(void* stream, int* device_status) {

@@ -4,17 +4,18 @@
 // barrier of the cluster, and their histograms are added up in the shared memory of the first of them.  What bounds it
 // is the chain of those meetings, not the bytes (4 MB at the most, read once or twice).
 // Measured against the copy, histogram pass, pick, stream pass and cooperative finalize it stands for: 65536 elements,
-// 0.1 %: 12.3 us for 41.7; 1000003 elements, 5 %: 26.2 us for 49.2 (reading and listing is half of that).
+// 0.1 %: 10.3 us for 41.7; 1000003 elements, 5 %: 24.1 us for 49.2 (reading and listing is half of that).
 //   sample      every CTA takes the same sample of at most kTopkSample elements, evenly spaced over the vector, and
 //               from it a bound L that very likely admits at least k elements and not many more.  No meeting: all
 //               CTAs find the same bound.
 //   list        every warp reads a slice of the vector and lists the elements whose key is at least L, in index order,
-//               in shared memory; their top 11 key bits are counted.
-//   levels      three radix levels (11 + 10 + 10 key bits) over the lists give the k-th largest key T and the number r
-//               of entries equal to T that still fit.
+//               in shared memory; they are counted in fine bins above L (bin_of).
+//   exact       the few elements of the k-th's bin go to the first CTA, which compares each with all the others: the k-th
+//               largest key T and the number r of entries equal to T that still fit.
 //   emit        counts of (key > T, key == T) per warp, prefix sums over warps and CTAs, packet in index order.
-// If the lists hold fewer than k elements, or one of them overflows (the sample said nothing about the vector, or most
-// of it is equal), the levels and the emit visit the slices themselves instead.  The result never depends on the sample.
+// If the bin holds too many elements, three radix levels (11 + 10 + 10 key bits) take the place of the last step; if the
+// lists hold fewer than k elements, or one of them overflows (the sample said nothing about the vector, or most of it is
+// equal), the levels and the emit visit the slices themselves instead.  The result never depends on the sample.
 #pragma once
 #include <cooperative_groups.h>
 
@@ -24,11 +25,18 @@
 
 namespace dgs {
 
-constexpr int kTopkThreads = 1024, kTopkWarps = kTopkThreads / 32;
+// Two variants.  Short vectors take 512 threads a CTA and fine bins with one exact step; the barriers of fewer warps are
+// shorter (65536 elements, 0.1 %: 10.3 us, 11.6 us with 1024 threads).  Long ones take 1024 threads, which list faster, and
+// three radix levels, since a bin of many candidates holds too many to compare (1000003 elements, 5 %: 24.1 us; 28.0 us
+// with 512 threads).
+constexpr uint32_t kTopkFine = 1u << 18;   // longest vector that takes the first
+__host__ __device__ constexpr int topk_threads(bool fine) { return fine ? 512 : 1024; }
 constexpr uint32_t kTopkMaxCluster = 16;   // (more than 8 is not portable to every GPU: the launch asks for it)
 constexpr int kBins2 = 1024;               // levels 2 and 3 (level 1: kBins1, the top 11 key bits)
-constexpr uint32_t kTopkSample = kTopkThreads;   // one element a thread
-constexpr uint32_t kTopkCap = 736;         // most elements a warp can list: 184 KB of lists per CTA
+constexpr uint32_t kTopkSample = 1024;
+constexpr uint32_t kTopkShort = 512;       // most elements in the k-th's bin that are ranked by comparing them
+// most elements a warp can list: 184 KB of lists per CTA
+__host__ __device__ constexpr uint32_t topk_cap(bool fine) { return 736u * 1024u / topk_threads(fine); }
 constexpr int kStatusRank = -1002;         // an entry got a rank that cannot be
 
 // Outcome of the last call's kernel on the device: 0, or a negative word if its packet is not complete.
@@ -38,18 +46,21 @@ struct TopkShared {
   uint32_t hist[kBins1];                     // this CTA's counts of the level in hand
   uint32_t sum1[kBins1], again1[kBins1];     // first CTA of the cluster: counts of all CTAs, level 1 (lists; slices)
   uint32_t sum2[kBins2], sum3[kBins2];       //                                               levels 2 and 3
-  uint32_t warp_sum[kTopkWarps];
-  uint2 warp_tot[kTopkWarps];                // (key > T, key == T) of each warp
+  uint32_t warp_sum[32];
+  uint2 warp_tot[32];                        // (key > T, key == T) of each warp
   uint2 cta_tot[kTopkMaxCluster];            // of each CTA of the cluster
   uint32_t overflow;                         // first CTA: some list was too short
-  uint32_t res[2];                           // of this CTA's own pick
-  uint4 told;                                // what the first CTA's pick found: bin, entries needed of it, total, overflow
+  uint32_t short_cnt, short_at;              // elements of this CTA in the k-th's bin; where they go
+  uint32_t short_all;                        // first CTA: of all CTAs
+  uint32_t res[3];                           // of this CTA's own pick
+  uint4 told;                                // what the first CTA found: bin, entries needed of it, total (0: a list
+                                             // was too short), entries in it; in the end T and r
 };
 
 // From a histogram of B bins in shared memory, counting from the top bin down, the bin that
 // holds the k-th entry and how many entries of that bin are needed.  Returns the total count; bin and need are valid
 // if it is at least k.  The same for every thread of the CTA.
-template <int B>
+template <int B, int kTopkThreads>
 __device__ uint32_t topk_pick(const uint32_t* hist, uint32_t k, uint32_t& bin, uint32_t& need, TopkShared& sh) {
   constexpr int PER = B / kTopkThreads;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -67,7 +78,7 @@ __device__ uint32_t topk_pick(const uint32_t* hist, uint32_t k, uint32_t& bin, u
   }
   if (lane == 31) sh.warp_sum[warp] = incl;
   __syncthreads();
-  const uint32_t w = sh.warp_sum[lane];       // as many warps as lanes
+  const uint32_t w = lane < kTopkThreads / 32 ? sh.warp_sum[lane] : 0u;
   uint32_t winc = w;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
@@ -81,6 +92,7 @@ __device__ uint32_t topk_pick(const uint32_t* hist, uint32_t k, uint32_t& bin, u
     if (above < k && k <= above + c[j]) {
       sh.res[0] = B - 1 - threadIdx.x * PER - j;
       sh.res[1] = k - above;
+      sh.res[2] = c[j];
     }
     above += c[j];
   }
@@ -90,9 +102,12 @@ __device__ uint32_t topk_pick(const uint32_t* hist, uint32_t k, uint32_t& bin, u
   return total;
 }
 
-__global__ void __launch_bounds__(kTopkThreads, 1) k_topk(const float* __restrict__ x, uint32_t n, uint32_t k,
+template <bool FINE>
+__global__ void __launch_bounds__(topk_threads(FINE), 1) k_topk(const float* __restrict__ x, uint32_t n, uint32_t k,
                                                          uint32_t* __restrict__ out_idx, float* __restrict__ out_val,
                                                          uint32_t cap) {
+  constexpr int kTopkThreads = topk_threads(FINE);
+  constexpr uint32_t kTopkWarps = kTopkThreads / 32;
   extern __shared__ __align__(16) unsigned char topk_dyn[];
   __shared__ TopkShared sh;
   namespace cg = cooperative_groups;
@@ -105,9 +120,10 @@ __global__ void __launch_bounds__(kTopkThreads, 1) k_topk(const float* __restric
     sh.hist[b] = 0;
     if (cta == 0) sh.sum1[b] = sh.again1[b] = 0;
   }
-  if (cta == 0) sh.sum2[tid] = sh.sum3[tid] = 0;
+  if (cta == 0)
+    for (uint32_t b = tid; b < (uint32_t)kBins2; b += kTopkThreads) sh.sum2[b] = sh.sum3[b] = 0;
   if (tid == 0) {
-    sh.overflow = 0;
+    sh.overflow = sh.short_cnt = sh.short_all = 0;
     if (cta == 0) g_topk_status = 0;
   }
   __syncthreads();
@@ -122,7 +138,8 @@ __global__ void __launch_bounds__(kTopkThreads, 1) k_topk(const float* __restric
   uint32_t L = 0;
   {
     const uint32_t s = min(n, kTopkSample);
-    if (tid < s) atomicAdd(sh.hist + (key_of(__ldg(x + (uint32_t)((uint64_t)tid * n / s))) >> 20), 1u);
+    for (uint32_t q = tid; q < s; q += kTopkThreads)
+      atomicAdd(sh.hist + (key_of(__ldg(x + (uint32_t)((uint64_t)q * n / s))) >> 20), 1u);
     __syncthreads();
     // Of k in n, k s / n are expected in the sample; four standard deviations and a few more, so that at least k
     // elements lie above the bound all but surely.  A sample of everything needs no margin.
@@ -132,7 +149,7 @@ __global__ void __launch_bounds__(kTopkThreads, 1) k_topk(const float* __restric
       want = (uint32_t)(mean + 4.f * sqrtf(mean)) + 8u;
     }
     uint32_t bin, need;
-    if (topk_pick<kBins1>(sh.hist, want, bin, need, sh) >= want) L = bin << 20;
+    if (topk_pick<kBins1, kTopkThreads>(sh.hist, want, bin, need, sh) >= want) L = bin << 20;
     for (uint32_t b = tid; b < (uint32_t)kBins1; b += kTopkThreads) sh.hist[b] = 0;
     __syncthreads();
   }
@@ -144,10 +161,17 @@ __global__ void __launch_bounds__(kTopkThreads, 1) k_topk(const float* __restric
   if ((reinterpret_cast<uintptr_t>(x) & 15u) == 0) {
     // 512 elements at a time, 16 bytes a lane: lane order is element order inside each of the four pieces of 128, so
     // four counts of a lane travel as four bytes through one prefix sum over the lanes
-    for (; from + 512u <= i1; from += 512u) {
-      float4 v[4];
+    // (the next tile is on its way while this one is listed)
+    float4 v[4], next[4];
+    auto load = [&](uint32_t at) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) v[j] = __ldg(reinterpret_cast<const float4*>(x + from) + j * 32 + lane);
+      for (int j = 0; j < 4; ++j) next[j] = __ldg(reinterpret_cast<const float4*>(x + at) + j * 32 + lane);
+    };
+    if (from + 512u <= i1) load(from);
+    for (; from + 512u <= i1; from += 512u) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[j] = next[j];
+      if (from + 1024u <= i1) load(from + 512u);
       uint32_t mask = 0, packed = 0;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -204,7 +228,7 @@ __global__ void __launch_bounds__(kTopkThreads, 1) k_topk(const float* __restric
   // counted from the list, where the lanes are full: counting while listing is an atomic per one or two elements
   for (uint32_t p = lane; p - lane < min(listed, cap); p += 32) {
     const bool valid = p < min(listed, cap);
-    hist_add(sh.hist, valid ? key_of(my_val[p]) >> 20 : 0u, valid, (int)lane);
+    hist_add(sh.hist, !valid ? 0u : FINE ? bin_of(key_of(my_val[p]), L) : key_of(my_val[p]) >> 20, valid, (int)lane);
   }
   __syncthreads();
   cl.barrier_wait();
@@ -224,8 +248,8 @@ __global__ void __launch_bounds__(kTopkThreads, 1) k_topk(const float* __restric
     cl.sync();
     if (cta == 0) {
       uint32_t fb, fn;
-      const uint32_t total = topk_pick<B>(sum, k_left, fb, fn, sh);
-      if (tid < C) cl.map_shared_rank(&sh, tid)->told = make_uint4(fb, fn, total, sh.overflow);
+      const uint32_t total = topk_pick<B, kTopkThreads>(sum, k_left, fb, fn, sh);
+      if (tid < C) cl.map_shared_rank(&sh, tid)->told = make_uint4(fb, fn, sh.overflow ? 0u : total, sh.res[2]);
     }
     cl.sync();
     const uint4 t = sh.told;
@@ -237,7 +261,7 @@ __global__ void __launch_bounds__(kTopkThreads, 1) k_topk(const float* __restric
   using Bins2 = std::integral_constant<int, kBins2>;
   uint32_t bin, need;
   const uint2 found = pick(sh.sum1, Bins1(), k, bin, need);
-  const bool slices = found.y != 0 || found.x < k;   // the same in the whole cluster
+  const bool slices = found.x < k;   // the same in the whole cluster
 
   // visits this warp's elements in index order, 32 at a time: fn(valid, index, value)
   auto each = [&](auto fn) {
@@ -253,24 +277,64 @@ __global__ void __launch_bounds__(kTopkThreads, 1) k_topk(const float* __restric
       }
     }
   };
-  if (slices) {
-    each([&](bool valid, uint32_t, float v) { hist_add(sh.hist, key_of(v) >> 20, valid, (int)lane); });
-    __syncthreads();
-    pick(sh.again1, Bins1(), k, bin, need);
-  }
-  uint32_t prefix = bin;
-#pragma unroll 1
-  for (int level = 2; level <= 3; ++level) {
-    const int shift = level == 2 ? 10 : 0;
+  uint32_t T, r;
+  if (FINE && !slices && found.y <= kTopkShort) {
+    // The elements of the k-th's bin go to the first CTA, which compares each with all the others.
+    uint32_t* const mine = sh.hist;
     each([&](bool valid, uint32_t, float v) {
       const uint32_t key = key_of(v);
-      if (valid && (key >> (shift + 10)) == prefix) atomicAdd(sh.hist + ((key >> shift) & 1023u), 1u);
+      if (valid && bin_of(key, L) == bin) mine[atomicAdd(&sh.short_cnt, 1u)] = key;
     });
     __syncthreads();
-    pick(level == 2 ? sh.sum2 : sh.sum3, Bins2(), need, bin, need);
-    prefix = (prefix << 10) | bin;
+    TopkShared* const head = cl.map_shared_rank(&sh, 0);
+    const uint32_t count = sh.short_cnt;
+    if (tid == 0) sh.short_at = atomicAdd(&head->short_all, count);
+    __syncthreads();
+    for (uint32_t q = tid; q < count; q += kTopkThreads) head->sum1[sh.short_at + q] = mine[q];
+    cl.sync();
+    if (cta == 0) {
+      for (uint32_t q = tid; q < found.y; q += kTopkThreads) {
+        const uint32_t key = sh.sum1[q];
+        uint32_t above = 0, same = 0;
+#pragma unroll 4
+        for (uint32_t o = 0; o < found.y; ++o) {
+          const uint32_t other = sh.sum1[o];
+          above += other > key ? 1u : 0u;
+          same += other == key ? 1u : 0u;
+        }
+        if (above < need && need <= above + same) {   // (the same for all that are equal)
+          sh.res[0] = key;
+          sh.res[1] = need - above;
+        }
+      }
+      __syncthreads();
+      if (tid < C) cl.map_shared_rank(&sh, tid)->told = make_uint4(sh.res[0], sh.res[1], 0, 0);
+    }
+    cl.sync();
+    T = sh.told.x;
+    r = sh.told.y;
+  } else {
+    // three radix levels (11 + 10 + 10 key bits) over the lists, or over the slices themselves
+    if (FINE || slices) {
+      each([&](bool valid, uint32_t, float v) { hist_add(sh.hist, key_of(v) >> 20, valid, (int)lane); });
+      __syncthreads();
+      pick(sh.again1, Bins1(), k, bin, need);
+    }
+    uint32_t prefix = bin;
+#pragma unroll 1
+    for (int level = 2; level <= 3; ++level) {
+      const int shift = level == 2 ? 10 : 0;
+      each([&](bool valid, uint32_t, float v) {
+        const uint32_t key = key_of(v);
+        if (valid && (key >> (shift + 10)) == prefix) atomicAdd(sh.hist + ((key >> shift) & 1023u), 1u);
+      });
+      __syncthreads();
+      pick(level == 2 ? sh.sum2 : sh.sum3, Bins2(), need, bin, need);
+      prefix = (prefix << 10) | bin;
+    }
+    T = prefix;
+    r = need;
   }
-  const uint32_t T = prefix, r = need;
 
   // how many of either kind each warp has, and the warps and CTAs before it
   uint32_t gt = 0, eq = 0;
@@ -281,7 +345,7 @@ __global__ void __launch_bounds__(kTopkThreads, 1) k_topk(const float* __restric
   });
   if (lane == 0) sh.warp_tot[warp] = make_uint2(gt, eq);
   __syncthreads();
-  const uint2 q = sh.warp_tot[lane];
+  const uint2 q = lane < kTopkWarps ? sh.warp_tot[lane] : make_uint2(0, 0);
   uint32_t gt_before = __reduce_add_sync(kFull, lane < warp ? q.x : 0u), eq_before = __reduce_add_sync(kFull, lane < warp ? q.y : 0u);
   const uint32_t gt_all = __reduce_add_sync(kFull, q.x), eq_all = __reduce_add_sync(kFull, q.y);
   if (tid < C) cl.map_shared_rank(&sh, tid)->cta_tot[cta] = make_uint2(gt_all, eq_all);

@@ -29,7 +29,7 @@ def vector(kind: str, n: int) -> np.ndarray:
     return x
 
 
-@pytest.mark.parametrize("n", [1, 31, 33, 4096, 4097, 65_535, 131_073, (1 << 20) - 1, 1 << 20])
+@pytest.mark.parametrize("n", [1, 31, 33, 4096, 4097, 65_535, 131_073, 1 << 18, (1 << 18) + 1, (1 << 20) - 1, 1 << 20])
 @pytest.mark.parametrize("kind", ["normal", "equal", "two", "few", "hidden", "corner"])
 def test_static_selection_edges(n, kind):
     x = vector(kind, n)
