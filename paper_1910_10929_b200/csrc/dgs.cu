@@ -936,7 +936,8 @@ int apply_impl(dgs_ctx* c, uint32_t worker, const dgs_packet* pkt) {
   const int stream_id = own ? c->slot_stream[slot] : peek_stream(c);   // after its push; else where a pull comes next
   const uint32_t gx = (pkt->count + kThreads - 1) / kThreads;
   int rc = DGS_OK;
-  if (pkt->count > 0 && !own) rc = fork_from_user(c, stream_id);
+  // theta and the D_q that are caught up may be what the caller's stream is still reading (nothing to do inside an event)
+  if (pkt->count > 0) rc = fork_from_user(c, stream_id);
   if (rc != DGS_OK) return rc;
   if (pkt->count == 0) {
     // nothing to subtract
@@ -1216,7 +1217,9 @@ int dgs_state_ptr(dgs_ctx* c, int which, uint32_t worker, const float** out) {
   switch (which) {
     case DGS_THETA: *out = c->at<float>(c->lay.theta); break;
     case DGS_D:
-      rc = catch_up_now(c, worker, 0);
+      rc = begin_call(c);
+      if (rc == DGS_OK) rc = fork_from_user(c, 0);   // the caller's stream may still be reading the vector as it is
+      if (rc == DGS_OK) rc = catch_up_now(c, worker, 0);
       if (rc != DGS_OK) return rc;
       *out = c->D_buf(worker);
       break;

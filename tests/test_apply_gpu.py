@@ -57,3 +57,31 @@ def test_a_packet_that_does_not_ascend_is_reported():
     val = torch.ones(3, device=DEV)
     ctx.server_apply(0, dgs.dgs_packet(idx.data_ptr(), val.data_ptr(), 3))
     assert ctx.status() != 0
+
+
+def test_an_own_packet_waits_for_the_callers_stream():
+    """The caller's stream reads theta and a difference late; an apply of the library's own packet, and the catch-up of
+    a difference that it or state() needs, must not be seen there."""
+    n, workers = 50_000, 2
+    wl = W.custom("late", [n], workers, 1, 5_000, grad_kind="normal")
+    ctx = dgs.Context.from_workload(wl, theta0=torch.from_numpy(wl.theta0()).to(DEV))
+    g = torch.from_numpy(wl.gradient(0)).to(DEV)
+    theta, D1 = ctx.state(dgs.DGS_THETA), ctx.state(dgs.DGS_D, 1)
+    ring = 40                                    # more packets than the log holds: worker 1's difference is caught up
+    for _ in range(ring):
+        pkt = ctx.worker_push(0, g)
+        ctx.flush()
+        torch.cuda.synchronize()
+        before = theta.clone(), D1.clone()
+        torch.cuda._sleep(200_000)
+        late = theta.clone(), D1.clone()
+        ctx.server_apply(0, pkt)
+        ctx.flush()
+        assert torch.equal(late[0], before[0]) and torch.equal(late[1], before[1])
+        assert not torch.equal(theta, before[0])
+    before = D1.clone()
+    torch.cuda._sleep(200_000)
+    late = D1.clone()
+    ctx.state(dgs.DGS_D, 1)
+    assert torch.equal(late, before) and not torch.equal(D1, before)
+    assert ctx.status() == 0
