@@ -2373,8 +2373,9 @@ __global__ void __maxnreg__(72) k_fold(const __grid_constant__ Workspace ws, con
   }
 }
 
-// Eager form, for a packet that is too long for the log (any count): buffer q < N is D_q, buffer N is theta.  Indices of one packet are distinct, so every
-// (buffer, entry) pair is touched by exactly one thread: plain load / subtract / store.
+// Eager form, for a packet that is too long for the log (any count): buffer q < N is D_q, buffer N is theta.  Indices of
+// one packet ascend, so every (buffer, entry) pair is touched by exactly one thread: plain load / subtract / store.  A
+// packet that does not ascend is reported.
 __global__ void __launch_bounds__(kThreads) k_scatter_sub(const uint32_t* __restrict__ idx,
                                                           const float* __restrict__ val, uint32_t count,
                                                           float* __restrict__ theta, float* __restrict__ D,
@@ -2385,11 +2386,9 @@ __global__ void __launch_bounds__(kThreads) k_scatter_sub(const uint32_t* __rest
   if (j >= count) return;
   const uint32_t i = idx[j];
   const float v = val[j];
-  if (i >= n) {
-    atomicMin(status, -2000);
-    return;
-  }
   const uint32_t q = blockIdx.y;
+  if (q == 0 && (i >= n || (j + 1 < count && idx[j + 1] <= i))) atomicMin(status, -2000);   // out of range, or not ascending
+  if (i >= n) return;
   float* p = (q == num_workers ? theta : D + (uint64_t)q * d_stride) + i;
   const float r = __fsub_rn(*p, v);
   *p = r;

@@ -59,6 +59,25 @@ def test_a_packet_that_does_not_ascend_is_reported():
     assert ctx.status() != 0
 
 
+@pytest.mark.parametrize("count", [3, 64, 65, 1_000])          # the library files packets of up to 64 entries here
+@pytest.mark.parametrize("fault", ["none", "duplicate", "descending", "beyond"])
+def test_faulty_packets_of_any_length_are_reported(count, fault):
+    n = 5_000
+    ctx = dgs.Context(n, 2, 0.1, 0.9, [0], [n], [10], [10], torch.zeros(n, device=DEV))
+    idx = np.arange(count, dtype=np.int64) * 4
+    at = count - 2                                               # the last pair, which may open a CTA's share
+    if fault == "duplicate":
+        idx[at + 1] = idx[at]
+    elif fault == "descending":
+        idx[at + 1] = idx[at] - 1
+    elif fault == "beyond":
+        idx[at + 1] = n
+    pair = torch.from_numpy(idx.astype(np.int32)).to(DEV), torch.ones(count, device=DEV)
+    ctx.server_apply(0, dgs.dgs_packet(pair[0].data_ptr(), pair[1].data_ptr(), count))
+    ctx.worker_pull(0)
+    assert (ctx.status() != 0) == (fault != "none")
+
+
 def test_an_own_packet_waits_for_the_callers_stream():
     """The caller's stream reads theta and a difference late; an apply of the library's own packet, and the catch-up of
     a difference that it or state() needs, must not be seen there."""
