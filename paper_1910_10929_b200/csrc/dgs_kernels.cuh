@@ -1450,7 +1450,9 @@ __global__ void __maxnreg__(64) k_finalize(const __grid_constant__ Workspace ws,
       }
     }
     __syncthreads();
-    // candidates above the k-th's bin are counted, those in it go to the layer's list
+    // Candidates above the k-th's bin are counted, those in it go to the layer's list.  (There are `pop` of them, the list's
+    // place holds that many.  Only where an earlier barrier gave up, and left its counts behind, does the list begin later:
+    // the bound keeps it in its place.)
     uint32_t hits = 0;
     count([&](int u, const LayerPick* t, bool valid, bool&) {
       const uint32_t b = bin_of(key_of(raw[u]), t->L), bin = t->bin;
@@ -1462,12 +1464,13 @@ __global__ void __maxnreg__(64) k_finalize(const __grid_constant__ Workspace ws,
 #pragma unroll
         for (int u = 0; u < kKeep; ++u) n += __popc(__ballot_sync(kFull, (hits >> u) & 1u));
         if (n) {
-          if (lane == 0) at = sh.tab[0].list_off + atomicAdd(ws.list_cnt, n);
+          if (lane == 0) at = atomicAdd(ws.list_cnt, n);
           at = __shfl_sync(kFull, at, 0);
+          uint2* const list = ws.list + sh.tab[0].list_off;
 #pragma unroll
           for (int u = 0; u < kKeep; ++u) {
-            const uint32_t m = __ballot_sync(kFull, (hits >> u) & 1u);
-            if ((hits >> u) & 1u) ws.list[at + __popc(m & lt)] = make_uint2(key_of(raw[u]), base + u * 32u + lane);
+            const uint32_t m = __ballot_sync(kFull, (hits >> u) & 1u), to = at + __popc(m & lt);
+            if (((hits >> u) & 1u) && to < sh.tab[0].pop) list[to] = make_uint2(key_of(raw[u]), base + u * 32u + lane);
             at += __popc(m);
           }
           hits = 0;
@@ -1488,12 +1491,13 @@ __global__ void __maxnreg__(64) k_finalize(const __grid_constant__ Workspace ws,
             mine |= in ? 1u << u : 0u;
             n += __popc(__ballot_sync(kFull, in));
           }
-          if (lane == 0) at = t->list_off + atomicAdd(ws.list_cnt + s_lo + near_t, n);
+          if (lane == 0) at = atomicAdd(ws.list_cnt + s_lo + near_t, n);
           at = __shfl_sync(kFull, at, 0);
+          uint2* const list = ws.list + t->list_off;
 #pragma unroll
           for (int u = 0; u < kKeep; ++u) {
-            const uint32_t m = __ballot_sync(kFull, (mine >> u) & 1u);
-            if ((mine >> u) & 1u) ws.list[at + __popc(m & lt)] = make_uint2(key_of(raw[u]), base + u * 32u + lane);
+            const uint32_t m = __ballot_sync(kFull, (mine >> u) & 1u), to = at + __popc(m & lt);
+            if (((mine >> u) & 1u) && to < t->pop) list[to] = make_uint2(key_of(raw[u]), base + u * 32u + lane);
             at += __popc(m);
           }
           hits &= ~mine;

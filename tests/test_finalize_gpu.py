@@ -45,3 +45,18 @@ def test_finalize_edges(sizes, ppm, kind):
         x[want] = 0.0
         assert np.array_equal(left, x), turn
     assert ctx.status() == 0
+
+
+def test_barriers_that_give_up_again_and_again():
+    """A selection whose barrier gave up leaves its counts behind: the lists of the later ones stay in their places, and
+    the arena beside them as it was."""
+    sizes = [40_000, 300, 513]
+    off = np.concatenate([[0], np.cumsum(sizes)[:-1]])
+    n, ks = sum(sizes), [400, 3, 5]
+    theta0 = torch.randn(n, device=DEV)
+    ctx = dgs.Context(n, 1, 0.1, 0.9, off, sizes, ks, ks, theta0, flags=dgs.DGS_TEST_STALLED_BARRIER | dgs.DGS_NO_SPECULATION)
+    for turn in range(60):       # every turn has its own k-th, so that every list is another bin's
+        g = torch.from_numpy(values("normal", n) * np.float32(1.3 ** (turn % 20))).to(DEV)
+        ctx.worker_push(0, g)
+        assert ctx.status() == dgs.DGS_ETIMEOUT
+    assert torch.equal(ctx.state(dgs.DGS_THETA), theta0)
