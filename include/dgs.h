@@ -210,7 +210,8 @@ int dgs_state_ptr(dgs_ctx* ctx, int which, uint32_t worker, const float** out);
 
 /* Overwrites a state vector from src (DEVICE f32[n]) on the stream: restores a
  * checkpoint, or loads a vector to be selected from with dgs_worker_pull.  The copy runs on the stream
- * given at dgs_init, after the work in flight on that vector; only DGS_U waits on the host. */
+ * given at dgs_init, after the work in flight on that vector; only DGS_U waits on the host.  src may be a state
+ * vector of the context itself: the copy then comes after all work in flight. */
 int dgs_state_load(dgs_ctx* ctx, int which, uint32_t worker, const float* src);
 
 /* Waits for all work in flight and returns the sticky device status word in

@@ -1270,6 +1270,12 @@ int dgs_state_load(dgs_ctx* c, int which, uint32_t worker, const float* src) {
       break;
     default: return DGS_EINVAL;
   }
+  // A vector of the library's own (the model into a worker's copy, say): events in flight may still be writing it.
+  const char* const s = reinterpret_cast<const char*>(src);
+  if (s >= c->base && s < c->base + c->lay.total) {
+    rc = dgs_flush(c);
+    if (rc != DGS_OK) return rc;
+  }
   rc = task_begin(c, t);
   if (rc != DGS_OK) return rc;
   DGS_CUDA(c, cudaMemcpyAsync(const_cast<float*>(dst), src, c->cfg.n * 4, cudaMemcpyDeviceToDevice, c->user));

@@ -39,3 +39,31 @@ def test_loads_between_events_in_flight(workers):
             ctypes.memmove(orc.state(cpu, q).ctypes.data, x.ctypes.data, x.nbytes)   # (the view is read-only)
     assert ctx.status() == 0
     compare_state(ctx, orc, workers, True)
+
+
+def test_loads_from_the_librarys_own_vectors():
+    """The model copied into a worker's local model, or another worker's, while events that change them are in flight."""
+    n, workers = 400_000, 6
+    wl = W.custom("own", [n], workers, 1, 5_000, grad_kind="normal")
+    theta0 = wl.theta0()
+    orc = oracle.Oracle.from_workload(wl, theta0=theta0, keep_local=True)
+    ctx = dgs.Context.from_workload(wl, theta0=torch.from_numpy(theta0).to(DEV), flags=dgs.DGS_KEEP_LOCAL_MODEL)
+    theta, local = ctx.state(dgs.DGS_THETA), [ctx.state(dgs.DGS_THETA_LOCAL, q) for q in range(workers)]
+    grads = []
+    for e in range(60):
+        g = np.random.default_rng(e).standard_normal(n, dtype=np.float32)
+        grads.append((g, torch.from_numpy(g).to(DEV)))
+    torch.cuda.synchronize()
+    for e, (g, gd) in enumerate(grads):
+        w = e % workers
+        ctx.event(w, gd)
+        orc.event(w, g)
+        if e % 4 == 3:
+            q = (e // 4) % workers
+            from_model = (e // 4) % 2 == 0
+            ctx.state_load(dgs.DGS_THETA_LOCAL, q, theta if from_model else local[w])
+            src = orc.state(oracle.THETA, 0) if from_model else orc.state(oracle.THETA_LOCAL, w)
+            src = src.copy()
+            ctypes.memmove(orc.state(oracle.THETA_LOCAL, q).ctypes.data, src.ctypes.data, src.nbytes)
+    assert ctx.status() == 0
+    compare_state(ctx, orc, workers, True)
