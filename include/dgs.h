@@ -198,7 +198,7 @@ int dgs_flush(dgs_ctx* ctx);
 /* The same event with HOST buffers (needs DGS_HOST_IO): copies grad (HOST f32[n],
  * ideally pinned) to the device, runs the event, copies the pull packet back into
  * out_idx / out_val (HOST, sum(k_pull) entries each, may be NULL to skip) and
- * waits for that work.  This is the end-to-end path: what a worker process
+ * waits for that work and for what earlier calls had enqueued.  This is the end-to-end path: what a worker process
  * without its own device buffers would call. */
 int dgs_event_host(dgs_ctx* ctx, uint32_t worker, const float* grad_host, uint32_t* out_idx, float* out_val);
 

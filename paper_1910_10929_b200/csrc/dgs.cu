@@ -417,12 +417,20 @@ int fork_from_user(dgs_ctx* c, int which) {
   return DGS_OK;
 }
 
-// Waits (on the host) for all internal streams and the caller's stream.
-int sync_all(dgs_ctx* c) {
-  for (int i = 0; i < kStreams; ++i)
-    if (c->st[i]) DGS_CUDA(c, cudaStreamSynchronize(c->st[i]));
-  DGS_CUDA(c, cudaStreamSynchronize(c->user));
+// Waits (on the host) for all internal streams ...
+int sync_library(dgs_ctx* c) {
+  for (int i = 0; i < kStreams; ++i) {
+    if (c->st[i] && c->dirty[i]) DGS_CUDA(c, cudaStreamSynchronize(c->st[i]));
+    c->dirty[i] = false;                     // nothing that the caller's stream would have to wait for
+  }
   c->alone = c->idle = true;
+  return DGS_OK;
+}
+// ... and the caller's stream (which has been made to wait for those that are not dirty).
+int sync_all(dgs_ctx* c) {
+  const int rc = sync_library(c);
+  if (rc != DGS_OK) return rc;
+  DGS_CUDA(c, cudaStreamSynchronize(c->user));
   return DGS_OK;
 }
 
@@ -1201,12 +1209,9 @@ int dgs_event_host(dgs_ctx* c, uint32_t worker, const float* grad_host, uint32_t
   cudaStream_t ps = c->st[stream_id];
   if (out_idx) DGS_CUDA(c, cudaMemcpyAsync(out_idx, g.idx, (uint64_t)g.count * 4, cudaMemcpyDeviceToHost, ps));
   if (out_val) DGS_CUDA(c, cudaMemcpyAsync(out_val, g.val, (uint64_t)g.count * 4, cudaMemcpyDeviceToHost, ps));
-  // push, apply and pull follow one another on this stream; what other calls have enqueued may still be running
-  DGS_CUDA(c, cudaStreamSynchronize(ps));
-  c->alone = c->idle = true;
-  for (int i = 0; i < kStreams; ++i)
-    if (i != stream_id && c->dirty[i]) c->alone = c->idle = false;
-  return DGS_OK;
+  // Push, apply and pull follow one another on this stream; what earlier calls have enqueued is complete as well when
+  // this one returns.
+  return sync_library(c);
 }
 
 int dgs_state_ptr(dgs_ctx* c, int which, uint32_t worker, const float** out) {

@@ -67,3 +67,26 @@ def test_loads_from_the_librarys_own_vectors():
             ctypes.memmove(orc.state(oracle.THETA_LOCAL, q).ctypes.data, src.ctypes.data, src.nbytes)
     assert ctx.status() == 0
     compare_state(ctx, orc, workers, True)
+
+
+def test_event_host_completes_what_was_enqueued_before():
+    """After dgs_event_host the host may read anything, without a join: here the packets of the events before it."""
+    n, workers = 3_000_000, 8
+    wl = W.custom("host", [n], workers, 1, 5_000, grad_kind="normal")
+    orc = oracle.Oracle.from_workload(wl)
+    ctx = dgs.Context.from_workload(wl, flags=dgs.DGS_HOST_IO)
+    g = np.random.default_rng(1).standard_normal(n, dtype=np.float32)
+    gd, gh = torch.from_numpy(g).to(DEV), torch.from_numpy(g).pin_memory()
+    side = torch.cuda.Stream()                       # not the caller's: ordered by the host alone
+    torch.cuda.synchronize()
+    for turn in range(4):
+        pulls = [ctx.event(w, gd)[1] for w in range(1, workers)]
+        ctx.event_host(0, gh)
+        with torch.cuda.stream(side):
+            got = [(ctx._view(p.idx, p.count, torch.int32).cpu().numpy().view(np.uint32),
+                    ctx._view(p.val, p.count, torch.float32).cpu().numpy()) for p in pulls]
+        for w, (gi, gv) in enumerate(got, start=1):
+            wi, wv = orc.event(w, g)[1]
+            assert np.array_equal(gi, wi) and np.array_equal(gv, wv), (turn, w)
+        orc.event(0, g)
+    assert ctx.status() == 0
