@@ -34,9 +34,8 @@
  *     was made.  Results (packets, state) are complete for that stream after dgs_flush,
  *     and for the host after any call that is documented to wait.  One host thread per
  *     context.
- *   - The library's streams are eight at most, and about half as many as there are workers; each
- *     is created when it is first needed, and a caller that calls dgs_flush after every event
- *     uses one.  The CUDA driver maps streams onto a fixed number of hardware queues, 8 unless the
+ *   - The library's streams are eight at most (two for a single worker); each is created when it
+ *     is first needed, and a caller that calls dgs_flush after every event uses one.  The CUDA driver maps streams onto a fixed number of hardware queues, 8 unless the
  *     environment variable CUDA_DEVICE_MAX_CONNECTIONS says otherwise, and streams that
  *     share a queue run one after the other.  The variable is read when the process creates
  *     its CUDA context, so a process that wants the overlap must set it (to 12 or more; 32

@@ -39,12 +39,13 @@ constexpr int kPullSlots = 8;             // pull packet slots
 constexpr int kVarSlots = 4;              // packet slots of the pull without secondary compression
 constexpr int kStreams = 8;               // most events in flight at a time
 constexpr int kSets = kStreams;           // scratch sets and spare velocity buffers: one of each per stream
-// Events in flight at a time: with more than about half of the workers in flight a selection finds no finished one to
-// take its bound from and waits for one that runs (8 workers, 124 M elements, a round of 8: 3.3 ms with 5 streams, 4.5 ms
-// with 7; 32 workers, 25.6 M elements, a round of 32: 2.5 ms with 4, 2.4 with 5, 2.2 with 7).
+// Events in flight at a time: the push of an event runs beside the pulls of the ones before it, those of the same worker
+// included, so even a few workers fill all of the streams.  Microseconds an event in runs of 256 without a join, 2 / 4 / 8
+// streams: 2 workers, 8.4 M elements: 53 / 39 / 36; 4 workers, 25.6 M: 82 / 65 / 57; 32 workers: 87 / 66 / 60.  A single
+// worker's events have one push and one pull at a time to overlap: 236 with two streams, 236 to 245 with more, 267 with one.
 int streams_for(const dgs_config* c) {
   if (c->flags & DGS_SINGLE_STREAM) return 1;   // kernels run one after the other, in call order
-  return (int)std::min<uint32_t>(kStreams, c->num_workers / 2 + 1);
+  return c->num_workers == 1 ? 2 : kStreams;
 }
 constexpr int kCaller = kStreams;         // the caller's stream, where the tracker names streams by number
 constexpr int kQueuesWanted = 12;         // hardware queues that keep the streams of two contexts and the caller's apart
@@ -219,7 +220,7 @@ void make_layout(const dgs_config* c, Layout* L) {
   L->log_sum = take((uint64_t)(L->log_ring + 1) * L->sum_stride * 4);
   L->blk_stride = align_up((c->n + kWarpTile - 1) / kWarpTile, 64);
   L->blk_max = take(N * L->blk_stride * 4);
-  L->L_next = take(2 * N * S * 4);
+  L->L_next = take(4 * N * S * 4);
   L->slack = take(2 * S * 4);
   L->u_slots = take((N + kSets) * sizeof(float*));
   L->status = take(4);
@@ -282,11 +283,15 @@ struct dgs_ctx {
   int finalize_max[3];   // most CTAs of the cooperative finalize kernel that can be resident at once, per mode
   uint64_t kind_seq[2];  // selections of each kind launched so far
   // Carried bounds: row (kind, worker) of L_next holds the bounds suggested by that worker's
-  // latest selection of that kind ([0] push, [1] pull).  row_age says in which state it was
+  // latest selection of that kind ([0] push, [1] pull).  There are two copies of a row, written in turn
+  // (row_copy: the latest): the worker's next selection need not wait until nobody reads the bounds of its
+  // last one.  With one copy, and one stream less than workers that arrive in turn, every selection read
+  // the row of the worker that came next, and no two events overlapped (8 workers, 2^20 elements: 34 us an event
+  // with 7 streams, 17 us with 6 or 8).  row_age says in which state it was
   // made: pushes the worker had done before (push), packets accumulated in D_w since its
   // previous pull (pull).  Thresholds grow with that age, so a row made at an age no larger
   // than the current one is a safe-side guess; the most recent such row is used.
-  std::vector<uint8_t> row_valid[2];
+  std::vector<uint8_t> row_valid[2], row_copy[2];
   std::vector<uint64_t> row_time[2], row_age[2];
   std::vector<uint64_t> pushes;  // pushes done per worker
   std::vector<int64_t> prev;
@@ -309,8 +314,8 @@ struct dgs_ctx {
   float* theta_local_buf(uint32_t q) const { return at<float>(lay.theta_local) + (uint64_t)q * lay.n_pad; }
   uint32_t* blk_max(uint32_t q) const { return at<uint32_t>(lay.blk_max) + (uint64_t)q * lay.blk_stride; }
   float** u_slot(uint32_t q) const { return at<float*>(lay.u_slots) + q; }
-  uint32_t* L_next(int pm, uint32_t w) const {
-    return at<uint32_t>(lay.L_next) + ((uint64_t)pm * cfg.num_workers + w) * cfg.num_segments;
+  uint32_t* L_next(int pm, int copy, uint32_t w) const {
+    return at<uint32_t>(lay.L_next) + ((uint64_t)(2 * pm + copy) * cfg.num_workers + w) * cfg.num_segments;
   }
 };
 
@@ -322,11 +327,11 @@ struct ResIds {
   uint32_t U(uint32_t w) const { return w; }
   uint32_t D(uint32_t q) const { return N + q; }
   uint32_t TL(uint32_t q) const { return 2 * N + q; }
-  uint32_t ROW(int kind, uint32_t w) const { return 3 * N + (uint32_t)kind * N + w; }
-  uint32_t THETA() const { return 5 * N; }
-  uint32_t SPARE(int j) const { return 5 * N + 1 + j; }
-  uint32_t SCR(int set) const { return 5 * N + 1 + kSets + set; }
-  uint32_t PKT(int slot) const { return 5 * N + 1 + 2 * kSets + slot; }   // push slots, then pull slots
+  uint32_t ROW(int kind, int copy, uint32_t w) const { return 3 * N + (uint32_t)(2 * kind + copy) * N + w; }
+  uint32_t THETA() const { return 7 * N; }
+  uint32_t SPARE(int j) const { return THETA() + 1 + j; }
+  uint32_t SCR(int set) const { return SPARE(kSets) + set; }
+  uint32_t PKT(int slot) const { return SCR(kSets) + slot; }   // push slots, then pull slots
   uint32_t VPKT(int slot) const { return PKT(kPushSlots + kPullSlots) + (uint32_t)slot; }
   uint32_t STAGE() const { return VPKT(kVarSlots); }
   uint32_t LOG(uint32_t slot) const { return STAGE() + 1 + slot; }
@@ -494,9 +499,10 @@ int fold_launch(dgs_ctx* c, const Workspace& ws, const SelArgs& a, uint32_t q, c
   const uint32_t first = (uint32_t)(c->applied[q] % c->log.ring);
   const uint32_t count = (uint32_t)(c->log_head - c->applied[q]);   // <= ring
   TimedLaunch tl(c, st, SCAN ? DGS_KERNEL_STREAM_PULL : DGS_KERNEL_CATCH_UP);
-  // Half the warps where many events share the GPU: with 8 streams a round of 32 arrivals on 11.7 M elements takes 3.21 ms
-  // with four warps a CTA and 3.42 ms with eight; with 5 streams a round of 8 on 124 M elements 3.15 ms and 3.08 ms.
-  const uint32_t warps = c->alone || c->streams <= 5 ? kFoldWarps : kFoldWarps / 2;
+  // Half the warps where several events share the GPU (a worker has one pull at a time, so it takes more than two workers).
+  // Eight / four warps a CTA, us an event in runs of 256: 2 workers, 8.4 M elements: 36 / 40, 62 layers of 11.7 M: 95 / 101;
+  // 3 workers, 25.6 M: 66 / 63; 8 workers: 61 / 57, 62 layers of 11.7 M: 83 / 78.
+  const uint32_t warps = c->alone || c->cfg.num_workers <= 2 ? kFoldWarps : kFoldWarps / 2;
   k_fold<SCAN><<<c->fold_grid, warps * 32, fold_dyn_bytes(warps, c->fold_ahead, ws.part_cap), st>>>(
       ws, a, c->log, first, count, (uint32_t)(c->applied[q] % (c->log.ring + 1)), (uint32_t)(c->log_head % (c->log.ring + 1)),
       c->fold_ahead);
@@ -563,7 +569,8 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
   // histogram route costs less than that on average.  (With one worker every pull is like the one before it.)
   if (KIND == 1 && age < 2 && c->cfg.num_workers > 1) row = -1;
   const bool single_pass = row >= 0;
-  a.L_next = c->L_next(KIND, worker);
+  const int next_copy = c->row_copy[KIND][worker] ^ 1;
+  a.L_next = c->L_next(KIND, next_copy, worker);
   a.slack = c->at<uint32_t>(c->lay.slack) + (uint64_t)KIND * c->cfg.num_segments;
   a.force_two_pass = single_pass ? 0 : 1;
   // CTAs of finalize: as many as keep the candidates (about 1.7 times the entries) in the threads' registers, but not
@@ -583,10 +590,10 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
     a.spin_limit = 4096;
   }
   a.seq = (uint32_t)c->kind_seq[KIND];
-  a.L_in = single_pass ? c->L_next(KIND, (uint32_t)row) : ws.L_safe;
+  a.L_in = single_pass ? c->L_next(KIND, c->row_copy[KIND][row], (uint32_t)row) : ws.L_safe;
   task.stream = stream_id;
-  if (single_pass && (uint32_t)row != worker) task.reads.push_back(R.ROW(KIND, (uint32_t)row));
-  if (a.speculate) task.writes.push_back(R.ROW(KIND, worker));
+  if (single_pass) task.reads.push_back(R.ROW(KIND, c->row_copy[KIND][row], (uint32_t)row));
+  if (a.speculate) task.writes.push_back(R.ROW(KIND, next_copy, worker));
   task.writes.push_back(R.SCR(stream_id));
   int rc = task_begin(c, task);
   if (rc != DGS_OK) return rc;
@@ -626,6 +633,7 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
   c->kind_seq[KIND] += 1;
   if (a.speculate) {
     c->row_valid[KIND][worker] = 1;
+    c->row_copy[KIND][worker] = (uint8_t)next_copy;
     c->row_time[KIND][worker] = c->kind_seq[KIND];
     c->row_age[KIND][worker] = age;
   }
@@ -769,6 +777,7 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
   }
   for (int k = 0; k < 2; ++k) {
     c->row_valid[k].assign(cfg->num_workers, 0);
+    c->row_copy[k].assign(cfg->num_workers, 0);
     c->row_time[k].assign(cfg->num_workers, 0);
     c->row_age[k].assign(cfg->num_workers, 0);
   }
@@ -825,7 +834,7 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
   }
   INIT_CUDA(cudaMemsetAsync(c->at<char>(L.log_sum), 0, (uint64_t)L.sum_stride * 4, st));   // no packet filed
   INIT_CUDA(cudaMemsetAsync(c->at<char>(L.blk_max), 0, N * L.blk_stride * 4, st));   // D = 0
-  INIT_CUDA(cudaMemsetAsync(c->at<char>(L.L_next), 0xFF, 2 * N * cfg->num_segments * 4, st));
+  INIT_CUDA(cudaMemsetAsync(c->at<char>(L.L_next), 0xFF, 4 * N * cfg->num_segments * 4, st));
   INIT_CUDA(cudaMemsetAsync(c->at<char>(L.slack), 0, 2ull * cfg->num_segments * 4, st));
   INIT_CUDA(cudaMemsetAsync(c->at<char>(L.status), 0, L.total - L.status, st));
   INIT_CUDA(cudaMemcpyAsync(c->at<char>(L.tiles), tiles.data(), tiles.size() * sizeof(Tile), cudaMemcpyHostToDevice, st));

@@ -60,7 +60,6 @@ struct SegDesc {
 };
 
 struct SegSel {        // per layer, finalize
-  uint32_t next;       // bound suggested for a later selection
   uint32_t prefix;     // radix levels over all candidates: key bits fixed so far
   uint32_t krem;       //   entries still to take at or below the fixed prefix
 };
@@ -119,7 +118,7 @@ struct SelArgs {
   float* theta_local;     // pull: theta_w or null
   uint32_t* blk_max;      // pull: per block of kWarpTile elements, an upper bound on the keys of D_w in it (or null)
   const uint32_t* L_in;   // [S] lower bounds guessed for this selection (single-pass route)
-  uint32_t* L_next;       // [S] receives the bounds this selection suggests for a later, similar one
+  uint32_t* L_next;       // [S] receives the bounds this selection suggests for a later, similar one (not L_in)
   uint32_t* slack;        // [S] eighths of k that the bounds of selections of this kind aim beyond the usual number
   uint32_t* pkt_idx;
   float* pkt_val;
@@ -1367,7 +1366,7 @@ __global__ void __maxnreg__(64) k_finalize(const __grid_constant__ Workspace ws,
             const uint32_t want = (uint32_t)min((uint64_t)spec_want(k) + (uint64_t)k * slack / 8u, (uint64_t)0xFFFFFFFFu);
             const uint32_t key = next_bound(ws, s, h, L, total, want, incl, sum, redo || a.force_two_pass, lane);
             if (lane == 0) {
-              ws.sel[s].next = key;                // (L_next may be the row that the other CTAs still read L from)
+              a.L_next[s] = key;
               if (slack && (a.seq & 31u) == 0) a.slack[s] = slack - 1u;
             }
           }
@@ -1512,14 +1511,12 @@ __global__ void __maxnreg__(64) k_finalize(const __grid_constant__ Workspace ws,
     redo = true;
   }
   const uint32_t touched = clo < chi ? s_last - s_lo + 1u : 0u;
-  // what the next selection expects to find cleared, and the bounds it may use
+  // what the next selection expects to find cleared
   {
     uint4* const h4 = reinterpret_cast<uint4*>(ws.hist1);
     for (size_t w = gthread; w < (size_t)S * (kBins1 / 4); w += nthreads) h4[w] = make_uint4(0, 0, 0, 0);
   }
   if (cta >= W) {
-    if (a.speculate)
-      for (uint32_t s = (cta - W) * kThreads + threadIdx.x; s < S; s += A * kThreads) a.L_next[s] = __ldcg(&ws.sel[s].next);
     for (uint32_t s = (cta - W) * kThreads + threadIdx.x; s < S; s += A * kThreads) ws.list_cnt[s] = 0;
   }
   uint2* const s_list = reinterpret_cast<uint2*>(sh.stream.hist);   // the list, where it is ranked in shared memory
