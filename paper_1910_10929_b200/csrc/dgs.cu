@@ -550,8 +550,9 @@ inline int packet_format_of(const dgs_ctx* c) {
 }
 
 template <int MODE>
-const void* finalize_kernel(const dgs_ctx* c) {
-  return c->cfg.num_segments > 1 ? (const void*)k_finalize<MODE, true> : (const void*)k_finalize<MODE, false>;
+const void* finalize_kernel(const dgs_ctx* c, bool big) {
+  if (c->cfg.num_segments > 1) return big ? (const void*)k_finalize<MODE, true, true> : (const void*)k_finalize<MODE, true, false>;
+  return big ? (const void*)k_finalize<MODE, false, true> : (const void*)k_finalize<MODE, false, false>;
 }
 
 template <int MODE>
@@ -581,6 +582,11 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
   const uint64_t cands = (uint64_t)a.pkt_count + a.pkt_count / 4 * 3 + 64ull * c->cfg.num_segments;
   const int fin_grid = (int)std::min<uint64_t>(std::min(c->finalize_max[MODE], c->alone ? 2 * c->sms : c->sms) - (int)advisers,
                                                std::max<uint64_t>(kFinalizeMin, (cands + kThreads * keep - 1) / (kThreads * keep)));
+  // More candidates than the registers of all CTAs hold: k_finalize<.., BIG>, but beside other kernels only for one layer
+  // and fifty times as many (runs of 32 events on 8.4 M elements, us an event without / with: one layer, 10 %, 20 times as
+  // many: 153 / 156; 50 %, 97 times: 823 / 733; 60 layers, 50 %: 750 / 818).
+  const uint64_t held = (uint64_t)fin_grid * kThreads * keep;
+  const bool big = c->alone ? cands > held : c->cfg.num_segments == 1 && cands > 50 * held;
   a.workers = (uint32_t)fin_grid;
   a.advisers = advisers;
   a.fold_grid = MODE == kPull ? (uint32_t)c->fold_grid : 0u;   // one CTA more plans the next pull's pass
@@ -624,7 +630,7 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
     // cooperative launch: the CTAs synchronise among themselves, so all must be resident
     TimedLaunch t(c, st, MODE == kPull ? DGS_KERNEL_FINALIZE_PULL : DGS_KERNEL_FINALIZE_PUSH);
     void* args[] = {(void*)&ws, (void*)&a};
-    DGS_CUDA(c, cudaLaunchCooperativeKernel(finalize_kernel<MODE>(c), dim3(fin_grid + advisers + (MODE == kPull ? 1 : 0)),
+    DGS_CUDA(c, cudaLaunchCooperativeKernel(finalize_kernel<MODE>(c, big), dim3(fin_grid + advisers + (MODE == kPull ? 1 : 0)),
                                             dim3(kThreads), args, finalize_dyn_bytes(c->cfg.num_segments), st));
     c->launches += 1;
   }
@@ -652,14 +658,18 @@ int occupancy_grids(dgs_ctx* c, int sms) {
   DGS_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_hist_all<MODE>, kThreads, 0));
   if (occ < 1) occ = 1;
   c->hist_grid[MODE] = std::min(sms * occ, kMaxGrid);
-  DGS_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, finalize_kernel<MODE>(c), kThreads,
-                                                            finalize_dyn_bytes(c->cfg.num_segments)));
-  if (occ < 1) {
-    c->last_cuda = (int)cudaErrorCooperativeLaunchTooLarge;
-    c->broken = true;
-    return DGS_ECUDA;
+  c->finalize_max[MODE] = kMaxWorkers;
+  for (const bool big : {false, true}) {
+    DGS_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, finalize_kernel<MODE>(c, big), kThreads,
+                                                              finalize_dyn_bytes(c->cfg.num_segments)));
+    if (occ < 1) {
+      c->last_cuda = (int)cudaErrorCooperativeLaunchTooLarge;
+      c->broken = true;
+      return DGS_ECUDA;
+    }
+    c->finalize_max[MODE] = std::min(c->finalize_max[MODE], sms * occ);
   }
-  c->finalize_max[MODE] = std::min(sms * occ, kMaxWorkers) - (MODE == kPull ? 1 : 0);
+  if (MODE == kPull) c->finalize_max[MODE] -= 1;   // the CTA that plans the next pass
   return DGS_OK;
 }
 

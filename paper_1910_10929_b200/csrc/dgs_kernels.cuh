@@ -1201,13 +1201,18 @@ __device__ __noinline__ uint32_t block_radix(const uint2* list, uint32_t pop, ui
 }
 
 // 64 registers a thread: finalize runs beside two CTAs of a push pass on an SM, which leave it that many
-template <int MODE, bool MANY>
-__global__ void __maxnreg__(64) k_finalize(const __grid_constant__ Workspace ws, const __grid_constant__ SelArgs a) {
+// BIG: for more candidates than the registers hold, where the kernel has the GPU to itself.  Such candidates are read again
+// in every phase, and a phase is a chain of trips to memory: four of them a lane are on their way instead of two, and a run
+// of candidates in one part needs neither a search nor a trip for its place.  Finalize of a pull, us, before / with BIG:
+// 2^24 elements, 10 %: 128 / 95, 50 %: 878 / 497; 2^27, 10 %: 1447 / 815.  Beside other kernels its registers cost more
+// than it gains (62 layers of 8.4 M elements, 1 %, runs of 32 events: 65 us an event without, 79 with).
+template <int MODE, bool MANY, bool BIG>
+__global__ void __maxnreg__(BIG ? 96 : 64) k_finalize(const __grid_constant__ Workspace ws, const __grid_constant__ SelArgs a) {
   constexpr int kPartCap = MODE == kPull ? kMaxParts : kMaxGrid;   // parts that the pass before, or a redo, can leave
   __shared__ __align__(16) FinalizeShared<kPartCap> sh;
   extern __shared__ __align__(16) unsigned char fin_dyn[];   // finalize_dyn_bytes(S) bytes
 
-  constexpr int PM = MODE == kPull ? 1 : 0, kKeep = finalize_keep(MANY);
+  constexpr int PM = MODE == kPull ? 1 : 0, kKeep = BIG ? 4 : finalize_keep(MANY);
   // CTAs [0, W) process the candidates, [W, W + A) look after the layers' bounds, and after k_fold one more plans the
   // next pass (it takes no part in the selection)
   const uint32_t cta = blockIdx.x, W = a.workers, A = a.advisers, S = ws.num_segs;
@@ -1250,11 +1255,23 @@ __global__ void __maxnreg__(64) k_finalize(const __grid_constant__ Workspace ws,
     const uint32_t part = part_of(sh.pre, lo, hi, p);
     return __ldcg(ws.part_slot0 + part) + (p - sh.pre[part]);
   };
+  uint32_t run_part = 0, run_slot = 0;   // BIG: part of the last load's first candidate, its first slot - pre
   auto load = [&](uint32_t base) {       // candidates base + 32 u + lane of this warp's run (beyond its end: the last one)
     uint32_t slot[kKeep];
+    bool one_part = false;
+    if (BIG) {
+      if (base == wlo || sh.pre[run_part + 1] <= base) {
+        run_part = base == wlo ? part0 : part_of(sh.pre, run_part + 1, part1, base);
+        run_slot = __ldcg(ws.part_slot0 + run_part) - sh.pre[run_part];
+      }
+      one_part = sh.pre[run_part + 1] >= min(base + 32u * kKeep, whi);   // no search, and no trip for the slots
+    }
 #pragma unroll
     for (int u = 0; u < kKeep; ++u)
-      if (base + u * 32u < whi) slot[u] = slot_of(min(base + u * 32u + lane, whi - 1u), part0, part1);
+      if (base + u * 32u < whi) {
+        const uint32_t p = min(base + u * 32u + lane, whi - 1u);
+        slot[u] = one_part ? run_slot + p : slot_of(p, part0, part1);
+      }
 #pragma unroll
     for (int u = 0; u < kKeep; ++u)
       if (base + u * 32u < whi) {
@@ -1388,7 +1405,7 @@ __global__ void __maxnreg__(64) k_finalize(const __grid_constant__ Workspace ws,
       chi = (uint32_t)min((uint64_t)C, (uint64_t)(cta + 1) * kWarps * per_warp);
       wlo = (uint32_t)min((uint64_t)chi, (uint64_t)clo + warp * per_warp);
       whi = (uint32_t)min((uint64_t)chi, (uint64_t)wlo + per_warp);
-      kept = per_warp <= 32u * kKeep;
+      kept = !BIG && per_warp <= 32u * kKeep;
       if (wlo < whi) {
         part0 = warp_part_of(sh.pre, parts, wlo, lane);
         part1 = warp_part_of(sh.pre, parts, whi - 1u, lane);
@@ -1575,6 +1592,15 @@ __global__ void __maxnreg__(64) k_finalize(const __grid_constant__ Workspace ws,
   } else {
     // Some bin holds more candidates than its list (many equal values, or a bound far below the k-th): three radix
     // levels (11 + 10 + 10 key bits) over all candidates, counted in global memory, the picks spread over the CTAs.
+    // A CTA counts the layer of its middle candidate in shared memory, others straight in global memory.  (All of them in
+    // global memory, where the keys crowd into a few dozen bins: 2^24 elements, 20 %: 1326 us instead of 323.)
+    uint32_t* const s_hist = sh.stream.hist;
+    uint32_t main_t = 0;
+    if (MANY && clo < chi) {
+      row_of(__ldcg(ws.cand_idx + slot_of(clo + (chi - clo) / 2u, 0, parts - 1u)));
+      main_t = near_t;
+    }
+    for (uint32_t b = threadIdx.x; b < (uint32_t)kBins1; b += kThreads) s_hist[b] = 0;
     if (!barrier()) return;              // the histograms are clear
 #pragma unroll 1
     for (int level = 1; level <= 3; ++level) {
@@ -1589,16 +1615,26 @@ __global__ void __maxnreg__(64) k_finalize(const __grid_constant__ Workspace ws,
             row_of(idx[u]);
             const uint32_t s = s_lo + near_t;
             const bool mine = base + u * 32u + lane < whi && (level == 1 || (key >> (sft + 10)) == __ldcg(&ws.sel[s].prefix));
-            const uint32_t at = s * (uint32_t)kBins1 + (level == 1 ? key >> 20 : (key >> sft) & 1023u);
+            const uint32_t bin = level == 1 ? key >> 20 : (key >> sft) & 1023u, at = s * (uint32_t)kBins1 + bin;
+            auto add = [&](uint32_t n) {
+              if (!MANY || near_t == main_t) atomicAdd(s_hist + bin, n); else atomicAdd(ws.hist1 + at, n);
+            };
             // lanes with the first one's bin are counted together: ties crowd into few bins
             const uint32_t m = __ballot_sync(kFull, mine);
             if (m) {
               const uint32_t lead = __shfl_sync(kFull, at, __ffs(m) - 1), same = __ballot_sync(kFull, mine && at == lead);
-              if (lane == __ffs(m) - 1) atomicAdd(ws.hist1 + lead, (uint32_t)__popc(same));
-              if (mine && at != lead) atomicAdd(ws.hist1 + at, 1u);
+              if (lane == __ffs(m) - 1) add(__popc(same));
+              if (mine && at != lead) add(1u);
             }
           }
       }
+      __syncthreads();
+      if (clo < chi)
+        for (uint32_t b = threadIdx.x; b < (uint32_t)kBins1; b += kThreads)
+          if (s_hist[b]) {
+            atomicAdd(ws.hist1 + (size_t)(s_lo + main_t) * kBins1 + b, s_hist[b]);
+            s_hist[b] = 0;
+          }
       if (!barrier()) return;
       for (uint32_t s = cta; s < S; s += W + A) {
         uint32_t bin, krem;

@@ -28,7 +28,8 @@ def values(kind: str, n: int) -> np.ndarray:
 
 @pytest.mark.parametrize("kind", ["normal", "ties", "narrow", "wide", "sparse"])
 @pytest.mark.parametrize("sizes,ppm", [([257], 100_000), ([65_536], 1000), ([300_001], 20_000), ([1 << 20], 400_000),
-                                       ([1] * 70 + [5_000] + [33] * 40 + [100_000], 10_000), ([700] * 90, 60_000)])
+                                       ([1] * 70 + [5_000] + [33] * 40 + [100_000], 10_000), ([700] * 90, 60_000),
+                                       ([400_000, 7, 300_001, 513], 500_000)])
 def test_finalize_edges(sizes, ppm, kind):
     n = sum(sizes)
     ks = [max(1, s * ppm // 1_000_000) for s in sizes]
