@@ -304,7 +304,8 @@ int dgs_free(dgs_ctx* ctx);
  *   n, k     1 <= k <= n <= DGS_STATIC_MAX_N; a larger n returns DGS_ELIMIT, other bad
  *            arguments DGS_EINVAL, and nothing is enqueued
  *   out_idx  DEVICE u32[k], out_val DEVICE f32[k]: the k entries of largest |x| (ties to
- *            the lowest index), ascending index, exactly as dgs_worker_pull would list them
+ *            the lowest index), ascending index, exactly as dgs_worker_pull would list them;
+ *            they must not overlap x, which may be read again while they are written
  *   stream   cudaStream_t; the work is enqueued there and the call returns
  *
  * The function calls no cudaMalloc / cudaFree and no allocating library routine.  The

@@ -1520,9 +1520,8 @@ extern "C" int dgs_topk_encode_static(const float* x, uint32_t n, uint32_t k, ui
   const uint32_t warps = (uint32_t)topk_threads(fine) / 32;
   uint32_t cluster = 1;
   while (cluster < d->max_cluster[fine] && cluster * warps * 32 < n) cluster *= 2;
-  // the lists hold a warp's whole slice where that fits (slices as k_topk cuts them)
-  const uint32_t unit = n >= cluster * warps * 512u ? 512u : 32u;
-  const uint32_t slice = ((n + unit - 1) / unit + cluster * warps - 1) / (cluster * warps) * unit;
+  // the lists hold all elements of a warp where that fits (shared out as in k_topk)
+  const uint32_t W = cluster * warps, unit = n >= W * 512u ? 512u : 32u, slice = ((n + unit - 1) / unit + W - 1) / W * unit;
   const uint32_t cap = std::min(topk_cap(fine), slice);
   const TopkLaunch l(fine, cluster, cap, static_cast<cudaStream_t>(stream));
   const cudaError_t e = fine ? cudaLaunchKernelEx(&l.cfg, k_topk<true>, x, n, k, out_idx, out_val, cap)

@@ -21,16 +21,21 @@ def vector(kind: str, n: int) -> np.ndarray:
         x[:] = np.where(rng.random(n) < 0.3, 1.0, -1.0 - 2.0 ** -20).astype(np.float32)
     elif kind == "few":          # fewer nonzero entries than are taken
         x[rng.random(n) < 0.999] = 0.0
-    elif kind == "hidden":       # large only where no sample is taken, or only where one is
-        s = (np.arange(min(n, 4096), dtype=np.uint64) * n // min(n, 4096)).astype(np.int64)
-        x[s] *= np.float32(1e4)
-    elif kind == "corner":       # everything large in one warp's slice
+    elif kind in ("hidden", "shown"):   # large only where the kernel takes no sample, or only where it takes one
+        m = min(n, 1024)
+        s = (np.arange(m, dtype=np.uint64) * n // m).astype(np.int64)
+        x[s] *= np.float32(1e4 if kind == "shown" else 1e-4)
+    elif kind == "sorted":       # a part of the vector holds all that is large: lists of some warps fill up
+        x = np.sort(np.abs(x))
+    elif kind == "zero":
+        x[:] = 0.0
+    elif kind == "corner":       # everything large lies together
         x[: n // 300 + 1] *= np.float32(1e4)
     return x
 
 
 @pytest.mark.parametrize("n", [1, 31, 33, 4096, 4097, 65_535, 131_073, 1 << 18, (1 << 18) + 1, (1 << 20) - 1, 1 << 20])
-@pytest.mark.parametrize("kind", ["normal", "equal", "two", "few", "hidden", "corner"])
+@pytest.mark.parametrize("kind", ["normal", "equal", "two", "few", "hidden", "shown", "sorted", "zero", "corner"])
 def test_static_selection_edges(n, kind):
     x = vector(kind, n)
     xd = torch.empty(n + 1, device=DEV)[n % 2:][:n]      # odd lengths also start off a 16-byte boundary
