@@ -385,11 +385,12 @@ def run_ours(args, wl, rank: int, world: int, local_rank: int, dist) -> dict:
     dom_ms, dom_cnt = stimes[dom]          # on its own (single-stream pass)
     ovl_ms, ovl_cnt = ktimes[dom]          # with the other streams' kernels beside it
     # algorithmic bytes per launch: the streaming passes move whole vectors; the apply reads the packet and
-    # lowers theta (8 K read + 8 K read-modify-write); a catch-up lowers one difference vector by the packets
-    # of one round of the workers (8 bytes per entry, N K entries)
+    # lowers theta (8 K read + 8 K read-modify-write); a pull's pass reads its difference vector and folds the packets
+    # of one round of the workers into it (8 bytes per entry, N K entries); a catch-up does the folding alone (it is
+    # launched only for a worker that is about to fall off the log, or before a two-pass selection)
     kernel_bytes = {
         "stream_push": 12 * wl.n, "finalize_push": None, "two_pass_push": 8 * wl.n,
-        "scatter": 16 * wl.K_push, "stream_pull": 4 * wl.n, "finalize_pull": None, "two_pass_pull": 4 * wl.n,
+        "scatter": 16 * wl.K_push, "stream_pull": 4 * wl.n + 8 * wl.K_push * N, "finalize_pull": None, "two_pass_pull": 4 * wl.n,
         "catch_up": 8 * wl.K_push * N,
     }
     achieved = kernel_bytes[dom] / (dom_ms * 1e-3 / max(dom_cnt, 1)) / 1e9
@@ -399,8 +400,6 @@ def run_ours(args, wl, rank: int, world: int, local_rank: int, dist) -> dict:
     def kernel_gbs(k, ms, cnt):
         if not cnt or ms <= 0:
             return None
-        if k == "catch_up":         # the apply's bytes of an event (N + 1 buffers) over scatter + catch-up time
-            return ab["apply"] * K / ((ms + ktimes["scatter"][0]) * 1e-3) / 1e9
         return kernel_bytes[k] / (ms * 1e-3 / cnt) / 1e9 if kernel_bytes[k] else None
 
     traffic, traffic_note = ncu_traffic(wl.name, dom)
@@ -438,8 +437,8 @@ def run_ours(args, wl, rank: int, world: int, local_rank: int, dist) -> dict:
                      "whole_event_frac": eff_gbs / peak,
                      "note": "achieved: CUDA events around each launch of the kernel in a pass of the same event "
                              f"loop ({Ks} events) that keeps every kernel on one stream, so the duration is the "
-                             "kernel's own; achieved_overlapped: the same in the multi-stream loop, where up to "
-                             "four push passes and the server-side kernels share the GPU and the bandwidth; "
+                             "kernel's own; achieved_overlapped: the same in the multi-stream loop, where the "
+                             "passes and small kernels of up to eight events share the GPU and the bandwidth; "
                              "whole_event_frac: algorithmic bytes of a whole event over the timed region"},
         "e2e": {"value": e2e_events / e2e_max, "unit": UNIT, "steps": Ke, "h2d_bytes_per_step": 4 * wl.n,
                 "d2h_bytes_per_step": 8 * wl.K_pull},

@@ -48,7 +48,7 @@ int streams_for(const dgs_config* c) {
   return c->num_workers == 1 ? 2 : kStreams;
 }
 constexpr int kCaller = kStreams;         // the caller's stream, where the tracker names streams by number
-constexpr int kQueuesWanted = 12;         // hardware queues that keep the streams of two contexts and the caller's apart
+constexpr int kQueuesWanted = 12;         // hardware queues for the streams of one context, the caller's and a few more
 constexpr int kLogRingMax = 128;            // most packets the apply log keeps
 constexpr int kLogSlack = 32;               // slots of the log beyond one per worker
 constexpr uint64_t kListCap = 4096;         // most entries of a layer's list of candidates in the k-th's bin
@@ -73,9 +73,9 @@ struct Layout {
   uint64_t tiles, segs, seg_off, blk_seg;
   ScratchLayout sc[kSets];
   uint64_t L_next, slack, u_slots, status, stats;
-  uint64_t log_ent, log_pos, log_sum;
+  uint64_t log_ent, log_pos, log_sum;   // ring of applied packets not yet folded into every D_q
   uint64_t blk_max;      // [N][blk_stride]: per block of kWarpTile elements, an upper bound on the keys of D_q in it
-  uint64_t blk_stride = 0;  // ring of applied packets not yet folded into every D_q
+  uint64_t blk_stride = 0;
   uint32_t log_ring = 0, log_stride = 0, pos_rows = 0, sum_stride = 0;
   uint32_t num_blocks = 0;
   uint64_t total = 0;

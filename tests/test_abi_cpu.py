@@ -51,7 +51,7 @@ def test_arena_sizing_scales_with_workers_and_flags():
     big = dgs.make_config(25_557_032, 32, 0.1, 0.9, [0], [25_557_032], [25_558], [25_558])
     need = dgs.dgs_arena_bytes(big)
     state = (2 * 32 + 1) * 25_557_032 * 4
-    # four spare velocity vectors, ten scratch sets (one per stream that selects) with two candidate buffers
+    # eight spare velocity vectors and eight scratch sets (one of each per stream) with two candidate buffers
     # of capacity n each, packet slots and the packet log
     assert state < need < 1.45 * state
 
@@ -92,7 +92,7 @@ def test_init_without_arena_is_rejected_before_any_gpu_work():
 
 def test_hardware_queues_reports_what_the_environment_says(monkeypatch):
     needed, configured = dgs.dgs_hardware_queues()
-    assert needed == 12                      # eleven streams of the library and the caller's
+    assert needed == 12                      # eight streams of the library, the caller's and a few more
     monkeypatch.setenv("CUDA_DEVICE_MAX_CONNECTIONS", "5")
     assert dgs.dgs_hardware_queues() == (12, 5)
     monkeypatch.delenv("CUDA_DEVICE_MAX_CONNECTIONS")

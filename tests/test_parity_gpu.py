@@ -176,10 +176,8 @@ def test_more_workers_than_packets_kept():
 
 
 def test_catch_up_takes_a_crowded_range_in_pieces():
-    # The ranges of the packet log come from the first packet: its entries lie in the first quarter
-    # of the vector, so one range covers the other three quarters.  All later packets fall there,
-    # and a worker that has missed a few of them finds more entries in that range than the
-    # catch-up's table holds at once.
+    # The first packet's entries lie in the first quarter of the vector, all later ones in its second half: a worker
+    # that has missed a few packets finds blocks without any entries, and blocks with more of them than are fetched ahead.
     n, N, E = 200_000, 8, 20
     wl = W.custom("moving", [n], N, E, 10_000, grad_kind="normal", grad_scale=1e-2, schedule_kind="cyclic")
     base = wl.gradient
