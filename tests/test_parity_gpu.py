@@ -361,19 +361,22 @@ def test_sweep_selection_at_the_bandwidth_bound_sizes(log2n, ppm):
     assert np.array_equal(bits(val), bits(x[want]))
 
 
-def test_sweep_scatter_into_33_buffers_matches_the_checker():
+@pytest.mark.parametrize("filed", [False, True])
+def test_sweep_scatter_into_33_buffers_matches_the_checker(filed):
     """The sweep's apply: the packet selected from a sweep vector (2^22 values, 1 %), given to
     dgs_server_apply as a foreign packet, is subtracted from theta and from 32 difference vectors
     (Algorithm 2, M <- M - decode(g); Eq. 3) -- compared with the CPU checker's apply, twice in a
-    row so that the second subtraction meets nonzero entries."""
+    row so that the second subtraction meets nonzero entries.  Filed in the log where the library's own
+    packets are as long, scattered at once where they are shorter."""
     n, N = 1 << 22, 32
     k = W.k_of(n, 10_000)
+    k_push = k if filed else 1
     x = W.sweep_values(n, index=22)
     chosen = oracle.topk(x, k).astype(np.uint32)
     vals = x[chosen]
     theta0 = W.custom("t", [n], N, 1, 10_000).theta0()
-    orc = oracle.Oracle(n, N, 0.1, 0.9, [0], [n], [k], [k], theta0)
-    ctx = dgs.Context(n, N, 0.1, 0.9, [0], [n], [k], [k], torch.from_numpy(theta0).to(DEV))
+    orc = oracle.Oracle(n, N, 0.1, 0.9, [0], [n], [k_push], [k], theta0)
+    ctx = dgs.Context(n, N, 0.1, 0.9, [0], [n], [k_push], [k], torch.from_numpy(theta0).to(DEV))
     idx_d = torch.from_numpy(chosen.view(np.int32)).to(DEV)
     val_d = torch.from_numpy(vals).to(DEV)
     pkt = dgs.dgs_packet(idx_d.data_ptr(), val_d.data_ptr(), k)
@@ -384,7 +387,7 @@ def test_sweep_scatter_into_33_buffers_matches_the_checker():
     assert np.array_equal(bits(ctx.state(dgs.DGS_THETA).cpu().numpy()), bits(orc.state(oracle.THETA)))
     for q in range(N):
         assert np.array_equal(bits(ctx.state(dgs.DGS_D, q).cpu().numpy()), bits(orc.state(oracle.D, q))), f"D[{q}]"
-    # the block bounds the scatter maintains still let a pull find the largest entries (Eq. 6a)
+    # the block bounds that either maintains still let a pull find the largest entries (Eq. 6a)
     gi, gv = packet_to_numpy(ctx, ctx.worker_pull(5))
     qi, qv = orc.pull(5)
     assert np.array_equal(gi, qi) and np.array_equal(bits(gv), bits(qv))
