@@ -275,6 +275,11 @@ __device__ __forceinline__ void flush_hist(uint32_t* s_hist, uint32_t* g_hist) {
   }
 }
 
+// One more candidate in a bin of layer `seg`: in shared memory for the CTA's main layer, else straight in global memory.
+__device__ __forceinline__ void count_bin(const Workspace& ws, uint32_t* s_hist, uint32_t main_seg, uint32_t seg, uint32_t bin) {
+  if (seg == main_seg) atomicAdd(s_hist + bin, 1u); else atomicAdd(ws.hist1 + (size_t)seg * kBins1 + bin, 1u);
+}
+
 // candidates of warps 0 .. warp-1 in this round, and of all warps
 __device__ __forceinline__ uint32_t round_offset(const uint32_t* wcnt, int warp, uint32_t& total) {
   uint32_t before = 0, tot = 0;
@@ -522,15 +527,14 @@ __device__ __forceinline__ uint32_t tile_mask_smem(const SelArgs& a, uint32_t ti
 }
 
 // ---- the same pass with TMA-staged tiles --------------------------------------------
-// Full tiles are brought into a ring of shared-memory stages by bulk asynchronous copies
-// (cp.async.bulk, completion counted on an mbarrier per stage), kStageTiles tiles of each
+// Blocks of kWarpTile elements are brought into a ring of shared-memory stages by bulk asynchronous copies
+// (cp.async.bulk, completion counted on an mbarrier per stage), one per warp of each
 // input per stage, so that several stages are in flight while the warps work on one: the
 // bytes in flight no longer depend on how many warps are waiting at a load.  One round of the
 // ordered append = one stage; the barrier between counting and writing is also the one after
 // which the stage of the round before is free, so a ring of kStages stages keeps kStages - 1
 // of them in flight.
-constexpr int kStageTiles = kWarps;                        // one tile per warp and stage
-constexpr int kStageFloats = kStageTiles * kWarpTile;      // per input array
+constexpr int kStageFloats = kWarps * kWarpTile;           // per input array: one block per warp and stage
 // The ring: three stages (96 KB, two CTAs per SM, 128 KB of the SM's shared memory in flight).
 struct StreamRing {
   static constexpr int kStages = 3;
@@ -566,105 +570,159 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
                ::"r"(smem_addr(dst)), "l"(src), "r"(bytes), "r"(smem_addr(bar)) : "memory");
 }
 
+// The layers that elements [base, base + len) lie in, `seg` the first of them: calls fn(layer, lo, hi, its bound) for each in
+// turn, elements base + lo .. base + hi - 1 being that layer's.  By a warp; 32 layers are looked up in one trip.
+template <typename Fn>
+__device__ __forceinline__ void each_layer(const Workspace& ws, const uint32_t* Larr, uint32_t seg, uint32_t base, uint32_t len,
+                                           Fn fn) {
+  uint32_t lo = 0;
+  for (uint32_t s0 = seg;; s0 += 32) {
+    const uint32_t s = min(s0 + (threadIdx.x & 31u), ws.num_segs - 1u);
+    const uint32_t end = min(__ldg(ws.seg_off + s + 1) - base, len), L = Larr[s];
+#pragma unroll 1
+    for (uint32_t j = 0; j < 32; ++j) {
+      const uint32_t hi = __shfl_sync(kFull, end, j);
+      fn(s0 + j, lo, hi, __shfl_sync(kFull, L, j));
+      if (hi == len) return;
+      lo = hi;
+    }
+  }
+}
+// A block that lies in several layers, or the vector's last, shorter one (a warp; element st * 32 + lane of the block is bit
+// st of the lane): every element is compared with the bound of its own layer.  su, sg: the block of the state vector and of
+// the gradient, in shared or global memory; seg: layer of its first element.  Returns the candidates, writes the new velocity.
 template <int MODE>
-__device__ void stream_tiles_tma(const Workspace& ws, const SelArgs& a, const uint32_t* Larr,
-                                 const float* __restrict__ in, float* __restrict__ out, uint32_t cta, uint32_t G,
-                                 StreamShared& sh, float* ring, uint64_t* full, int* s_dead) {
+__device__ __noinline__ uint32_t mixed_mask(const Workspace& ws, const SelArgs& a, const uint32_t* Larr, const float* su,
+                                            const float* sg, float* out, uint32_t base, uint32_t len, uint32_t seg) {
+  const uint32_t lane = threadIdx.x & 31u;
+  float x[kRaggedSteps];
+#pragma unroll
+  for (int st = 0; st < kRaggedSteps; ++st) {
+    const uint32_t off = st * 32u + lane;
+    x[st] = off < len ? combine<MODE>(su[off], sg[off], a.m, a.lr) : 0.f;
+  }
+  uint32_t mask = 0;
+  each_layer(ws, Larr, seg, base, len, [&](uint32_t, uint32_t lo, uint32_t hi, uint32_t L) {
+    const float Lf = __uint_as_float(L);   // |x| >= Lf  <=>  key(x) >= L for finite x (no flush-to-zero)
+#pragma unroll
+    for (int st = 0; st < kRaggedSteps; ++st) {
+      const uint32_t off = st * 32u + lane;
+      if (off >= lo && off < hi && fabsf(x[st]) >= Lf) mask |= 1u << st;
+    }
+  });
+#pragma unroll
+  for (int st = 0; st < kRaggedSteps; ++st) {
+    const uint32_t off = st * 32u + lane;
+    if (off < len) out[base + off] = (mask >> st) & 1u ? x[st] : unsent<MODE>(x[st], a.inv_m);
+  }
+  return mask;
+}
+// Writes its candidates from slot `pos` on, in index order; those of layer main_seg are counted in `hist`.
+template <int MODE>
+__device__ __noinline__ void mixed_emit(const Workspace& ws, const SelArgs& a, const uint32_t* Larr, uint32_t mask, const float* su,
+                                        const float* sg, uint32_t base, uint32_t len, uint32_t seg, uint32_t pos, uint32_t main_seg,
+                                        uint32_t* hist) {
+  const uint32_t lane = threadIdx.x & 31u, lt = lanemask_lt();
+  each_layer(ws, Larr, seg, base, len, [&](uint32_t s, uint32_t lo, uint32_t hi, uint32_t L) {
+#pragma unroll 2
+    for (uint32_t st = lo / 32u; st * 32u < hi; ++st) {
+      const uint32_t off = st * 32u + lane;
+      const bool cand = ((mask >> st) & 1u) && off >= lo && off < hi;
+      const uint32_t b = __ballot_sync(kFull, cand);
+      if (cand) {
+        const uint32_t to = pos + __popc(b & lt);
+        const float v = combine<MODE>(su[off], sg[off], a.m, a.lr);
+        ws.cand_idx[to] = base + off;
+        ws.cand_val[to] = v;
+        count_bin(ws, hist, main_seg, s, bin_of(key_of(v), L));
+      }
+      pos += __popc(b);
+    }
+  });
+}
+
+// The pass runs over the blocks of the flat vector, kWarps of them a round, and takes no notice of where layers begin: a
+// block inside one layer is compared with that layer's bound, one that lies in several element by element, and the ring
+// never runs empty in between.  The candidates of the layer in the middle of the CTA's share are counted in shared memory,
+// those of others straight in global memory.  (A layer at a time, the ring restarted and the histogram flushed for each and
+// one warp at work on its ragged ends, 11.7 M elements in 62 layers took 54 us, and the CTAs with the small layers 58 us where
+// the others took 24; now 37 us.)
+template <int MODE>
+__device__ void stream_blocks_tma(const Workspace& ws, const SelArgs& a, const uint32_t* Larr, const float* __restrict__ in,
+                                  float* __restrict__ out, uint32_t cta, uint32_t G, StreamShared& sh, float* ring, uint64_t* full,
+                                  int* s_dead) {
   using R = StreamRing;
   static_assert(MODE != kPull, "a pull's pass is k_fold");
   static_assert(R::kStages >= 2, "the ring needs a stage in flight besides the one being read");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t t0 = part_first_tile(cta, G, ws.num_tiles), t1 = part_first_tile(cta + 1, G, ws.num_tiles);
-  const uint32_t lt = lanemask_lt();
-  for (int b = threadIdx.x; b < kBins1; b += kThreads) sh.hist[b] = 0;
+  const uint32_t NB = ws.num_blocks, S = ws.num_segs, n = ws.n, whole_blocks = n / kWarpTile;
+  const uint32_t t0 = part_first_tile(cta, G, NB), t1 = part_first_tile(cta + 1, G, NB);
+  const uint32_t f1 = min(t1, whole_blocks);    // blocks [t0, f1) come through the ring; the vector's last one may be shorter
+  const uint32_t rounds = (t1 - t0 + kWarps - 1) / kWarps;
+  auto issue = [&](uint32_t r) {                // thread 0 only; round r has a whole block
+    const uint32_t st = r % R::kStages, first = t0 + r * kWarps;
+    const uint32_t bytes = min((uint32_t)kWarps, f1 - first) * kWarpTile * 4;
+    const size_t elem = (size_t)first * kWarpTile;
+    float* dst = ring + (size_t)st * (R::kStageBytes / 4);
+    mbar_expect_tx(full + st, bytes * 2);
+    bulk_load(dst, in + elem, bytes, full + st);
+    bulk_load(dst + kStageFloats, a.grad + elem, bytes, full + st);
+  };
+  auto fetched = [&](uint32_t r) { return t0 + r * kWarps < f1; };   // (the shorter block may be alone in its round)
   if (threadIdx.x == 0) {
-    sh.cursor = 0;
     *s_dead = 0;
     if (cta == 0) ws.sync[kParts] = G;
     for (int st = 0; st < R::kStages; ++st) mbar_init(full + st, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    for (uint32_t r = 0; r < (uint32_t)R::kStages - 1 && r < rounds && fetched(r); ++r) issue(r);
+  }
+  for (int b = threadIdx.x; b < kBins1; b += kThreads) sh.hist[b] = 0;
+  const uint32_t slot0 = t0 * kWarpTile;        // first slot of this CTA's region
+  const uint32_t main_seg = S == 1 || t0 >= t1 ? 0u : __ldg(ws.blk_seg + t0 + (t1 - t0) / 2);
+  // layer of the first element of this warp's block
+  uint32_t seg = S == 1 || t0 + warp >= t1 ? 0u : __ldg(ws.blk_seg + t0 + warp);
+  uint32_t seg_end = S == 1 ? n : __ldg(ws.seg_off + seg + 1), L = Larr[seg];
+  __syncthreads();
+  uint32_t cur = 0;   // candidates appended so far (same in every thread)
+  for (uint32_t r = 0; r < rounds; ++r) {
+    const uint32_t st = r % R::kStages, blk = t0 + r * kWarps + warp, base = blk * kWarpTile;
+    if (blk < t1 && base >= seg_end) {
+      seg = __ldg(ws.blk_seg + blk);
+      seg_end = __ldg(ws.seg_off + seg + 1);
+      L = Larr[seg];
+    }
+    const bool landed = !fetched(r) || mbar_wait(full + st, (r / R::kStages) & 1u);
+    if (!landed) *s_dead = 1;
+    const float* const su = ring + (size_t)st * (R::kStageBytes / 4) + warp * kWarpTile;
+    const bool plain = blk < f1 && base + kWarpTile <= seg_end;
+    uint32_t mask = 0;
+    if (blk < t1 && landed) {
+      if (plain) {
+        mask = tile_mask_smem<MODE>(a, base, su, su + kStageFloats, L, lane, out);
+      } else {                                  // (the shorter block straight from global memory)
+        mask = mixed_mask<MODE>(ws, a, Larr, blk < f1 ? su : in + base, blk < f1 ? su + kStageFloats : a.grad + base, out, base,
+                                min((uint32_t)kWarpTile, n - base), seg);
+      }
+    }
+    const uint32_t count = __reduce_add_sync(kFull, (uint32_t)__popc(mask));
+    if (lane == 0) sh.wcnt[r & 1][warp] = count;
+    __syncthreads();   // the counts of this round are known, and every warp has left the stage of the round before
+    if (*s_dead) break;
+    const uint32_t ahead = r + R::kStages - 1;
+    if (threadIdx.x == 0 && ahead < rounds && fetched(ahead)) issue(ahead);   // into the stage of the round before
+    uint32_t total;
+    const uint32_t pos = slot0 + cur + round_offset(sh.wcnt[r & 1], warp, total);
+    cur += total;
+    if (count == 0) continue;
+    if (plain) {
+      tile_emit(ws, base, mask, pos, lane, [&](uint32_t off) { return combine<MODE>(su[off], su[kStageFloats + off], a.m, a.lr); },
+                [&](uint32_t, uint32_t key) { count_bin(ws, sh.hist, main_seg, seg, bin_of(key, L)); });
+    } else {
+      mixed_emit<MODE>(ws, a, Larr, mask, blk < f1 ? su : in + base, blk < f1 ? su + kStageFloats : a.grad + base, base,
+                       min((uint32_t)kWarpTile, n - base), seg, pos, main_seg, sh.hist);
+    }
   }
   __syncthreads();
-  if (t0 >= t1) {
-    if (threadIdx.x == 0) {
-      ws.part_cands[cta] = 0;
-      ws.part_slot0[cta] = 0;
-    }
-    return;
-  }
-  const uint32_t slot0 = ws.tiles[t0].start;
-  const uint32_t seg_first = ws.tiles[t0].seg, seg_last = ws.tiles[t1 - 1].seg;
-  uint32_t uses = 0;  // stage uses so far (same in every thread): stage = use % kStages, parity = (use / kStages) & 1
-  uint32_t cur = 0;   // candidates appended so far (same in every thread)
-  for (uint32_t s = seg_first; s <= seg_last; ++s) {
-    const uint32_t a0 = max(t0, ws.segs[s].tile_begin), a1 = min(t1, ws.segs[s].tile_end);
-    const uint32_t L = Larr[s];
-    // only the first and the last tile of a layer can be ragged
-    const bool head = ws.tiles[a0].len != kWarpTile;
-    const bool tail = (a1 - 1 > a0 || !head) && ws.tiles[a1 - 1].len != kWarpTile;
-    const uint32_t f0 = a0 + (head ? 1u : 0u), f1 = a1 - (tail ? 1u : 0u);   // full tiles [f0, f1)
-    // a ragged tile is one warp's work; the warp tells the others how many candidates it appended
-    auto ragged = [&](uint32_t t) {
-      if (warp == 0) {
-        const Tile tile = ws.tiles[t];
-        float x[kRaggedSteps];
-        const uint32_t flags = ragged_mask<MODE>(a, tile, L, lane, in, out, x);
-        const uint32_t count = __reduce_add_sync(kFull, (uint32_t)__popc(flags));
-        ragged_emit(ws, sh, tile, flags, L, slot0 + cur, lane, lt, x);
-        if (lane == 0) sh.cursor = count;
-      }
-      __syncthreads();
-      cur += sh.cursor;
-      __syncthreads();
-    };
-    if (head) ragged(a0);
-    const uint32_t nfull = f1 > f0 ? f1 - f0 : 0;
-    const uint32_t nchunks = (nfull + kStageTiles - 1) / kStageTiles;
-    const uint32_t e0 = nfull ? ws.tiles[f0].start : 0;   // first element of the full tiles (multiple of kWarpTile)
-    auto issue = [&](uint32_t chunk, uint32_t use) {      // thread 0 only
-      const uint32_t st = use % R::kStages;
-      const uint32_t tiles_here = min((uint32_t)kStageTiles, nfull - chunk * kStageTiles);
-      const uint32_t bytes = tiles_here * kWarpTile * 4;
-      const size_t elem = (size_t)e0 + (size_t)chunk * kStageFloats;
-      float* dst = ring + (size_t)st * (R::kStageBytes / 4);
-      mbar_expect_tx(full + st, bytes * 2);
-      bulk_load(dst, in + elem, bytes, full + st);
-      bulk_load(dst + kStageFloats, a.grad + elem, bytes, full + st);
-    };
-    uint32_t issued = 0;                                  // thread 0: chunks asked for
-    if (threadIdx.x == 0)
-      for (; issued < (uint32_t)R::kStages - 1 && issued < nchunks; ++issued) issue(issued, uses + issued);
-    uint32_t done = 0;
-    for (uint32_t c = 0; c < nchunks; ++c, ++done) {
-      const uint32_t use = uses + done, st = use % R::kStages;
-      const bool landed = mbar_wait(full + st, (use / R::kStages) & 1u);
-      if (!landed) *s_dead = 1;
-      const uint32_t tl = c * kStageTiles + warp;          // this warp's tile among the full ones
-      const float* su = ring + (size_t)st * (R::kStageBytes / 4) + warp * kWarpTile;
-      uint32_t mask = 0;
-      if (tl < nfull && landed) mask = tile_mask_smem<MODE>(a, e0 + tl * kWarpTile, su, su + kStageFloats, L, lane, out);
-      const uint32_t count = __reduce_add_sync(kFull, (uint32_t)__popc(mask));
-      if (lane == 0) sh.wcnt[use & 1][warp] = count;
-      __syncthreads();   // the counts of this round are known, and every warp has left the stage of the round before
-      if (*s_dead) break;
-      if (threadIdx.x == 0 && issued < nchunks) {          // into the stage of the round before
-        issue(issued, uses + issued);
-        ++issued;
-      }
-      uint32_t total;
-      const uint32_t base = slot0 + cur + round_offset(sh.wcnt[use & 1], warp, total);
-      cur += total;
-      tile_emit(ws, e0 + tl * kWarpTile, mask, base, lane, [&](uint32_t off) {
-        return combine<MODE>(su[off], su[kStageFloats + off], a.m, a.lr);
-      }, [&](uint32_t, uint32_t key) { atomicAdd(sh.hist + bin_of(key, L), 1u); });
-    }
-    if (*s_dead) break;
-    uses += done;
-    __syncthreads();   // every warp has left the last stage (the next layer's first copies go anywhere in the ring)
-    if (tail) ragged(a1 - 1);
-    flush_hist(sh.hist, ws.hist1 + (size_t)s * kBins1);
-    __syncthreads();
-  }
   if (*s_dead) {
     // a copy did not land in time: report, give the copies still in flight one more bounded wait, leave
     if (threadIdx.x == 0) {
@@ -675,6 +733,8 @@ __device__ void stream_tiles_tma(const Workspace& ws, const SelArgs& a, const ui
       }
     }
     __syncthreads();
+  } else {
+    flush_hist(sh.hist, ws.hist1 + (size_t)main_seg * kBins1);
   }
   if (threadIdx.x == 0) {
     ws.part_cands[cta] = cur;
@@ -1802,7 +1862,7 @@ __global__ void __launch_bounds__(kThreads) k_pick_lower(Workspace ws) {
 
 // ---- stand-alone stream pass with the carried bound -------------------------------
 template <int MODE>
-__global__ void __maxnreg__(64) k_stream(Workspace ws, SelArgs a) {
+__global__ void __maxnreg__(64) k_stream(const __grid_constant__ Workspace ws, const __grid_constant__ SelArgs a) {
   extern __shared__ __align__(128) unsigned char dyn_smem[];   // the ring of stages
   __shared__ StreamShared sh;
   __shared__ __align__(8) uint64_t full[StreamRing::kStages];
@@ -1810,8 +1870,8 @@ __global__ void __maxnreg__(64) k_stream(Workspace ws, SelArgs a) {
   const float* in = *a.u_cur_slot;
   float* out = *a.u_spare_slot;
   if (blockIdx.x == 0 && threadIdx.x == 0) ws.sync[kBarCount] = ws.sync[kFail] = 0;   // for the finalize launch that follows
-  stream_tiles_tma<MODE>(ws, a, a.L_in, in, out, blockIdx.x, gridDim.x, sh, reinterpret_cast<float*>(dyn_smem), full,
-                         &s_dead);
+  stream_blocks_tma<MODE>(ws, a, a.L_in, in, out, blockIdx.x, gridDim.x, sh, reinterpret_cast<float*>(dyn_smem), full,
+                          &s_dead);
 }
 
 // ---- pull without secondary compression: every nonzero entry of D_w -------------------
@@ -2117,44 +2177,64 @@ __device__ __forceinline__ uint32_t lane_offsets(uint32_t count, uint32_t lt, ui
   return ex;
 }
 
-// A block that is not a full one inside one layer (layer `seg` is its first): every element is compared with the
-// bound of its own layer.  Appends the candidates from slot `at` on, returns how many; top: largest key.
+// A block in shared memory that is not a full one inside one layer (layer `seg` is its first): every element is compared
+// with the bound of its own layer, a layer at a time.  Appends the candidates from slot `at` on, returns how many; top: this
+// lane's largest key.  A layer with few entries to send has a bound that admits most of it, so there may be 16 a lane.
+// (One element after the other, each with a look at its layer's bound: 15,000 to 21,000 cycles a block, and the warp
+// with three of them kept a pass of 45,000 cycles waiting for another 45,000.  11.7 M elements in 62 layers, alone: 49 us, now
+// 42, with 0.5 M entries to fold in, 86 us, now 74, with 3.7 M.)
 template <bool SCAN>
 __device__ __noinline__ uint32_t scan_mixed(const Workspace& ws, const SelArgs& a, const float* t, uint32_t base, uint32_t seg,
-                                            uint32_t at, uint32_t& top) {
-  const int lane = threadIdx.x & 31;
-  const uint32_t len = min((uint32_t)kWarpTile, ws.n - base), S = ws.num_segs;
-  uint32_t mask = 0, best = 0, s = seg;
-  auto layer_of = [&](uint32_t off) {
-    while (s + 1 < S && __ldg(ws.seg_off + s + 1) <= base + off) ++s;
-  };
-  for (uint32_t e = 0; e < 16; ++e) {
-    const uint32_t off = lane * 16 + e;
-    if (off < len) {
-      const uint32_t key = key_of(t[tile_place(off)]);
-      best = max(best, key);
-      if (SCAN) {
-        layer_of(off);
-        if (key >= a.L_in[s]) mask |= 1u << e;
-      }
-    }
+                                            uint32_t at, uint32_t main_seg, uint32_t* hist, uint32_t& top) {
+  const uint32_t lane = threadIdx.x & 31u, sw = (lane >> 1) & 3u;
+  const uint32_t len = min((uint32_t)kWarpTile, ws.n - base);
+  const uint32_t len_here = min(16u, max(len, lane * 16u) - lane * 16u);   // of this lane's 16 elements, those in the vector
+  uint32_t key[16], best = 0;
+#pragma unroll
+  for (int j = 0; j < kVecIters; ++j) {
+    const uint4 q = *reinterpret_cast<const uint4*>(t + (lane * 4u + ((uint32_t)j ^ sw)) * 4u);
+    key[4 * j] = q.x;
+    key[4 * j + 1] = q.y;
+    key[4 * j + 2] = q.z;
+    key[4 * j + 3] = q.w;
   }
-  __syncwarp();
+#pragma unroll
+  for (int e = 0; e < 16; ++e) {
+    key[e] &= 0x7FFFFFFFu;
+    if ((uint32_t)e < len_here) best = max(best, key[e]);
+  }
   top = best;
   if (!SCAN) return 0;
+  uint32_t mask = 0;
+  // of this lane's 16 elements, those that lie in [lo, hi)
+  auto part = [&](uint32_t lo, uint32_t hi) {
+    const uint32_t first = min(16u, max(lo, lane * 16u) - lane * 16u), end = min(16u, max(hi, lane * 16u) - lane * 16u);
+    return (1u << end) - (1u << first);
+  };
+  each_layer(ws, a.L_in, seg, base, len, [&](uint32_t, uint32_t lo, uint32_t hi, uint32_t L) {
+    const uint32_t here = part(lo, hi);
+    if (here) {
+      uint32_t m = 0;
+#pragma unroll
+      for (int e = 0; e < 16; ++e) m |= key[e] >= L ? 1u << e : 0u;
+      mask |= m & here;
+    }
+    __syncwarp();
+  });
   uint32_t total;
   uint32_t pos = at + lane_offsets(__popc(mask), lanemask_lt(), total);
-  s = seg;
-  for (uint32_t m = mask; m; m &= m - 1) {
-    const uint32_t off = lane * 16 + __ffs(m) - 1;
-    const float v = t[tile_place(off)];
-    layer_of(off);
-    ws.cand_idx[pos] = base + off;
-    ws.cand_val[pos] = v;
-    ++pos;
-    atomicAdd(ws.hist1 + (size_t)s * kBins1 + bin_of(key_of(v), a.L_in[s]), 1u);
-  }
-  __syncwarp();
+  if (total)
+    each_layer(ws, a.L_in, seg, base, len, [&](uint32_t s, uint32_t lo, uint32_t hi, uint32_t L) {
+      for (uint32_t m = mask & part(lo, hi); m; m &= m - 1) {
+        const uint32_t off = lane * 16u + __ffs(m) - 1u;
+        const float v = t[tile_place(off)];
+        ws.cand_idx[pos] = base + off;
+        ws.cand_val[pos] = v;
+        ++pos;
+        count_bin(ws, hist, main_seg, s, bin_of(key_of(v), L));
+      }
+      __syncwarp();
+    });
   return total;
 }
 
@@ -2207,9 +2287,9 @@ __global__ void __maxnreg__(72) k_fold(const __grid_constant__ Workspace ws, con
         const uint32_t bound = __ldcg(a.blk_max + b);
         uint32_t s = S == 1 ? 0u : __ldg(ws.blk_seg + b);
         uint32_t L = a.L_in[s];
-        if (S > 1) {   // the lowest bound of the layers that have a part of the block
+        if (S > 1) {   // the lowest bound of the layers that have a part of the block (read in any case if there are many)
           const uint64_t end = (uint64_t)(b + 1) * kWarpTile;
-          while (s + 1 < S && __ldg(ws.seg_off + s + 1) < end) L = min(L, a.L_in[++s]);
+          for (int j = 0; j < 4 && L && s + 1 < S && __ldg(ws.seg_off + s + 1) < end; ++j) L = j < 3 ? min(L, a.L_in[++s]) : 0u;
         }
         on = bound >= L;
       }
@@ -2380,12 +2460,11 @@ __global__ void __maxnreg__(72) k_fold(const __grid_constant__ Workspace ws, con
           ws.cand_idx[pos] = base + off;
           ws.cand_val[pos] = c;
           ++pos;
-          const uint32_t bin = bin_of(key_of(c), L);
-          atomicAdd(seg == main_seg ? sh.hist + bin : ws.hist1 + (size_t)seg * kBins1 + bin, 1u);
+          count_bin(ws, sh.hist, main_seg, seg, bin_of(key_of(c), L));
         }
       }
     } else {
-      cands += scan_mixed<SCAN>(ws, a, t, base, seg, slot0 + cands, top);
+      cands += scan_mixed<SCAN>(ws, a, t, base, seg, slot0 + cands, main_seg, sh.hist, top);
       top = __reduce_max_sync(kFull, top);
     }
     if (lane == 0) a.blk_max[blk] = top;     // the block's bound is exact again (entries sent later only lower it)
