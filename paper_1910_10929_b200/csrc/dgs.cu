@@ -580,12 +580,18 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
   const uint32_t advisers = std::min<uint32_t>(32u, (c->cfg.num_segments + 2 * kWarps - 1) / (2 * kWarps));
   const uint64_t keep = finalize_keep(c->cfg.num_segments > 1);
   const uint64_t cands = (uint64_t)a.pkt_count + a.pkt_count / 4 * 3 + 64ull * c->cfg.num_segments;
-  const int fin_grid = (int)std::min<uint64_t>(std::min(c->finalize_max[MODE], c->alone ? 2 * c->sms : c->sms) - (int)advisers,
-                                               std::max<uint64_t>(kFinalizeMin, (cands + kThreads * keep - 1) / (kThreads * keep)));
+  uint64_t want = std::max<uint64_t>(kFinalizeMin, (cands + kThreads * keep - 1) / (kThreads * keep));
+  // Beside other kernels an eighth of that, but not fewer than 48: what its CTAs hold is taken from the passes, which have
+  // the bytes to move, and a selection that takes longer only waits for its turn later.  Rounds of 32 arrivals, ms, with as many
+  // as keep the candidates (one per SM at most) / 100 / 50 / 24: 11.7 M elements in 62 layers: 3.09 / 2.94 / 2.85 / 2.92; 124 M:
+  // 11.57 / 11.31 / 11.25 / 11.23; 8 arrivals on 124 M in 148 layers: 2.91 / 2.86 / 2.85 / 2.87.
+  if (!c->alone) want = std::min(want, std::max<uint64_t>(48, want / 8));
+  const uint64_t most = (uint64_t)(std::min(c->finalize_max[MODE], c->alone ? 2 * c->sms : c->sms) - (int)advisers);
+  const int fin_grid = (int)std::min(most, want);
   // More candidates than the registers of all CTAs hold: k_finalize<.., BIG>, but beside other kernels only for one layer
   // and fifty times as many (runs of 32 events on 8.4 M elements, us an event without / with: one layer, 10 %, 20 times as
   // many: 153 / 156; 50 %, 97 times: 823 / 733; 60 layers, 50 %: 750 / 818).
-  const uint64_t held = (uint64_t)fin_grid * kThreads * keep;
+  const uint64_t held = (c->alone ? (uint64_t)fin_grid : most) * kThreads * keep;
   const bool big = c->alone ? cands > held : c->cfg.num_segments == 1 && cands > 50 * held;
   a.workers = (uint32_t)fin_grid;
   a.advisers = advisers;
