@@ -499,10 +499,10 @@ int fold_launch(dgs_ctx* c, const Workspace& ws, const SelArgs& a, uint32_t q, c
   const uint32_t first = (uint32_t)(c->applied[q] % c->log.ring);
   const uint32_t count = (uint32_t)(c->log_head - c->applied[q]);   // <= ring
   TimedLaunch tl(c, st, SCAN ? DGS_KERNEL_STREAM_PULL : DGS_KERNEL_CATCH_UP);
-  // Half the warps where several events share the GPU (a worker has one pull at a time, so it takes more than two workers).
+  // Fewer warps where several events share the GPU (a worker has one pull at a time, so it takes more than two workers).
   // Eight / four warps a CTA, us an event in runs of 256: 2 workers, 8.4 M elements: 36 / 40, 62 layers of 11.7 M: 95 / 101;
   // 3 workers, 25.6 M: 66 / 63; 8 workers: 61 / 57, 62 layers of 11.7 M: 83 / 78.
-  const uint32_t warps = c->alone || c->cfg.num_workers <= 2 ? kFoldWarps : kFoldWarps / 2;
+  const uint32_t warps = c->alone || c->cfg.num_workers <= 2 ? kFoldWarps : kFoldWarpsBeside;
   k_fold<SCAN><<<c->fold_grid, warps * 32, fold_dyn_bytes(warps, c->fold_ahead, ws.part_cap), st>>>(
       ws, a, c->log, first, count, (uint32_t)(c->applied[q] % (c->log.ring + 1)), (uint32_t)(c->log_head % (c->log.ring + 1)),
       c->fold_ahead);

@@ -37,7 +37,8 @@ constexpr uint32_t kFull = 0xFFFFFFFFu;
 constexpr uint32_t kSpecSlack = 64; // a carried bound aims at max(1.5 k, k + 64) candidates next time
 constexpr int kMaxGrid = 512;       // upper bound on the grid of a stream pass (= parts of the candidate buffer)
 constexpr int kMaxFoldGrid = 320;   // upper bound on the grid of a pull's pass (every warp of it is a part)
-constexpr int kMaxParts = kMaxFoldGrid * kWarps;   // upper bound on the parts of the candidate buffer
+constexpr int kFoldWarps = 10;      // most warps of a CTA of a pull's pass
+constexpr int kMaxParts = (kMaxFoldGrid * kFoldWarps + 255) / 256 * 256;   // upper bound on the parts of the candidate buffer (a multiple of kThreads)
 constexpr uint32_t kFoldSlack = 64; // part_cap is at least that much longer than a CTA's share (its tables round to groups and words)
 constexpr int kMaxWorkers = 320;    // upper bound on the grid of finalize
 constexpr uint32_t kSpinLimit = 1u << 22;  // bounded waits: give up and report after this many polls
@@ -2017,15 +2018,18 @@ __global__ void __launch_bounds__(kThreads) k_apply_log(const uint32_t* __restri
 // Blocks are skipped when no packet has an entry in them and (SCAN) their bound lies below L.  The blocks of a CTA
 // that are left are dealt out to its warps in eight runs of about equal cost; a warp is a part of the candidate
 // buffer, so the candidates are in index order without any barrier between the warps.
-// What bounds it is the chain of a block (positions -> entries -> subtract -> scan) times the blocks of a warp, so the
-// grid is two CTAs per SM.  Measured alone, in place of a catch-up by ranges of the log followed by the pull's own
+// What bounds it is the warps' instructions: about 300 for a block without entries, 600 with 20 of them, one after the other,
+// at half of the issue rate with 16 warps on an SM.  (More blocks of a warp on their way do not help: three or four instead
+// of two: 2^26 elements without entries 74 and 84 us for 75.)  So the grid is two CTAs per SM, with ten warps each where
+// the pull has the GPU to itself.  Eight / ten / twelve warps, alone: 2^26 elements without entries 73 / 67 / 67 us; 11.7 M in 62
+// layers with 3.7 M entries 75 / 60 / 66; 124 M in 148 layers, 8 packets 122 / 111 / 106; 25.6 M 22.3 / 20.7 / 20.3.  Measured alone, in place of a catch-up by ranges of the log followed by the pull's own
 // pass over D: 11.7 M elements in 62 layers, 3.7 M entries of 32 packets: 92 us for 272 + 62; 25.6 M elements, 0.8 M
 // entries: 46 us for 78 + 28; 124 M elements, 4.0 M entries: 220 us for 434 + 211.
-// The grid is the same whether a CTA has kFoldWarps warps or half as many, and so is the plan for it: a pull that has
-// the GPU to itself takes the full number, one that shares it with the push passes of later events the half (a round
-// of 32 arrivals on 124 M elements: 12.6 ms with four warps, 13.7 ms with eight, whose buffers and threads slow the
-// pushes down; one arrival at a time on 25.6 M elements with 8 workers: 196 us with eight, 210 us with four).
-constexpr int kFoldWarps = kWarps;
+// The grid is the same whether a CTA has kFoldWarps warps or fewer, and so is the plan for it: a pull that has
+// the GPU to itself takes the full number, one that shares it with the push passes of later events four (a round
+// of 32 arrivals on 124 M elements: 11.6 ms with four warps, 11.7 ms with eight and 12.7 ms with two, whose buffers and threads
+// slow the pushes down; one arrival at a time on 25.6 M elements with 8 workers: 127 us with ten, 129 us with eight).
+constexpr int kFoldWarpsBeside = 4;
 struct FoldStage {                  // one block of one warp
   float tile[kWarpTile];
   uint2 runs[32];                   // the packets with entries in the block, in order, see BlockRuns
@@ -2258,9 +2262,13 @@ __global__ void __maxnreg__(72) k_fold(const __grid_constant__ Workspace ws, con
 
   // this CTA's blocks [b0, b1)
   uint32_t b0 = part_first_tile(cta, G, NB), b1 = part_first_tile(cta + 1, G, NB);
-  if (SCAN && ws.plan != nullptr && ld_volatile(ws.sync + kPlanParts) == G && __ldcg(ws.plan + G) == NB) {
-    b0 = __ldcg(ws.plan + cta);
-    b1 = __ldcg(ws.plan + cta + 1);
+  if (SCAN && ws.plan != nullptr) {            // (one trip)
+    const uint32_t of = ld_volatile(ws.sync + kPlanParts), end = __ldcg(ws.plan + G);
+    const uint32_t p0 = __ldcg(ws.plan + cta), p1 = __ldcg(ws.plan + cta + 1);
+    if (of == G && end == NB) {
+      b0 = p0;
+      b1 = p1;
+    }
   }
   const uint32_t mine = b0 < b1 ? b1 - b0 : 0u, words = (mine + 31u) / 32u;   // words of `live`
 
@@ -2327,7 +2335,7 @@ __global__ void __maxnreg__(72) k_fold(const __grid_constant__ Workspace ws, con
       all += sh.warp_sum[w];                     // < 2^32 / 8: a share has fewer than 2^20 blocks
     }
     // first warp whose run begins in this thread's blocks or later: the smallest k with k all / nw >= at
-    uint32_t k = sum ? (uint32_t)(((uint64_t)at * nw + all - 1) / all) : nw;
+    uint32_t k = sum ? (at * nw + all - 1) / all : nw;     // (below 2^32: nw <= 10, and a block costs at most 255)
     while (k > 0 && sum && (k - 1) * all / nw >= at) --k;
     while (k < nw && k * all / nw < at) ++k;
     if (sum && k < nw && k * all / nw < at + sum) {
