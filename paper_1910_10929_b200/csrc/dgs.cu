@@ -574,12 +574,13 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
   a.L_next = c->L_next(KIND, next_copy, worker);
   a.slack = c->at<uint32_t>(c->lay.slack) + (uint64_t)KIND * c->cfg.num_segments;
   a.force_two_pass = single_pass ? 0 : 1;
-  // CTAs of finalize: as many as keep the candidates (about 1.7 times the entries) in the threads' registers, but not
-  // fewer than 32, since every step of a warp is a chain, and no more than one per SM (see k_finalize).  A warp per two
-  // layers for the advice.
+  // CTAs of finalize: as many as keep the candidates in the threads' registers, but not fewer than 32, since every step of a
+  // warp is a chain, and no more than two per SM.  There are 2 to 4 times as many candidates as entries; where the kernel has
+  // the GPU to itself it is sized for 3 (one arrival at a time on 25.6 M elements: 128.5 us sized for 1.75, 123 for 3; on 11.7 M
+  // in 62 layers its two finalize kernels take 28 and 31 us instead of 34 and 36).  A warp per two layers for the advice.
   const uint32_t advisers = std::min<uint32_t>(32u, (c->cfg.num_segments + 2 * kWarps - 1) / (2 * kWarps));
   const uint64_t keep = finalize_keep(c->cfg.num_segments > 1);
-  const uint64_t cands = (uint64_t)a.pkt_count + a.pkt_count / 4 * 3 + 64ull * c->cfg.num_segments;
+  const uint64_t cands = (c->alone ? 3ull * a.pkt_count : (uint64_t)a.pkt_count + a.pkt_count / 4 * 3) + 64ull * c->cfg.num_segments;
   uint64_t want = std::max<uint64_t>(kFinalizeMin, (cands + kThreads * keep - 1) / (kThreads * keep));
   // Beside other kernels an eighth of that, but not fewer than 48: what its CTAs hold is taken from the passes, which have
   // the bytes to move, and a selection that takes longer only waits for its turn later.  Rounds of 32 arrivals, ms, with as many
