@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "dgs_kernels.cuh"
+#include "dgs_one.cuh"
 #include "dgs_topk.cuh"
 
 using namespace dgs;
@@ -52,6 +53,8 @@ constexpr int kQueuesWanted = 12;         // hardware queues for the streams of 
 constexpr int kLogRingMax = 128;            // most packets the apply log keeps
 constexpr int kLogSlack = 32;               // slots of the log beyond one per worker
 constexpr uint64_t kListCap = 4096;         // most entries of a layer's list of candidates in the k-th's bin
+constexpr uint64_t kOneMaxN = 3ull << 19;   // longest vector whose selections are one kernel each
+constexpr uint32_t kOneGridBeside = 64;     // most CTAs of that kernel beside other events
 
 inline uint64_t align_up(uint64_t x, uint64_t a) { return (x + a - 1) / a * a; }
 
@@ -280,6 +283,8 @@ struct dgs_ctx {
   // that waits): the event in hand starts on an idle GPU.
   bool alone;
   int hist_grid[3];      // CTAs of the whole-input histogram pass, per mode
+  int one_max[3];        // most CTAs of pass and finalize in one kernel, per mode
+  uint32_t pair[kSets];  // pair of sync words that the last selection on each scratch set has used
   int finalize_max[3];   // most CTAs of the cooperative finalize kernel that can be resident at once, per mode
   uint64_t whole_layers;  // elements of layers that may be candidates as a whole (several layers)
   uint64_t kind_seq[2];  // selections of each kind launched so far
@@ -495,18 +500,24 @@ void catch_up_deps(const dgs_ctx* c, uint32_t q, Task* t) {
 }
 // The launch itself, on a stream that task_begin has prepared with those dependencies: the filed packets that D_q
 // has not seen yet, and with SCAN the stream pass of a pull in the same trip over D_q.
+FoldRange fold_range(const dgs_ctx* c, uint32_t q) {
+  const uint32_t ring = c->log.ring;
+  FoldRange f;
+  f.first = (uint32_t)(c->applied[q] % ring);
+  f.count = (uint32_t)(c->log_head - c->applied[q]);   // <= ring
+  f.row0 = (uint32_t)(c->applied[q] % (ring + 1));
+  f.row1 = (uint32_t)(c->log_head % (ring + 1));
+  f.ahead = c->fold_ahead;
+  return f;
+}
 template <bool SCAN>
 int fold_launch(dgs_ctx* c, const Workspace& ws, const SelArgs& a, uint32_t q, cudaStream_t st) {
-  const uint32_t first = (uint32_t)(c->applied[q] % c->log.ring);
-  const uint32_t count = (uint32_t)(c->log_head - c->applied[q]);   // <= ring
   TimedLaunch tl(c, st, SCAN ? DGS_KERNEL_STREAM_PULL : DGS_KERNEL_CATCH_UP);
   // Fewer warps where several events share the GPU (a worker has one pull at a time, so it takes more than two workers).
   // Eight / four warps a CTA, us an event in runs of 256: 2 workers, 8.4 M elements: 36 / 40, 62 layers of 11.7 M: 95 / 101;
   // 3 workers, 25.6 M: 66 / 63; 8 workers: 61 / 57, 62 layers of 11.7 M: 83 / 78.
   const uint32_t warps = c->alone || c->cfg.num_workers <= 2 ? kFoldWarps : kFoldWarpsBeside;
-  k_fold<SCAN><<<c->fold_grid, warps * 32, fold_dyn_bytes(warps, c->fold_ahead, ws.part_cap), st>>>(
-      ws, a, c->log, first, count, (uint32_t)(c->applied[q] % (c->log.ring + 1)), (uint32_t)(c->log_head % (c->log.ring + 1)),
-      c->fold_ahead);
+  k_fold<SCAN><<<c->fold_grid, warps * 32, fold_dyn_bytes(warps, c->fold_ahead, ws.part_cap), st>>>(ws, a, c->log, fold_range(c, q));
   DGS_CUDA(c, cudaGetLastError());
   c->launches += 1;
   c->applied[q] = c->log_head;
@@ -556,6 +567,10 @@ const void* finalize_kernel(const dgs_ctx* c, bool big) {
   return big ? (const void*)k_finalize<MODE, false, true> : (const void*)k_finalize<MODE, false, false>;
 }
 
+uint32_t one_bytes(const dgs_ctx* c, int mode) {
+  return one_dyn_bytes(mode, c->cfg.num_segments, c->fold_ahead, c->ws[0].part_cap);
+}
+
 template <int MODE>
 int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age, int stream_id, Task& task) {
   constexpr int KIND = MODE == kPull ? 1 : 0;
@@ -601,6 +616,21 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
   a.workers = (uint32_t)fin_grid;
   a.advisers = advisers;
   a.fold_grid = MODE == kPull ? (uint32_t)c->fold_grid : 0u;   // one CTA more plans the next pull's pass
+  // Short vectors: pass and finalize in one kernel.  Beside other events the host is what such vectors wait for, 3 us a launch
+  // (rounds of 12 arrivals on 409 K elements: 205 us with two kernels a selection, 164 with one; of 27 on 131 K: 471, 391; of 28
+  // on 880 K, 1.4 %: 494, 452; but 2^21 elements: 20 us an event with two, 27 with one).  Alone it is the GPU, and only a pull of
+  // one layer gains: its pass takes little longer with half of the CTAs (2^20 elements: pull 22.3 / 19.6 us, push 19.6 / 20.2;
+  // in 60 layers 40 / 42 and 31 / 34).  While launches are timed each kernel stays on its own.
+  const uint32_t others = advisers + (MODE == kPull ? 1u : 0u);
+  uint32_t one_grid = std::min<uint32_t>(c->alone ? kOneMaxGrid : kOneGridBeside, (c->lay.num_blocks + kWarps - 1) / kWarps);
+  one_grid = std::min<uint32_t>(std::max<uint32_t>(one_grid, (uint32_t)kFinalizeMin + others), (uint32_t)c->one_max[MODE]);
+  const bool one = c->cfg.n <= kOneMaxN && (c->alone ? MODE == kPull && c->cfg.num_segments == 1 : true) && !big && !c->timing &&
+                   one_grid > others && (c->lay.num_blocks + one_grid - 1) / one_grid + kFoldSlack <= ws.part_cap;
+  if (one) {
+    a.workers = std::min<uint32_t>(a.workers, one_grid - others);
+    if (MODE == kPull) a.fold_grid = one_grid;
+  }
+  a.pair = c->pair[stream_id] ^= 1u;
   a.packet_format = packet_format_of(c);
   if (c->cfg.flags & DGS_TEST_STALLED_BARRIER) {
     a.phantom_workers = 1;
@@ -628,16 +658,23 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
     DGS_CUDA(c, cudaGetLastError());
     c->launches += 2;
   }
-  if constexpr (MODE == kPull) {
+  if (one) {
+    FoldRange f = MODE == kPull ? fold_range(c, worker) : FoldRange{};
+    void* args[] = {(void*)&ws, (void*)&a, (void*)&c->log, (void*)&f};
+    DGS_CUDA(c, cudaLaunchCooperativeKernel(one_kernel(MODE, c->cfg.num_segments > 1), dim3(one_grid), dim3(kThreads), args,
+                                            one_bytes(c, MODE), st));
+    c->launches += 1;
+    if (MODE == kPull) c->applied[worker] = c->log_head;
+  } else if constexpr (MODE == kPull) {
     rc = fold_launch<true>(c, ws, a, worker, st);
     if (rc != DGS_OK) return rc;
   } else {
     TimedLaunch t(c, st, DGS_KERNEL_STREAM_PUSH);
-    k_stream<MODE><<<c->stream_grid[MODE], kThreads, StreamRing::kBytes, st>>>(ws, a);
+    k_stream<MODE><<<c->stream_grid[MODE], kThreads, PushRing::kBytes, st>>>(ws, a);
     DGS_CUDA(c, cudaGetLastError());
     c->launches += 1;
   }
-  {
+  if (!one) {
     // cooperative launch: the CTAs synchronise among themselves, so all must be resident
     TimedLaunch t(c, st, MODE == kPull ? DGS_KERNEL_FINALIZE_PULL : DGS_KERNEL_FINALIZE_PUSH);
     void* args[] = {(void*)&ws, (void*)&a};
@@ -657,12 +694,30 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
   return DGS_OK;
 }
 
+// Grid of k_fold and the room for its tables and buffers.
+constexpr int kFoldMaxDyn = 208 * 1024;   // beside its static shared memory
+int fold_setup(dgs_ctx* c, int sms) {
+  c->fold_grid = (int)std::min<uint32_t>((c->lay.num_blocks + 7) / 8, (uint32_t)std::min(2 * sms, kMaxFoldGrid));
+  // A quarter more than the mean number of entries of a block, for a worker that has missed a packet per worker.
+  const uint64_t mean = std::min<uint64_t>(c->cfg.num_workers, 32) * c->lay.K[0] * kWarpTile / c->cfg.n;
+  c->fold_ahead = (uint32_t)std::min<uint64_t>(192, std::max<uint64_t>(64, align_up(mean + mean / 4, 64)));
+  // Eight even shares: where most of the vector is cold, the shares of the CTAs that have only cold blocks grow
+  // (a share never gets longer than an even one without a plan).
+  const uint32_t even = (c->lay.num_blocks + c->fold_grid - 1) / c->fold_grid + kFoldSlack;
+  const uint32_t cap = (uint32_t)align_up(std::max<uint32_t>(even, std::min<uint32_t>(32768u, 8 * even)), 128);
+  for (int k = 0; k < kSets; ++k) c->ws[k].part_cap = cap;
+  DGS_CUDA(c, cudaFuncSetAttribute(k_fold<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFoldMaxDyn));
+  DGS_CUDA(c, cudaFuncSetAttribute(k_fold<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFoldMaxDyn));
+  if (fold_dyn_bytes(kFoldWarps, c->fold_ahead, cap) > (uint32_t)kFoldMaxDyn) return DGS_EINVAL;   // (n < 2^32 keeps an even share well below)
+  return DGS_OK;
+}
+
 template <int MODE>
 int occupancy_grids(dgs_ctx* c, int sms) {
   int occ = 0;
   if constexpr (MODE != kPull) {
-    DGS_CUDA(c, cudaFuncSetAttribute(k_stream<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, StreamRing::kBytes));
-    DGS_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_stream<MODE>, kThreads, StreamRing::kBytes));
+    DGS_CUDA(c, cudaFuncSetAttribute(k_stream<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, PushRing::kBytes));
+    DGS_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_stream<MODE>, kThreads, PushRing::kBytes));
     if (occ < 1) occ = 1;
     c->stream_grid[MODE] = std::min(sms * occ, kMaxGrid);
   }
@@ -681,24 +736,13 @@ int occupancy_grids(dgs_ctx* c, int sms) {
     c->finalize_max[MODE] = std::min(c->finalize_max[MODE], sms * occ);
   }
   if (MODE == kPull) c->finalize_max[MODE] -= 1;   // the CTA that plans the next pass
-  return DGS_OK;
-}
-
-// Grid of k_fold and the room for its tables and buffers.
-constexpr int kFoldMaxDyn = 208 * 1024;   // beside its static shared memory
-int fold_setup(dgs_ctx* c, int sms) {
-  c->fold_grid = (int)std::min<uint32_t>((c->lay.num_blocks + 7) / 8, (uint32_t)std::min(2 * sms, kMaxFoldGrid));
-  // A quarter more than the mean number of entries of a block, for a worker that has missed a packet per worker.
-  const uint64_t mean = std::min<uint64_t>(c->cfg.num_workers, 32) * c->lay.K[0] * kWarpTile / c->cfg.n;
-  c->fold_ahead = (uint32_t)std::min<uint64_t>(192, std::max<uint64_t>(64, align_up(mean + mean / 4, 64)));
-  // Eight even shares: where most of the vector is cold, the shares of the CTAs that have only cold blocks grow
-  // (a share never gets longer than an even one without a plan).
-  const uint32_t even = (c->lay.num_blocks + c->fold_grid - 1) / c->fold_grid + kFoldSlack;
-  const uint32_t cap = (uint32_t)align_up(std::max<uint32_t>(even, std::min<uint32_t>(32768u, 8 * even)), 128);
-  for (int k = 0; k < kSets; ++k) c->ws[k].part_cap = cap;
-  DGS_CUDA(c, cudaFuncSetAttribute(k_fold<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFoldMaxDyn));
-  DGS_CUDA(c, cudaFuncSetAttribute(k_fold<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFoldMaxDyn));
-  if (fold_dyn_bytes(kFoldWarps, c->fold_ahead, cap) > (uint32_t)kFoldMaxDyn) return DGS_EINVAL;   // (n < 2^32 keeps an even share well below)
+  c->one_max[MODE] = 0;
+  if (c->cfg.n <= kOneMaxN && one_bytes(c, MODE) <= (uint32_t)kFoldMaxDyn) {
+    const void* const f = one_kernel(MODE, c->cfg.num_segments > 1);
+    DGS_CUDA(c, cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kFoldMaxDyn));
+    DGS_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f, kThreads, one_bytes(c, MODE)));
+    c->one_max[MODE] = std::min(kOneMaxGrid, sms * occ);
+  }
   return DGS_OK;
 }
 
@@ -788,6 +832,7 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
   c->base = static_cast<char*>(cfg->arena);
   c->user = c->st[kCaller] = static_cast<cudaStream_t>(cfg->stream);
   c->push_count = 0;
+  for (uint32_t& p : c->pair) p = 0;
   c->inv_m = 1.0f / cfg->momentum;  // one IEEE division; the kernels multiply by this constant
   c->timestamp = 0;
   c->launches = 0;
@@ -824,8 +869,8 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
   INIT_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
   if (!coop) return fail(DGS_ECUDA);
   c->sms = sms;
-  if (occupancy_grids<kPushSam>(c, sms) != DGS_OK || occupancy_grids<kPushResidual>(c, sms) != DGS_OK ||
-      occupancy_grids<kPull>(c, sms) != DGS_OK || fold_setup(c, sms) != DGS_OK)
+  if (fold_setup(c, sms) != DGS_OK || occupancy_grids<kPushSam>(c, sms) != DGS_OK || occupancy_grids<kPushResidual>(c, sms) != DGS_OK ||
+      occupancy_grids<kPull>(c, sms) != DGS_OK)
     return fail(DGS_ECUDA);
   INIT_CUDA(cudaEventCreateWithFlags(&c->ev_in, cudaEventDisableTiming));
   if (stream_ready(c, 0) != DGS_OK) return fail(DGS_ECUDA);

@@ -74,7 +74,9 @@ struct LayerPick {     // finalize: what a CTA knows of a layer that its candida
 };
 
 // word indices in Workspace::sync
-enum SyncWord : int { kBarCount = 0, kFail = 3, kParts = 4, kPlanParts = 5, kNumSyncWords = 8 };
+// (the barrier's count and the flags of layers whose guesses failed: two pairs, which the selections on a scratch set take in
+// turn, see SelArgs::pair)
+enum SyncWord : int { kBarCount = 0, kFail = 2, kParts = 4, kPlanParts = 5, kNumSyncWords = 8 };
 
 struct Workspace {
   const Tile* tiles;
@@ -130,6 +132,7 @@ struct SelArgs {
   uint32_t workers;       // CTAs of finalize that process the candidates
   uint32_t advisers;      // further ones that check the guesses and suggest the next bounds
   uint32_t seq;           // selections of this kind launched before
+  uint32_t pair;          // which of the two pairs of sync words this selection uses: 0 or 1, the one before it used the other
   uint32_t fold_grid;     // pull: CTAs of the pass before this finalize (0: it was not k_fold, nothing to plan)
   uint32_t phantom_workers;  // testing only: CTAs the finalize barrier waits for beyond those launched (0 in normal use)
   uint32_t spin_limit;    // polls after which a bounded wait gives up (0: kSpinLimit)
@@ -536,9 +539,10 @@ __device__ __forceinline__ uint32_t tile_mask_smem(const SelArgs& a, uint32_t ti
 // which the stage of the round before is free, so a ring of kStages stages keeps kStages - 1
 // of them in flight.
 constexpr int kStageFloats = kWarps * kWarpTile;           // per input array: one block per warp and stage
-// The ring: three stages (96 KB, two CTAs per SM, 128 KB of the SM's shared memory in flight).
+// The ring: three stages (96 KB, two CTAs per SM, 128 KB of the SM's shared memory in flight); two where the pass is short.
+template <int STAGES>
 struct StreamRing {
-  static constexpr int kStages = 3;
+  static constexpr int kStages = STAGES;
   static constexpr int kStageBytes = 2 * kStageFloats * 4;                // 16 KB per input
   static constexpr int kBytes = kStages * kStageBytes;
 };
@@ -648,11 +652,10 @@ __device__ __noinline__ void mixed_emit(const Workspace& ws, const SelArgs& a, c
 // those of others straight in global memory.  (A layer at a time, the ring restarted and the histogram flushed for each and
 // one warp at work on its ragged ends, 11.7 M elements in 62 layers took 54 us, and the CTAs with the small layers 58 us where
 // the others took 24; now 37 us.)
-template <int MODE>
+template <int MODE, typename R>
 __device__ void stream_blocks_tma(const Workspace& ws, const SelArgs& a, const uint32_t* Larr, const float* __restrict__ in,
                                   float* __restrict__ out, uint32_t cta, uint32_t G, StreamShared& sh, float* ring, uint64_t* full,
                                   int* s_dead) {
-  using R = StreamRing;
   static_assert(MODE != kPull, "a pull's pass is k_fold");
   static_assert(R::kStages >= 2, "the ring needs a stage in flight besides the one being read");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -884,7 +887,7 @@ __device__ __forceinline__ void number_parts(const Workspace& ws, uint32_t parts
 
 // From the histogram of a whole layer (top 11 key bits; cleared here): L_safe = lower edge of the bin holding the k-th
 // largest key, L_wide = a bound that admits about max(1.5 k, k+64) entries.  By one CTA.
-__device__ void pick_lower(const Workspace& ws, uint32_t s, uint32_t k, unsigned long long* s_warp, uint32_t* s_res) {
+static __device__ void pick_lower(const Workspace& ws, uint32_t s, uint32_t k, unsigned long long* s_warp, uint32_t* s_res) {
   uint32_t bin, krem, wbin = 0, wrem = 0;
   uint32_t* const h = ws.hist1 + (size_t)s * kBins1;
   const uint32_t want = spec_want(k), total = block_pick<kBins1>(h, k, bin, krem, s_warp, s_res);
@@ -900,18 +903,18 @@ __device__ void pick_lower(const Workspace& ws, uint32_t s, uint32_t k, unsigned
 
 // Barrier among the CTAs of finalize (all resident: cooperative launch).  One arrival
 // counter that only grows: the i-th barrier of a launch is passed when the counter has
-// reached i*W (the stream pass that precedes every finalize launch clears the counter).
+// reached i*W (it is cleared by the pass before finalize, or, where both are one kernel, by the selection before).
 // Bounded: returns false, with the status word set, if the others do not arrive.
-__device__ bool worker_barrier(uint32_t* sync, uint32_t W, int* status, int* s_ok, uint32_t& target,
+static __device__ bool worker_barrier(uint32_t* count, uint32_t W, int* status, int* s_ok, uint32_t& target,
                                uint32_t limit = kSpinLimit) {
   target += W;
   __syncthreads();
   if (threadIdx.x == 0) {
     int ok = 1;
     __threadfence();
-    atomicAdd(sync + kBarCount, 1u);
+    atomicAdd(count, 1u);
     uint32_t spins = 0;
-    while ((int32_t)(ld_volatile(sync + kBarCount) - target) < 0) {
+    while ((int32_t)(ld_volatile(count) - target) < 0) {
       if (++spins > limit) {
         ok = 0;
         atomicMin(status, kStatusTimeout);
@@ -952,7 +955,7 @@ constexpr int kTouch = 40;      // layers of a CTA whose picks fit in shared mem
 
 constexpr int kListSmem = kThreads;    // entries of the list that are ranked in shared memory (one layer)
 template <int MAXPARTS>
-struct FinalizeShared {
+struct __align__(16) FinalizeShared {
   StreamShared stream;                 // redo of the passes (guess failed); its histogram also serves the warps' radix steps
   unsigned long long warp_scan[kWarps];
   uint32_t res[3];
@@ -1083,7 +1086,7 @@ __device__ __forceinline__ uint32_t next_bound(const Workspace& ws, uint32_t s, 
 
 // The k-th largest of the `pop` keys of a list, all of them in [base, base + 2^bits), by one warp; hist: 128 words of
 // shared memory of its own.  Returns T and, in r, how many of the keys equal to T are among the k.
-__device__ __noinline__ uint32_t warp_radix(const uint2* list, uint32_t pop, uint32_t k, uint32_t base, int bits, uint32_t* hist,
+static __device__ __noinline__ uint32_t warp_radix(const uint2* list, uint32_t pop, uint32_t k, uint32_t base, int bits, uint32_t* hist,
                                                int lane, uint32_t& r) {
   if (pop <= 32u) {                              // ranks by comparing with every other key
     const uint32_t key = (uint32_t)lane < pop ? __ldcg(&list[lane].x) : 0u;
@@ -1142,7 +1145,9 @@ __device__ __noinline__ uint32_t warp_radix(const uint2* list, uint32_t pop, uin
 // about the same, judged by what this pass cost each CTA.  What has to be read and folded in clusters in the
 // tensors with the largest updates, and those are the same for every worker; with equal ranges a few CTAs do most
 // of the work.  Done by a CTA of its own beside the finalize, so that it adds nothing to the chain.
-__device__ void plan_parts(const Workspace& ws, uint32_t G, FinalizeShared<kMaxParts>& sh) {
+template <int MAXPARTS>
+__device__ void plan_parts(const Workspace& ws, uint32_t G, FinalizeShared<MAXPARTS>& sh) {
+  static_assert(MAXPARTS >= 512 + kMaxFoldGrid, "two tables in the place of the parts");
   uint32_t* const before = sh.pre;             // [G] cost of the CTAs before this one
   uint32_t* const first = sh.pre + 512;        // [G + 1] where they began
   uint32_t* const cost = sh.stream.hist;       // [G]
@@ -1208,10 +1213,10 @@ __device__ __noinline__ bool redo_passes(const Workspace& ws, const SelArgs& a, 
                                          unsigned long long* s_warp, uint32_t* s_res, int* s_ok, uint32_t Wb, uint32_t spin_limit,
                                          uint32_t& bar_target) {
   const uint32_t cta = blockIdx.x, G = a.workers + a.advisers, S = ws.num_segs;
-  auto barrier = [&]() { return worker_barrier(ws.sync, Wb, ws.status, s_ok, bar_target, spin_limit); };
+  auto barrier = [&]() { return worker_barrier(ws.sync + kBarCount + a.pair, Wb, ws.status, s_ok, bar_target, spin_limit); };
   for (size_t w = (size_t)cta * kThreads + threadIdx.x; w < (size_t)S * kBins1; w += (size_t)G * kThreads) ws.hist1[w] = 0;
   for (uint32_t s = cta * kThreads + threadIdx.x; s < S; s += G * kThreads) ws.list_cnt[s] = 0;
-  if (cta == 0 && threadIdx.x == 0) ws.sync[kFail] = 0;
+  if (cta == 0 && threadIdx.x == 0) ws.sync[kFail + a.pair] = 0;
   if (!barrier()) return false;
   hist_all_tiles<MODE>(ws, a, in, cta, G, st.hist);
   if (!barrier()) return false;
@@ -1225,7 +1230,7 @@ __device__ __noinline__ bool redo_passes(const Workspace& ws, const SelArgs& a, 
 }
 
 // The k-th largest of the `pop` keys of a list, all of them in [base, base + 2^bits), by the whole CTA; hist: 256 words.
-__device__ __noinline__ uint32_t block_radix(const uint2* list, uint32_t pop, uint32_t k, uint32_t base, int bits, uint32_t* hist,
+static __device__ __noinline__ uint32_t block_radix(const uint2* list, uint32_t pop, uint32_t k, uint32_t base, int bits, uint32_t* hist,
                                              uint32_t* s_res, uint32_t& r) {
   const int lane = threadIdx.x & 31;
   uint32_t prefix = 0;
@@ -1270,39 +1275,41 @@ __device__ __noinline__ uint32_t block_radix(const uint2* list, uint32_t pop, ui
 // of candidates in one part needs neither a search nor a trip for its place.  Finalize of a pull, us, before / with BIG:
 // 2^24 elements, 10 %: 128 / 95, 50 %: 878 / 497; 2^27, 10 %: 1447 / 815.  Beside other kernels its registers cost more
 // than it gains (62 layers of 8.4 M elements, 1 %, runs of 32 events: 65 us an event without, 79 with).
-template <int MODE, bool MANY, bool BIG>
-__global__ void __maxnreg__(BIG ? 96 : 64) k_finalize(const __grid_constant__ Workspace ws, const __grid_constant__ SelArgs a) {
-  constexpr int kPartCap = MODE == kPull ? kMaxParts : kMaxGrid;   // parts that the pass before, or a redo, can leave
-  __shared__ __align__(16) FinalizeShared<kPartCap> sh;
-  extern __shared__ __align__(16) unsigned char fin_dyn[];   // finalize_dyn_bytes(S) bytes
-
+// PASSED: in one kernel with the pass before it, all of whose CTAs come here; `bar_target`: their number.  in, out: the state
+// vector that the pass has read, and for a push the one that it has written.
+template <int MODE, bool MANY, bool BIG, int MAXPARTS, bool PASSED>
+__device__ __forceinline__ void finalize(const Workspace& ws, const SelArgs& a, const float* in, float* out,
+                                         FinalizeShared<MAXPARTS>& sh, unsigned char* fin_dyn, uint32_t bar_target) {
   constexpr int PM = MODE == kPull ? 1 : 0, kKeep = BIG ? 4 : finalize_keep(MANY);
   // CTAs [0, W) process the candidates, [W, W + A) look after the layers' bounds, and after k_fold one more plans the
   // next pass (it takes no part in the selection)
   const uint32_t cta = blockIdx.x, W = a.workers, A = a.advisers, S = ws.num_segs;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t gthread = cta * kThreads + threadIdx.x, nthreads = (W + A) * kThreads, lt = lanemask_lt(), le = lt | (1u << lane);
+  // the barrier counts W + A arrivals; a test can make it wait for CTAs that do not exist, with a short limit,
+  // to see the bounded wait give up (every CTA then leaves with DGS_ETIMEOUT in the status word)
+  const uint32_t Wb = W + A + a.phantom_workers, spin_limit = a.spin_limit ? a.spin_limit : kSpinLimit;
+  if (PASSED) {
+    if (cta >= W + A + (MODE == kPull ? 1u : 0u)) {      // nothing to do here: the others only wait for its pass
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(ws.sync + kBarCount + a.pair, 1u);
+      }
+      return;
+    }
+    const uint32_t all = bar_target + a.phantom_workers;
+    bar_target = 0;
+    if (!worker_barrier(ws.sync + kBarCount + a.pair, all, ws.status, &sh.ok, bar_target, spin_limit)) return;
+  }
   if constexpr (MODE == kPull) {
     if (cta == W + A) {
       plan_parts(ws, a.fold_grid, sh);
       return;
     }
   }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t gthread = cta * kThreads + threadIdx.x, nthreads = (W + A) * kThreads, lt = lanemask_lt(), le = lt | (1u << lane);
-  // the barrier counts W + A arrivals; a test can make it wait for CTAs that do not exist, with a short limit,
-  // to see the bounded wait give up (every CTA then leaves with DGS_ETIMEOUT in the status word)
-  const uint32_t Wb = W + A + a.phantom_workers, spin_limit = a.spin_limit ? a.spin_limit : kSpinLimit;
-  uint32_t bar_target = 0;
-  auto barrier = [&]() { return worker_barrier(ws.sync, Wb, ws.status, &sh.ok, bar_target, spin_limit); };
+  auto barrier = [&]() { return worker_barrier(ws.sync + kBarCount + a.pair, Wb, ws.status, &sh.ok, bar_target, spin_limit); };
 
-  // pointers are read once, before anything may exchange them
-  const float* in = nullptr;
-  float* out = nullptr;
-  if (MODE == kPull) {
-    in = a.D;
-  } else {
-    in = *a.u_cur_slot;
-    out = *a.u_spare_slot;
-  }
   const uint32_t* seg_off = ws.seg_off;
   if (MANY && S <= (uint32_t)kSegCap) {
     uint32_t* const sm = reinterpret_cast<uint32_t*>(fin_dyn);
@@ -1454,7 +1461,7 @@ __global__ void __maxnreg__(BIG ? 96 : 64) k_finalize(const __grid_constant__ Wo
         } else if (a.speculate && lane == 0) {
           a.slack[s] = min(slack + 4u, 16u);       // (selections in flight beside this one may write it too: it is advice)
         }
-        if (flag && lane == 0) atomicOr(ws.sync + kFail, flag);
+        if (flag && lane == 0) atomicOr(ws.sync + kFail + a.pair, flag);
         seen += total;
       }
       if (lane == 0 && seen) atomicAdd(ws.stats + 2, (unsigned long long)seen);
@@ -1462,7 +1469,7 @@ __global__ void __maxnreg__(BIG ? 96 : 64) k_finalize(const __grid_constant__ Wo
     } else {
       // flat numbering of the candidates (the stream pass is complete: an earlier kernel, or the barrier above)
       parts = ld_volatile(ws.sync + kParts);
-      number_parts<kPartCap>(ws, parts, sh.pre, sh.warp_scan);
+      number_parts<MAXPARTS>(ws, parts, sh.pre, sh.warp_scan);
       const uint32_t C = sh.pre[parts];
       const uint32_t per_warp = (uint32_t)(((uint64_t)C + W * kWarps * 32u - 1u) / (W * kWarps * 32u)) * 32u;
       clo = (uint32_t)min((uint64_t)C, (uint64_t)cta * kWarps * per_warp);
@@ -1586,7 +1593,7 @@ __global__ void __maxnreg__(BIG ? 96 : 64) k_finalize(const __grid_constant__ Wo
       __syncwarp();
     });
     if (!barrier()) return;
-    flags = ld_volatile(ws.sync + kFail);
+    flags = ld_volatile(ws.sync + kFail + a.pair);
     if (!(flags & 1u) || redo) break;
     if (!barrier()) return;              // everyone has seen the flags
     redo = true;
@@ -1842,6 +1849,17 @@ __global__ void __maxnreg__(BIG ? 96 : 64) k_finalize(const __grid_constant__ Wo
   }
 }
 
+template <int MODE, bool MANY, bool BIG>
+__global__ void __maxnreg__(BIG ? 96 : 64) k_finalize(const __grid_constant__ Workspace ws, const __grid_constant__ SelArgs a) {
+  constexpr int kPartCap = MODE == kPull ? kMaxParts : kMaxGrid;   // parts that the pass before, or a redo, can leave
+  __shared__ FinalizeShared<kPartCap> sh;
+  extern __shared__ __align__(16) unsigned char fin_dyn[];   // finalize_dyn_bytes(S) bytes
+  // pointers are read once, before anything may exchange them
+  const float* const in = MODE == kPull ? a.D : *a.u_cur_slot;
+  float* const out = MODE == kPull ? nullptr : *a.u_spare_slot;
+  finalize<MODE, MANY, BIG, kPartCap, false>(ws, a, in, out, sh, fin_dyn, 0u);
+}
+
 // ---- the two passes as kernels of their own, for a selection with nothing to go by -------
 template <int MODE>
 __global__ void __launch_bounds__(kThreads, 4) k_hist_all(Workspace ws, SelArgs a) {
@@ -1861,18 +1879,19 @@ __global__ void __launch_bounds__(kThreads) k_pick_lower(Workspace ws) {
   }
 }
 
+using PushRing = StreamRing<3>;
 // ---- stand-alone stream pass with the carried bound -------------------------------
 template <int MODE>
 __global__ void __maxnreg__(64) k_stream(const __grid_constant__ Workspace ws, const __grid_constant__ SelArgs a) {
   extern __shared__ __align__(128) unsigned char dyn_smem[];   // the ring of stages
   __shared__ StreamShared sh;
-  __shared__ __align__(8) uint64_t full[StreamRing::kStages];
+  __shared__ __align__(8) uint64_t full[PushRing::kStages];
   __shared__ int s_dead;
   const float* in = *a.u_cur_slot;
   float* out = *a.u_spare_slot;
-  if (blockIdx.x == 0 && threadIdx.x == 0) ws.sync[kBarCount] = ws.sync[kFail] = 0;   // for the finalize launch that follows
-  stream_blocks_tma<MODE>(ws, a, a.L_in, in, out, blockIdx.x, gridDim.x, sh, reinterpret_cast<float*>(dyn_smem), full,
-                          &s_dead);
+  if (blockIdx.x == 0 && threadIdx.x < 2) ws.sync[kBarCount + threadIdx.x] = ws.sync[kFail + threadIdx.x] = 0;   // for the finalize that follows
+  stream_blocks_tma<MODE, PushRing>(ws, a, a.L_in, in, out, blockIdx.x, gridDim.x, sh, reinterpret_cast<float*>(dyn_smem), full,
+                                    &s_dead);
 }
 
 // ---- pull without secondary compression: every nonzero entry of D_w -------------------
@@ -1881,7 +1900,7 @@ __global__ void __maxnreg__(64) k_stream(const __grid_constant__ Workspace ws, c
 // This kernel copies the first `capacity` of them into the packet, clears them in D_w (Eq. 4:
 // v_k becomes M), adds them to theta_w if kept (Eq. 5), and writes the count.
 constexpr int kStatusLimit = -6;   // = DGS_ELIMIT
-__global__ void __launch_bounds__(kThreads) k_emit_all(Workspace ws, float* __restrict__ D,
+static __global__ void __launch_bounds__(kThreads) k_emit_all(Workspace ws, float* __restrict__ D,
                                                        float* __restrict__ theta_local,
                                                        uint32_t* __restrict__ blk_max, uint32_t* __restrict__ out_idx,
                                                        float* __restrict__ out_val, uint32_t* __restrict__ out_count,
@@ -1967,7 +1986,7 @@ __device__ __forceinline__ uint32_t warp_lower_bound(const uint32_t* __restrict_
 // Each of the remaining CTAs finds where kThreads blocks of the vector begin in this packet: the packet's part that
 // falls into them is found by two searches, its entries are counted per block in shared memory, and a prefix sum
 // gives the positions.
-__global__ void __launch_bounds__(kThreads) k_apply_log(const uint32_t* __restrict__ idx,
+static __global__ void __launch_bounds__(kThreads) k_apply_log(const uint32_t* __restrict__ idx,
                                                         const float* __restrict__ val, uint32_t count,
                                                         float* __restrict__ theta, uint64_t n, int* status,
                                                         PacketLog lg, uint32_t slot, uint32_t row, uint32_t copy_ctas) {
@@ -2034,6 +2053,11 @@ struct FoldStage {                  // one block of one warp
   float tile[kWarpTile];
   uint2 runs[32];                   // the packets with entries in the block, in order, see BlockRuns
   uint2 ent[1];                     // [ahead] entries that are fetched while the block before is worked on
+};
+struct FoldRange {                  // what a pass folds in
+  uint32_t first, count;            // packets: first slot of the log, number
+  uint32_t row0, row1;              // rows of running sums before and after them
+  uint32_t ahead;                   // entries of a block that are fetched ahead
 };
 struct FoldShared {
   uint32_t hist[kBins1];            // SCAN: candidates of the CTA's main layer, by bin_of
@@ -2129,7 +2153,7 @@ __device__ __forceinline__ uint32_t subtract_group(float* tile, uint2 q, bool ha
 // What of a block was not fetched ahead: entries of the first 32 packets beyond the first `ahead` (a multiple of 32),
 // and the packets after the first 32 (a worker that has been away for long).  128 entries are on their way while 128 are
 // subtracted (a block with 1500 entries is a warp's whole share: with 32 on their way it took 50,000 cycles).
-__device__ __noinline__ uint32_t fold_rest(const PacketLog& lg, uint32_t first, uint32_t count, uint32_t ahead, uint32_t blk, uint32_t n,
+static __device__ __noinline__ uint32_t fold_rest(const PacketLog& lg, uint32_t first, uint32_t count, uint32_t ahead, uint32_t blk, uint32_t n,
                                            FoldStage* st) {
   constexpr int kDeep = 4;
   const int lane = threadIdx.x & 31;
@@ -2244,12 +2268,11 @@ __device__ __noinline__ uint32_t scan_mixed(const Workspace& ws, const SelArgs& 
 
 // 72 registers a thread: with 64 the loop over the blocks spills a few (a round of 32 arrivals on 124 M elements: 14.1 ms
 // against 11.9), with 80 and 96 fewer warps of other kernels fit beside it (12.4 ms, 12.4 ms).
-template <bool SCAN>
-__global__ void __maxnreg__(72) k_fold(const __grid_constant__ Workspace ws, const __grid_constant__ SelArgs a,
-                                       const __grid_constant__ PacketLog lg, uint32_t first, uint32_t count, uint32_t row0,
-                                       uint32_t row1, uint32_t ahead) {
-  __shared__ FoldShared sh;
-  extern __shared__ __align__(16) unsigned char fold_dyn[];
+// ONE: in one kernel with finalize.
+template <bool SCAN, bool ONE>
+__device__ __forceinline__ void fold_blocks(const Workspace& ws, const SelArgs& a, const PacketLog& lg, const FoldRange& f,
+                                            FoldShared& sh, unsigned char* fold_dyn) {
+  const uint32_t first = f.first, count = f.count, row0 = f.row0, row1 = f.row1, ahead = f.ahead;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t tid = threadIdx.x, nt = blockDim.x, nw = nt / 32u, cta = blockIdx.x, G = gridDim.x;
   const uint32_t lt = lanemask_lt(), le = lt | (1u << lane);
@@ -2279,7 +2302,9 @@ __global__ void __maxnreg__(72) k_fold(const __grid_constant__ Workspace ws, con
     sh.read = 0;
     if (SCAN && cta == 0) {
       ws.sync[kParts] = G * nw;
-      ws.sync[kBarCount] = ws.sync[kFail] = 0;   // for the finalize launch that follows
+      // for the next selection, and for the finalize that follows
+      ws.sync[kBarCount + (a.pair ^ 1u)] = ws.sync[kFail + (a.pair ^ 1u)] = 0;
+      if (!ONE) ws.sync[kBarCount + a.pair] = ws.sync[kFail + a.pair] = 0;
     }
   }
 
@@ -2499,11 +2524,18 @@ __global__ void __maxnreg__(72) k_fold(const __grid_constant__ Workspace ws, con
     }
   }
 }
+template <bool SCAN>
+__global__ void __maxnreg__(72) k_fold(const __grid_constant__ Workspace ws, const __grid_constant__ SelArgs a,
+                                       const __grid_constant__ PacketLog lg, const __grid_constant__ FoldRange f) {
+  __shared__ FoldShared sh;
+  extern __shared__ __align__(16) unsigned char fold_dyn[];
+  fold_blocks<SCAN, false>(ws, a, lg, f, sh, fold_dyn);
+}
 
 // Eager form, for a packet that is too long for the log (any count): buffer q < N is D_q, buffer N is theta.  Indices of
 // one packet ascend, so every (buffer, entry) pair is touched by exactly one thread: plain load / subtract / store.  A
 // packet that does not ascend is reported.
-__global__ void __launch_bounds__(kThreads) k_scatter_sub(const uint32_t* __restrict__ idx,
+static __global__ void __launch_bounds__(kThreads) k_scatter_sub(const uint32_t* __restrict__ idx,
                                                           const float* __restrict__ val, uint32_t count,
                                                           float* __restrict__ theta, float* __restrict__ D,
                                                           uint64_t d_stride, uint32_t num_workers, uint64_t n,

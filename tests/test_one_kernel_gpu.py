@@ -1,0 +1,57 @@
+"""Selections of short vectors, whose pass and finalize are one kernel beside other events (and for a pull of one layer also
+alone), in turn with those that are two: at the smallest sizes, at the longest short vector and one element more.  State and
+packets, bit for bit against the CPU checker."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_1910_10929_b200 as dgs
+import workloads as W
+from _replay import bits, compare_state, packet_to_numpy
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+LONGEST = 3 << 19
+
+
+@pytest.mark.parametrize("sizes,workers,ppm,join", [
+    ([1], 3, 1_000_000, 3),
+    ([513], 4, 20_000, 1),
+    ([64 * 8 * 512 + 1], 5, 30_000, 4),               # a block more than one for every warp
+    ([70_001, 3, 500, 9_000], 3, 10_000, 5),
+    ([1] * 400 + [20_000], 4, 600_000, 7),            # more layers than a CTA's table in shared memory holds
+    ([LONGEST], 3, 2_000, 4),
+    ([LONGEST + 1], 3, 2_000, 4),
+    ([1 << 19, 1 << 19], 3, 50_000, 100),             # dense, never alone
+])
+@pytest.mark.parametrize("flags", [0, dgs.DGS_RESIDUAL_MODE])
+def test_one_kernel_and_two_in_turn(sizes, workers, ppm, join, flags):
+    events = 6 * workers
+    wl = W.custom("one", sizes, workers, events, ppm, grad_kind="normal")
+    n, theta0 = sum(sizes), wl.theta0()
+    orc = oracle.Oracle.from_workload(wl, theta0=theta0, residual_mode=bool(flags))
+    ctx = dgs.Context.from_workload(wl, theta0=torch.from_numpy(theta0).to(DEV), flags=flags, pull_all_capacity=n)
+    rng = np.random.default_rng(n)
+    grads = [rng.standard_normal(n, dtype=np.float32) for _ in range(5)]
+    on_gpu = [torch.from_numpy(g).to(DEV) for g in grads]
+    torch.cuda.synchronize()
+    for e in range(events):
+        w, g = e % workers, e % 5
+        if e % 9 == 5:                                # a pull without secondary compression on the same scratch
+            push = ctx.worker_push(w, on_gpu[g])
+            ctx.server_apply(w, push)
+            gi, gv = ctx.var_packet(ctx.worker_pull_all(w))
+            oi, ov = orc.push(w, grads[g])
+            orc.apply(w, oi, ov)
+            qi, qv, _ = orc.pull_all(w, n)
+            assert np.array_equal(gi.cpu().numpy().view(np.uint32), qi) and np.array_equal(bits(gv.cpu().numpy()), bits(qv))
+            continue
+        got = ctx.event(w, on_gpu[g])
+        want = orc.event(w, grads[g])
+        if e % join == join - 1 or e == events - 1:
+            for p, ref in zip(got, want):
+                gi, gv = packet_to_numpy(ctx, p)
+                assert np.array_equal(gi, ref[0]) and np.array_equal(bits(gv), bits(ref[1])), e
+    assert ctx.status() == 0
+    compare_state(ctx, orc, workers, False)
