@@ -564,8 +564,8 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 // bounded wait: false if the copies did not land within the poll limit
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-  for (uint32_t spins = 0; spins < kSpinLimit; ++spins)
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32_t limit) {
+  for (; limit; --limit)
     if (mbar_try_wait(bar, parity)) return true;
   return false;
 }
@@ -652,10 +652,12 @@ __device__ __noinline__ void mixed_emit(const Workspace& ws, const SelArgs& a, c
 // those of others straight in global memory.  (A layer at a time, the ring restarted and the histogram flushed for each and
 // one warp at work on its ragged ends, 11.7 M elements in 62 layers took 54 us, and the CTAs with the small layers 58 us where
 // the others took 24; now 37 us.)
+// If a copy does not land in time the status word says so and *s_dead is set: the CTA's counts are then not complete, and a late
+// copy may still write to the ring.  `phantom` is for tests: arrivals that the last CTA's copies wait for and that never come.
 template <int MODE, typename R>
 __device__ void stream_blocks_tma(const Workspace& ws, const SelArgs& a, const uint32_t* Larr, const float* __restrict__ in,
                                   float* __restrict__ out, uint32_t cta, uint32_t G, StreamShared& sh, float* ring, uint64_t* full,
-                                  int* s_dead) {
+                                  int* s_dead, uint32_t phantom, uint32_t spin_limit) {
   static_assert(MODE != kPull, "a pull's pass is k_fold");
   static_assert(R::kStages >= 2, "the ring needs a stage in flight besides the one being read");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -676,7 +678,7 @@ __device__ void stream_blocks_tma(const Workspace& ws, const SelArgs& a, const u
   if (threadIdx.x == 0) {
     *s_dead = 0;
     if (cta == 0) ws.sync[kParts] = G;
-    for (int st = 0; st < R::kStages; ++st) mbar_init(full + st, 1);
+    for (int st = 0; st < R::kStages; ++st) mbar_init(full + st, 1u + (cta + 1 == G ? phantom : 0u));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     for (uint32_t r = 0; r < (uint32_t)R::kStages - 1 && r < rounds && fetched(r); ++r) issue(r);
   }
@@ -695,7 +697,7 @@ __device__ void stream_blocks_tma(const Workspace& ws, const SelArgs& a, const u
       seg_end = __ldg(ws.seg_off + seg + 1);
       L = Larr[seg];
     }
-    const bool landed = !fetched(r) || mbar_wait(full + st, (r / R::kStages) & 1u);
+    const bool landed = !fetched(r) || mbar_wait(full + st, (r / R::kStages) & 1u, spin_limit);
     if (!landed) *s_dead = 1;
     const float* const su = ring + (size_t)st * (R::kStageBytes / 4) + warp * kWarpTile;
     const bool plain = blk < f1 && base + kWarpTile <= seg_end;
@@ -732,8 +734,8 @@ __device__ void stream_blocks_tma(const Workspace& ws, const SelArgs& a, const u
     if (threadIdx.x == 0) {
       atomicMin(ws.status, kStatusTimeout);
       for (int st = 0; st < R::kStages; ++st) {
-        mbar_wait(full + st, 0);
-        mbar_wait(full + st, 1);
+        mbar_wait(full + st, 0, spin_limit);
+        mbar_wait(full + st, 1, spin_limit);
       }
     }
     __syncthreads();
@@ -1298,7 +1300,7 @@ __device__ __forceinline__ void finalize(const Workspace& ws, const SelArgs& a, 
       }
       return;
     }
-    const uint32_t all = bar_target + a.phantom_workers;
+    const uint32_t all = bar_target + (MODE == kPull ? a.phantom_workers : 0u);   // (a push: a CTA of its pass does not come)
     bar_target = 0;
     if (!worker_barrier(ws.sync + kBarCount + a.pair, all, ws.status, &sh.ok, bar_target, spin_limit)) return;
   }
@@ -1891,7 +1893,7 @@ __global__ void __maxnreg__(64) k_stream(const __grid_constant__ Workspace ws, c
   float* out = *a.u_spare_slot;
   if (blockIdx.x == 0 && threadIdx.x < 2) ws.sync[kBarCount + threadIdx.x] = ws.sync[kFail + threadIdx.x] = 0;   // for the finalize that follows
   stream_blocks_tma<MODE, PushRing>(ws, a, a.L_in, in, out, blockIdx.x, gridDim.x, sh, reinterpret_cast<float*>(dyn_smem), full,
-                                    &s_dead);
+                                    &s_dead, 0u, kSpinLimit);
 }
 
 // ---- pull without secondary compression: every nonzero entry of D_w -------------------

@@ -18,8 +18,9 @@ __global__ void __maxnreg__(80) k_one_push(const __grid_constant__ Workspace ws,
   float* out = *a.u_spare_slot;
   if (blockIdx.x == 0 && threadIdx.x == 0) ws.sync[kBarCount + (a.pair ^ 1u)] = ws.sync[kFail + (a.pair ^ 1u)] = 0;   // for the next selection
   stream_blocks_tma<MODE, OnePushRing>(ws, a, a.L_in, in, out, blockIdx.x, gridDim.x, sh, reinterpret_cast<float*>(dyn_smem), full,
-                                       &s_dead);
+                                       &s_dead, a.phantom_workers, a.spin_limit ? a.spin_limit : kSpinLimit);
   __syncthreads();
+  if (s_dead) return;   // finalize's tables would lie where a late copy may land; the others give up at the barrier
   finalize<MODE, MANY, false, 256, true>(ws, a, in, out, *reinterpret_cast<OneShared<MODE>*>(dyn_smem),
                                          dyn_smem + sizeof(OneShared<MODE>), gridDim.x);
 }

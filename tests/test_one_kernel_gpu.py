@@ -1,6 +1,8 @@
 """Selections of short vectors, whose pass and finalize are one kernel beside other events (and for a pull of one layer also
 alone), in turn with those that are two: at the smallest sizes, at the longest short vector and one element more.  State and
 packets, bit for bit against the CPU checker."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -55,3 +57,29 @@ def test_one_kernel_and_two_in_turn(sizes, workers, ppm, join, flags):
                 assert np.array_equal(gi, ref[0]) and np.array_equal(bits(gv), bits(ref[1])), e
     assert ctx.status() == 0
     compare_state(ctx, orc, workers, False)
+
+
+def test_a_pass_that_cannot_end_goes_no_further():
+    """With DGS_TEST_STALLED_BARRIER the barrier between a pull's pass and its finalize waits for a CTA that does not exist, and
+    the copies of the last CTA of a push's pass for an arrival that never comes: that CTA must leave at once, since finalize's
+    tables lie where its copies land, and the others give up at the barrier.  Nothing after it may run."""
+    n, k, workers = 300_000, 300, 3
+    theta0 = torch.randn(n, device=DEV)
+    ctx = dgs.Context(n, workers, 0.1, 0.9, [0], [n], [k], [k], theta0, flags=dgs.DGS_TEST_STALLED_BARRIER)
+    grad = torch.randn(n, device=DEV)
+    torch.cuda.synchronize()
+    t0 = time.perf_counter()
+    for turn in range(6):                             # (the pairs of sync words are taken in turn)
+        at = ctx.launch_count()
+        ctx.worker_pull(turn % workers)               # alone; nothing to go by: two kernels for its bound, then one
+        assert ctx.launch_count() == at + 3
+        ctx.worker_push(turn % workers, grad)         # beside the pull
+        assert ctx.launch_count() == at + (4 if turn else 6)   # the first push has nothing to go by either
+        assert ctx.status() == dgs.DGS_ETIMEOUT
+    assert time.perf_counter() - t0 < 20.0
+    assert ctx.stats()[3] == 0                        # no finalize has looked at a candidate
+    assert torch.equal(ctx.state(dgs.DGS_THETA), theta0)
+    for w in range(workers):
+        assert not ctx.state(dgs.DGS_U, w).any() and not ctx.state(dgs.DGS_D, w).any()
+    ctx.close()
+    test_one_kernel_and_two_in_turn([n], workers, 1_000, 3, 0)   # a context made afterwards runs clean
