@@ -281,7 +281,9 @@ struct dgs_ctx {
   uint32_t fold_ahead;   // entries of a block it fetches ahead
   // No pull has been enqueued since the caller's stream was last made to wait for everything (dgs_flush, or a call
   // that waits): the event in hand starts on an idle GPU.
-  bool alone;
+  bool idle_gpu;
+  bool lone;             // the last calls between two such joins held one pull
+  uint32_t pulls;        // since the last join
   int hist_grid[3];      // CTAs of the whole-input histogram pass, per mode
   int one_max[3];        // most CTAs of pass and finalize in one kernel, per mode
   uint32_t pair[kSets];  // pair of sync words that the last selection on each scratch set has used
@@ -428,13 +430,26 @@ int fork_from_user(dgs_ctx* c, int which) {
   return DGS_OK;
 }
 
+// Everything that was in flight is complete, or the caller's stream waits for it.
+void joined(dgs_ctx* c) {
+  if (c->pulls) c->lone = c->pulls == 1;
+  c->pulls = 0;
+  c->idle = c->idle_gpu = true;
+}
+// Whether the event in hand has the GPU to itself.  The one that opens a round of several does not: the others are enqueued
+// right behind it, and a finalize sized for an idle GPU, whose CTAs must all be resident, waits for room beside their passes and
+// keeps them waiting.  What follows a join is taken to be as many events as between the last two.  (Rounds of 8 arrivals on
+// 124 M elements in 148 layers, us, every event after a join taken for alone / this: 3022 / 2877; of 32 on 11.7 M in 62 layers
+// 2870 / 2789; of 8 on 8.4 M in 2000 layers 1280 / 1115; one arrival at a time the same.)
+bool has_gpu(const dgs_ctx* c) { return c->idle_gpu && c->lone; }
+
 // Waits (on the host) for all internal streams ...
 int sync_library(dgs_ctx* c) {
   for (int i = 0; i < kStreams; ++i) {
     if (c->st[i] && c->dirty[i]) DGS_CUDA(c, cudaStreamSynchronize(c->st[i]));
     c->dirty[i] = false;                     // nothing that the caller's stream would have to wait for
   }
-  c->alone = c->idle = true;
+  joined(c);
   return DGS_OK;
 }
 // ... and the caller's stream (which has been made to wait for those that are not dirty).
@@ -516,7 +531,7 @@ int fold_launch(dgs_ctx* c, const Workspace& ws, const SelArgs& a, uint32_t q, c
   // Fewer warps where several events share the GPU (a worker has one pull at a time, so it takes more than two workers).
   // Eight / four warps a CTA, us an event in runs of 256: 2 workers, 8.4 M elements: 36 / 40, 62 layers of 11.7 M: 95 / 101;
   // 3 workers, 25.6 M: 66 / 63; 8 workers: 61 / 57, 62 layers of 11.7 M: 83 / 78.
-  const uint32_t warps = c->alone || c->cfg.num_workers <= 2 ? kFoldWarps : kFoldWarpsBeside;
+  const uint32_t warps = has_gpu(c) || c->cfg.num_workers <= 2 ? kFoldWarps : kFoldWarpsBeside;
   k_fold<SCAN><<<c->fold_grid, warps * 32, fold_dyn_bytes(warps, c->fold_ahead, ws.part_cap), st>>>(ws, a, c->log, fold_range(c, q));
   DGS_CUDA(c, cudaGetLastError());
   c->launches += 1;
@@ -585,7 +600,7 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
   // fewer than k candidates (four workers drawn at random), each then starting over inside finalize.  The
   // histogram route costs less than that on average.  (With one worker every pull is like the one before it.)
   if (KIND == 1 && age < 2 && c->cfg.num_workers > 1) row = -1;
-  const bool single_pass = row >= 0;
+  const bool single_pass = row >= 0, alone = has_gpu(c);
   const int next_copy = c->row_copy[KIND][worker] ^ 1;
   a.L_next = c->L_next(KIND, next_copy, worker);
   a.slack = c->at<uint32_t>(c->lay.slack) + (uint64_t)KIND * c->cfg.num_segments;
@@ -598,21 +613,21 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
   const uint64_t keep = finalize_keep(c->cfg.num_segments > 1);
   // Layers that are small enough to be candidates as a whole (see next_bound) often are: 60 layers of 2^20 elements, alone, 18.3
   // and 20.8 us without them, 16.5 and 18.2 with.
-  const uint64_t cands = c->alone ? std::max<uint64_t>(3ull * a.pkt_count + 64ull * c->cfg.num_segments, c->whole_layers)
+  const uint64_t cands = alone ? std::max<uint64_t>(3ull * a.pkt_count + 64ull * c->cfg.num_segments, c->whole_layers)
                                   : (uint64_t)a.pkt_count + a.pkt_count / 4 * 3 + 64ull * c->cfg.num_segments;
   uint64_t want = std::max<uint64_t>(kFinalizeMin, (cands + kThreads * keep - 1) / (kThreads * keep));
   // Beside other kernels an eighth of that, but not fewer than 48: what its CTAs hold is taken from the passes, which have
   // the bytes to move, and a selection that takes longer only waits for its turn later.  Rounds of 32 arrivals, ms, with as many
   // as keep the candidates (one per SM at most) / 100 / 50 / 24: 11.7 M elements in 62 layers: 3.09 / 2.94 / 2.85 / 2.92; 124 M:
   // 11.57 / 11.31 / 11.25 / 11.23; 8 arrivals on 124 M in 148 layers: 2.91 / 2.86 / 2.85 / 2.87.
-  if (!c->alone) want = std::min(want, std::max<uint64_t>(48, want / 8));
-  const uint64_t most = (uint64_t)(std::min(c->finalize_max[MODE], c->alone ? 2 * c->sms : c->sms) - (int)advisers);
+  if (!alone) want = std::min(want, std::max<uint64_t>(48, want / 8));
+  const uint64_t most = (uint64_t)(std::min(c->finalize_max[MODE], alone ? 2 * c->sms : c->sms) - (int)advisers);
   const int fin_grid = (int)std::min(most, want);
   // More candidates than the registers of all CTAs hold: k_finalize<.., BIG>, but beside other kernels only for one layer
   // and fifty times as many (runs of 32 events on 8.4 M elements, us an event without / with: one layer, 10 %, 20 times as
   // many: 153 / 156; 50 %, 97 times: 823 / 733; 60 layers, 50 %: 750 / 818).
-  const uint64_t held = (c->alone ? (uint64_t)fin_grid : most) * kThreads * keep;
-  const bool big = c->alone ? cands > held : c->cfg.num_segments == 1 && cands > 50 * held;
+  const uint64_t held = (alone ? (uint64_t)fin_grid : most) * kThreads * keep;
+  const bool big = alone ? cands > held : c->cfg.num_segments == 1 && cands > 50 * held;
   a.workers = (uint32_t)fin_grid;
   a.advisers = advisers;
   a.fold_grid = MODE == kPull ? (uint32_t)c->fold_grid : 0u;   // one CTA more plans the next pull's pass
@@ -622,9 +637,9 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
   // one layer gains: its pass takes little longer with half of the CTAs (2^20 elements: pull 22.3 / 19.6 us, push 19.6 / 20.2;
   // in 60 layers 40 / 42 and 31 / 34).  While launches are timed each kernel stays on its own.
   const uint32_t others = advisers + (MODE == kPull ? 1u : 0u);
-  uint32_t one_grid = std::min<uint32_t>(c->alone ? kOneMaxGrid : kOneGridBeside, (c->lay.num_blocks + kWarps - 1) / kWarps);
+  uint32_t one_grid = std::min<uint32_t>(alone ? kOneMaxGrid : kOneGridBeside, (c->lay.num_blocks + kWarps - 1) / kWarps);
   one_grid = std::min<uint32_t>(std::max<uint32_t>(one_grid, (uint32_t)kFinalizeMin + others), (uint32_t)c->one_max[MODE]);
-  const bool one = c->cfg.n <= kOneMaxN && (c->alone ? MODE == kPull && c->cfg.num_segments == 1 : true) && !big && !c->timing &&
+  const bool one = c->cfg.n <= kOneMaxN && (alone ? MODE == kPull && c->cfg.num_segments == 1 : true) && !big && !c->timing &&
                    one_grid > others && (c->lay.num_blocks + one_grid - 1) / one_grid + kFoldSlack <= ws.part_cap;
   if (one) {
     a.workers = std::min<uint32_t>(a.workers, one_grid - others);
@@ -838,7 +853,8 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
   c->launches = 0;
   c->last_cuda = 0;
   c->broken = false;
-  c->alone = true;
+  c->idle_gpu = c->lone = true;
+  c->pulls = 0;
   c->timing = false;
   for (int i = 0; i < DGS_NUM_KERNELS; ++i) {
     c->time_ms[i] = 0.0;
@@ -1117,7 +1133,8 @@ int pull_impl(dgs_ctx* c, uint32_t worker, dgs_packet* out) {
   c->prev[worker] = (int64_t)c->timestamp;
   c->pull_count += 1;
   c->worker_stream[worker] = -1;
-  c->alone = false;
+  c->idle_gpu = false;
+  c->pulls += 1;
   if (out) {
     out->idx = a.pkt_idx;
     out->val = a.pkt_val;
@@ -1171,7 +1188,8 @@ int pull_all_impl(dgs_ctx* c, uint32_t worker, dgs_var_packet* out) {
   c->pull_count += 1;
   c->worker_stream[worker] = -1;
   c->var_count += 1;
-  c->alone = false;
+  c->idle_gpu = false;
+  c->pulls += 1;
   if (out) {
     out->idx = vi;
     out->val = vv;
@@ -1250,8 +1268,7 @@ int dgs_flush(dgs_ctx* c) {
     c->dirty[i] = false;
     c->waited_seq[kCaller][i] = c->task_seq;
   }
-  c->idle = true;
-  c->alone = true;
+  joined(c);
   return DGS_OK;
 }
 

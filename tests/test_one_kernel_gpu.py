@@ -83,3 +83,36 @@ def test_a_pass_that_cannot_end_goes_no_further():
         assert not ctx.state(dgs.DGS_U, w).any() and not ctx.state(dgs.DGS_D, w).any()
     ctx.close()
     test_one_kernel_and_two_in_turn([n], workers, 1_000, 3, 0)   # a context made afterwards runs clean
+
+
+def one_layer(n, k, workers):
+    """A context of one layer, and an event that returns how many kernels its push was."""
+    ctx = dgs.Context(n, workers, 0.1, 0.9, [0], [n], [k], [k], torch.zeros(n, device=DEV))
+    grads = [torch.randn(n, device=DEV) for _ in range(workers)]
+
+    def event(w):
+        before = ctx.launch_count()
+        pkt = ctx.worker_push(w, grads[w])
+        launches = ctx.launch_count() - before
+        ctx.server_apply(w, pkt)
+        ctx.worker_pull(w)
+        return launches
+    return ctx, event
+
+
+def test_an_event_that_opens_a_round_is_not_alone():
+    """Alone on the GPU a push of a short vector is two kernels, beside other events one.  The event after a join is taken to be
+    alone if the one before the join was, and to open a round if a round was before the join."""
+    ctx, event = one_layer(300_000, 300, 3)
+    for _ in range(2):
+        for w in range(3):
+            event(w)
+        ctx.flush()
+    assert [event(w) for w in range(3)] == [1, 1, 1]
+    ctx.flush()
+    event(0)
+    ctx.flush()
+    ctx.flush()                                   # a join with nothing before it says nothing
+    assert event(1) == 2
+    assert ctx.status() == 0
+    assert [event(w) for w in range(3)] == [2, 1, 1]
