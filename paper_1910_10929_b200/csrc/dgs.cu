@@ -586,6 +586,21 @@ uint32_t one_bytes(const dgs_ctx* c, int mode) {
   return one_dyn_bytes(mode, c->cfg.num_segments, c->fold_ahead, c->ws[0].part_cap);
 }
 
+// CTAs of finalize beside other kernels, of the `want` that keep the candidates in registers.  What its CTAs hold is taken from the
+// passes, which have the bytes to move, and with many workers a selection that takes longer only waits for its turn later: an
+// eighth, but not fewer than 48.  With few workers an event waits for the one before it, and there is not enough in flight to
+// fill the time: all of them up to three workers, 96 up to seven.  us, all (one per SM at most) / 96 / 48: 62 layers of 11.7 M, 32
+// arrivals of 1 worker 6090 / - / 9724, 2: 2637 / - / 2940, 3: 2443 / 2328 / 2495, 4: 2447 / 2346 / 2343, 6: 2485 / 2355 / 2330, 8:
+// 2524 / - / 2286, 32: 3045 / - / 2786; rounds of 3 arrivals 300 / 313 / 337, 4: 356 / 365 / 407, 6: 510 / 494 / 525, 8: 680 / - / 649;
+// 60 layers of 25 M, 1 %: 3: 484 / 508 / 570, 4: 604 / 618 / 683, 6: 913 / 899 / 929, 8: 1210 / - / 1217, 16: 2500 / - / 2380.
+constexpr uint64_t finalize_beside(uint32_t workers, uint64_t want) {
+  const uint64_t few = workers >= 8 ? 48 : 96, less = want / 8 > few ? want / 8 : few;
+  return workers <= 3 || want < less ? want : less;
+}
+static_assert(finalize_beside(1, 204) == 204 && finalize_beside(3, 204) == 204, "a chain of events");
+static_assert(finalize_beside(4, 204) == 96 && finalize_beside(7, 60) == 60, "");
+static_assert(finalize_beside(8, 204) == 48 && finalize_beside(32, 800) == 100 && finalize_beside(32, 33) == 33, "");
+
 template <int MODE>
 int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age, int stream_id, Task& task) {
   constexpr int KIND = MODE == kPull ? 1 : 0;
@@ -616,11 +631,7 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
   const uint64_t cands = alone ? std::max<uint64_t>(3ull * a.pkt_count + 64ull * c->cfg.num_segments, c->whole_layers)
                                   : (uint64_t)a.pkt_count + a.pkt_count / 4 * 3 + 64ull * c->cfg.num_segments;
   uint64_t want = std::max<uint64_t>(kFinalizeMin, (cands + kThreads * keep - 1) / (kThreads * keep));
-  // Beside other kernels an eighth of that, but not fewer than 48: what its CTAs hold is taken from the passes, which have
-  // the bytes to move, and a selection that takes longer only waits for its turn later.  Rounds of 32 arrivals, ms, with as many
-  // as keep the candidates (one per SM at most) / 100 / 50 / 24: 11.7 M elements in 62 layers: 3.09 / 2.94 / 2.85 / 2.92; 124 M:
-  // 11.57 / 11.31 / 11.25 / 11.23; 8 arrivals on 124 M in 148 layers: 2.91 / 2.86 / 2.85 / 2.87.
-  if (!alone) want = std::min(want, std::max<uint64_t>(48, want / 8));
+  if (!alone) want = finalize_beside(c->cfg.num_workers, want);
   const uint64_t most = (uint64_t)(std::min(c->finalize_max[MODE], alone ? 2 * c->sms : c->sms) - (int)advisers);
   const int fin_grid = (int)std::min(most, want);
   // More candidates than the registers of all CTAs hold: k_finalize<.., BIG>, but beside other kernels only for one layer
