@@ -525,13 +525,21 @@ FoldRange fold_range(const dgs_ctx* c, uint32_t q) {
   f.ahead = c->fold_ahead;
   return f;
 }
+// Warps of a CTA of the pass: ten where the pull has the GPU to itself, as with a single worker, whose pulls follow one another;
+// eight where one other pull may be in flight (a worker has one at a time), four beside more.  us, 16 arrivals, eight / ten: 1
+// worker, 8.4 M elements 3045 / 2976, 62 layers of 11.7 M 4774 / 4700; 2 workers 615 / 640, 1518 / 1536.  us an event in runs of
+// 256, eight / four: 2 workers, 8.4 M: 36 / 40, 62 layers of 11.7 M: 95 / 101; 3 workers, 25.6 M: 66 / 63; 8 workers: 61 / 57, 62
+// layers of 11.7 M: 83 / 78.  (Vectors of 500 M elements with many entries, where an SM has room for one CTA of ten warps or two of
+// eight: pass of a pull alone 1308 / 1342.)
+constexpr uint32_t fold_warps(uint32_t workers, bool alone) {
+  return alone || workers == 1 ? kFoldWarps : workers == 2 ? kWarps : kFoldWarpsBeside;
+}
+static_assert(fold_warps(32, true) == 10 && fold_warps(1, false) == 10 && fold_warps(2, false) == 8 && fold_warps(3, false) == 4, "");
+
 template <bool SCAN>
 int fold_launch(dgs_ctx* c, const Workspace& ws, const SelArgs& a, uint32_t q, cudaStream_t st) {
   TimedLaunch tl(c, st, SCAN ? DGS_KERNEL_STREAM_PULL : DGS_KERNEL_CATCH_UP);
-  // Fewer warps where several events share the GPU (a worker has one pull at a time, so it takes more than two workers).
-  // Eight / four warps a CTA, us an event in runs of 256: 2 workers, 8.4 M elements: 36 / 40, 62 layers of 11.7 M: 95 / 101;
-  // 3 workers, 25.6 M: 66 / 63; 8 workers: 61 / 57, 62 layers of 11.7 M: 83 / 78.
-  const uint32_t warps = has_gpu(c) || c->cfg.num_workers <= 2 ? kFoldWarps : kFoldWarpsBeside;
+  const uint32_t warps = fold_warps(c->cfg.num_workers, has_gpu(c));
   k_fold<SCAN><<<c->fold_grid, warps * 32, fold_dyn_bytes(warps, c->fold_ahead, ws.part_cap), st>>>(ws, a, c->log, fold_range(c, q));
   DGS_CUDA(c, cudaGetLastError());
   c->launches += 1;
