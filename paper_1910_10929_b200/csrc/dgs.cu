@@ -54,6 +54,17 @@ constexpr int kLogRingMax = 128;            // most packets the apply log keeps
 constexpr int kLogSlack = 32;               // slots of the log beyond one per worker
 constexpr uint64_t kListCap = 4096;         // most entries of a layer's list of candidates in the k-th's bin
 constexpr uint64_t kOneMaxN = 3ull << 19;   // longest vector whose selections are one kernel each
+// ... beside other events: with more layers a CTA has more bounds to pick for, and finalize has fewer CTAs in that kernel.  Rounds of 12
+// and 16 arrivals, us, two kernels a selection / one: one layer: 0.5 M elements 313 / 235, 1.05 M 250 / 180, 1.5 M 262 / 200; 2 layers:
+// 1.05 M 212 / 206, 1.2 M 215 / 222; 8: 0.7 M 279 / 191, 1.05 M 216 / 218, 1.2 M 219 / 232; 20: 0.7 M 241 / 228, 0.9 M 225 / 231; 60: 0.5 M
+// 317 / 255, 0.7 M 249 / 249, 0.88 M 251 / 266; 200: 0.25 M 307 / 280, 0.5 M 314 / 316, 0.7 M 330 / 356; 1000: 0.25 M 675 / 712, at 2 % 815 /
+// 932.  Dense selections differ less: 1.5 M elements in one layer, 20 %: 1090 / 1075; 0.5 M in 60, 20 %: 645 / 648.
+constexpr uint64_t one_max_beside(uint32_t layers) {
+  constexpr uint64_t least = 1ull << 19, most = 1ull << 20;
+  if (layers == 1) return kOneMaxN;
+  return layers > 512 ? 0 : layers < 64 ? most - ((uint64_t)layers << 13) : least;
+}
+static_assert(one_max_beside(63) >= one_max_beside(64) && one_max_beside(2) < kOneMaxN, "fewer elements for more layers");
 constexpr uint32_t kOneGridBeside = 64;     // most CTAs of that kernel beside other events
 
 inline uint64_t align_up(uint64_t x, uint64_t a) { return (x + a - 1) / a * a; }
@@ -651,14 +662,15 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
   a.advisers = advisers;
   a.fold_grid = MODE == kPull ? (uint32_t)c->fold_grid : 0u;   // one CTA more plans the next pull's pass
   // Short vectors: pass and finalize in one kernel.  Beside other events the host is what such vectors wait for, 3 us a launch
-  // (rounds of 12 arrivals on 409 K elements: 205 us with two kernels a selection, 164 with one; of 27 on 131 K: 471, 391; of 28
-  // on 880 K, 1.4 %: 494, 452; but 2^21 elements: 20 us an event with two, 27 with one).  Alone it is the GPU, and only a pull of
-  // one layer gains: its pass takes little longer with half of the CTAs (2^20 elements: pull 22.3 / 19.6 us, push 19.6 / 20.2;
-  // in 60 layers 40 / 42 and 31 / 34).  While launches are timed each kernel stays on its own.
+  // (see one_max_beside; 2^21 elements: 20 us an event with two kernels a selection, 27 with one).  Alone it is the GPU, and only a
+  // pull of one layer gains: its pass takes little longer with half of the CTAs (2^20 elements: pull 22.3 / 19.6 us, push 19.6 /
+  // 20.2; in 60 layers 40 / 42 and 31 / 34; select from 1.5 M elements, 0.1 to 3 %: 34-41 / 32-37, 5 %: 46 / 46).  While launches are
+  // timed each kernel stays on its own.
   const uint32_t others = advisers + (MODE == kPull ? 1u : 0u);
   uint32_t one_grid = std::min<uint32_t>(alone ? kOneMaxGrid : kOneGridBeside, (c->lay.num_blocks + kWarps - 1) / kWarps);
   one_grid = std::min<uint32_t>(std::max<uint32_t>(one_grid, (uint32_t)kFinalizeMin + others), (uint32_t)c->one_max[MODE]);
-  const bool one = c->cfg.n <= kOneMaxN && (alone ? MODE == kPull && c->cfg.num_segments == 1 : true) && !big && !c->timing &&
+  const uint64_t one_max_n = !alone ? one_max_beside(c->cfg.num_segments) : MODE == kPull && c->cfg.num_segments == 1 ? kOneMaxN : 0;
+  const bool one = c->cfg.n <= one_max_n && !big && !c->timing &&
                    one_grid > others && (c->lay.num_blocks + one_grid - 1) / one_grid + kFoldSlack <= ws.part_cap;
   if (one) {
     a.workers = std::min<uint32_t>(a.workers, one_grid - others);
@@ -771,7 +783,7 @@ int occupancy_grids(dgs_ctx* c, int sms) {
   }
   if (MODE == kPull) c->finalize_max[MODE] -= 1;   // the CTA that plans the next pass
   c->one_max[MODE] = 0;
-  if (c->cfg.n <= kOneMaxN && one_bytes(c, MODE) <= (uint32_t)kFoldMaxDyn) {
+  if (c->cfg.n <= one_max_beside(c->cfg.num_segments) && one_bytes(c, MODE) <= (uint32_t)kFoldMaxDyn) {
     const void* const f = one_kernel(MODE, c->cfg.num_segments > 1);
     DGS_CUDA(c, cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kFoldMaxDyn));
     DGS_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f, kThreads, one_bytes(c, MODE)));

@@ -25,7 +25,7 @@ LONGEST = 3 << 19
     ([1] * 400 + [20_000], 4, 600_000, 7),            # more layers than a CTA's table in shared memory holds
     ([LONGEST], 3, 2_000, 4),
     ([LONGEST + 1], 3, 2_000, 4),
-    ([1 << 19, 1 << 19], 3, 50_000, 100),             # dense, never alone
+    ([1 << 19, (1 << 19) - 20_000], 3, 50_000, 100),  # dense, alone only at the start and after a pull without compression
 ])
 @pytest.mark.parametrize("flags", [0, dgs.DGS_RESIDUAL_MODE])
 def test_one_kernel_and_two_in_turn(sizes, workers, ppm, join, flags):
@@ -85,9 +85,11 @@ def test_a_pass_that_cannot_end_goes_no_further():
     test_one_kernel_and_two_in_turn([n], workers, 1_000, 3, 0)   # a context made afterwards runs clean
 
 
-def one_layer(n, k, workers):
-    """A context of one layer, and an event that returns how many kernels its push was."""
-    ctx = dgs.Context(n, workers, 0.1, 0.9, [0], [n], [k], [k], torch.zeros(n, device=DEV))
+def launch_counter(sizes, workers):
+    """A context that keeps a hundredth of every layer, and an event that returns how many kernels its push was."""
+    n, ks = sum(sizes), [max(1, x // 100) for x in sizes]
+    off = np.concatenate([[0], np.cumsum(sizes)[:-1]])
+    ctx = dgs.Context(n, workers, 0.1, 0.9, off, sizes, ks, ks, torch.zeros(n, device=DEV))
     grads = [torch.randn(n, device=DEV) for _ in range(workers)]
 
     def event(w):
@@ -103,7 +105,7 @@ def one_layer(n, k, workers):
 def test_an_event_that_opens_a_round_is_not_alone():
     """Alone on the GPU a push of a short vector is two kernels, beside other events one.  The event after a join is taken to be
     alone if the one before the join was, and to open a round if a round was before the join."""
-    ctx, event = one_layer(300_000, 300, 3)
+    ctx, event = launch_counter([300_000], 3)
     for _ in range(2):
         for w in range(3):
             event(w)
@@ -116,3 +118,22 @@ def test_an_event_that_opens_a_round_is_not_alone():
     assert event(1) == 2
     assert ctx.status() == 0
     assert [event(w) for w in range(3)] == [2, 1, 1]
+
+
+@pytest.mark.parametrize("sizes,kernels", [
+    ([LONGEST], 1),
+    ([LONGEST + 1], 2),
+    ([1 << 19, (1 << 19) - (2 << 13)], 1),            # two layers: 2^20 elements but 2^13 for each
+    ([1 << 19, (1 << 19) - (2 << 13) + 1], 2),
+    ([8_192] * 64, 1),                                # 2^19 from 64 layers on
+    ([8_192] * 63 + [8_193], 2),
+    ([64] * 512, 1),
+    ([64] * 513, 2),
+])
+def test_which_selections_beside_other_events_are_one_kernel(sizes, kernels):
+    ctx, event = launch_counter(sizes, 3)
+    for _ in range(2):
+        for w in range(3):
+            event(w)
+    assert [event(w) for w in range(3)] == [kernels] * 3
+    assert ctx.status() == 0
