@@ -25,6 +25,7 @@
 #include <utility>
 #include <vector>
 
+#include "dgs_apply.cuh"
 #include "dgs_kernels.cuh"
 #include "dgs_one.cuh"
 #include "dgs_topk.cuh"
