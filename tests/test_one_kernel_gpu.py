@@ -1,6 +1,7 @@
 """Selections of short vectors, whose pass and finalize are one kernel beside other events (and for a pull of one layer also
 alone), in turn with those that are two: at the smallest sizes, at the longest short vector and one element more.  State and
 packets, bit for bit against the CPU checker."""
+import ctypes
 import time
 
 import numpy as np
@@ -136,4 +137,39 @@ def test_which_selections_beside_other_events_are_one_kernel(sizes, kernels):
         for w in range(3):
             event(w)
     assert [event(w) for w in range(3)] == [kernels] * 3
+    assert ctx.status() == 0
+
+
+@pytest.mark.parametrize("sizes", [[300_000], [100_000, 700, 50_000]])
+@pytest.mark.parametrize("flags", [0, dgs.DGS_RESIDUAL_MODE])
+def test_a_guess_that_fails_starts_over_inside_the_kernel(sizes, flags):
+    """Every second round all values are a thousandth of what the carried bounds were made for, and no candidate is found."""
+    workers, n = 3, sum(sizes)
+    wl = W.custom("redo", sizes, workers, 1, 10_000, grad_kind="normal")
+    orc = oracle.Oracle.from_workload(wl, residual_mode=bool(flags))
+    ctx = dgs.Context.from_workload(wl, flags=flags)
+    rng = np.random.default_rng(n)
+    nothing = torch.zeros(n, device=DEV)
+    for turn in range(6):
+        scale = np.float32(1e-3 if turn % 2 else 1.0)
+        grads = [rng.standard_normal(n, dtype=np.float32) * scale for _ in range(workers)]
+        on_gpu = [torch.from_numpy(g).to(DEV) for g in grads]
+        if turn % 2:
+            for w in range(workers):
+                for mine, its in ((dgs.DGS_U, oracle.U), (dgs.DGS_D, oracle.D)):
+                    ctx.state_load(mine, w, nothing)
+                    ctypes.memset(orc.state(its, w).ctypes.data, 0, 4 * n)
+        torch.cuda.synchronize()
+        before, launches = ctx.stats(), ctx.launch_count()
+        for w in range(workers):
+            got = ctx.event(w, on_gpu[w])
+            want = orc.event(w, grads[w])
+        if turn > 1:
+            assert ctx.launch_count() - launches == 3 * workers      # push, apply, pull: a kernel each
+        if turn % 2:
+            assert ctx.stats()[1] > before[1]
+        for p, ref in zip(got, want):
+            gi, gv = packet_to_numpy(ctx, p)
+            assert np.array_equal(gi, ref[0]) and np.array_equal(bits(gv), bits(ref[1])), turn
+        compare_state(ctx, orc, workers, False)
     assert ctx.status() == 0
