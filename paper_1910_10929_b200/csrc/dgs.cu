@@ -525,8 +525,7 @@ void catch_up_deps(const dgs_ctx* c, uint32_t q, Task* t) {
   for (uint64_t p = c->applied[q]; p < c->log_head; ++p) t->reads.push_back(R.LOG((uint32_t)(p % c->log.ring)));
   t->writes.push_back(R.D(q));
 }
-// The launch itself, on a stream that task_begin has prepared with those dependencies: the filed packets that D_q
-// has not seen yet, and with SCAN the stream pass of a pull in the same trip over D_q.
+// The filed packets that D_q has not seen yet.
 FoldRange fold_range(const dgs_ctx* c, uint32_t q) {
   const uint32_t ring = c->log.ring;
   FoldRange f;
@@ -543,15 +542,22 @@ FoldRange fold_range(const dgs_ctx* c, uint32_t q) {
 // 256, eight / four: 2 workers, 8.4 M: 36 / 40, 62 layers of 11.7 M: 95 / 101; 3 workers, 25.6 M: 66 / 63; 8 workers: 61 / 57, 62
 // layers of 11.7 M: 83 / 78.  (Vectors of 500 M elements with many entries, where an SM has room for one CTA of ten warps or two of
 // eight: pass of a pull alone 1308 / 1342.)
-constexpr uint32_t fold_warps(uint32_t workers, bool alone) {
-  return alone || workers == 1 ? kFoldWarps : workers == 2 ? kWarps : kFoldWarpsBeside;
+// The pull that opens a round (idle) takes ten as well where it is a long one of a long vector, us a round, four / ten: 25.6 M
+// elements, 32 workers 2072 / 2057, 16: 1026 / 1028, 8: 531 / 536; 124 M, 32 workers 11,130 / 11,060; but 8.4 M, 32 workers 1038 / 1059, 4:
+// 166 / 178; 62 layers of 11.7 M, 32 workers 2779 / 2791.
+constexpr uint32_t fold_warps(uint32_t workers, uint64_t n, bool idle, bool alone) {
+  return alone || workers == 1 || (idle && workers >= 16 && n >= 1ull << 24) ? kFoldWarps : workers == 2 ? kWarps : kFoldWarpsBeside;
 }
-static_assert(fold_warps(32, true) == 10 && fold_warps(1, false) == 10 && fold_warps(2, false) == 8 && fold_warps(3, false) == 4, "");
+static_assert(fold_warps(32, 1000, true, true) == 10 && fold_warps(1, 1000, false, false) == 10, "alone");
+static_assert(fold_warps(2, 1ull << 25, true, false) == 8 && fold_warps(3, 1ull << 25, true, false) == 4, "a few in flight");
+static_assert(fold_warps(16, 1ull << 24, true, false) == 10 && fold_warps(16, 1ull << 24, false, false) == 4, "");
 
+// The launch itself, on a stream that task_begin has prepared with those dependencies; with SCAN the stream pass of a pull
+// in the same trip over D_q.
 template <bool SCAN>
 int fold_launch(dgs_ctx* c, const Workspace& ws, const SelArgs& a, uint32_t q, cudaStream_t st) {
   TimedLaunch tl(c, st, SCAN ? DGS_KERNEL_STREAM_PULL : DGS_KERNEL_CATCH_UP);
-  const uint32_t warps = fold_warps(c->cfg.num_workers, has_gpu(c));
+  const uint32_t warps = fold_warps(c->cfg.num_workers, c->cfg.n, c->idle_gpu, has_gpu(c));
   k_fold<SCAN><<<c->fold_grid, warps * 32, fold_dyn_bytes(warps, c->fold_ahead, ws.part_cap), st>>>(ws, a, c->log, fold_range(c, q));
   DGS_CUDA(c, cudaGetLastError());
   c->launches += 1;
