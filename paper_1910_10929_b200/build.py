@@ -10,7 +10,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libdgs.so")
 SOURCES = [os.path.join(CSRC, "dgs.cu"), os.path.join(CSRC, "dgs_one.cu")]
-DEPENDS = SOURCES + [os.path.join(CSRC, f) for f in ("dgs_apply.cuh", "dgs_kernels.cuh", "dgs_one.cuh", "dgs_topk.cuh")] + [os.path.join(ROOT, "include", "dgs.h")]
+DEPENDS = SOURCES + [os.path.join(CSRC, f) for f in ("dgs_apply.cuh", "dgs_arrivals.h", "dgs_kernels.cuh", "dgs_one.cuh", "dgs_topk.cuh")] + [os.path.join(ROOT, "include", "dgs.h")]
 
 NVCC_FLAGS = [
     "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",

@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "dgs_apply.cuh"
+#include "dgs_arrivals.h"
 #include "dgs_kernels.cuh"
 #include "dgs_one.cuh"
 #include "dgs_topk.cuh"
@@ -294,8 +295,7 @@ struct dgs_ctx {
   // No pull has been enqueued since the caller's stream was last made to wait for everything (dgs_flush, or a call
   // that waits): the event in hand starts on an idle GPU.
   bool idle_gpu;
-  bool lone;             // the last calls between two such joins held one pull
-  uint32_t pulls;        // since the last join
+  Arrivals arrivals;
   int hist_grid[3];      // CTAs of the whole-input histogram pass, per mode
   int one_max[3];        // most CTAs of pass and finalize in one kernel, per mode
   uint32_t pair[kSets];  // pair of sync words that the last selection on each scratch set has used
@@ -444,8 +444,7 @@ int fork_from_user(dgs_ctx* c, int which) {
 
 // Everything that was in flight is complete, or the caller's stream waits for it.
 void joined(dgs_ctx* c) {
-  if (c->pulls) c->lone = c->pulls == 1;
-  c->pulls = 0;
+  c->arrivals.joined();
   c->idle = c->idle_gpu = true;
 }
 // Whether the event in hand has the GPU to itself.  The one that opens a round of several does not: the others are enqueued
@@ -453,7 +452,7 @@ void joined(dgs_ctx* c) {
 // keeps them waiting.  What follows a join is taken to be as many events as between the last two.  (Rounds of 8 arrivals on
 // 124 M elements in 148 layers, us, every event after a join taken for alone / this: 3022 / 2877; of 32 on 11.7 M in 62 layers
 // 2870 / 2789; of 8 on 8.4 M in 2000 layers 1280 / 1115; one arrival at a time the same.)
-bool has_gpu(const dgs_ctx* c) { return c->idle_gpu && c->lone; }
+bool has_gpu(const dgs_ctx* c) { return c->idle_gpu && c->arrivals.lone(); }
 
 // Waits (on the host) for all internal streams ...
 int sync_library(dgs_ctx* c) {
@@ -613,19 +612,20 @@ uint32_t one_bytes(const dgs_ctx* c, int mode) {
 }
 
 // CTAs of finalize beside other kernels, of the `want` that keep the candidates in registers.  What its CTAs hold is taken from the
-// passes, which have the bytes to move, and with many workers a selection that takes longer only waits for its turn later: an
-// eighth, but not fewer than 48.  With few workers an event waits for the one before it, and there is not enough in flight to
-// fill the time: all of them up to three workers, 96 up to seven.  us, all (one per SM at most) / 96 / 48: 62 layers of 11.7 M, 32
-// arrivals of 1 worker 6090 / - / 9724, 2: 2637 / - / 2940, 3: 2443 / 2328 / 2495, 4: 2447 / 2346 / 2343, 6: 2485 / 2355 / 2330, 8:
-// 2524 / - / 2286, 32: 3045 / - / 2786; rounds of 3 arrivals 300 / 313 / 337, 4: 356 / 365 / 407, 6: 510 / 494 / 525, 8: 680 / - / 649;
-// 60 layers of 25 M, 1 %: 3: 484 / 508 / 570, 4: 604 / 618 / 683, 6: 913 / 899 / 929, 8: 1210 / - / 1217, 16: 2500 / - / 2380.
-constexpr uint64_t finalize_beside(uint32_t workers, uint64_t want) {
-  const uint64_t few = workers >= 8 ? 48 : 96, less = want / 8 > few ? want / 8 : few;
-  return workers <= 3 || want < less ? want : less;
+// passes, which have the bytes to move, and with many events side by side a selection that takes longer only waits for its turn
+// later: an eighth, but not fewer than 48, and not fewer than 96 with four to seven.  Where an event waits for the one before it,
+// all.  us, all (one per SM at most) / 96 / 48, 62 layers of 11.7 M: 32 arrivals in turn of 1 worker 6090 / - / 9724, 2: 2637 / - / 2940,
+// 4: 2447 / 2346 / 2343, 6: 2485 / 2355 / 2330, 8: 2524 / - / 2286, 32: 3045 / - / 2786; rounds of 4: 356 / 365 / 407, 6: 510 / 494 / 525,
+// 8: 680 / - / 649; workers drawn at random, rounds of 8: 1184 / 1253 / 1668, 32: 4970 / 4955 / 5535.  60 layers of 25 M, 1 %, rounds of 4:
+// 604 / 618 / 683, 6: 913 / 899 / 929, 8: 1210 / - / 1217, 16: 2500 / - / 2380; at random, 0.3 %, 8: 1520 / 1686 / 2071, 32: 6395 / 6540 / 7455.
+// One layer of 25 M, 0.1 %, at random, 8: 1190 / 1202 / 1381, 32: 4786 / 4831 / 5395.
+constexpr uint64_t finalize_beside(uint32_t abreast, uint64_t want) {
+  const uint64_t few = abreast >= 8 ? 48 : 96, less = want / 8 > few ? want / 8 : few;
+  return abreast < 4 || want < less ? want : less;
 }
-static_assert(finalize_beside(1, 204) == 204 && finalize_beside(3, 204) == 204, "a chain of events");
-static_assert(finalize_beside(4, 204) == 96 && finalize_beside(7, 60) == 60, "");
-static_assert(finalize_beside(8, 204) == 48 && finalize_beside(32, 800) == 100 && finalize_beside(32, 33) == 33, "");
+static_assert(finalize_beside(1, 204) == 204, "a chain of events");
+static_assert(finalize_beside(4, 204) == 96 && finalize_beside(4, 60) == 60, "");
+static_assert(finalize_beside(8, 204) == 48 && finalize_beside(8, 800) == 100 && finalize_beside(8, 33) == 33, "");
 
 template <int MODE>
 int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age, int stream_id, Task& task) {
@@ -657,7 +657,7 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
   const uint64_t cands = alone ? std::max<uint64_t>(3ull * a.pkt_count + 64ull * c->cfg.num_segments, c->whole_layers)
                                   : (uint64_t)a.pkt_count + a.pkt_count / 4 * 3 + 64ull * c->cfg.num_segments;
   uint64_t want = std::max<uint64_t>(kFinalizeMin, (cands + kThreads * keep - 1) / (kThreads * keep));
-  if (!alone) want = finalize_beside(c->cfg.num_workers, want);
+  if (!alone) want = finalize_beside(c->arrivals.abreast(), want);
   const uint64_t most = (uint64_t)(std::min(c->finalize_max[MODE], alone ? 2 * c->sms : c->sms) - (int)advisers);
   const int fin_grid = (int)std::min(most, want);
   // More candidates than the registers of all CTAs hold: k_finalize<.., BIG>, but beside other kernels only for one layer
@@ -891,8 +891,8 @@ int dgs_init(const dgs_config* cfg, dgs_ctx** out) {
   c->launches = 0;
   c->last_cuda = 0;
   c->broken = false;
-  c->idle_gpu = c->lone = true;
-  c->pulls = 0;
+  c->idle_gpu = true;
+  c->arrivals = Arrivals(cfg->num_workers);
   c->timing = false;
   for (int i = 0; i < DGS_NUM_KERNELS; ++i) {
     c->time_ms[i] = 0.0;
@@ -1044,6 +1044,7 @@ int push_impl(dgs_ctx* c, uint32_t worker, const float* grad, dgs_packet* out, i
   a.m = c->cfg.momentum;
   a.lr = c->cfg.lr;
   a.inv_m = c->inv_m;
+  c->arrivals.arrived(worker);
   Task task;
   task.writes = {R.U(worker), R.SPARE(stream_id), R.PKT(slot)};
   if (grad_is_stage) task.reads.push_back(R.STAGE());
@@ -1146,6 +1147,7 @@ int pull_impl(dgs_ctx* c, uint32_t worker, dgs_packet* out) {
   const Layout& L = c->lay;
   const ResIds R{c->cfg.num_workers};
   const int slot = kPushSlots + (int)(c->pull_count % kPullSlots);
+  if (c->worker_stream[worker] < 0) c->arrivals.arrived(worker);
   const int stream_id = c->worker_stream[worker] >= 0 ? c->worker_stream[worker] : take_stream(c);
   int rc = fork_from_user(c, stream_id);  // the caller may still be reading an older pull packet on its stream
   if (rc != DGS_OK) return rc;
@@ -1172,7 +1174,6 @@ int pull_impl(dgs_ctx* c, uint32_t worker, dgs_packet* out) {
   c->pull_count += 1;
   c->worker_stream[worker] = -1;
   c->idle_gpu = false;
-  c->pulls += 1;
   if (out) {
     out->idx = a.pkt_idx;
     out->val = a.pkt_val;
@@ -1187,6 +1188,7 @@ int pull_all_impl(dgs_ctx* c, uint32_t worker, dgs_var_packet* out) {
   const Layout& L = c->lay;
   const ResIds R{c->cfg.num_workers};
   const int vslot = (int)(c->var_count % kVarSlots);
+  if (c->worker_stream[worker] < 0) c->arrivals.arrived(worker);
   const int stream_id = c->worker_stream[worker] >= 0 ? c->worker_stream[worker] : take_stream(c);
   int rc = fork_from_user(c, stream_id);  // the caller may still be reading an older packet on its stream
   if (rc != DGS_OK) return rc;
@@ -1227,7 +1229,6 @@ int pull_all_impl(dgs_ctx* c, uint32_t worker, dgs_var_packet* out) {
   c->worker_stream[worker] = -1;
   c->var_count += 1;
   c->idle_gpu = false;
-  c->pulls += 1;
   if (out) {
     out->idx = vi;
     out->val = vv;
