@@ -537,7 +537,8 @@ FoldRange fold_range(const dgs_ctx* c, uint32_t q) {
 }
 // Warps of a CTA of the pass: ten where the pull has the GPU to itself, as with a single worker, whose pulls follow one another;
 // eight where one other pull may be in flight (a worker has one at a time), four beside more.  us, 16 arrivals, eight / ten: 1
-// worker, 8.4 M elements 3045 / 2976, 62 layers of 11.7 M 4774 / 4700; 2 workers 615 / 640, 1518 / 1536.  us an event in runs of
+// worker, 8.4 M elements 3045 / 2976, 62 layers of 11.7 M 4774 / 4700; 2 workers 615 / 640, 1518 / 1536; but rounds of 2 workers on
+// 19 M 173 / 174, on 50 M, where the passes are long beside everything else, 361 / 348.  us an event in runs of
 // 256, eight / four: 2 workers, 8.4 M: 36 / 40, 62 layers of 11.7 M: 95 / 101; 3 workers, 25.6 M: 66 / 63; 8 workers: 61 / 57, 62
 // layers of 11.7 M: 83 / 78.  (Vectors of 500 M elements with many entries, where an SM has room for one CTA of ten warps or two of
 // eight: pass of a pull alone 1308 / 1342.)
@@ -545,10 +546,11 @@ FoldRange fold_range(const dgs_ctx* c, uint32_t q) {
 // elements, 32 workers 2072 / 2057, 16: 1026 / 1028, 8: 531 / 536; 124 M, 32 workers 11,130 / 11,060; but 8.4 M, 32 workers 1038 / 1059, 4:
 // 166 / 178; 62 layers of 11.7 M, 32 workers 2779 / 2791.
 constexpr uint32_t fold_warps(uint32_t workers, uint64_t n, bool idle, bool alone) {
-  return alone || workers == 1 || (idle && workers >= 16 && n >= 1ull << 24) ? kFoldWarps : workers == 2 ? kWarps : kFoldWarpsBeside;
+  if (alone || workers == 1 || (workers == 2 && n >= 1ull << 25) || (idle && workers >= 16 && n >= 1ull << 24)) return kFoldWarps;
+  return workers == 2 ? kWarps : kFoldWarpsBeside;
 }
 static_assert(fold_warps(32, 1000, true, true) == 10 && fold_warps(1, 1000, false, false) == 10, "alone");
-static_assert(fold_warps(2, 1ull << 25, true, false) == 8 && fold_warps(3, 1ull << 25, true, false) == 4, "a few in flight");
+static_assert(fold_warps(2, 1ull << 24, true, false) == 8 && fold_warps(2, 1ull << 25, false, false) == 10 && fold_warps(3, 1ull << 25, true, false) == 4, "a few in flight");
 static_assert(fold_warps(16, 1ull << 24, true, false) == 10 && fold_warps(16, 1ull << 24, false, false) == 4, "");
 
 // The launch itself, on a stream that task_begin has prepared with those dependencies; with SCAN the stream pass of a pull
