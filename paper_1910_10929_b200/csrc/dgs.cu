@@ -651,12 +651,14 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
   // CTAs of finalize: as many as keep the candidates in the threads' registers, but not fewer than 32, since every step of a
   // warp is a chain, and no more than two per SM.  There are 2 to 4 times as many candidates as entries; where the kernel has
   // the GPU to itself it is sized for 3 (one arrival at a time on 25.6 M elements: 128.5 us sized for 1.75, 123 for 3; on 11.7 M
-  // in 62 layers its two finalize kernels take 28 and 31 us instead of 34 and 36).  A warp per two layers for the advice.
+  // in 62 layers its two finalize kernels take 28 and 31 us instead of 34 and 36), and where it opens a round whose events wait for one
+  // another (workers drawn at random, rounds of 4, us, without / with: 17 M elements 646 / 609, 60 layers of 25 M 1034 / 969; of 16: 2005 /
+  // 1961, 3198 / 3116).  A warp per two layers for the advice.
   const uint32_t advisers = std::min<uint32_t>(32u, (c->cfg.num_segments + 2 * kWarps - 1) / (2 * kWarps));
   const uint64_t keep = finalize_keep(c->cfg.num_segments > 1);
   // Layers that are small enough to be candidates as a whole (see next_bound) often are: 60 layers of 2^20 elements, alone, 18.3
   // and 20.8 us without them, 16.5 and 18.2 with.
-  const uint64_t cands = alone ? std::max<uint64_t>(3ull * a.pkt_count + 64ull * c->cfg.num_segments, c->whole_layers)
+  const uint64_t cands = alone || (c->idle_gpu && c->arrivals.chained()) ? std::max<uint64_t>(3ull * a.pkt_count + 64ull * c->cfg.num_segments, c->whole_layers)
                                   : (uint64_t)a.pkt_count + a.pkt_count / 4 * 3 + 64ull * c->cfg.num_segments;
   uint64_t want = std::max<uint64_t>(kFinalizeMin, (cands + kThreads * keep - 1) / (kThreads * keep));
   if (!alone) want = finalize_beside(c->arrivals.abreast(), want);

@@ -25,11 +25,13 @@ class Arrivals {
   }
   // Between the last two joins that had any there was one arrival.
   bool lone() const { return batch_ == 1; }
+  // Lately an event had to wait for one of the three before it.
+  bool chained() const { return count_ < near4_; }
   // How many events run side by side: 8 (or more), 4 to 7 (reported as 4), or fewer (1).  That many have to come between two joins,
   // and lately, for as long as every worker takes to come twice, none may have waited for one so few arrivals before it.
   uint32_t abreast() const {
     const uint64_t batch = std::max(batch_, count_ - joined_at_);
-    return batch >= 8 && count_ >= near8_ ? 8 : batch >= 5 && count_ >= near4_ ? 4 : 1;
+    return batch >= 8 && count_ >= near8_ ? 8 : batch >= 5 && !chained() ? 4 : 1;
   }
 
  private:
