@@ -255,7 +255,10 @@ enum {
 
 /* Measurement aid (no counterpart in the paper).  While on, every kernel launch of
  * this context is bracketed by two CUDA events on the stream it runs on (at most
- * 65536 launches between two reads are recorded). */
+ * 65536 launches between two reads are recorded).  A selection from a short vector that is one
+ * kernel otherwise runs as its two parts, DGS_KERNEL_STREAM_* and DGS_KERNEL_FINALIZE_*, while
+ * timing is on: the results are the same, but the times are of kernels that an untimed run does
+ * not launch. */
 int dgs_timing_enable(dgs_ctx* ctx, int on);
 
 /* Waits for all work in flight; ms[i] / count[i] receive the summed device time in

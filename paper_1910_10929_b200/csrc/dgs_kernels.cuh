@@ -86,7 +86,7 @@ struct Workspace {
   uint32_t num_blocks;    // blocks of kWarpTile elements (the last one may be partial)
   const uint32_t* blk_seg;   // [num_blocks] layer of the first element of each block
   // candidates: part p (CTA p of the grid that ran a push's stream pass, warp p of a pull's) owns the slots
-  // starting at the first element of its first tile
+  // starting at the first element of its first block (of its first tile, where a selection has started over)
   uint32_t* cand_idx;     // [n]
   float* cand_val;        // [n]
   uint32_t* part_cands;   // [kMaxParts] candidates written by each part
@@ -1266,8 +1266,9 @@ static __device__ __noinline__ uint32_t block_radix(const uint2* list, uint32_t 
 
 // 64 registers a thread: beside other kernels whatever the small ones hold is taken from the passes.  Runs without a join,
 // us an event with 64 / 72 / 80 / 96 / 128: 62 layers of 11.7 M elements, 32 workers: 94 / 94 / 98 / 107 / 114; one layer of
-// 25.6 M: 59.9 / 59.5 / 60.0 / 60.4 / 62.6.  Alone, 96 are 1 to 3 % faster.  (Shared memory is not what binds here: 13.3 KB
-// for a pull instead of 20.5 KB, with the parts numbered in groups of four, changed none of these by more than 0.5 %.)
+// 25.6 M: 59.9 / 59.5 / 60.0 / 60.4 / 62.6.  Alone, 96 are 1 to 3 % faster.  (Shared memory is not what binds here: with
+// eight warps a CTA in the pull's pass, 13.3 KB for a pull instead of 20.5 KB, with the parts numbered in groups of four, changed
+// none of these by more than 0.5 %; with the parts of ten it is 23.5 KB.)
 // BIG: for more candidates than the registers hold, where the kernel has the GPU to itself.  Such candidates are read again
 // in every phase, and a phase is a chain of trips to memory: four of them a lane are on their way instead of two, and a run
 // of candidates in one part needs neither a search nor a trip for its place.  Finalize of a pull, us, before / with BIG:
@@ -1925,7 +1926,7 @@ struct PacketLog {
 // Every D[i] sees the same subtractions in the same order as if the packets had been applied one by one, with one trip
 // to memory instead of one per packet.  Only 128-byte lines that hold an entry are written back.
 // Blocks are skipped when no packet has an entry in them and (SCAN) their bound lies below L.  The blocks of a CTA
-// that are left are dealt out to its warps in eight runs of about equal cost; a warp is a part of the candidate
+// that are left are dealt out to its warps in runs of about equal cost; a warp is a part of the candidate
 // buffer, so the candidates are in index order without any barrier between the warps.
 // What bounds it is the warps' instructions: about 300 for a block without entries, 600 with 20 of them, one after the other,
 // at half of the issue rate with 16 warps on an SM.  (More blocks of a warp on their way do not help: three or four instead
@@ -2210,7 +2211,9 @@ __device__ __forceinline__ void fold_blocks(const Workspace& ws, const SelArgs& 
         const uint32_t bound = __ldcg(a.blk_max + b);
         uint32_t s = S == 1 ? 0u : __ldg(ws.blk_seg + b);
         uint32_t L = a.L_in[s];
-        if (S > 1) {   // the lowest bound of the layers that have a part of the block (read in any case if there are many)
+        // The lowest bound of the layers that have a part of the block.  A block in five or more is always read: it holds three of
+        // them whole, and of every layer something is sent.
+        if (S > 1) {
           const uint64_t end = (uint64_t)(b + 1) * kWarpTile;
           for (int j = 0; j < 4 && L && s + 1 < S && __ldg(ws.seg_off + s + 1) < end; ++j) L = j < 3 ? min(L, a.L_in[++s]) : 0u;
         }
@@ -2247,7 +2250,7 @@ __device__ __forceinline__ void fold_blocks(const Workspace& ws, const SelArgs& 
     all = 0;
     for (uint32_t w = 0; w < nw; ++w) {
       if (w == (uint32_t)warp) at += all;
-      all += sh.warp_sum[w];                     // < 2^32 / 8: a share has fewer than 2^20 blocks
+      all += sh.warp_sum[w];                     // (a share has fewer than 2^20 blocks, and a block costs at most 255)
     }
     // first warp whose run begins in this thread's blocks or later: the smallest k with k all / nw >= at
     uint32_t k = sum ? (at * nw + all - 1) / all : nw;     // (below 2^32: nw <= 10, and a block costs at most 255)
