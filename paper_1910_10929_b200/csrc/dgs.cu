@@ -661,7 +661,7 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
   const uint64_t cands = alone || (c->idle_gpu && c->arrivals.chained()) ? std::max<uint64_t>(3ull * a.pkt_count + 64ull * c->cfg.num_segments, c->whole_layers)
                                   : (uint64_t)a.pkt_count + a.pkt_count / 4 * 3 + 64ull * c->cfg.num_segments;
   uint64_t want = std::max<uint64_t>(kFinalizeMin, (cands + kThreads * keep - 1) / (kThreads * keep));
-  if (!alone) want = finalize_beside(c->arrivals.abreast(), want);
+  if (!alone) want = finalize_beside(c->streams > 1 ? c->arrivals.abreast() : 1, want);
   const uint64_t most = (uint64_t)(std::min(c->finalize_max[MODE], alone ? 2 * c->sms : c->sms) - (int)advisers);
   const int fin_grid = (int)std::min(most, want);
   // More candidates than the registers of all CTAs hold: k_finalize<.., BIG>, but beside other kernels only for one layer
