@@ -658,17 +658,23 @@ int launch_select(dgs_ctx* c, const SelArgs& a_in, uint32_t worker, uint64_t age
   const uint64_t keep = finalize_keep(c->cfg.num_segments > 1);
   // Layers that are small enough to be candidates as a whole (see next_bound) often are: 60 layers of 2^20 elements, alone, 18.3
   // and 20.8 us without them, 16.5 and 18.2 with.
-  const uint64_t cands = alone || (c->idle_gpu && c->arrivals.chained()) ? std::max<uint64_t>(3ull * a.pkt_count + 64ull * c->cfg.num_segments, c->whole_layers)
+  const bool opens_chain = !alone && c->idle_gpu && c->arrivals.chained();
+  const uint64_t cands = alone || opens_chain ? std::max<uint64_t>(3ull * a.pkt_count + 64ull * c->cfg.num_segments, c->whole_layers)
                                   : (uint64_t)a.pkt_count + a.pkt_count / 4 * 3 + 64ull * c->cfg.num_segments;
   uint64_t want = std::max<uint64_t>(kFinalizeMin, (cands + kThreads * keep - 1) / (kThreads * keep));
   if (!alone) want = finalize_beside(c->streams > 1 ? c->arrivals.abreast() : 1, want);
-  const uint64_t most = (uint64_t)(std::min(c->finalize_max[MODE], alone ? 2 * c->sms : c->sms) - (int)advisers);
+  // Two CTAs an SM where it has the GPU to itself, as where it opens a chain of events of a single worker.  (Selections from 2^26
+  // elements, 10 %, by one worker, two between joins: the first on one CTA an SM 733 us, on two 530; but rounds of 4 at random,
+  // 8.4 M elements, 2 %: 506 / 560.)
+  const bool wide = alone || (opens_chain && c->cfg.num_workers == 1);
+  const uint64_t most = (uint64_t)(std::min(c->finalize_max[MODE], wide ? 2 * c->sms : c->sms) - (int)advisers);
   const int fin_grid = (int)std::min(most, want);
   // More candidates than the registers of all CTAs hold: k_finalize<.., BIG>, but beside other kernels only for one layer
   // and fifty times as many (runs of 32 events on 8.4 M elements, us an event without / with: one layer, 10 %, 20 times as
-  // many: 153 / 156; 50 %, 97 times: 823 / 733; 60 layers, 50 %: 750 / 818).
-  const uint64_t held = (alone ? (uint64_t)fin_grid : most) * kThreads * keep;
-  const bool big = alone ? cands > held : c->cfg.num_segments == 1 && cands > 50 * held;
+  // many: 153 / 156; 50 %, 97 times: 823 / 733; 60 layers, 50 %: 750 / 818), or where it opens a chain of events (rounds of 2 and 4 at
+  // random, 8.4 M elements, 10 %: 1027 / 930, 1360 / 1281).
+  const uint64_t held = (wide ? (uint64_t)fin_grid : most) * kThreads * keep;
+  const bool big = wide ? cands > held : c->cfg.num_segments == 1 && cands > (opens_chain ? held : 50 * held);
   a.workers = (uint32_t)fin_grid;
   a.advisers = advisers;
   a.fold_grid = MODE == kPull ? (uint32_t)c->fold_grid : 0u;   // one CTA more plans the next pull's pass
